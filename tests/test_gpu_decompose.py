@@ -114,3 +114,38 @@ def test_zero_matrix_and_errors(dv, ctx):
     assert e.value.code == dv.DVQLS_ERR_INVALID_ARG
     # the context stays usable after an error
     same(run_dense(dv, ctx, np.eye(8), 0.0, 8), odec.decompose(np.eye(8), 0.0, 8))
+
+
+@pytest.mark.parametrize("n,L_max", [(7, 100), (7, 2048), (8, 1), (4, 256)])
+@pytest.mark.parametrize("step", [0.0, 2.0 ** -40, 2.0 ** -20])
+def test_dense_selection_among_near_equal_keys(dv, ctx, n, L_max, step):
+    """One entry per X-mask: 4^n coefficients of (nearly) one magnitude, so the
+    cut falls among equal or almost equal keys and position decides."""
+    N = 1 << n
+    A = np.zeros((N, N))
+    A[:, 0] = 1.0 + step * np.arange(N)
+    same(run_dense(dv, ctx, A, 0.0, L_max), odec.decompose(A, 0.0, L_max))
+
+
+def test_banded_selection_among_equal_keys(dv, ctx):
+    """The same for states of more than 2^12 amplitudes: three masks with flat spectra."""
+    n = 13
+    bands = np.zeros((3, 1 << n))
+    bands[:, 0] = (1.0, -1.0, 1.0)
+    for L_max in (5, 2000):
+        same(run_banded(dv, ctx, n, [0, 1, 6], bands, 0.0, L_max), odec.decompose_banded(n, np.array([0, 1, 6]), bands, 0.0, L_max))
+
+
+@pytest.mark.parametrize("n", [6, 11])
+def test_outputs_off_their_natural_alignment(dv, ctx, n):
+    """A device buffer that is not aligned to its element is filled all the same."""
+    offsets, bands = wl.toeplitz_bands(n, [3.3, -0.9])
+    ref = odec.decompose_banded(n, offsets, bands, 0.0, 16)
+    raw = torch.zeros(16 * 16 + 4, device="cuda", dtype=torch.uint8)
+    xm = torch.zeros(16, device="cuda", dtype=torch.int32)
+    zm = np.zeros(16, np.uint32)
+    bv = torch.tensor(bands, device="cuda")
+    L, _, _ = dv.dvqls_pauli_decompose_banded(ctx, n, offsets, bv, 0.0, 16, raw[4:], xm, zm)
+    got = raw[4:].cpu().numpy().tobytes()
+    assert L == ref["L_out"] and np.array_equal(np.frombuffer(got, np.complex128)[:L], ref["coef"])
+    assert np.array_equal(xm.cpu().numpy()[:L].astype(np.uint32), ref["x"]) and np.array_equal(zm[:L], ref["z"])
