@@ -38,6 +38,29 @@ def test_forward_and_gradient_match_oracle(dv, ctx, I, H, O, B):
         dv.dvqls_ws_destroy(ws)
 
 
+# Tile edges of the 64 x 64 products and of the batch splits, device and host
+# arrays.  FP32 sums of at most 1,100 terms: 1,100 x 2^-24 = 7e-5 of the size of
+# the terms at worst, so 1e-4 of the largest entry.
+@pytest.mark.parametrize("I,H,O,B", [(1, 1, 1, 1), (64, 64, 64, 64), (5, 65, 63, 129), (7, 128, 65, 1100)])
+@pytest.mark.parametrize("device", [False, True])
+def test_gradient_at_tile_edges(dv, ctx, I, H, O, B, device):
+    import torch
+    p, X, T, M = random_net(I, H, O, B, I + H + O + B)
+    p *= np.float32(1.0 / np.sqrt(max(1, H / 32)))
+    M[0, 0] = 1.0
+    ws = dv.dvqls_ws_create(ctx, I, H, O, p)
+    try:
+        g = np.zeros(p.size, np.float32)
+        batch = [torch.from_numpy(a).cuda() for a in (X, T, M)] if device else (X, T, M)
+        loss = dv.dvqls_ws_grad(ws, B, *batch, g)
+        l_ref = omlp.loss(p.astype(np.float64), X, T, M, I, H, O)
+        g_ref = omlp.grad(p.astype(np.float64), X, T, M, I, H, O)
+        assert abs(loss - l_ref) <= 1e-4 * max(1.0, abs(l_ref))
+        assert np.abs(g - g_ref).max() <= 1e-4 * max(1.0, np.abs(g_ref).max())
+    finally:
+        dv.dvqls_ws_destroy(ws)
+
+
 def test_train_step_is_adam_on_the_gradient(dv, ctx):
     I, H, O, B = 7, 16, 9, 20
     p, X, T, M = random_net(I, H, O, B, 5)
