@@ -7,7 +7,8 @@
 //                       Pauli-string matvec, by conjugate gradients (A~
 //                       Hermitian positive definite), falling back to CG on
 //                       the normal equations A~^dag A~ x = A~^dag b when CG
-//                       breaks down; FP64, bounded iteration count.
+//                       breaks down; FP64, bounded iteration count.  The terms
+//                       of one X-mask act as one diagonal, formed once per call.
 //   dvqls_optimize      Adam on alpha with the batched cost and parameter-
 //                       shift gradient each iteration, many instances in
 //                       lock step; an instance stops when F >= target.
@@ -50,13 +51,14 @@ __device__ double2 block_sum2_all(double2 v, double2* red) {
     return s;
 }
 
+// One CTA per instance; the FP64 state build (build_state_f64) bounds it.
 __global__ void __launch_bounds__(FT) k_fidelity(const FidInst* __restrict__ insts, int* status) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ double2 red[FT / 32];
+    __shared__ double rnx[FT / 32];
     const FidInst I = insts[blockIdx.x];
     const int N = 1 << I.n;
-    double2* psi = reinterpret_cast<double2*>(smem);
-    double2* scs = psi + N;
+    double* psi = reinterpret_cast<double*>(smem);
     for (int a = threadIdx.x; a < I.P; a += FT) {
         const double al = I.alpha[a];
         if (!isfinite(al)) atomicCAS(status, 0, DEV_NONFINITE_INPUT);
@@ -65,16 +67,33 @@ __global__ void __launch_bounds__(FT) k_fidelity(const FidInst* __restrict__ ins
         I.cs[a] = make_double2(c, s);
     }
     __syncthreads();
-    build_state<double>(psi, scs, I.n, I.d, I.P, I.cs, 0);
+    build_state_f64(psi, I.n, I.d, I.P, I.cs, 0);
     double2 ov = make_double2(0.0, 0.0), nx = make_double2(0.0, 0.0);
     for (int j = threadIdx.x; j < N; j += FT) {
-        const double2 x = I.xhat[j], p = psi[j];
-        ov.x += x.x * p.x + x.y * p.y;  // conj(x) p
-        ov.y += x.x * p.y - x.y * p.x;
+        const double2 x = I.xhat[j];
+        const double p = psi[f64_pad(j)];  // the state is real
+        ov.x += x.x * p;  // conj(x) p
+        ov.y -= x.y * p;
         nx.x += x.x * x.x + x.y * x.y;
     }
-    ov = block_sum2_all(ov, red);
-    nx = block_sum2_all(nx, red);
+    for (int o = 16; o; o >>= 1) {
+        ov.x += __shfl_xor_sync(0xffffffffu, ov.x, o);
+        ov.y += __shfl_xor_sync(0xffffffffu, ov.y, o);
+        nx.x += __shfl_xor_sync(0xffffffffu, nx.x, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        red[threadIdx.x >> 5] = ov;
+        rnx[threadIdx.x >> 5] = nx.x;
+    }
+    __syncthreads();
+    if (threadIdx.x >= 8) return;
+    ov = red[threadIdx.x];
+    nx.x = rnx[threadIdx.x];
+    for (int o = 4; o; o >>= 1) {
+        ov.x += __shfl_xor_sync(0xffu, ov.x, o);
+        ov.y += __shfl_xor_sync(0xffu, ov.y, o);
+        nx.x += __shfl_xor_sync(0xffu, nx.x, o);
+    }
     if (threadIdx.x == 0) {
         if (!(nx.x > 0.0) || !isfinite(nx.x)) atomicCAS(status, 0, DEV_BAD_NORM);
         *I.F = (ov.x * ov.x + ov.y * ov.y) / nx.x;
@@ -120,12 +139,18 @@ __device__ double2 dotc(int N, const double2* a, const double2* b, double2* red)
     return block_sum2_all(s, red);
 }
 
-// Single CTA conjugate gradients; vectors in global memory (L2-resident).
+struct LcuGroups;
+__device__ bool grouped(const LcuGroups* g);  // the X-mask diagonals were formed
+
+// Single CTA conjugate gradients term by term, for LCUs whose diagonals are not
+// formed (too many masks or terms, or N above CGR_MAXN); vectors in global
+// memory (L2-resident).
 // out: [0] iterations, [1] relative residual, [2] 1 if converged, [3] 1 if
 // the normal equations were used.
 __global__ void __launch_bounds__(CGT) k_cg(int n, int L, const double2* coef, const uint32_t* xm, const uint32_t* zm,
                                            const double2* b, double2* x, double2* r, double2* p, double2* Ap,
-                                           double2* tmp, double tol, int max_iter, double* out) {
+                                           double2* tmp, double tol, int max_iter, double* out, const LcuGroups* g) {
+    if (grouped(g)) return;  // k_cg_diag has solved it
     __shared__ double2 red[CGT / 32];
     const int N = 1 << n;
     {  // one CTA per right-hand side: vectors of N entries each, four result words
@@ -202,6 +227,285 @@ __global__ void __launch_bounds__(CGT) k_cg(int n, int L, const double2* coef, c
     }
 }
 
+// ------------------------------------------- CG on X-mask diagonals
+// Terms with the same X-mask x act together as one diagonal: A~ v [j] = sum_x
+// d_x[j] v[j ^ x] with d_x[j] = sum of c_l i^popc(x & z_l) (-1)^popc(z_l & (j ^ x))
+// over the terms of x.  The diagonals are formed once per call, so a matvec
+// costs one multiply-add per amplitude and distinct mask instead of one per
+// term (7 against 64 for the top terms of a tridiagonal matrix), and only its
+// real half when every diagonal and the right-hand side are real.  FP64 bounds
+// these solves: its instructions issue at 1/64 of the FP32 rate.
+constexpr int GRP_MAXL = 2048;  // terms the grouping kernel takes
+constexpr int GRP_MAXX = 64;    // distinct masks the solver takes; more: term by term
+constexpr int CGR_T = 256;
+constexpr int CGR_MAXN = 4096;  // amplitudes (16 per thread)
+
+struct LcuGroups {
+    int nx;   // distinct X-masks (above GRP_MAXX: the diagonals are not formed)
+    int im;   // some diagonal has an imaginary part
+    int off[GRP_MAXX + 1];
+    uint32_t x[GRP_MAXX];
+};
+
+__device__ bool grouped(const LcuGroups* g) { return g && g->nx <= GRP_MAXX; }
+
+// One CTA: the terms of each distinct mask, masks in order of first
+// appearance, the terms of a mask in their order (list).
+__global__ void __launch_bounds__(1024) k_lcu_group(int n, int L, const uint32_t* __restrict__ xm, LcuGroups* g, int* list) {
+    __shared__ uint32_t sx[GRP_MAXL];
+    __shared__ unsigned short first[GRP_MAXL], count[GRP_MAXL];  // first term of the mask; its terms (at the first)
+    __shared__ int nx;
+    const uint32_t mask = (1u << n) - 1u;
+    if (threadIdx.x == 0) nx = 0;
+    for (int l = threadIdx.x; l < L; l += 1024) sx[l] = xm[l] & mask;
+    __syncthreads();
+    for (int l = threadIdx.x; l < L; l += 1024) {
+        int f = l, c = 0;
+        for (int k = L - 1; k >= 0; --k)
+            if (sx[k] == sx[l]) {
+                f = k;
+                ++c;
+            }
+        first[l] = (unsigned short)f;
+        count[l] = (unsigned short)c;
+        if (f == l) atomicAdd(&nx, 1);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        g->nx = nx;
+        g->im = 0;
+    }
+    if (nx > GRP_MAXX) return;
+    if (threadIdx.x == 0) g->off[nx] = L;
+    for (int l = threadIdx.x; l < L; l += 1024) {
+        int at = 0, rank = 0, grp = 0;
+        for (int k = 0; k < L; ++k) {
+            if (first[k] == k && k < first[l]) {
+                at += count[k];
+                ++grp;
+            }
+            if (k < l && first[k] == first[l]) ++rank;
+        }
+        list[at + rank] = l;
+        if (first[l] == l) {
+            g->off[grp] = at;
+            g->x[grp] = sx[l];
+        }
+    }
+}
+
+// Diagonal blockIdx.y: real parts at re[y N + j], imaginary parts at im[y N + j].
+__global__ void __launch_bounds__(256) k_lcu_diag(int n, const double2* __restrict__ coef, const uint32_t* __restrict__ zm,
+                                                  LcuGroups* g, const int* __restrict__ list, double* re, double* im) {
+    const int y = blockIdx.y, N = 1 << n, j = blockIdx.x * 256 + threadIdx.x;
+    if (g->nx > GRP_MAXX || y >= g->nx) return;
+    const uint32_t x = g->x[y], src = uint32_t(j) ^ x;
+    double dr = 0.0, di = 0.0;
+    for (int k = g->off[y]; k < g->off[y + 1]; ++k) {
+        const int l = list[k];
+        const uint32_t z = zm[l] & uint32_t(N - 1);
+        const double2 c = coef[l];
+        double cr, ci;  // c_l i^popc(x & z)
+        switch (__popc(x & z) & 3) {
+            case 0: cr = c.x; ci = c.y; break;
+            case 1: cr = -c.y; ci = c.x; break;
+            case 2: cr = -c.x; ci = -c.y; break;
+            default: cr = c.y; ci = -c.x; break;
+        }
+        const bool neg = __popc(z & src) & 1;
+        dr += neg ? -cr : cr;
+        if (ci != 0.0) di += neg ? -ci : ci;
+    }
+    if (j >= N) return;
+    re[(size_t)y * N + j] = dr;
+    im[(size_t)y * N + j] = di;
+    if (di != 0.0) g->im = 1;
+}
+
+// Sum over the CTA in every thread; red alternates between two rows so that
+// one barrier is enough.  The FP64 adds of a full tree in each thread would
+// cost more than a matvec.
+__device__ __forceinline__ double cgr_sum(double v, double (*red)[CGR_T / 32], int& turn) {
+    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) red[turn][threadIdx.x >> 5] = v;
+    __syncthreads();
+    double s = red[turn][threadIdx.x & 7];
+    for (int o = 4; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    turn ^= 1;
+    return s;
+}
+
+// The CG of one right-hand side by one CTA, EPT amplitudes per thread (j = t +
+// 256 e): x and r in registers, p (and the normal equations' A~ p) in shared
+// memory, the diagonals from L1 / L2.  Same steps, breakdown test and result
+// words as k_cg.
+template <int EPT, bool CPLX>
+__device__ void cgr_solve(int n, const LcuGroups& G, const double* __restrict__ re, const double* __restrict__ im,
+                          const double2* b, double2* xo, double* sp, double tol, int max_iter, double* out) {
+    constexpr int C = CPLX ? 2 : 1;  // real planes per vector
+    __shared__ double red[2][CGR_T / 32];
+    __shared__ double sc[3];  // step alpha, beta, relative residual
+    const int N = 1 << n, t = threadIdx.x, nx = G.nx;
+    int turn = 0;
+    double* st = sp + C * N;
+    auto live = [&](int e) { return t + CGR_T * e < N; };
+    // y = A~ src (adj: A~^dag src), src in shared memory
+    auto matvec = [&](const double* src, bool adj, double (&yr)[EPT], double (&yi)[EPT]) {
+#pragma unroll
+        for (int e = 0; e < EPT; ++e) yr[e] = yi[e] = 0.0;
+        for (int g = 0; g < nx; ++g) {
+            const int x = int(G.x[g]);
+            const double* dr = re + (size_t)g * N;
+            const double* di = im + (size_t)g * N;
+#pragma unroll
+            for (int e = 0; e < EPT; ++e) {
+                const int j = t + CGR_T * e;
+                if (j >= N) break;
+                const int s = j ^ x, k = adj ? s : j;  // (A~^dag)[j, s] = conj(A~[s, j]), the diagonal's entry s
+                const double a = src[s], d = dr[k];
+                yr[e] = fma(d, a, yr[e]);
+                if (CPLX) {
+                    const double ai = src[N + s], ei = adj ? -di[k] : di[k];
+                    yr[e] = fma(-ei, ai, yr[e]);
+                    yi[e] = fma(d, ai, yi[e]);
+                    yi[e] = fma(ei, a, yi[e]);
+                }
+            }
+        }
+    };
+    double xr[EPT], xi[EPT], rr_[EPT], ri[EPT], qr[EPT], qi[EPT];
+    for (int normal = 0; normal < 2; ++normal) {
+#pragma unroll
+        for (int e = 0; e < EPT; ++e) {
+            const double2 v = live(e) ? b[t + CGR_T * e] : make_double2(0.0, 0.0);
+            rr_[e] = v.x;
+            ri[e] = v.y;
+            xr[e] = xi[e] = 0.0;
+        }
+        auto put = [&](double* dst, const double (&vr)[EPT], const double (&vi)[EPT]) {
+#pragma unroll
+            for (int e = 0; e < EPT; ++e)
+                if (live(e)) {
+                    dst[t + CGR_T * e] = vr[e];
+                    if (CPLX) dst[N + t + CGR_T * e] = vi[e];
+                }
+        };
+        if (normal) {  // the right-hand side A~^dag b
+            put(sp, rr_, ri);
+            __syncthreads();
+            matvec(sp, true, rr_, ri);
+            __syncthreads();
+        }
+        put(sp, rr_, ri);
+        double acc = 0.0;
+#pragma unroll
+        for (int e = 0; e < EPT; ++e) {
+            acc = fma(rr_[e], rr_[e], acc);
+            if (CPLX) acc = fma(ri[e], ri[e], acc);
+        }
+        double rr = cgr_sum(acc, red, turn);  // its barrier also publishes p
+        const double rhs = sqrt(rr);
+        bool broke = false;
+        int it = 0;
+        double rel = rhs > 0.0 ? 1.0 : 0.0;
+        while (it < max_iter && rel > tol) {
+            double dot = 0.0;
+            if (normal) {
+                matvec(sp, false, qr, qi);
+                put(st, qr, qi);
+                __syncthreads();
+                matvec(st, true, qr, qi);
+            } else {
+                matvec(sp, false, qr, qi);
+            }
+#pragma unroll
+            for (int e = 0; e < EPT; ++e)
+                if (live(e)) {
+                    dot = fma(sp[t + CGR_T * e], qr[e], dot);
+                    if (CPLX) dot = fma(sp[N + t + CGR_T * e], qi[e], dot);
+                }
+            const double pAp = cgr_sum(dot, red, turn);
+            if (!(pAp > 0.0)) {
+                broke = true;
+                break;
+            }
+            if (t < 32) sc[0] = rr / pAp;  // a division in every warp would cost as much as a dot product
+            __syncthreads();
+            const double a = sc[0];
+            acc = 0.0;
+#pragma unroll
+            for (int e = 0; e < EPT; ++e)
+                if (live(e)) {
+                    xr[e] = fma(a, sp[t + CGR_T * e], xr[e]);
+                    rr_[e] = fma(-a, qr[e], rr_[e]);
+                    acc = fma(rr_[e], rr_[e], acc);
+                    if (CPLX) {
+                        xi[e] = fma(a, sp[N + t + CGR_T * e], xi[e]);
+                        ri[e] = fma(-a, qi[e], ri[e]);
+                        acc = fma(ri[e], ri[e], acc);
+                    }
+                }
+            const double rr2 = cgr_sum(acc, red, turn);
+            if (t < 32) sc[1] = rr2 / rr;
+            else if (t < 64) sc[2] = rhs > 0.0 ? sqrt(rr2) / rhs : 0.0;
+            __syncthreads();
+            const double bet = sc[1];
+            rel = sc[2];
+            rr = rr2;
+#pragma unroll
+            for (int e = 0; e < EPT; ++e)
+                if (live(e)) {
+                    sp[t + CGR_T * e] = fma(bet, sp[t + CGR_T * e], rr_[e]);
+                    if (CPLX) sp[N + t + CGR_T * e] = fma(bet, sp[N + t + CGR_T * e], ri[e]);
+                }
+            __syncthreads();
+            ++it;
+        }
+        if (!broke) {
+#pragma unroll
+            for (int e = 0; e < EPT; ++e)
+                if (live(e)) xo[t + CGR_T * e] = make_double2(xr[e], xi[e]);
+            if (t == 0) {
+                out[0] = it;
+                out[1] = rel;
+                out[2] = rel <= tol ? 1.0 : 0.0;
+                out[3] = normal;
+            }
+            return;
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int e = 0; e < EPT; ++e)
+        if (live(e)) xo[t + CGR_T * e] = make_double2(xr[e], xi[e]);
+    if (t == 0) {
+        out[0] = max_iter;
+        out[1] = INFINITY;
+        out[2] = 0.0;
+        out[3] = 1.0;
+    }
+}
+
+template <int EPT>
+__global__ void __launch_bounds__(CGR_T) k_cg_diag(int n, const LcuGroups* __restrict__ g, const double* __restrict__ re,
+                                                   const double* __restrict__ im, const double2* b, double2* x, double tol,
+                                                   int max_iter, double* out) {
+    extern __shared__ __align__(16) unsigned char cgr_smem[];
+    __shared__ LcuGroups G;
+    const int N = 1 << n;
+    if (g->nx > GRP_MAXX) return;  // k_cg solves it term by term
+    for (int k = threadIdx.x; k < int(sizeof G / 4); k += CGR_T)
+        reinterpret_cast<int*>(&G)[k] = reinterpret_cast<const int*>(g)[k];
+    b += (size_t)blockIdx.x * N;
+    x += (size_t)blockIdx.x * N;
+    out += 4 * blockIdx.x;
+    bool cplx = false;
+    for (int j = threadIdx.x; j < N; j += CGR_T) cplx |= b[j].y != 0.0;
+    double* sp = reinterpret_cast<double*>(cgr_smem);
+    if (__syncthreads_or(cplx) || G.im) cgr_solve<EPT, true>(n, G, re, im, b, x, sp, tol, max_iter, out);
+    else cgr_solve<EPT, false>(n, G, re, im, b, x, sp, tol, max_iter, out);
+}
+
 // One Adam update of the active angles: element i is angle gmap[i], whose
 // instance has the bias corrections c1[i] = 1 - beta1^t and c2[i] = 1 - beta2^t.
 __global__ void k_adam(int count, const int* __restrict__ gmap, const double* __restrict__ g, double* alpha,
@@ -268,7 +572,7 @@ extern "C" int dvqls_fidelity(dvqls_ctx* ctx, const dvqls_ansatz* an, const doub
     I.F = (double*)(ctx->ws + o_F);
     memcpy(ctx->pin + p_t, &I, sizeof I);
     DVQLS_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->ws + o_t, ctx->pin + p_t, sizeof I, cudaMemcpyHostToDevice, ctx->stream));
-    const size_t smem = size_t(N + P) * 16;
+    const size_t smem = f64_state_doubles(n, P) * 8;
     DVQLS_CUDA_TRY(ctx, allow_dynamic_smem((const void*)k_fidelity));
     k_fidelity<<<1, FT, smem, ctx->stream>>>((const FidInst*)(ctx->ws + o_t), ctx->d_status);
     DVQLS_CUDA_TRY(ctx, cudaGetLastError());
@@ -509,6 +813,10 @@ extern "C" int dvqls_lcu_solve_batched(dvqls_ctx* ctx, int n, const dvqls_lcu* l
     const bool multi = nrhs == 1 && N >= CGM_MIN_N;  // one large system: the grid-wide CG
     const int G = multi ? (int)std::min<long long>(N / CGM_T, (long long)ctx->num_sms * 8) : 0;
     const size_t o_sc = ar.reserve(64), o_part = ar.reserve(size_t(std::max(G, 1)) * 8);
+    const bool diag = !multi && N <= CGR_MAXN && L <= GRP_MAXL;
+    const size_t planes = diag ? size_t(std::min<long long>(std::min(L, GRP_MAXX), N)) * size_t(N) * 8 : 0;
+    const size_t o_grp = ar.reserve(sizeof(LcuGroups)), o_list = ar.reserve(size_t(diag ? L : 1) * 4);
+    const size_t o_re = ar.reserve(planes), o_im = ar.reserve(planes);
     int rc = ensure_workspace(ctx, ar.total());
     if (!rc) rc = ensure_pinned(ctx, pin.total());
     if (!rc) rc = pin_acquire(ctx);
@@ -525,9 +833,30 @@ extern "C" int dvqls_lcu_solve_batched(dvqls_ctx* ctx, int n, const dvqls_lcu* l
                       (double*)(ws + o_part), G);
         if (rc) return rc;
     } else {
-        k_cg<<<nrhs, CGT, 0, ctx->stream>>>(n, L, coef, xm, zm, bd, (double2*)(ws + o_x), (double2*)(ws + o_r),
-                                            (double2*)(ws + o_p), (double2*)(ws + o_ap), (double2*)(ws + o_tmp), tol,
-                                            max_iter, out);
+        LcuGroups* grp = diag ? (LcuGroups*)(ws + o_grp) : nullptr;
+        if (diag) {
+            const int* list = (const int*)(ws + o_list);
+            double *re = (double*)(ws + o_re), *im = (double*)(ws + o_im);
+            double2* xd = (double2*)(ws + o_x);
+            k_lcu_group<<<1, 1024, 0, ctx->stream>>>(n, L, xm, grp, (int*)(ws + o_list));
+            k_lcu_diag<<<dim3(ceil_div(N, 256), (unsigned)(planes / (size_t(N) * 8))), 256, 0, ctx->stream>>>(
+                n, coef, zm, grp, list, re, im);
+            auto solve = [&](auto kern) -> cudaError_t {
+                const cudaError_t e = allow_dynamic_smem((const void*)kern);
+                if (e != cudaSuccess) return e;
+                kern<<<nrhs, CGR_T, size_t(N) * 32, ctx->stream>>>(n, grp, re, im, bd, xd, tol, max_iter, out);
+                return cudaGetLastError();
+            };
+            DVQLS_CUDA_TRY(ctx, n <= 8    ? solve(k_cg_diag<1>)
+                                : n == 9  ? solve(k_cg_diag<2>)
+                                : n == 10 ? solve(k_cg_diag<4>)
+                                : n == 11 ? solve(k_cg_diag<8>)
+                                          : solve(k_cg_diag<16>));
+        }
+        if (!diag || L > GRP_MAXX)  // at most GRP_MAXX terms have at most as many masks
+            k_cg<<<nrhs, CGT, 0, ctx->stream>>>(n, L, coef, xm, zm, bd, (double2*)(ws + o_x), (double2*)(ws + o_r),
+                                                (double2*)(ws + o_p), (double2*)(ws + o_ap), (double2*)(ws + o_tmp), tol,
+                                                max_iter, out, grp);
     }
     DVQLS_CUDA_TRY(ctx, cudaGetLastError());
     rc = pin_release(ctx);
@@ -574,7 +903,6 @@ static int optimize(dvqls_ctx* ctx, int count, const dvqls_instance* inst, const
     cudaSetDevice(ctx->device);
     std::vector<int> P(count), N(count), L(count);
     std::vector<long long> aoff(count + 1, 0), xoff(count + 1, 0), loff(count + 1, 0), boff(count + 1, 0);
-    int nmax = 1;
     for (int i = 0; i < count; ++i) {
         const dvqls_instance& q = inst[i];
         if (q.ansatz.n < 1 || q.ansatz.n > DVQLS_MAX_SMEM_QUBITS || q.ansatz.depth < 0 || q.lcu.L < 1 || !q.alpha ||
@@ -583,7 +911,6 @@ static int optimize(dvqls_ctx* ctx, int count, const dvqls_instance* inst, const
         P[i] = q.ansatz.n * (q.ansatz.depth + 1);
         N[i] = 1 << q.ansatz.n;
         L[i] = q.lcu.L;
-        nmax = std::max(nmax, q.ansatz.n);
         aoff[i + 1] = aoff[i] + P[i];
         xoff[i + 1] = xoff[i] + N[i];
         loff[i + 1] = loff[i] + L[i];
@@ -670,7 +997,8 @@ static int optimize(dvqls_ctx* ctx, int count, const dvqls_instance* inst, const
         results[i].cost = NAN;
         results[i].fidelity = NAN;
     }
-    const size_t fsmem = (size_t(1) << nmax) * 16 + size_t(*std::max_element(P.begin(), P.end())) * 16;
+    size_t fsmem = 0;
+    for (int i = 0; i < count; ++i) fsmem = std::max(fsmem, f64_state_doubles(inst[i].ansatz.n, P[i]) * 8);
     DVQLS_CUDA_TRY(ctx, allow_dynamic_smem((const void*)k_fidelity));
     std::vector<int> active(count);
     for (int i = 0; i < count; ++i) active[i] = i;

@@ -22,24 +22,17 @@ struct V2<double> {
     using t = double2;
 };
 
-template <typename R2>
-__device__ __forceinline__ R2 neg2(R2 v) {
-    v.x = -v.x;
-    v.y = -v.y;
-    return v;
-}
-
 __device__ __forceinline__ int czring_parity(int i, int n) {
     int p = __popc(i & (i >> 1) & ((1 << (n - 1)) - 1));
     if (n >= 3) p += (i >> (n - 1)) & i & 1;
     return p & 1;
 }
 
-// psi = V(alpha_s)|0> in shared memory, all threads of the CTA (blockDim.x
-// of them) taking part; ends with a barrier.  cs holds (cos, sin) of the half
-// angles: [0, P) at alpha, [P, 2P) at alpha + pi/2, [2P, 3P) at alpha - pi/2;
-// shift s selects alpha (s = 0), alpha + pi/2 e_k (s = 2k+1) or
-// alpha - pi/2 e_k (s = 2k+2).  scs receives the P (cos, sin) pairs used.
+// The state builders below form psi = V(alpha_s)|0> and end with a barrier.  cs
+// holds (cos, sin) of the half angles: [0, P) at alpha, [P, 2P) at alpha + pi/2,
+// [2P, 3P) at alpha - pi/2; shift s selects alpha (s = 0), alpha + pi/2 e_k
+// (s = 2k+1) or alpha - pi/2 e_k (s = 2k+2).  scs receives the P (cos, sin) pairs
+// used.
 // Barrier over the threads that build a state: the whole block (bar = 0) or
 // the NTH threads that share named barrier `bar`.
 __device__ __forceinline__ void group_sync(int bar, int NTH) {
@@ -47,101 +40,11 @@ __device__ __forceinline__ void group_sync(int bar, int NTH) {
     else asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(NTH) : "memory");
 }
 
-// Builds shifted state s with threads t = 0 .. NTH-1 of a group.
-template <typename R>
-__device__ void build_state_group(typename V2<R>::t* psi, typename V2<R>::t* scs, int n, int d, int P,
-                                  const double2* cs, int s, int t, int NTH, int bar) {
-    using R2 = typename V2<R>::t;
-    const int N = 1 << n;
-    int k = -1, which = 0;
-    if (s > 0) {
-        k = (s - 1) >> 1;
-        which = ((s - 1) & 1) ? 2 : 1;
-    }
-    for (int a = t; a < P; a += NTH) {
-        const double2 v = cs[(a == k ? which : 0) * P + a];
-        R2 r;
-        r.x = (R)v.x;
-        r.y = (R)v.y;
-        scs[a] = r;
-    }
-    group_sync(bar, NTH);
-    for (int i = t; i < N; i += NTH) {  // initial Ry layer on |0>: a product state
-        R v = (R)1;
-        for (int q = 0; q < n; ++q) v *= ((i >> q) & 1) ? scs[q].y : scs[q].x;
-        R2 r;
-        r.x = v;
-        r.y = (R)0;
-        psi[i] = r;
-    }
-    group_sync(bar, NTH);
-    // Layers: the CZ ring (diagonal) is applied while loading the first pass;
-    // the Ry rotations of qubits q and q+1 are fused into one pass over groups
-    // of four amplitudes (bits q, q+1 = 00, 01, 10, 11), so a layer takes
-    // ceil(n/2) passes and barriers.
-    for (int layer = 1; layer <= d; ++layer) {
-        for (int q = 0; q < n; q += 2) {
-            const R c0 = scs[layer * n + q].x, s0 = scs[layer * n + q].y;
-            if (q + 1 < n) {
-                const R c1 = scs[layer * n + q + 1].x, s1 = scs[layer * n + q + 1].y;
-                for (int p = t; p < N / 4; p += NTH) {
-                    const int i00 = ((p >> q) << (q + 2)) | (p & ((1 << q) - 1));
-                    const int i01 = i00 | (1 << q), i10 = i00 | (2 << q), i11 = i00 | (3 << q);
-                    R2 a = psi[i00], b = psi[i01], c = psi[i10], e = psi[i11];
-                    if (q == 0) {
-                        if (czring_parity(i00, n)) a = neg2(a);
-                        if (czring_parity(i01, n)) b = neg2(b);
-                        if (czring_parity(i10, n)) c = neg2(c);
-                        if (czring_parity(i11, n)) e = neg2(e);
-                    }
-                    R2 a1, b1, c1r, e1;  // Ry on qubit q: pairs (a, b) and (c, e)
-                    a1.x = c0 * a.x - s0 * b.x;
-                    a1.y = c0 * a.y - s0 * b.y;
-                    b1.x = s0 * a.x + c0 * b.x;
-                    b1.y = s0 * a.y + c0 * b.y;
-                    c1r.x = c0 * c.x - s0 * e.x;
-                    c1r.y = c0 * c.y - s0 * e.y;
-                    e1.x = s0 * c.x + c0 * e.x;
-                    e1.y = s0 * c.y + c0 * e.y;
-                    R2 u;  // Ry on qubit q+1: pairs (a1, c1r) and (b1, e1)
-                    u.x = c1 * a1.x - s1 * c1r.x;
-                    u.y = c1 * a1.y - s1 * c1r.y;
-                    psi[i00] = u;
-                    u.x = s1 * a1.x + c1 * c1r.x;
-                    u.y = s1 * a1.y + c1 * c1r.y;
-                    psi[i10] = u;
-                    u.x = c1 * b1.x - s1 * e1.x;
-                    u.y = c1 * b1.y - s1 * e1.y;
-                    psi[i01] = u;
-                    u.x = s1 * b1.x + c1 * e1.x;
-                    u.y = s1 * b1.y + c1 * e1.y;
-                    psi[i11] = u;
-                }
-            } else {
-                for (int p = t; p < N / 2; p += NTH) {
-                    const int i0 = ((p >> q) << (q + 1)) | (p & ((1 << q) - 1)), i1 = i0 | (1 << q);
-                    R2 a = psi[i0], b = psi[i1];
-                    if (q == 0) {
-                        if (czring_parity(i0, n)) a = neg2(a);
-                        if (czring_parity(i1, n)) b = neg2(b);
-                    }
-                    R2 u, v;
-                    u.x = c0 * a.x - s0 * b.x;
-                    u.y = c0 * a.y - s0 * b.y;
-                    v.x = s0 * a.x + c0 * b.x;
-                    v.y = s0 * a.y + c0 * b.y;
-                    psi[i0] = u;
-                    psi[i1] = v;
-                }
-            }
-            group_sync(bar, NTH);
-        }
-    }
-}
-
-// The same state with real amplitudes (every gate of the ansatz is real),
-// multiplied by `scale`, in precision R: psi[0 .. 2^n), scs[0 .. P) as
-// (cos, sin).
+// Shifted state s in precision R, real (every gate of the ansatz is), multiplied
+// by `scale`, by threads t = 0 .. NTH-1 of a group: psi[0 .. 2^n), scs[0 .. P) as
+// (cos, sin).  The CZ ring (diagonal) is applied while loading a layer's first
+// pass; the Ry rotations of qubits q and q+1 are fused into one pass over groups
+// of four amplitudes, so a layer takes ceil(n/2) passes and barriers.
 template <typename R>
 __device__ inline void build_state_real(R* psi, typename V2<R>::t* scs, int n, int d, int P, const double2* cs, int s,
                                         int t, int NTH, int bar, R scale) {
@@ -449,10 +352,128 @@ __device__ inline void build_state_regs(void* psi, float* scratch, float2* scs, 
     group_sync(bar, 256);
 }
 
-template <typename R>
-__device__ void build_state(typename V2<R>::t* psi, typename V2<R>::t* scs, int n, int d, int P,
-                            const double2* cs, int s) {
-    build_state_group<R>(psi, scs, n, d, P, cs, s, threadIdx.x, blockDim.x, 0);
+// ---- FP64 state in shared memory for 256 threads, n <= 12.
+//
+// FP64 instructions bound it (they issue at 1/64 of the FP32 rate), so the Ry
+// rotations run in the scaled form of ry_scaled (one FMA per amplitude instead
+// of two instructions), NB qubits per pass over 2^NB amplitudes in registers,
+// with one multiply per amplitude and layer for the product of the layer's
+// factors, and the initial product state comes from two factor tables.
+// Amplitude i sits at word i + (i >> 4).
+__host__ __device__ inline int f64_pad(int i) { return i + (i >> 4); }
+// Doubles: psi, the rotations, a factor per layer, the two factor tables.
+__host__ __device__ inline size_t f64_state_doubles(int n, int P) {
+    const size_t N = size_t(1) << n;
+    return N + (N >> 4) + P + (P / n - 1) + (N < 32 ? N : 32) + (N < 32 ? 1 : N >> 5);
+}
+
+// Scaled rotation of (c, s): |r| <= 1 leaves bit 62 of r free for the form.
+__device__ __forceinline__ double f64_rot(double c, double s) {
+    const bool sf = fabs(c) < fabs(s);
+    const double r = sf ? c / s : s / c;
+    return __hiloint2double(__double2hiint(r) | (sf ? 0x40000000 : 0), __double2loint(r));
+}
+
+template <int NB>
+__device__ __forceinline__ void f64_pass(double* psi, int n, int b, const double* rot, int t, bool first,
+                                         const double* lowt, const double* hight, double fac) {
+    for (int g = t; g < (1 << n) >> NB; g += 256) {
+        const int i0 = ((g >> b) << (b + NB)) | (g & ((1 << b) - 1));
+        double v[1 << NB];
+#pragma unroll
+        for (int r = 0; r < (1 << NB); ++r) {
+            const int i = i0 | (r << b);
+            v[r] = lowt ? lowt[i & 31] * hight[i >> 5] : psi[f64_pad(i)];
+            if (first)  // the CZ ring, applied while loading the layer's first pass
+                v[r] = __hiloint2double(__double2hiint(v[r]) ^ (czring_parity(i, n) << 31), __double2loint(v[r]));
+        }
+#pragma unroll
+        for (int k = 0; k < NB; ++k) {
+            const double w = rot[b + k];
+            const bool sf = __double2hiint(w) & 0x40000000;
+            const double q = __hiloint2double(__double2hiint(w) & ~0x40000000, __double2loint(w));
+#pragma unroll
+            for (int r = 0; r < (1 << NB); ++r)
+                if (!((r >> k) & 1)) {
+                    const double a0 = v[r], a1 = v[r | (1 << k)];
+                    if (sf) {
+                        v[r] = fma(q, a0, -a1);
+                        v[r | (1 << k)] = fma(q, a1, a0);
+                    } else {
+                        v[r] = fma(-q, a1, a0);
+                        v[r | (1 << k)] = fma(q, a0, a1);
+                    }
+                }
+        }
+        if (b + NB == n) {
+#pragma unroll
+            for (int r = 0; r < (1 << NB); ++r) v[r] *= fac;
+        }
+#pragma unroll
+        for (int r = 0; r < (1 << NB); ++r) psi[f64_pad(i0 | (r << b))] = v[r];
+    }
+    __syncthreads();
+}
+
+// psi(alpha_s) in FP64: buf holds f64_state_doubles(n, P) doubles, psi first.
+// cs as for build_state_real.  Ends with a barrier.  Whole CTA of 256 threads.
+__device__ inline void build_state_f64(double* buf, int n, int d, int P, const double2* cs, int s) {
+    const int N = 1 << n, t = threadIdx.x;
+    double* rot = buf + N + (N >> 4);
+    double* facs = rot + P;
+    double* lowt = facs + d;
+    double* hight = lowt + (N < 32 ? N : 32);
+    int k = -1, which = 0;
+    if (s > 0) {
+        k = (s - 1) >> 1;
+        which = ((s - 1) & 1) ? 2 : 1;
+    }
+    auto angle = [&](int a) { return cs[(a == k ? which : 0) * P + a]; };
+    for (int a = n + t; a < P; a += 256) {
+        const double2 v = angle(a);
+        rot[a] = f64_rot(v.x, v.y);
+    }
+    for (int layer = 1 + (t ^ 255); layer <= d; layer += 256) {  // the last threads: the first ones hold rotations
+        double f = 1.0;
+        for (int q = 0; q < n; ++q) {
+            const double2 v = angle(layer * n + q);
+            f *= fabs(v.x) < fabs(v.y) ? v.y : v.x;
+        }
+        facs[layer - 1] = f;
+    }
+    auto bits = [&](int i, int q0, int q1) {  // factors of qubits q0 .. q1 - 1 of the product state
+        double v = 1.0;
+        for (int q = q0; q < q1; ++q) {
+            const double2 c = angle(q);
+            v *= ((i >> (q - q0)) & 1) ? c.y : c.x;
+        }
+        return v;
+    };
+    const int nl = n < 5 ? n : 5, nh = N >> nl;
+    if (t >= 64 && t - 64 < (1 << nl)) lowt[t - 64] = bits(t - 64, 0, nl);
+    if (t >= 96 && t - 96 < nh) hight[t - 96] = bits(t - 96, nl, n);
+    __syncthreads();
+    if (d == 0) {
+        for (int i = t; i < N; i += 256) buf[f64_pad(i)] = lowt[i & 31] * hight[i >> 5];
+        __syncthreads();
+        return;
+    }
+    // qubits per pass: at least 128 groups where the state has them (four warps, one per scheduler)
+    const int nb = n <= 9 ? 2 : n == 10 ? 3 : 4;
+    for (int layer = 1; layer <= d; ++layer) {
+        const double* lr = rot + layer * n;
+        const double fac = facs[layer - 1];
+        for (int b = 0; b < n; b += nb) {
+            const bool first = b == 0;
+            const double* tab = first && layer == 1 ? lowt : nullptr;
+            switch (min(nb, n - b)) {
+                case 1: f64_pass<1>(buf, n, b, lr, t, first, tab, hight, fac); break;
+                case 2: f64_pass<2>(buf, n, b, lr, t, first, tab, hight, fac); break;
+                case 3: f64_pass<3>(buf, n, b, lr, t, first, tab, hight, fac); break;
+                default: f64_pass<4>(buf, n, b, lr, t, first, tab, hight, fac); break;
+            }
+        }
+    }
 }
 
 }  // namespace dvqls
