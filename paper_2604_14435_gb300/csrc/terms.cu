@@ -57,7 +57,7 @@ struct Inst {
     float4* cf;      // L or null: ctil as float pairs
     void* bop;       // tensor-core tiles: the b rows of the B operand, TC_BOP_STAGE bytes per stage, or null
     void* wht;       // Walsh-Hadamard classes: the class table (WHT_TABLE_BYTES), or null
-    float2* bf;      // Walsh-Hadamard classes: b in FP32, or null
+    void* bf;        // Walsh-Hadamard classes: b as float2, or in fixed point as longlong2 (FP64), or null
     double2* cs;     // 3P: (cos, sin) of half angles: base, +pi/2, -pi/2
     double* bn2;     // ||b||^2
     double2* Dpart;  // S*T*T*ks
@@ -2187,9 +2187,10 @@ constexpr size_t WHT_OFF_DX = (WHT_OFF_PR + 2 * WHT_MAXP + 15) & ~size_t(15);  /
 constexpr size_t WHT_OFF_DO = WHT_OFF_DX + 4 * 64;                  // int term-class offsets [65]
 constexpr size_t WHT_OFF_DT = WHT_OFF_DO + 4 * 65;                  // uint16 terms by class [64]
 constexpr size_t WHT_OFF_EZ = (WHT_OFF_DT + 2 * 64 + 15) & ~size_t(15);  // uint16 z_l ^ z_m by class
-constexpr size_t WHT_OFF_EK = (WHT_OFF_EZ + 2 * WHT_MAXP + 15) & ~size_t(15);  // float2 signed weights by class
-constexpr size_t WHT_OFF_KEY = WHT_OFF_EK + 8 * WHT_MAXP;  // the inputs the table was built from: int L,
-                                                              // uint32 x[64], z[64], double2 coef[64]
+constexpr size_t WHT_OFF_EK = (WHT_OFF_EZ + 2 * WHT_MAXP + 15) & ~size_t(15);  // signed weights by class: float2, or
+                                                                               // double (FP64)
+constexpr size_t WHT_OFF_KEY = WHT_OFF_EK + 8 * WHT_MAXP;  // the inputs the table was built from: int L (negative
+                                                              // for FP64 weights), uint32 x[64], z[64], double2 coef[64]
 constexpr size_t WHT_OFF_SUM = WHT_OFF_KEY + 16 + 8 * 64 + 16 * 64;  // uint64 checksum of bytes [0, WHT_OFF_SUM)
 constexpr size_t WHT_OFF_BIM = WHT_OFF_SUM + 8;  // int: b has a nonzero imaginary part (rewritten every call)
 constexpr size_t WHT_TABLE_BYTES = WHT_OFF_SUM + 16;                   // header: int pair classes, term classes
@@ -2214,11 +2215,22 @@ __device__ inline unsigned long long wht_checksum(const unsigned char* tb, unsig
     return s;
 }
 
+// Fixed point of the FP64 classes: 1.0 = 2^W64_FRAC.  b is scaled by a power of
+// two so that ||b|| <= 1.
+constexpr int W64_FRAC = 62;
+__device__ __forceinline__ int w64_bexp(double bn2) {
+    int ex;
+    frexp(sqrt(bn2), &ex);  // ||b|| <= 2^ex
+    return min(max(ex, -1000), 1000);  // an invalid ||b||^2 is reported by k_prepare
+}
+
 // Class tables of one instance (one CTA of 256 per instance): pairs (l <= m)
 // sorted by x_l ^ x_m (bitonic sort of (mask, pair) keys), each with its
 // transform index z_l ^ z_m and its weight (-1)^popc(z_l & x) Re(w_lm),
-// doubled for l < m, as a float pair; terms by x_l; and b as float2.  Runs
-// after k_prepare (which forms the weights).
+// doubled for l < m, as a float pair (or a double, F64); terms by x_l; and b as
+// float2 (or in fixed point, F64).  Runs after k_prepare (which forms the
+// weights).
+template <bool F64>
 __global__ void __launch_bounds__(WHT_CT) k_wht_classes(const Inst* __restrict__ insts) {
     pdl_wait();
     pdl_trigger();
@@ -2232,8 +2244,14 @@ __global__ void __launch_bounds__(WHT_CT) k_wht_classes(const Inst* __restrict__
     bool im = false;
     for (long long j = t; I.b && j < N; j += WHT_CT) {  // the local cost has no b here (|+>^n is implied)
         const double2 v = I.b[j];
-        I.bf[j] = make_float2((float)v.x, (float)v.y);
-        im |= (float)v.y != 0.f;
+        if (F64) {
+            const double sc = scalbn(1.0, W64_FRAC - w64_bexp(*I.bn2));
+            reinterpret_cast<longlong2*>(I.bf)[j] = make_longlong2(__double2ll_rn(v.x * sc), __double2ll_rn(v.y * sc));
+            im |= v.y != 0.0;
+        } else {
+            reinterpret_cast<float2*>(I.bf)[j] = make_float2((float)v.x, (float)v.y);
+            im |= (float)v.y != 0.f;
+        }
     }
     if (__syncthreads_or(im) != 0) {
         if (t == 0) *reinterpret_cast<int*>(tb + WHT_OFF_BIM) = 1;
@@ -2256,10 +2274,13 @@ __global__ void __launch_bounds__(WHT_CT) k_wht_classes(const Inst* __restrict__
         differs = kx[t] != I.xm[t] || kz[t] != I.zm[t] || __double_as_longlong(c.x) != __double_as_longlong(k.x) ||
                   __double_as_longlong(c.y) != __double_as_longlong(k.y);
     }
-    if (t == 0 && *kL != L) differs = true;
+    const int tag = F64 ? -L : L;
+    if (t == 0 && *kL != tag) differs = true;
     __shared__ unsigned long long red[WHT_CT / 32];
     unsigned long long* ksum = reinterpret_cast<unsigned long long*>(tb + WHT_OFF_SUM);
     if (!__syncthreads_or(differs) && wht_checksum(tb, red) == *ksum) return;  // still valid, untouched
+    int P2 = 2;  // the pairs are sorted within the next power of two
+    while (P2 < np) P2 <<= 1;
     for (int e = np + t; e < 4096; e += WHT_CT) key[e] = ~0ull;
     __syncthreads();
     for (int q = t; q < L * L; q += WHT_CT) {  // pair (l, m), l <= m, at e = l L - l (l - 1) / 2 + m - l
@@ -2269,9 +2290,9 @@ __global__ void __launch_bounds__(WHT_CT) k_wht_classes(const Inst* __restrict__
                 ((unsigned long long)(sx[l] ^ sx[m]) << 16) | (unsigned long long)(l | (m << 8));
     }
     __syncthreads();
-    for (int k = 2; k <= 4096; k <<= 1)
+    for (int k = 2; k <= P2; k <<= 1)
         for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int e = t; e < 4096; e += WHT_CT) {
+            for (int e = t; e < P2; e += WHT_CT) {
                 const int p = e ^ j;
                 if (p > e) {
                     const unsigned long long a = key[e], b = key[p];
@@ -2325,9 +2346,13 @@ __global__ void __launch_bounds__(WHT_CT) k_wht_classes(const Inst* __restrict__
         pr[e] = uint16_t(p);
         const uint32_t zl = sz[l], zm = sz[m];
         reinterpret_cast<uint16_t*>(tb + WHT_OFF_EZ)[e] = uint16_t((zl ^ zm) & uint32_t(N - 1));
-        const float4 wv = I.wf[l * L + m];
         const float sg = ((__popc(zl & x) & 1) ? -1.f : 1.f) * (l < m ? 2.f : 1.f);  // exact scaling
-        reinterpret_cast<float2*>(tb + WHT_OFF_EK)[e] = make_float2(sg * wv.x, sg * wv.y);
+        if (F64) {
+            reinterpret_cast<double*>(tb + WHT_OFF_EK)[e] = (double)sg * I.w[l * L + m].x;
+        } else {
+            const float4 wv = I.wf[l * L + m];
+            reinterpret_cast<float2*>(tb + WHT_OFF_EK)[e] = make_float2(sg * wv.x, sg * wv.y);
+        }
     }
     if (t == WHT_CT - 1) co[tsum[WHT_CT - 1] + cnt] = np;  // the end of the last class
     __shared__ int sfirst[64];  // term k is the first with its mask
@@ -2371,7 +2396,7 @@ __global__ void __launch_bounds__(WHT_CT) k_wht_classes(const Inst* __restrict__
         kz[t] = I.zm[t];
         kc[t] = I.coef[t];
     }
-    if (t == 0) *kL = L;
+    if (t == 0) *kL = tag;
     __syncthreads();  // every word of the table is written
     const unsigned long long sum = wht_checksum(tb, red);
     if (t == 0) *ksum = sum;
@@ -2623,7 +2648,7 @@ __global__ void __launch_bounds__(WHT_NT, 4) k_terms_wht(const Inst* __restrict_
             szl[t] = t < L ? I.zm[t] : 0u;
             dre[t] = dim[t] = 0.f;
         }
-        for (int j = t; !I.local && j < (1 << I.n); j += WHT_NT) sb[j] = I.bf[j];
+        for (int j = t; !I.local && j < (1 << I.n); j += WHT_NT) sb[j] = reinterpret_cast<const float2*>(I.bf)[j];
         build_state_regs<false>(psi, scratch, scs, I.n, I.d, I.P, I.cs, s + I.s0, t, 0, 1.f);  // ends with a barrier
         float S = 0.f, E = 0.f;
         if (I.local) {
@@ -2682,6 +2707,225 @@ __global__ void __launch_bounds__(WHT_NT, 4) k_terms_wht(const Inst* __restrict_
 inline size_t wht_smem_bytes(int Pmax) {
     const size_t N = size_t(1) << WHT_MAXN;
     return 4 * (N + 8 * (N + N / 32) + 2 * (N + N / 32)) + 8 * N + 8 * (size_t)Pmax;
+}
+
+// ------------------------------------- Walsh-Hadamard classes in FP64
+// DVQLS_FP64 with L <= 64 and n <= 10: the same classes, for the same terms.
+// The FP64 tiles spend one DFMA per term and amplitude on a pipe that issues 2
+// per clock and SM (n = 10, L = 64: 2.2 M DFMAs, 1.1 M cycles per state).  Here
+// the transforms run in 64-bit fixed point on the integer pipes: the state has
+// norm one, so sum_i |psi[i] psi[i ^ x]| <= 1 and every partial sum of a
+// transform stays within 1.0 = 2^62 -- the adds are exact.  An amplitude and a
+// product are rounded once each, to 2^-63 absolute (an FP64 rounding of an
+// amplitude near 2^-5, the mean at n = 10, is 2^-58).  What is left on the FP64
+// pipe is the state build and one FMA per term for the weighted sums.
+// One CTA of 8 warps per item, two CTAs per SM (the transform of 2^10 values
+// holds 64 registers a lane), so one CTA's state build overlaps the other's
+// transforms.
+// n = 10, L = 64, 101 shifts of one system: 623 us by the tiles, 72 us by the
+// classes; 48 systems of n = 6..10: 8,646 us against 600 us.
+constexpr int W64_ROW = (1 << WHT_MAXN) + (1 << WHT_MAXN) / 32;
+
+// a b for a, b in fixed point, rounded to nearest.
+__device__ __forceinline__ long long w64_mul(long long a, long long b) {
+    const unsigned long long lo = (unsigned long long)a * (unsigned long long)b;
+    return (__mul64hi(a, b) << 2) + (long long)(lo >> 62) + (long long)((lo >> 61) & 1ull);
+}
+
+// Transform of v (index (r << 5) | lane) into the warp's row, at i + (i >> 5)
+// for 2^10 values (A = 32: through the row, lane bits become register bits), else at i.
+template <int A, int LOGA>
+__device__ __forceinline__ void w64_transform(long long (&v)[A], long long* row, int N, int lane) {
+    auto regs = [&]() {
+#pragma unroll
+        for (int kb = 0; kb < LOGA; ++kb)
+#pragma unroll
+            for (int r = 0; r < A; ++r)
+                if (!((r >> kb) & 1)) {
+                    const long long a = v[r], b = v[r | (1 << kb)];
+                    v[r] = a + b;
+                    v[r | (1 << kb)] = a - b;
+                }
+    };
+    regs();
+    if constexpr (A == 32) {
+#pragma unroll
+        for (int r = 0; r < 32; ++r) row[r * 33 + lane] = v[r];
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 32; ++j) v[j] = row[lane * 33 + j];  // index (lane << 5) | j
+        __syncwarp();
+        regs();
+#pragma unroll
+        for (int j = 0; j < 32; ++j) row[lane * 33 + j] = v[j];
+    } else {
+        const int nl = N < 32 ? __ffs(N) - 1 : 5;
+        for (int b = 0; b < nl; ++b)
+#pragma unroll
+            for (int r = 0; r < A; ++r) {
+                const long long p = __shfl_xor_sync(0xffffffffu, v[r], 1 << b);
+                v[r] = ((lane >> b) & 1) ? p - v[r] : v[r] + p;
+            }
+        if (lane < N || N >= 32) {
+#pragma unroll
+            for (int r = 0; r < A; ++r) row[(r << 5) | lane] = v[r];
+        }
+    }
+    __syncwarp();
+}
+
+// The pair classes (flavours 0..n of the local cost) and, for the global cost,
+// the term classes of one state q, dealt to the warps; the warp's sums of its
+// lanes in D (flavour 0) and E (the others), delta~ to dre / dim.
+template <int A, int LOGA>
+__device__ void w64_item(const Inst& I, int s, const long long* q, long long* row, double* dre, double* dim,
+                         const uint32_t* szl, double& D, double& E, int lane) {
+    constexpr bool PAD = A == 32;
+    const int n = I.n, N = 1 << n, L = I.L, w = threadIdx.x >> 5, lm = N < 32 ? N - 1 : 31;
+    const unsigned char* tb = reinterpret_cast<const unsigned char*>(I.wht);
+    const int ncls = reinterpret_cast<const int*>(tb)[0], nd = reinterpret_cast<const int*>(tb)[1];
+    const uint32_t* cx = reinterpret_cast<const uint32_t*>(tb + WHT_OFF_CX);
+    const int* co = reinterpret_cast<const int*>(tb + WHT_OFF_CO);
+    const uint16_t* pr = reinterpret_cast<const uint16_t*>(tb + WHT_OFF_PR);
+    const uint16_t* ez = reinterpret_cast<const uint16_t*>(tb + WHT_OFF_EZ);
+    const double* ek = reinterpret_cast<const double*>(tb + WHT_OFF_EK);
+    const uint32_t* dx = reinterpret_cast<const uint32_t*>(tb + WHT_OFF_DX);
+    const int* dof = reinterpret_cast<const int*>(tb + WHT_OFF_DO);
+    const uint16_t* dt = reinterpret_cast<const uint16_t*>(tb + WHT_OFF_DT);
+    double2* Gp = (s == 0 && I.Gpart) ? reinterpret_cast<double2*>(I.Gpart) : nullptr;
+    const double unit = scalbn(1.0, -W64_FRAC);
+    const int parts = 1 + *reinterpret_cast<const int*>(tb + WHT_OFF_BIM);
+    const int pairs = ncls * I.F, jobs = pairs + (I.local ? 0 : nd * parts);
+    auto at = [&](uint32_t z) { return row[PAD ? z + (z >> 5) : z]; };
+#pragma unroll 1
+    for (int j = w; j < jobs; j += WHT_NT / 32) {
+        long long v[A];
+        if (j >= pairs) {
+            const int c = (j - pairs) / parts, part = (j - pairs) - c * parts, x = int(dx[c]);
+            const longlong2* qb = reinterpret_cast<const longlong2*>(I.bf);
+#pragma unroll
+            for (int r = 0; r < A; ++r) {  // conj(b[i ^ x]) psi[i], its real or imaginary part
+                const int i = (r << 5) | (lane & lm), k = (i ^ x) & (N - 1);
+                v[r] = w64_mul(part ? -qb[k].y : qb[k].x, q[i]);
+            }
+            w64_transform<A, LOGA>(v, row, N, lane);
+            const double sc = scalbn(1.0, w64_bexp(*I.bn2) - W64_FRAC);
+            for (int e = dof[c] + lane; e < dof[c + 1]; e += 32) {
+                const int l = dt[e];
+                (part ? dim : dre)[l] = (double)at(szl[l] & uint32_t(N - 1)) * sc;
+            }
+            __syncwarp();
+            continue;
+        }
+        const int f = j / ncls, c = j - f * ncls;
+        const int x = int(cx[c] ^ (f ? 1u << (f - 1) : 0u));  // X_j between the two terms (local cost)
+#pragma unroll
+        for (int r = 0; r < A; ++r) {
+            const int i = (r << 5) | (lane & lm);
+            v[r] = w64_mul(q[i], q[(i ^ x) & (N - 1)]);  // masks >= 2^n are reported, never followed
+        }
+        w64_transform<A, LOGA>(v, row, N, lane);
+        const int e0 = co[c], e1 = co[c + 1];
+        if (f == 0) {
+            for (int e = e0 + lane; e < e1; e += 32) D = fma(ek[e], (double)at(ez[e]), D);
+        } else {
+            for (int e = e0 + lane; e < e1; e += 32) {
+                const double k = ek[e];
+                E = fma((szl[pr[e] & 0xFF] >> (f - 1)) & 1u ? -k : k, (double)at(ez[e]), E);
+            }
+        }
+        if (Gp)  // the beta output of the unshifted state
+            for (int e = e0 + lane; e < e1; e += 32) {
+                const int p = pr[e], l = p & 0xFF, m = p >> 8;
+                double beta = (double)at(ez[e]) * unit;
+                if (__popc(szl[l] & uint32_t(x)) & 1) beta = -beta;
+                Gp[(long long)l * L + m] = make_double2(beta, 0.0);
+                Gp[(long long)m * L + l] = make_double2(beta, 0.0);
+            }
+        __syncwarp();
+    }
+}
+
+inline size_t w64_smem_bytes(int Pmax) {
+    return 8 * (f64_state_doubles(WHT_MAXN, Pmax) + (size_t(1) << WHT_MAXN) + 8 * size_t(W64_ROW));
+}
+
+__global__ void __launch_bounds__(WHT_NT, 2) k_terms_wht64(const Inst* __restrict__ insts, int count, long long total,
+                                                           unsigned long long* queue) {
+    pdl_wait();
+    pdl_trigger();
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ uint32_t szl[TT];
+    __shared__ double dre[TT], dim[TT], red[WHT_NT / 32], redE[WHT_NT / 32];
+    __shared__ double2 redT[2];
+    __shared__ long long s_item;
+    const int t = threadIdx.x, w = t >> 5, lane = t & 31;
+    long long* q = reinterpret_cast<long long*>(smem);        // 2^WHT_MAXN
+    long long* row = q + (1 << WHT_MAXN) + w * W64_ROW;         // this warp's transform row
+    double* st = reinterpret_cast<double*>(q + (1 << WHT_MAXN) + 8 * W64_ROW);
+    for (;;) {
+        if (t == 0) s_item = (long long)atomicAdd(queue, 1ull);
+        __syncthreads();
+        const long long gi = s_item;
+        __syncthreads();
+        if (gi >= total) break;
+        const Inst& I = insts[find_instance(insts, count, gi)];
+        const int s = int(gi - I.item_base), L = I.L, N = 1 << I.n;
+        if (t < TT) {
+            szl[t] = t < L ? I.zm[t] : 0u;
+            dre[t] = dim[t] = 0.0;
+        }
+        build_state_f64(st, I.n, I.d, I.P, I.cs, s + I.s0);
+        const double one = scalbn(1.0, W64_FRAC);
+        for (int i = t; i < N; i += WHT_NT) q[i] = __double2ll_rn(st[f64_pad(i)] * one);
+        __syncthreads();
+        double D = 0.0, E = 0.0;
+        switch (I.n) {
+            case 10: w64_item<32, 5>(I, s, q, row, dre, dim, szl, D, E, lane); break;
+            case 9: w64_item<16, 4>(I, s, q, row, dre, dim, szl, D, E, lane); break;
+            case 8: w64_item<8, 3>(I, s, q, row, dre, dim, szl, D, E, lane); break;
+            case 7: w64_item<4, 2>(I, s, q, row, dre, dim, szl, D, E, lane); break;
+            case 6: w64_item<2, 1>(I, s, q, row, dre, dim, szl, D, E, lane); break;
+            default: w64_item<1, 0>(I, s, q, row, dre, dim, szl, D, E, lane); break;  // n <= 5
+        }
+        for (int o = 16; o; o >>= 1) D += __shfl_xor_sync(0xffffffffu, D, o);
+        if (I.local)
+            for (int o = 16; o; o >>= 1) E += __shfl_xor_sync(0xffffffffu, E, o);
+        if (lane == 0) {
+            red[w] = D;
+            redE[w] = E;
+        }
+        __syncthreads();
+        if (!I.local && t < TT) {  // T = sum_l c~_l delta~_l
+            double2 T = make_double2(0.0, 0.0);
+            if (t < L) {
+                const double2 c = I.ctil[t];
+                const double dr = dre[t], di = dim[t];
+                T = make_double2(c.x * dr - c.y * di, c.x * di + c.y * dr);
+                if (s == 0 && I.dpart) reinterpret_cast<double2*>(I.dpart)[t] = make_double2(dr, di);
+            }
+            for (int o = 16; o; o >>= 1) {
+                T.x += __shfl_xor_sync(0xffffffffu, T.x, o);
+                T.y += __shfl_xor_sync(0xffffffffu, T.y, o);
+            }
+            if (lane == 0) redT[w] = T;
+        }
+        __syncthreads();
+        const double unit = scalbn(1.0, -W64_FRAC);
+        if (t == 0) {
+            double Ds = 0.0, Es = 0.0;
+            for (int k = 0; k < WHT_NT / 32; ++k) {
+                Ds += red[k];
+                if (I.local) Es += redE[k];
+            }
+            I.Dpart[(long long)s * I.F] = make_double2(Ds * unit, 0.0);
+            if (I.local) I.Dpart[(long long)s * I.F + 1] = make_double2(Es * unit, 0.0);
+            else I.Tpart[s] = make_double2(redT[0].x + redT[1].x, redT[0].y + redT[1].y);
+        } else if (I.local && t >= 2 && t < I.F) {  // slot 0 of a shift holds D, slot 1 E, the rest zero
+            I.Dpart[(long long)s * I.F + t] = make_double2(0.0, 0.0);
+        }
+        __syncthreads();
+    }
 }
 
 // ---------------------------------------------------------------- combine
@@ -2894,7 +3138,8 @@ static int launch_pass(dvqls_ctx* ctx, cudaStream_t st, const Inst* dtable, cons
     }
     if (ps.wht) {
         if (marks) prof_begin(ctx, 0);
-        DVQLS_CUDA_TRY(ctx, launch_pdl(k_wht_classes, dim3(ps.count), dim3(WHT_CT), 0, st, dtable));
+        DVQLS_CUDA_TRY(ctx, launch_pdl(ps.fp32 ? k_wht_classes<false> : k_wht_classes<true>, dim3(ps.count), dim3(WHT_CT), 0,
+                                       st, dtable));
         if (marks) prof_end(ctx);
     }
     if (ps.tc && ps.st_grid > 0) {  // shifted states of the on-chip instances, packed for the term kernel
@@ -2915,7 +3160,7 @@ static int launch_pass(dvqls_ctx* ctx, cudaStream_t st, const Inst* dtable, cons
     }
     if (marks) prof_begin(ctx, 1);
     if (ps.wht)
-        DVQLS_CUDA_TRY(ctx, launch_pdl(k_terms_wht, dim3(ps.grid), dim3(WHT_NT), ps.smem, st, dtable, ps.count,
+        DVQLS_CUDA_TRY(ctx, launch_pdl(ps.fp32 ? k_terms_wht : k_terms_wht64, dim3(ps.grid), dim3(WHT_NT), ps.smem, st, dtable, ps.count,
                                        ps.total, ctx->d_queue));
     else if (ps.tc)
         DVQLS_CUDA_TRY(ctx, launch_pdl(k_terms_tc, dim3(ps.grid), dim3(TCT), ps.smem, st, dtable, ps.count, ps.total,
@@ -3042,11 +3287,13 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
     }
     cudaSetDevice(ctx->device);
     const bool fp32 = precision != DVQLS_FP64;
-    // Walsh-Hadamard classes serve the global cost when every LCU fits one
-    // 64-term tile and every state n <= 10 qubits; tensor-core tiles when
-    // every LCU fits one tile (asked for directly, or as the fallback of the
-    // classes); anything else runs the FP32 CUDA-core tiles.
-    bool wht = precision == DVQLS_FP32_WHT;
+    // Walsh-Hadamard classes serve the calls that ask for them, and FP64, when
+    // every LCU fits one 64-term tile and every state n <= 10 qubits (FP64: even
+    // with a class per pair, a transform in fixed point costs less than the
+    // N DFMAs of its term; see k_terms_wht64); tensor-core tiles when asked for
+    // directly, or as the fallback of the global cost's classes; anything else
+    // runs the CUDA-core tiles.
+    bool wht = precision == DVQLS_FP32_WHT || precision == DVQLS_FP64;
     for (const auto& h : hi) wht = wht && h.T == 1 && h.n <= WHT_MAXN;
     bool tc = !wht && (precision == DVQLS_FP32_TC || (precision == DVQLS_FP32_WHT && !local));
     int copy_nmax = 0, split_nmax = 0;
@@ -3077,11 +3324,11 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
                 st_smem = std::max(st_smem, tcs_smem(h.n, h.P));
             }
     if (st_grid > 0) DVQLS_CUDA_TRY(ctx, allow_dynamic_smem((const void*)k_tc_states));
-    const size_t smem = wht  ? wht_smem_bytes(Pmax)
+    const size_t smem = wht  ? (fp32 ? wht_smem_bytes(Pmax) : w64_smem_bytes(Pmax))
                         : tc ? tc_smem_bytes(tc_nsm, copy_nmax, split_nmax, readout)
                         : fp32 ? smem_bytes<float>(nmax, Pmax) : smem_bytes<double>(nmax, Pmax);
     const size_t r2 = fp32 ? 8 : 16;
-    auto kfun = wht ? (const void*)k_terms_wht
+    auto kfun = wht ? (fp32 ? (const void*)k_terms_wht : (const void*)k_terms_wht64)
                 : tc ? (const void*)k_terms_tc
                 : fp32 ? (const void*)k_terms_smem<float> : (const void*)k_terms_smem<double>;
     DVQLS_CUDA_TRY(ctx, allow_dynamic_smem(kfun));
@@ -3172,7 +3419,7 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
         o.cf = fp32 ? ar.reserve(L * 16) : 0;
         o.bop = tc && !local ? ar.reserve(size_t(tc_bop_stages(h.N)) * TC_BOP_STAGE) : 0;
         o.wht = wht ? ar.reserve(WHT_TABLE_BYTES) : 0;
-        o.bf = wht ? ar.reserve(size_t(h.N) * 8) : 0;
+        o.bf = wht ? ar.reserve(size_t(h.N) * (fp32 ? 8 : 16)) : 0;
         o.cs = ar.reserve(size_t(3) * h.P * 16);
         o.bn2 = ar.reserve(8);
         o.Dp = ar.reserve(size_t(h.S) * h.F * h.T * h.T * kp * 16);
@@ -3244,7 +3491,7 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
         I.cf = fp32 ? (float4*)(ws + o.cf) : nullptr;
         I.bop = tc && !local ? (void*)(ws + o.bop) : nullptr;
         I.wht = wht ? (void*)(ws + o.wht) : nullptr;
-        I.bf = wht ? (float2*)(ws + o.bf) : nullptr;
+        I.bf = wht ? (void*)(ws + o.bf) : nullptr;
         I.cs = (double2*)(ws + o.cs);
         I.bn2 = (double*)(ws + o.bn2);
         I.Dpart = (double2*)(ws + o.Dp);
