@@ -66,6 +66,7 @@ struct Inst {
     void* dpart;     // ks*L   (shift 0 only; null when delta is not requested)
     double* NsDs;    // 3S: N_s, Re D_s, Im D_s
     void* states;    // n > 12: the S shifted states in HBM (S x N), else null
+    void* chain;     // n > 12: the unshifted state after every pass (2d + 1 states), or null when S = 1
     void* tcst;      // tensor-core pass, n <= 12: the S shifted states as packed FP16 pairs (S x N words), else null
     double* cost;
     double* grad;    // P or null
@@ -553,12 +554,70 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 3 : 1) k_terms_smem(const
 // chunks (CZ ring signs and the Ry rotations of qubits 0..11 in shared memory)
 // and one pass over column tiles of HC consecutive low indices x all high
 // indices (Ry of qubits 12..; a warp reads whole 128-byte rows).
+//
+// A shifted state equals the unshifted one up to the layer of its angle, so
+// the unshifted state is built first, keeping it after every pass (`chain`),
+// and a shifted state starts from there: at the low pass of its angle's layer,
+// or at the high pass when its qubit is one of 12.. (the low pass before it is
+// the unshifted state's).  Half the passes of S full builds, with the same
+// operations on every amplitude.  The shifted states are taken through all
+// their layers in groups that stay in L2 (HBM_GROUP bytes; of 129 MB), so HBM
+// sees little more than a state's last write.  Two n = 20 instances of depth 10
+// (882 states): 25.0 ms for full builds of all states, pass by pass.  The uneven
+// batch they belong to: 67.8 ms with those, 57.1 without groups, 57.8 with
+// groups of 96 MB, 54.8 with 64, 56.4 with 32, 58.1 with 20.
 constexpr int LOQ = 12, LOC = 1 << LOQ, HC = 32;
+constexpr size_t HBM_GROUP = size_t(64) << 20;
+
+// Launch with programmatic stream serialization (the kernel starts with
+// pdl_wait, so it observes everything its predecessor wrote).
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                              Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
+
+// Where pass `hi` of layer `layer` (layer 0: the product state, written only)
+// reads and writes the state of shift sg of the instance (0: unshifted).
+template <typename R>
+__device__ __forceinline__ void hbm_io(const Inst& I, int sg, int layer, bool hi, const R*& src, R*& dst) {
+    const size_t N = size_t(1) << I.n;
+    R* own = reinterpret_cast<R*>(I.states) + (size_t)(sg - I.s0) * N;
+    R* chain = reinterpret_cast<R*>(I.chain);
+    if (sg == 0 && !chain) {
+        src = dst = own;
+        return;
+    }
+    auto full = [&](int l) { return chain + (size_t)(2 * l) * N; };      // after layer l
+    auto half = [&](int l) { return chain + (size_t)(2 * l - 1) * N; };  // after the low pass of layer l
+    if (sg == 0) {
+        src = layer == 0 ? nullptr : hi ? half(layer) : full(layer - 1);
+        const bool last = layer == I.d && (hi || layer == 0) && I.s0 == 0;
+        dst = last ? own : layer == 0 ? full(0) : hi ? full(layer) : half(layer);
+        return;
+    }
+    const int k = (sg - 1) >> 1;
+    dst = own;
+    src = own;
+    if (layer > 0 && k / I.n == layer) {
+        if (!hi) src = full(layer - 1);
+        else if (k % I.n >= LOQ) src = half(layer);
+    }
+}
 
 template <typename R>
-__device__ __forceinline__ void shift_angle(const Inst& I, int s, int a, R& c, R& sn) {
+__device__ __forceinline__ void shift_angle(const Inst& I, int sg, int a, R& c, R& sn) {
     int k = -1, which = 0;
-    const int sg = s + I.s0;  // the shift's index in the instance
     if (sg > 0) {
         k = (sg - 1) >> 1;
         which = ((sg - 1) & 1) ? 2 : 1;
@@ -569,15 +628,16 @@ __device__ __forceinline__ void shift_angle(const Inst& I, int s, int a, R& c, R
 }
 
 template <typename R>
-__global__ void __launch_bounds__(256) k_hbm_init(const Inst* __restrict__ insts, int idx) {
+__global__ void __launch_bounds__(256) k_hbm_init(const Inst* __restrict__ insts, int idx, int sg0) {
+    pdl_wait();
+    pdl_trigger();
     // The product state factorises over bit groups: amplitude i of this chunk
     // is t0[i & 63] t1[(i >> 6) & 63] h, the factors of qubits 0..5, 6..11 and
     // of the chunk's high bits (two multiplies per amplitude).
     const Inst& I = insts[idx];
     __shared__ R cq[32], sq[32], t0[64], t1[64], hc;
-    const int s = blockIdx.y, n = I.n, t = threadIdx.x;
-    const size_t N = size_t(1) << n;
-    if (t < n) shift_angle<R>(I, s, t, cq[t], sq[t]);
+    const int sg = sg0 + blockIdx.y, n = I.n, t = threadIdx.x;
+    if (t < n) shift_angle<R>(I, sg, t, cq[t], sq[t]);
     __syncthreads();
     if (t < 128) {
         const int g = t >> 6, k = t & 63;
@@ -590,7 +650,10 @@ __global__ void __launch_bounds__(256) k_hbm_init(const Inst* __restrict__ insts
         hc = v;
     }
     __syncthreads();
-    R* st = reinterpret_cast<R*>(I.states) + s * N + ((size_t)blockIdx.x << LOQ);
+    const R* src;
+    R* st;
+    hbm_io<R>(I, sg, 0, false, src, st);
+    st += (size_t)blockIdx.x << LOQ;
     constexpr int VE = 16 / sizeof(R);
 #pragma unroll 4
     for (int e4 = t; e4 < LOC / VE; e4 += 256) {
@@ -607,19 +670,24 @@ __global__ void __launch_bounds__(256) k_hbm_init(const Inst* __restrict__ insts
 }
 
 template <typename R>
-__global__ void __launch_bounds__(256) k_hbm_lo(const Inst* __restrict__ insts, int idx, int layer) {
+__global__ void __launch_bounds__(256) k_hbm_lo(const Inst* __restrict__ insts, int idx, int layer, int sg0) {
+    pdl_wait();
+    pdl_trigger();
     extern __shared__ __align__(16) unsigned char sm[];
     R* w = reinterpret_cast<R*>(sm);
     const Inst& I = insts[idx];
     __shared__ R cq[LOQ], sq[LOQ];
-    const int s = blockIdx.y, n = I.n, base = blockIdx.x << LOQ;
-    const size_t N = size_t(1) << n;
-    if (threadIdx.x < LOQ) shift_angle<R>(I, s, layer * n + threadIdx.x, cq[threadIdx.x], sq[threadIdx.x]);
-    R* st = reinterpret_cast<R*>(I.states) + s * N + base;
+    const int sg = sg0 + blockIdx.y, n = I.n, base = blockIdx.x << LOQ;
+    if (threadIdx.x < LOQ) shift_angle<R>(I, sg, layer * n + threadIdx.x, cq[threadIdx.x], sq[threadIdx.x]);
+    const R* src;
+    R* dst;
+    hbm_io<R>(I, sg, layer, false, src, dst);
+    src += base;
+    dst += base;
     constexpr int VE = 16 / sizeof(R);  // amplitudes per 16-byte vector: all of a thread's loads in flight
 #pragma unroll
     for (int e4 = threadIdx.x; e4 < LOC / VE; e4 += 256) {
-        const uint4 u = reinterpret_cast<const uint4*>(st)[e4];
+        const uint4 u = reinterpret_cast<const uint4*>(src)[e4];
         R v[VE];
         memcpy(v, &u, 16);
 #pragma unroll
@@ -641,7 +709,7 @@ __global__ void __launch_bounds__(256) k_hbm_lo(const Inst* __restrict__ insts, 
     }
 #pragma unroll
     for (int e4 = threadIdx.x; e4 < LOC / VE; e4 += 256)
-        reinterpret_cast<uint4*>(st)[e4] = reinterpret_cast<const uint4*>(w)[e4];
+        reinterpret_cast<uint4*>(dst)[e4] = reinterpret_cast<const uint4*>(w)[e4];
 }
 
 // The same low-qubit pass for FP32 states with the chunk in registers, 16
@@ -657,28 +725,33 @@ __global__ void __launch_bounds__(256) k_hbm_lo(const Inst* __restrict__ insts, 
 // eight consecutive threads, 64 bytes apart, fall in eight different bank
 // groups; the two half-warps of a 256-strided read sit 16 banks apart).
 __device__ __forceinline__ int lo_pad(int e) { return e + ((e >> 5) << 2) + ((e >> 8) << 4); }
-__global__ void __launch_bounds__(256) k_hbm_lo_regs(const Inst* __restrict__ insts, int idx, int layer) {
+__global__ void __launch_bounds__(256) k_hbm_lo_regs(const Inst* __restrict__ insts, int idx, int layer, int sg0) {
+    pdl_wait();
+    pdl_trigger();
     constexpr int PADW = LOC + (LOC >> 5) * 4 + (LOC >> 8) * 16;
     __shared__ __align__(16) float scr[2][PADW];
     __shared__ float rq[LOQ], fq[LOQ];
     __shared__ int sfq[LOQ];
     const Inst& I = insts[idx];
-    const int s = blockIdx.y, n = I.n, base = blockIdx.x << LOQ, t = threadIdx.x;
-    const size_t N = size_t(1) << n;
+    const int sg = sg0 + blockIdx.y, n = I.n, base = blockIdx.x << LOQ, t = threadIdx.x;
     if (t < LOQ) {  // the rotations in scaled form; their factors are applied at the store
         float c, sn;
-        shift_angle<float>(I, s, layer * n + t, c, sn);
+        shift_angle<float>(I, sg, layer * n + t, c, sn);
         const RyScaled q = ry_scaled(c, sn);
         rq[t] = q.r;
         fq[t] = q.fac;
         sfq[t] = q.sform;
     }
-    float* st = reinterpret_cast<float*>(I.states) + s * N + base;
+    const float* src;
+    float* st;
+    hbm_io<float>(I, sg, layer, false, src, st);
+    src += base;
+    st += base;
     float v[16];
     // layout A: amplitude 16 t + r
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-        const float4 x = reinterpret_cast<const float4*>(st)[4 * t + c];
+        const float4 x = reinterpret_cast<const float4*>(src)[4 * t + c];
         v[4 * c + 0] = x.x;
         v[4 * c + 1] = x.y;
         v[4 * c + 2] = x.z;
@@ -726,21 +799,24 @@ __global__ void __launch_bounds__(256) k_hbm_lo_regs(const Inst* __restrict__ in
 }
 
 template <typename R>
-__global__ void __launch_bounds__(256) k_hbm_hi(const Inst* __restrict__ insts, int idx, int layer) {
+__global__ void __launch_bounds__(256) k_hbm_hi(const Inst* __restrict__ insts, int idx, int layer, int sg0) {
+    pdl_wait();
+    pdl_trigger();
     extern __shared__ __align__(16) unsigned char sm[];
     R* w = reinterpret_cast<R*>(sm);  // [H][HC]
     const Inst& I = insts[idx];
     __shared__ R cq[32], sq[32];
-    const int s = blockIdx.y, n = I.n, H = 1 << (n - LOQ), lo0 = blockIdx.x * HC;
-    const size_t N = size_t(1) << n;
+    const int sg = sg0 + blockIdx.y, n = I.n, H = 1 << (n - LOQ), lo0 = blockIdx.x * HC;
     if (threadIdx.x < n - LOQ)
-        shift_angle<R>(I, s, layer * n + LOQ + threadIdx.x, cq[threadIdx.x], sq[threadIdx.x]);
-    R* st = reinterpret_cast<R*>(I.states) + s * N;
+        shift_angle<R>(I, sg, layer * n + LOQ + threadIdx.x, cq[threadIdx.x], sq[threadIdx.x]);
+    const R* src;
+    R* st;
+    hbm_io<R>(I, sg, layer, true, src, st);
     constexpr int VE = 16 / sizeof(R);  // 16-byte vectors of a row's HC columns
 #pragma unroll 8
     for (int e4 = threadIdx.x; e4 < H * HC / VE; e4 += 256) {
         const int e = e4 * VE;
-        reinterpret_cast<uint4*>(w)[e4] = *reinterpret_cast<const uint4*>(st + ((size_t)(e / HC) << LOQ) + lo0 + e % HC);
+        reinterpret_cast<uint4*>(w)[e4] = *reinterpret_cast<const uint4*>(src + ((size_t)(e / HC) << LOQ) + lo0 + e % HC);
     }
     __syncthreads();
     for (int q = 0; q < n - LOQ; ++q) {
@@ -769,26 +845,31 @@ __global__ void __launch_bounds__(256) k_hbm_hi(const Inst* __restrict__ insts, 
 // and the tile is stored from there (a warp writes one 128-byte row segment per
 // register).  One barrier per tile instead of one per qubit.
 template <int LOGH>
-__global__ void __launch_bounds__(256) k_hbm_hi_regs(const Inst* __restrict__ insts, int idx, int layer) {
+__global__ void __launch_bounds__(256) k_hbm_hi_regs(const Inst* __restrict__ insts, int idx, int layer, int sg0) {
+    pdl_wait();
+    pdl_trigger();
     constexpr int H = 1 << LOGH, RG = H / 8;
     __shared__ float scr[H * 33];
     __shared__ float rq[LOGH], fq[LOGH];
     __shared__ int sfq[LOGH];
     const Inst& I = insts[idx];
-    const int s = blockIdx.y, n = I.n, lo0 = blockIdx.x * 32, t = threadIdx.x, lane = t & 31, w = t >> 5;
-    const size_t N = size_t(1) << n;
+    const int sg = sg0 + blockIdx.y, n = I.n, lo0 = blockIdx.x * 32, t = threadIdx.x, lane = t & 31, w = t >> 5;
     if (t < LOGH) {  // the rotations in scaled form; their factors are applied at the store
         float c, sn;
-        shift_angle<float>(I, s, layer * n + LOQ + t, c, sn);
+        shift_angle<float>(I, sg, layer * n + LOQ + t, c, sn);
         const RyScaled q = ry_scaled(c, sn);
         rq[t] = q.r;
         fq[t] = q.fac;
         sfq[t] = q.sform;
     }
-    float* st = reinterpret_cast<float*>(I.states) + s * N + lo0 + lane;
+    const float* src;
+    float* st;
+    hbm_io<float>(I, sg, layer, true, src, st);
+    src += lo0 + lane;
+    st += lo0 + lane;
     float v[RG];
 #pragma unroll
-    for (int r = 0; r < RG; ++r) v[r] = st[(size_t)((r << 3) | w) << LOQ];
+    for (int r = 0; r < RG; ++r) v[r] = src[(size_t)((r << 3) | w) << LOQ];
     __syncthreads();
 #pragma unroll
     for (int kb = 0; kb < LOGH - 3; ++kb)  // h bit 3 + kb: qubit 15 + kb, register bit kb
@@ -808,35 +889,64 @@ __global__ void __launch_bounds__(256) k_hbm_hi_regs(const Inst* __restrict__ in
     for (int r = 0; r < RG; ++r) st[(size_t)((w << (LOGH - 3)) | r) << LOQ] = v[r] * fac;
 }
 
+// States of the shifts s0 .. s0 + S - 1 of instance idx (its record in device
+// memory has `chain` unless S = 1 and s0 = 0).
 template <typename R>
-int build_hbm_states(dvqls_ctx* ctx, const Inst* dtable, int idx, int n, int d, int S, bool marks) {
+int build_hbm_states(dvqls_ctx* ctx, cudaStream_t st, const Inst* dtable, int idx, int n, int d, int s0, int S, bool marks) {
     const int chunks = 1 << (n - LOQ), tiles = LOC / HC;
     const size_t lo_smem = sizeof(R) * LOC, hi_smem = sizeof(R) * ((size_t)chunks * HC);
     DVQLS_CUDA_TRY(ctx, allow_dynamic_smem((const void*)k_hbm_lo<R>));
     DVQLS_CUDA_TRY(ctx, allow_dynamic_smem((const void*)k_hbm_hi<R>));
-    if (marks) prof_begin(ctx, 3);  // one profiling mark per kernel
-    k_hbm_init<R><<<dim3(chunks, S), 256, 0, ctx->stream>>>(dtable, idx);
-    if (marks) prof_end(ctx);
-    for (int layer = 1; layer <= d; ++layer) {
+    // one profiling mark per kernel
+    auto init = [&](int sg0, int count) -> int {
+        if (marks) prof_begin(ctx, 3);
+        DVQLS_CUDA_TRY(ctx, launch_pdl(k_hbm_init<R>, dim3(chunks, count), dim3(256), 0, st, dtable, idx, sg0));
+        if (marks) prof_end(ctx);
+        return DVQLS_OK;
+    };
+    auto lo = [&](int layer, int sg0, int count) -> int {
         if (marks) prof_begin(ctx, 3);
         if constexpr (sizeof(R) == 4)
-            k_hbm_lo_regs<<<dim3(chunks, S), 256, 0, ctx->stream>>>(dtable, idx, layer);
+            DVQLS_CUDA_TRY(ctx, launch_pdl(k_hbm_lo_regs, dim3(chunks, count), dim3(256), 0, st, dtable, idx, layer, sg0));
         else
-            k_hbm_lo<R><<<dim3(chunks, S), 256, lo_smem, ctx->stream>>>(dtable, idx, layer);
+            DVQLS_CUDA_TRY(ctx, launch_pdl(k_hbm_lo<R>, dim3(chunks, count), dim3(256), lo_smem, st, dtable, idx, layer, sg0));
         if (marks) prof_end(ctx);
+        return DVQLS_OK;
+    };
+    auto hi = [&](int layer, int sg0, int count) -> int {
         if (marks) prof_begin(ctx, 3);
+        const dim3 g(LOC / 32, count);
         if (sizeof(R) == 4 && n == 20)
-            k_hbm_hi_regs<8><<<dim3(LOC / 32, S), 256, 0, ctx->stream>>>(dtable, idx, layer);
+            DVQLS_CUDA_TRY(ctx, launch_pdl(k_hbm_hi_regs<8>, g, dim3(256), 0, st, dtable, idx, layer, sg0));
         else if (sizeof(R) == 4 && n == 19)
-            k_hbm_hi_regs<7><<<dim3(LOC / 32, S), 256, 0, ctx->stream>>>(dtable, idx, layer);
+            DVQLS_CUDA_TRY(ctx, launch_pdl(k_hbm_hi_regs<7>, g, dim3(256), 0, st, dtable, idx, layer, sg0));
         else if (sizeof(R) == 4 && n == 18)
-            k_hbm_hi_regs<6><<<dim3(LOC / 32, S), 256, 0, ctx->stream>>>(dtable, idx, layer);
+            DVQLS_CUDA_TRY(ctx, launch_pdl(k_hbm_hi_regs<6>, g, dim3(256), 0, st, dtable, idx, layer, sg0));
         else
-            k_hbm_hi<R><<<dim3(tiles, S), 256, hi_smem, ctx->stream>>>(dtable, idx, layer);
+            DVQLS_CUDA_TRY(ctx, launch_pdl(k_hbm_hi<R>, dim3(tiles, count), dim3(256), hi_smem, st, dtable, idx, layer, sg0));
         if (marks) prof_end(ctx);
+        return DVQLS_OK;
+    };
+    const int end = s0 + S, deepest = end > 1 ? (end - 2) / 2 / n : 0;  // the last layer with a shifted angle
+    int rc = init(0, 1);
+    // the unshifted state: to the end when it is wanted, else as far as a shift starts from it
+    for (int layer = 1; layer <= (s0 == 0 ? d : deepest) && !rc; ++layer) {
+        rc = lo(layer, 0, 1);
+        if (!rc) rc = hi(layer, 0, 1);
     }
-    DVQLS_CUDA_TRY(ctx, cudaGetLastError());
-    return DVQLS_OK;
+    const int group = (int)std::max<size_t>(1, HBM_GROUP / (sizeof(R) << n));
+    for (int g0 = std::max(1, s0); g0 < end && !rc; g0 += group) {
+        const int g1 = std::min(end, g0 + group);
+        // shifts below sg1: 2 n per layer, the two of a qubit side by side
+        auto below = [&](int sg1) { return std::min(g1, sg1) - g0; };
+        if (below(2 * n + 1) > 0) rc = init(g0, below(2 * n + 1));
+        for (int layer = std::max(1, (g0 - 1) / 2 / n); layer <= d && !rc; ++layer) {
+            const int cl = below(2 * n * layer + 1 + 2 * LOQ), ch = below(2 * n * (layer + 1) + 1);
+            if (cl > 0) rc = lo(layer, g0, cl);
+            if (!rc && ch > 0) rc = hi(layer, g0, ch);
+        }
+    }
+    return rc;
 }
 
 // Amplitudes per work item for states in HBM (each FP32 sum runs over half
@@ -3069,7 +3179,7 @@ __global__ void __launch_bounds__(NT) k_combine_partials(const double* __restric
 
 // ------------------------------------------------------------------- host
 struct HostInst {
-    int n, d, L, P, S, T, ks, F;
+    int n, d, L, P, S, T, ks, F, s0;
     long long N;
     int order;  // position in the caller's array
     bool hbm;   // n > 12: states built in HBM
@@ -3103,24 +3213,6 @@ struct PassShape {
     int bop_fused;   // 1: those CTAs are part of k_prepare (every state has <= TC_BOP_FUSED_N amplitudes)
 };
 
-// Launch with programmatic stream serialization (the kernel starts with
-// pdl_wait, so it observes everything its predecessor wrote).
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                              Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
-}
-
 // The kernel sequence of one cost pass on stream `st`: queue reset, prepare,
 // state passes of the instances with states in HBM, term tiles, combine.
 static int launch_pass(dvqls_ctx* ctx, cudaStream_t st, const Inst* dtable, const PassShape& ps,
@@ -3151,11 +3243,8 @@ static int launch_pass(dvqls_ctx* ctx, cudaStream_t st, const Inst* dtable, cons
     for (int oi = 0; oi < ps.count; ++oi) {
         const HostInst& h = *tab[oi];
         if (!h.hbm) continue;
-        cudaStream_t keep = ctx->stream;
-        ctx->stream = st;
-        const int rc = ps.fp32 ? build_hbm_states<float>(ctx, dtable, oi, h.n, h.d, h.S, marks)
-                               : build_hbm_states<double>(ctx, dtable, oi, h.n, h.d, h.S, marks);
-        ctx->stream = keep;
+        const int rc = ps.fp32 ? build_hbm_states<float>(ctx, st, dtable, oi, h.n, h.d, h.s0, h.S, marks)
+                               : build_hbm_states<double>(ctx, st, dtable, oi, h.n, h.d, h.s0, h.S, marks);
         if (rc) return rc;
     }
     if (marks) prof_begin(ctx, 1);
@@ -3273,6 +3362,7 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
                                  range->s1, h.S);
             h.S = range->s1 - range->s0;
         }
+        h.s0 = range ? range->s0 : 0;
         h.T = ceil_div(L, TT);
         h.N = 1LL << n;
         h.order = i;
@@ -3362,7 +3452,7 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
     struct Off {
         size_t coef, xm, zm, alpha, b;       // staged inputs (ws) ...
         size_t pcoef, pxm, pzm, palpha, pb;  // ... and their pinned slots
-        size_t ctil, w, wf, cf, bop, wht, bf, cs, bn2, Dp, Tp, Gp, dp, NsDs, cost, grad, beta, delta, states, tcst;
+        size_t ctil, w, wf, cf, bop, wht, bf, cs, bn2, Dp, Tp, Gp, dp, NsDs, cost, grad, beta, delta, states, chain, tcst;
         size_t pcost, pgrad, pbeta, pdelta;
     };
     std::vector<Off> off(count);
@@ -3428,6 +3518,7 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
         o.dp = delta_out ? ar.reserve(size_t(kp) * L * r2) : 0;
         o.NsDs = ar.reserve(size_t(h.S) * 24);
         o.states = h.hbm ? ar.reserve(size_t(h.S) * size_t(h.N) * (r2 / 2)) : 0;  // real amplitudes
+        o.chain = h.hbm && h.S + h.s0 > 1 ? ar.reserve((2 * size_t(h.d) + 1) * size_t(h.N) * (r2 / 2)) : 0;
         o.tcst = tc && !h.hbm ? ar.reserve(size_t(h.S) * size_t(h.N) * 4) : 0;     // packed FP16 pairs
     }
     int rc = ensure_workspace(ctx, ar.total());
@@ -3500,6 +3591,7 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
         I.dpart = delta_out ? (void*)(ws + o.dp) : nullptr;
         I.NsDs = (double*)(ws + o.NsDs);
         I.states = h.hbm ? (void*)(ws + o.states) : nullptr;
+        I.chain = h.hbm && h.S + h.s0 > 1 ? (void*)(ws + o.chain) : nullptr;
         I.tcst = tc && !h.hbm ? (void*)(ws + o.tcst) : nullptr;
         // Device outputs are written in place by the combine kernel.
         I.cost = dev_cost ? costs + i : (double*)(ws + o.cost);
@@ -3775,7 +3867,7 @@ int fidelity_hbm(dvqls_ctx* ctx, int n, int d, const double* alpha, const double
     rc = pin_release(ctx);
     if (rc) return rc;
     k_fid_angles<<<1, FIDH_T, 0, ctx->stream>>>(dt, ctx->d_status);
-    rc = build_hbm_states<double>(ctx, dt, 0, n, d, 1, false);
+    rc = build_hbm_states<double>(ctx, ctx->stream, dt, 0, n, d, 0, 1, false);
     if (rc) return rc;
     k_fid_partial<<<nb, FIDH_T, 0, ctx->stream>>>(dt, xd, (double*)(ctx->ws + o_pt));
     k_fid_final<<<1, 32, 0, ctx->stream>>>((const double*)(ctx->ws + o_pt), nb, ctx->d_status,

@@ -99,3 +99,28 @@ def test_split_rejects_bad_ranges(dv, ctx):
         dv.dvqls_combine_partials(ctx, n, d, zero, torch.zeros(1, device="cuda", dtype=torch.float64),
                                   torch.zeros(n * (d + 1), device="cuda", dtype=torch.float64))
     assert e.value.code == dv.DVQLS_ERR_NUMERIC
+
+
+@pytest.mark.parametrize("prec", [0, 1, 2])
+def test_ranges_that_start_inside_the_ansatz(dv, ctx, prec):
+    """States in HBM start from the unshifted state at the layer (and, for
+    qubits 12.., the half layer) of their angle: ranges that begin and end on
+    low and high qubits of every layer, without shift 0, add up to the whole."""
+    n, d, L = 14, 2, 3
+    rng = np.random.default_rng(21)
+    N, P = 1 << n, n * (d + 1)
+    xs, zs = rng.integers(0, N, L).astype(np.uint32), rng.integers(0, N, L).astype(np.uint32)
+    coef = np.ascontiguousarray(rng.normal(size=L) + 1j * rng.normal(size=L)).view(np.float64)
+    b = np.ascontiguousarray(rng.normal(size=N) + 1j * rng.normal(size=N)).view(np.float64)
+    alpha = rng.uniform(-np.pi, np.pi, P)
+    an, lcu = dv.make_ansatz(n, d), dv.make_lcu(L, coef, xs, zs)
+    whole = np.zeros((2 * P + 1, 4))
+    dv.dvqls_cost_grad_partials(ctx, an, alpha, lcu, b, prec, 0, 2 * P + 1, whole)
+    cuts = [0, 1, 2 * 13 + 1, 2 * n + 1, 2 * n + 24, 2 * (n + 13), 4 * n, 4 * n + 2, 2 * P, 2 * P + 1]
+    got = np.zeros_like(whole)
+    for a, e in zip(cuts[:-1], cuts[1:]):
+        part = np.zeros_like(whole)
+        dv.dvqls_cost_grad_partials(ctx, an, alpha, lcu, b, prec, a, e, part)
+        assert np.all(part[:a] == 0) and np.all(part[e:] == 0)
+        got += part
+    assert np.array_equal(got, whole)  # the same operations on every amplitude
