@@ -51,14 +51,13 @@ __device__ double2 block_sum2_all(double2 v, double2* red) {
     return s;
 }
 
-// One CTA per instance; the FP64 state build (build_state_f64) bounds it.
+// One CTA per instance; the state in fixed point (build_state_fx), the overlap in FP64.
 __global__ void __launch_bounds__(FT) k_fidelity(const FidInst* __restrict__ insts, int* status) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ double2 red[FT / 32];
     __shared__ double rnx[FT / 32];
     const FidInst I = insts[blockIdx.x];
     const int N = 1 << I.n;
-    double* psi = reinterpret_cast<double*>(smem);
     for (int a = threadIdx.x; a < I.P; a += FT) {
         const double al = I.alpha[a];
         if (!isfinite(al)) atomicCAS(status, 0, DEV_NONFINITE_INPUT);
@@ -67,11 +66,11 @@ __global__ void __launch_bounds__(FT) k_fidelity(const FidInst* __restrict__ ins
         I.cs[a] = make_double2(c, s);
     }
     __syncthreads();
-    build_state_f64(psi, I.n, I.d, I.P, I.cs, 0);
+    const Fx* psi = build_state_fx(smem, I.n, I.d, I.P, I.cs, 0);
     double2 ov = make_double2(0.0, 0.0), nx = make_double2(0.0, 0.0);
     for (int j = threadIdx.x; j < N; j += FT) {
         const double2 x = I.xhat[j];
-        const double p = psi[f64_pad(j)];  // the state is real
+        const double p = fx_to(psi[j]);  // the state is real
         ov.x += x.x * p;  // conj(x) p
         ov.y -= x.y * p;
         nx.x += x.x * x.x + x.y * x.y;
@@ -572,7 +571,7 @@ extern "C" int dvqls_fidelity(dvqls_ctx* ctx, const dvqls_ansatz* an, const doub
     I.F = (double*)(ctx->ws + o_F);
     memcpy(ctx->pin + p_t, &I, sizeof I);
     DVQLS_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->ws + o_t, ctx->pin + p_t, sizeof I, cudaMemcpyHostToDevice, ctx->stream));
-    const size_t smem = f64_state_doubles(n, P) * 8;
+    const size_t smem = fx_smem(n, P);
     DVQLS_CUDA_TRY(ctx, allow_dynamic_smem((const void*)k_fidelity));
     k_fidelity<<<1, FT, smem, ctx->stream>>>((const FidInst*)(ctx->ws + o_t), ctx->d_status);
     DVQLS_CUDA_TRY(ctx, cudaGetLastError());
@@ -998,7 +997,7 @@ static int optimize(dvqls_ctx* ctx, int count, const dvqls_instance* inst, const
         results[i].fidelity = NAN;
     }
     size_t fsmem = 0;
-    for (int i = 0; i < count; ++i) fsmem = std::max(fsmem, f64_state_doubles(inst[i].ansatz.n, P[i]) * 8);
+    for (int i = 0; i < count; ++i) fsmem = std::max(fsmem, fx_smem(inst[i].ansatz.n, P[i]));
     DVQLS_CUDA_TRY(ctx, allow_dynamic_smem((const void*)k_fidelity));
     std::vector<int> active(count);
     for (int i = 0; i < count; ++i) active[i] = i;

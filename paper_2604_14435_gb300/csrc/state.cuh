@@ -352,77 +352,152 @@ __device__ inline void build_state_regs(void* psi, float* scratch, float2* scs, 
     group_sync(bar, 256);
 }
 
-// ---- FP64 state in shared memory for 256 threads, n <= 12.
+// ---- The state in 64-bit fixed point, for 256 threads, n <= 12 (FP64 precision).
 //
-// FP64 instructions bound it (they issue at 1/64 of the FP32 rate), so the Ry
-// rotations run in the scaled form of ry_scaled (one FMA per amplitude instead
-// of two instructions), NB qubits per pass over 2^NB amplitudes in registers,
-// with one multiply per amplitude and layer for the product of the layer's
-// factors, and the initial product state comes from two factor tables.
-// Amplitude i sits at word i + (i >> 4).
-__host__ __device__ inline int f64_pad(int i) { return i + (i >> 4); }
-// Doubles: psi, the rotations, a factor per layer, the two factor tables.
-__host__ __device__ inline size_t f64_state_doubles(int n, int P) {
-    const size_t N = size_t(1) << n;
-    return N + (N >> 4) + P + (P / n - 1) + (N < 32 ? N : 32) + (N < 32 ? 1 : N >> 5);
+// FP64 instructions issue at 1/64 of the FP32 rate, six integer multiply-adds
+// and a shift in less time than one of them.  The state has norm
+// one, so every amplitude and every cos and sin is h 2^30 + l in units of 2^-60
+// (|h| <= 2^30, l in [-2^29, 2^29)), and c a + t b is six multiply-adds and a
+// shift, rounded to nearest at 2^-60; the two products of low parts, below a
+// quarter of that unit and of mean zero, are dropped.  An FP64 rotation rounds an
+// amplitude near 2^-5 (the mean at n = 10) at 2^-58, so this is no less exact
+// (gradients of 48 systems of n = 6..10 against a 64-bit reference: 8.5e-16
+// relative, FP64 states 1.1e-15).
+// n = 10, depth 4: 20 k cycles for a state and CTA, 60 k in FP64 with the state in
+// shared memory.
+constexpr int FX_BITS = 60;
+struct Fx {
+    int h, l;
+};
+__device__ __forceinline__ Fx fx_split(long long y) {  // y: the value + 2^29
+    Fx r;
+    r.h = int(y >> 30);
+    r.l = int(uint32_t(y) & 0x3FFFFFFFu) - (1 << 29);
+    return r;
+}
+__device__ __forceinline__ Fx fx_from(double v) { return fx_split(__double2ll_rn(v * 0x1p60) + (1LL << 29)); }
+__device__ __forceinline__ double fx_to(Fx a) { return double((long long)a.h * (1LL << 30) + a.l) * 0x1p-60; }
+__device__ __forceinline__ Fx fx_neg(Fx a) { return Fx{-a.h, -a.l}; }  // l = -2^29 gives 2^29, which the products take
+// a b in units of 2^-60, rounded to nearest.
+__device__ __forceinline__ long long fx_mul(Fx a, Fx b) {
+    const long long x = (1LL << 29) + (long long)a.h * b.l + (long long)a.l * b.h;
+    return (x >> 30) + (long long)a.h * b.h;
+}
+// c a + t b, rounded; |c a + t b| <= 1.
+__device__ __forceinline__ Fx fx_rot(Fx a, Fx b, Fx c, Fx t) {
+    // 2^59 carries the 2^29 that fx_split wants
+    const long long x = ((1LL << 29) + (1LL << 59)) + (long long)a.h * c.l + (long long)a.l * c.h + (long long)b.h * t.l +
+                        (long long)b.l * t.h;
+    return fx_split((x >> 30) + (long long)a.h * c.h + (long long)b.h * t.h);
 }
 
-// Scaled rotation of (c, s): |r| <= 1 leaves bit 62 of r free for the form.
-__device__ __forceinline__ double f64_rot(double c, double s) {
-    const bool sf = fabs(c) < fabs(s);
-    const double r = sf ? c / s : s / c;
-    return __hiloint2double(__double2hiint(r) | (sf ? 0x40000000 : 0), __double2loint(r));
-}
-
-template <int NB>
-__device__ __forceinline__ void f64_pass(double* psi, int n, int b, const double* rot, int t, bool first,
-                                         const double* lowt, const double* hight, double fac) {
-    for (int g = t; g < (1 << n) >> NB; g += 256) {
-        const int i0 = ((g >> b) << (b + NB)) | (g & ((1 << b) - 1));
-        double v[1 << NB];
+// Ry of the qubits on lane bits 0 .. nb - 1 (first qubit q0) and register bits.
+template <int A>
+__device__ __forceinline__ void fx_lanes(Fx (&v)[A], int lane, int b0, int nb, const int4* ang) {
+    for (int j = 0; j < nb; ++j) {
+        const int4 q = ang[j];
+        const Fx c{q.x, q.y}, sn{q.z, q.w}, t = (lane >> (b0 + j)) & 1 ? sn : fx_neg(sn);
 #pragma unroll
-        for (int r = 0; r < (1 << NB); ++r) {
-            const int i = i0 | (r << b);
-            v[r] = lowt ? lowt[i & 31] * hight[i >> 5] : psi[f64_pad(i)];
-            if (first)  // the CZ ring, applied while loading the layer's first pass
-                v[r] = __hiloint2double(__double2hiint(v[r]) ^ (czring_parity(i, n) << 31), __double2loint(v[r]));
+        for (int r = 0; r < A; ++r) {
+            Fx p;
+            p.h = __shfl_xor_sync(0xffffffffu, v[r].h, 1 << (b0 + j));
+            p.l = __shfl_xor_sync(0xffffffffu, v[r].l, 1 << (b0 + j));
+            v[r] = fx_rot(v[r], p, c, t);
         }
-#pragma unroll
-        for (int k = 0; k < NB; ++k) {
-            const double w = rot[b + k];
-            const bool sf = __double2hiint(w) & 0x40000000;
-            const double q = __hiloint2double(__double2hiint(w) & ~0x40000000, __double2loint(w));
-#pragma unroll
-            for (int r = 0; r < (1 << NB); ++r)
-                if (!((r >> k) & 1)) {
-                    const double a0 = v[r], a1 = v[r | (1 << k)];
-                    if (sf) {
-                        v[r] = fma(q, a0, -a1);
-                        v[r | (1 << k)] = fma(q, a1, a0);
-                    } else {
-                        v[r] = fma(-q, a1, a0);
-                        v[r | (1 << k)] = fma(q, a0, a1);
-                    }
-                }
-        }
-        if (b + NB == n) {
-#pragma unroll
-            for (int r = 0; r < (1 << NB); ++r) v[r] *= fac;
-        }
-#pragma unroll
-        for (int r = 0; r < (1 << NB); ++r) psi[f64_pad(i0 | (r << b))] = v[r];
     }
-    __syncthreads();
+}
+template <int A, int LOGA>
+__device__ __forceinline__ void fx_regs(Fx (&v)[A], const int4* ang) {
+#pragma unroll
+    for (int kb = 0; kb < LOGA; ++kb) {
+        const int4 q = ang[kb];
+        const Fx c{q.x, q.y}, sn{q.z, q.w}, ns = fx_neg(sn);
+#pragma unroll
+        for (int r = 0; r < A; ++r)
+            if (!((r >> kb) & 1)) {
+                const Fx a0 = v[r], a1 = v[r | (1 << kb)];
+                v[r] = fx_rot(a0, a1, c, ns);
+                v[r | (1 << kb)] = fx_rot(a1, a0, c, sn);
+            }
+    }
+}
+__device__ __forceinline__ Fx fx_sign(Fx a, int flip) { return flip ? fx_neg(a) : a; }
+
+// Place of element i in a transpose buffer: both mappings below take a
+// half-warp's 16 elements to 16 different bank pairs.
+__device__ __forceinline__ int fx_at(int i) { return i ^ ((i >> 4) & 15); }
+// Shared memory of build_state_fx, in bytes: P angles of 16 bytes and two buffers
+// of 2^n amplitudes.
+__host__ __device__ inline size_t fx_smem(int n, int P) { return 16 * (size_t(P) + (size_t(1) << n)); }
+
+// n >= 8: A = 2^n / 256 amplitudes per thread.  Mapping 0: i = (r << 8) | (w << 5) |
+// lane (qubits 0..4 on lanes, 5..7 on warps), mapping 1: i = (r << 8) | (lane << 3) | w
+// (3..7 on lanes, 0..2 on warps); one transpose per layer brings the three
+// qubits of the warp bits onto lanes, alternating the mappings, as
+// state_regs_multiwarp.
+template <int A, int LOGA>
+__device__ void fx_multiwarp(Fx* out, Fx* scr, const int4* ang, const Fx* lowt, const Fx* hight, int n, int d, int t) {
+    const int lane = t & 31, w = t >> 5, N = 1 << n;
+    auto index = [&](int M, int r) { return M == 0 ? (r << 8) | (w << 5) | lane : (r << 8) | (lane << 3) | w; };
+    Fx v[A];
+#pragma unroll
+    for (int r = 0; r < A; ++r) {
+        const int i = index(0, r);
+        v[r] = fx_split(fx_mul(lowt[i & 31], hight[i >> 5]) + (1LL << 29));
+    }
+    int M = 0;
+    for (int layer = 1; layer <= d; ++layer) {
+        const int4* la = ang + layer * n;
+#pragma unroll
+        for (int r = 0; r < A; ++r) v[r] = fx_sign(v[r], czring_parity(index(M, r), n));
+        fx_lanes<A>(v, lane, 0, 5, la + (M == 0 ? 0 : 3));
+        fx_regs<A, LOGA>(v, la + 8);
+        Fx* buf = scr + (layer & 1) * N;
+#pragma unroll
+        for (int r = 0; r < A; ++r) buf[fx_at(index(M, r))] = v[r];
+        __syncthreads();
+        M ^= 1;
+#pragma unroll
+        for (int r = 0; r < A; ++r) v[r] = buf[fx_at(index(M, r))];
+        // mapping 0: lanes 0..2 hold qubits 0..2; mapping 1: lanes 2..4 hold qubits 5..7
+        fx_lanes<A>(v, lane, M == 0 ? 0 : 2, 3, la + (M == 0 ? 0 : 5));
+    }
+#pragma unroll
+    for (int r = 0; r < A; ++r) out[index(M, r)] = v[r];
 }
 
-// psi(alpha_s) in FP64: buf holds f64_state_doubles(n, P) doubles, psi first.
-// cs as for build_state_real.  Ends with a barrier.  Whole CTA of 256 threads.
-__device__ inline void build_state_f64(double* buf, int n, int d, int P, const double2* cs, int s) {
+// n <= 7: one warp holds the state, A = max(1, 2^n / 32) amplitudes per lane.
+template <int A, int LOGA>
+__device__ void fx_warp(Fx* out, const int4* ang, const Fx* lowt, const Fx* hight, int n, int d, int lane) {
+    const int N = 1 << n, li = N < 32 ? lane & (N - 1) : lane, nl = n < 5 ? n : 5;
+    Fx v[A];
+#pragma unroll
+    for (int r = 0; r < A; ++r) v[r] = fx_split(fx_mul(lowt[li], hight[r]) + (1LL << 29));
+    for (int layer = 1; layer <= d; ++layer) {
+        const int4* la = ang + layer * n;
+#pragma unroll
+        for (int r = 0; r < A; ++r) v[r] = fx_sign(v[r], czring_parity((r << 5) | li, n));
+        fx_lanes<A>(v, lane, 0, nl, la);
+        fx_regs<A, LOGA>(v, la + 5);
+    }
+    __syncwarp();  // the tables are read: out may lie over their end
+    if (lane < N || N >= 32) {
+#pragma unroll
+        for (int r = 0; r < A; ++r) out[(r << 5) | lane] = v[r];
+    }
+}
+
+// psi(alpha_s): returns where its 2^n amplitudes lie in smem (fx_smem(n, P)
+// bytes).  cs as for build_state_real.  Whole CTA of 256 threads; ends with a
+// barrier.
+__device__ inline Fx* build_state_fx(unsigned char* smem, int n, int d, int P, const double2* cs, int s) {
     const int N = 1 << n, t = threadIdx.x;
-    double* rot = buf + N + (N >> 4);
-    double* facs = rot + P;
-    double* lowt = facs + d;
-    double* hight = lowt + (N < 32 ? N : 32);
+    int4* angw = reinterpret_cast<int4*>(smem);
+    Fx* scr = reinterpret_cast<Fx*>(angw + P);  // two buffers; the factor tables start in the one first written at layer 2
+    Fx* lowt = scr;
+    Fx* hight = lowt + (N < 32 ? N : 32);
+    // the result: not the buffer of the last transpose, whose reads may still go on
+    Fx* out = scr + (n < 8 ? 1 : (d + 1) & 1) * N;
     int k = -1, which = 0;
     if (s > 0) {
         k = (s - 1) >> 1;
@@ -431,49 +506,39 @@ __device__ inline void build_state_f64(double* buf, int n, int d, int P, const d
     auto angle = [&](int a) { return cs[(a == k ? which : 0) * P + a]; };
     for (int a = n + t; a < P; a += 256) {
         const double2 v = angle(a);
-        rot[a] = f64_rot(v.x, v.y);
+        const Fx c = fx_from(v.x), sn = fx_from(v.y);
+        angw[a] = make_int4(c.h, c.l, sn.h, sn.l);
     }
-    for (int layer = 1 + (t ^ 255); layer <= d; layer += 256) {  // the last threads: the first ones hold rotations
-        double f = 1.0;
-        for (int q = 0; q < n; ++q) {
-            const double2 v = angle(layer * n + q);
-            f *= fabs(v.x) < fabs(v.y) ? v.y : v.x;
-        }
-        facs[layer - 1] = f;
-    }
-    auto bits = [&](int i, int q0, int q1) {  // factors of qubits q0 .. q1 - 1 of the product state
+    // the initial Ry layer on |0> is a product state: factors of qubits 0..4 and of the others
+    const int nl = n < 5 ? n : 5, nh = N >> nl;
+    const int nlow = 1 << nl;
+    for (int e = t ^ 255; e < nlow + nh; e += 256) {
+        const bool lo = e < nlow;
+        const int i = lo ? e : e - nlow, q0 = lo ? 0 : nl, q1 = lo ? nl : n;
         double v = 1.0;
         for (int q = q0; q < q1; ++q) {
             const double2 c = angle(q);
             v *= ((i >> (q - q0)) & 1) ? c.y : c.x;
         }
-        return v;
-    };
-    const int nl = n < 5 ? n : 5, nh = N >> nl;
-    if (t >= 64 && t - 64 < (1 << nl)) lowt[t - 64] = bits(t - 64, 0, nl);
-    if (t >= 96 && t - 96 < nh) hight[t - 96] = bits(t - 96, nl, n);
+        (lo ? lowt : hight)[i] = fx_from(v);
+    }
     __syncthreads();
-    if (d == 0) {
-        for (int i = t; i < N; i += 256) buf[f64_pad(i)] = lowt[i & 31] * hight[i >> 5];
-        __syncthreads();
-        return;
-    }
-    // qubits per pass: at least 128 groups where the state has them (four warps, one per scheduler)
-    const int nb = n <= 9 ? 2 : n == 10 ? 3 : 4;
-    for (int layer = 1; layer <= d; ++layer) {
-        const double* lr = rot + layer * n;
-        const double fac = facs[layer - 1];
-        for (int b = 0; b < n; b += nb) {
-            const bool first = b == 0;
-            const double* tab = first && layer == 1 ? lowt : nullptr;
-            switch (min(nb, n - b)) {
-                case 1: f64_pass<1>(buf, n, b, lr, t, first, tab, hight, fac); break;
-                case 2: f64_pass<2>(buf, n, b, lr, t, first, tab, hight, fac); break;
-                case 3: f64_pass<3>(buf, n, b, lr, t, first, tab, hight, fac); break;
-                default: f64_pass<4>(buf, n, b, lr, t, first, tab, hight, fac); break;
+    switch (n) {
+        case 8: fx_multiwarp<1, 0>(out, scr, angw, lowt, hight, n, d, t); break;
+        case 9: fx_multiwarp<2, 1>(out, scr, angw, lowt, hight, n, d, t); break;
+        case 10: fx_multiwarp<4, 2>(out, scr, angw, lowt, hight, n, d, t); break;
+        case 11: fx_multiwarp<8, 3>(out, scr, angw, lowt, hight, n, d, t); break;
+        case 12: fx_multiwarp<16, 4>(out, scr, angw, lowt, hight, n, d, t); break;
+        default:
+            if (t < 32) {
+                if (n == 7) fx_warp<4, 2>(out, angw, lowt, hight, n, d, t);
+                else if (n == 6) fx_warp<2, 1>(out, angw, lowt, hight, n, d, t);
+                else fx_warp<1, 0>(out, angw, lowt, hight, n, d, t);
             }
-        }
+            break;
     }
+    __syncthreads();
+    return out;
 }
 
 }  // namespace dvqls

@@ -57,7 +57,7 @@ struct Inst {
     float4* cf;      // L or null: ctil as float pairs
     void* bop;       // tensor-core tiles: the b rows of the B operand, TC_BOP_STAGE bytes per stage, or null
     void* wht;       // Walsh-Hadamard classes: the class table (WHT_TABLE_BYTES), or null
-    void* bf;        // Walsh-Hadamard classes: b as float2, or in fixed point as longlong2 (FP64), or null
+    void* bf;        // Walsh-Hadamard classes: b as float2, or in fixed point as int4 (FP64), or null
     double2* cs;     // 3P: (cos, sin) of half angles: base, +pi/2, -pi/2
     double* bn2;     // ||b||^2
     double2* Dpart;  // S*T*T*ks
@@ -2289,7 +2289,7 @@ constexpr int WHT_MAXP = 64 * 65 / 2;  // pairs l <= m of a 64-term LCU
 constexpr int WHT_NT = 256;
 constexpr int WHT_MAXN = 10;
 constexpr int WHT_CT = 1024;  // threads of the class-table kernel
-// Per-instance class table, built on the device by k_wht_classes (bytes):
+// Per-instance class table, built on the device by k_wht_prepare (bytes):
 constexpr size_t WHT_OFF_CX = 16;                                   // uint32 class masks [WHT_MAXP]
 constexpr size_t WHT_OFF_CO = WHT_OFF_CX + 4 * WHT_MAXP;            // int class offsets [WHT_MAXP + 1]
 constexpr size_t WHT_OFF_PR = WHT_OFF_CO + 4 * (WHT_MAXP + 1);      // uint16 pairs l | m << 8 by class
@@ -2299,217 +2299,230 @@ constexpr size_t WHT_OFF_DT = WHT_OFF_DO + 4 * 65;                  // uint16 te
 constexpr size_t WHT_OFF_EZ = (WHT_OFF_DT + 2 * 64 + 15) & ~size_t(15);  // uint16 z_l ^ z_m by class
 constexpr size_t WHT_OFF_EK = (WHT_OFF_EZ + 2 * WHT_MAXP + 15) & ~size_t(15);  // signed weights by class: float2, or
                                                                                // double (FP64)
-constexpr size_t WHT_OFF_KEY = WHT_OFF_EK + 8 * WHT_MAXP;  // the inputs the table was built from: int L (negative
-                                                              // for FP64 weights), uint32 x[64], z[64], double2 coef[64]
-constexpr size_t WHT_OFF_SUM = WHT_OFF_KEY + 16 + 8 * 64 + 16 * 64;  // uint64 checksum of bytes [0, WHT_OFF_SUM)
-constexpr size_t WHT_OFF_BIM = WHT_OFF_SUM + 8;  // int: b has a nonzero imaginary part (rewritten every call)
-constexpr size_t WHT_TABLE_BYTES = WHT_OFF_SUM + 16;                   // header: int pair classes, term classes
-
-// 64-bit checksum of a table (sum of mixed, position-tagged 32-bit words;
-// valid in every thread of the block).
-__device__ inline unsigned long long wht_checksum(const unsigned char* tb, unsigned long long* red) {
-    const uint32_t* wds = reinterpret_cast<const uint32_t*>(tb);
-    unsigned long long h = 0;
-    for (int i = threadIdx.x; i < int(WHT_OFF_SUM / 4); i += blockDim.x) {
-        unsigned long long z = ((unsigned long long)wds[i] | ((unsigned long long)i << 32)) + 0x9E3779B97F4A7C15ull;
-        z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-        z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-        h += z ^ (z >> 31);
-    }
-    for (int o = 16; o; o >>= 1) h += __shfl_xor_sync(0xffffffffu, h, o);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = h;
-    __syncthreads();
-    unsigned long long s = 0;
-    for (int k = 0; k < int(blockDim.x >> 5); ++k) s += red[k];
-    return s;
-}
-
-// Fixed point of the FP64 classes: 1.0 = 2^W64_FRAC.  b is scaled by a power of
-// two so that ||b|| <= 1.
-constexpr int W64_FRAC = 62;
+constexpr size_t WHT_OFF_BIM = WHT_OFF_EK + 8 * WHT_MAXP;  // int: b has a nonzero imaginary part
+constexpr size_t WHT_TABLE_BYTES = WHT_OFF_BIM + 16;          // header: int pair classes, term classes
+// Fixed point of the FP64 classes (units of 2^-FX_BITS): b is scaled by a power
+// of two so that ||b|| <= 1.
 __device__ __forceinline__ int w64_bexp(double bn2) {
     int ex;
     frexp(sqrt(bn2), &ex);  // ||b|| <= 2^ex
     return min(max(ex, -1000), 1000);  // an invalid ||b||^2 is reported by k_prepare
 }
 
-// Class tables of one instance (one CTA of 256 per instance): pairs (l <= m)
-// sorted by x_l ^ x_m (bitonic sort of (mask, pair) keys), each with its
-// transform index z_l ^ z_m and its weight (-1)^popc(z_l & x) Re(w_lm),
-// doubled for l < m, as a float pair (or a double, F64); terms by x_l; and b as
-// float2 (or in fixed point, F64).  Runs after k_prepare (which forms the
-// weights).
+// What a class pass needs of one instance (one CTA each), in one launch: the
+// input checks, ||b||^2, c~, the half-angle tables and b as float2 (or in fixed
+// point, F64) -- k_prepare's part -- and the class table: the pairs (l <= m) by
+// x_l ^ x_m (within a class by m, then l), each with its transform index
+// z_l ^ z_m and its weight (-1)^popc(z_l & x) Re(w_lm), doubled for l < m, as a
+// float pair (or a double, F64); the terms by x_l.
+//
+// Masks are below 2^10, so the pairs are dealt to their classes by counting:
+// eight warps each rank a run of pairs within its classes (match_any finds the
+// lanes of one class, a count per warp and mask carries over), one scan over the
+// 1,024 masks gives every class its place.  A bitonic sort of 4,096 keys took 60 us,
+// and keeping the table from call to call under a checksum 16 us after k_prepare's
+// 8; this takes 15 in all (L = 64, n = 10).
+constexpr int WHT_RANK_WARPS = 8;  // warps 8 .. 15 rank, 0 .. 7 take b, 16 .. 31 the angles
+__device__ __forceinline__ void wht_pair(int e, int& l, int& m) {  // pair number e = m (m + 1) / 2 + l
+    m = int((sqrtf(8.f * float(e) + 1.f) - 1.f) * 0.5f);
+    if (m * (m + 1) / 2 > e) --m;
+    if ((m + 1) * (m + 2) / 2 <= e) ++m;
+    l = e - m * (m + 1) / 2;
+}
 template <bool F64>
-__global__ void __launch_bounds__(WHT_CT) k_wht_classes(const Inst* __restrict__ insts) {
-    pdl_wait();
+__global__ void __launch_bounds__(WHT_CT) k_wht_prepare(const Inst* __restrict__ insts, int* status,
+                                                        unsigned long long* queue) {
     pdl_trigger();
-    const Inst I = insts[blockIdx.x];
-    if (!I.wht) return;
-    __shared__ unsigned long long key[4096];
+    constexpr int BINS = 1 << WHT_MAXN;
+    static_assert(BINS == WHT_CT, "one thread per mask");
     __shared__ uint32_t sx[64], sz[64];
+    __shared__ double2 sc[64];
+    __shared__ unsigned short cnt[WHT_RANK_WARPS][BINS], rank[WHT_MAXP];
+    __shared__ int start[BINS], part[32], cpart[32];
+    __shared__ double red[8], s_bn2;
+    __shared__ int s_im;
+    __shared__ unsigned s_first[2];
+    const Inst I = insts[blockIdx.x];
+    const int L = I.L, t = threadIdx.x, w = t >> 5, lane = t & 31, np = L * (L + 1) / 2;
+    const int N = 1 << I.n, run = (np + WHT_RANK_WARPS - 1) / WHT_RANK_WARPS;
     unsigned char* tb = reinterpret_cast<unsigned char*>(I.wht);
-    const int L = I.L, t = threadIdx.x, np = L * (L + 1) / 2;
-    const long long N = 1LL << I.n;
-    bool im = false;
-    for (long long j = t; I.b && j < N; j += WHT_CT) {  // the local cost has no b here (|+>^n is implied)
-        const double2 v = I.b[j];
-        if (F64) {
-            const double sc = scalbn(1.0, W64_FRAC - w64_bexp(*I.bn2));
-            reinterpret_cast<longlong2*>(I.bf)[j] = make_longlong2(__double2ll_rn(v.x * sc), __double2ll_rn(v.y * sc));
-            im |= v.y != 0.0;
-        } else {
-            reinterpret_cast<float2*>(I.bf)[j] = make_float2((float)v.x, (float)v.y);
-            im |= (float)v.y != 0.f;
-        }
-    }
-    if (__syncthreads_or(im) != 0) {
-        if (t == 0) *reinterpret_cast<int*>(tb + WHT_OFF_BIM) = 1;
-    } else if (t == 0) {
-        *reinterpret_cast<int*>(tb + WHT_OFF_BIM) = 0;
-    }
-    if (t < 64) {
-        sx[t] = t < L ? I.xm[t] : 0u;
-        sz[t] = t < L ? I.zm[t] : 0u;
-    }
-    // The table is a function of L, the masks and the coefficients alone: when
-    // the copy kept with it matches them exactly, it is still valid.
-    int* kL = reinterpret_cast<int*>(tb + WHT_OFF_KEY);
-    uint32_t* kx = reinterpret_cast<uint32_t*>(tb + WHT_OFF_KEY + 16);
-    uint32_t* kz = kx + 64;
-    double2* kc = reinterpret_cast<double2*>(tb + WHT_OFF_KEY + 16 + 8 * 64);
-    bool differs = false;
+    if (queue && blockIdx.x == 0 && t == 0) *queue = 0ull;  // the term kernel's work queue
+    for (int k = t; k < WHT_RANK_WARPS * BINS / 2; k += WHT_CT) reinterpret_cast<uint32_t*>(cnt)[k] = 0u;
+    if (t == 0) s_im = 0;
     if (t < L) {
-        const double2 c = I.coef[t], k = kc[t];
-        differs = kx[t] != I.xm[t] || kz[t] != I.zm[t] || __double_as_longlong(c.x) != __double_as_longlong(k.x) ||
-                  __double_as_longlong(c.y) != __double_as_longlong(k.y);
-    }
-    const int tag = F64 ? -L : L;
-    if (t == 0 && *kL != tag) differs = true;
-    __shared__ unsigned long long red[WHT_CT / 32];
-    unsigned long long* ksum = reinterpret_cast<unsigned long long*>(tb + WHT_OFF_SUM);
-    if (!__syncthreads_or(differs) && wht_checksum(tb, red) == *ksum) return;  // still valid, untouched
-    int P2 = 2;  // the pairs are sorted within the next power of two
-    while (P2 < np) P2 <<= 1;
-    for (int e = np + t; e < 4096; e += WHT_CT) key[e] = ~0ull;
-    __syncthreads();
-    for (int q = t; q < L * L; q += WHT_CT) {  // pair (l, m), l <= m, at e = l L - l (l - 1) / 2 + m - l
-        const int l = q / L, m = q % L;
-        if (l <= m)
-            key[l * L - l * (l - 1) / 2 + (m - l)] =
-                ((unsigned long long)(sx[l] ^ sx[m]) << 16) | (unsigned long long)(l | (m << 8));
+        const uint32_t x = I.xm[t], z = I.zm[t];
+        const double2 c = I.coef[t];
+        if (x >= uint32_t(N) || z >= uint32_t(N)) set_status(status, DEV_BAD_MASK);
+        if (!isfinite(c.x) || !isfinite(c.y)) set_status(status, DEV_NONFINITE_INPUT);
+        sx[t] = x & uint32_t(N - 1);  // masks >= 2^n are reported, never followed
+        sz[t] = z & uint32_t(N - 1);
+        const double2 r = ctil_of(I, t);
+        sc[t] = r;
+        I.ctil[t] = r;
+        if (I.cf) I.cf[t] = split_ff(r);
     }
     __syncthreads();
-    for (int k = 2; k <= P2; k <<= 1)
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int e = t; e < P2; e += WHT_CT) {
-                const int p = e ^ j;
-                if (p > e) {
-                    const unsigned long long a = key[e], b = key[p];
-                    if (((e & k) == 0) == (a > b)) {
-                        key[e] = b;
-                        key[p] = a;
-                    }
-                }
+    double2 b[4];  // warps 0 .. 7: the instance's b (the local cost's is implied)
+    if (w < 8) {
+        double acc = !I.b && t == 0 ? 1.0 : 0.0;
+        bool im = false;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int j = t + 256 * k;
+            b[k] = I.b && j < N ? I.b[j] : make_double2(0.0, 0.0);
+            acc += b[k].x * b[k].x + b[k].y * b[k].y;
+            im |= F64 ? b[k].y != 0.0 : (float)b[k].y != 0.f;
+        }
+        for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (lane == 0) red[w] = acc;
+        if (im) s_im = 1;
+    } else if (w < 8 + WHT_RANK_WARPS) {
+        const int v = w - 8, e1 = min(np, (v + 1) * run);
+        unsigned short* c = cnt[v];
+        for (int e0 = v * run; e0 < e1; e0 += 32) {
+            const int e = e0 + lane;
+            const unsigned act = __ballot_sync(0xffffffffu, e < e1);
+            if (e < e1) {
+                int l, m;
+                wht_pair(e, l, m);
+                const uint32_t x = sx[l] ^ sx[m];
+                const unsigned same = __match_any_sync(act, x);
+                const int before = c[x];
+                rank[e] = (unsigned short)(before + __popc(same & ((1u << lane) - 1u)));
+                __syncwarp(act);
+                if (lane == __ffs(same) - 1) c[x] = (unsigned short)(before + __popc(same));
             }
-            __syncthreads();
+            __syncwarp();
         }
-    // Class numbers: a class starts where the mask changes; its number is the
-    // count of starts up to it (block prefix sum over 4096 / WHT_CT keys per
-    // thread).
-    constexpr int PER = 4096 / WHT_CT, LANE_N = WHT_CT / 32;
-    __shared__ int tsum[WHT_CT];
-    uint32_t* cx = reinterpret_cast<uint32_t*>(tb + WHT_OFF_CX);
-    int* co = reinterpret_cast<int*>(tb + WHT_OFF_CO);
-    uint16_t* pr = reinterpret_cast<uint16_t*>(tb + WHT_OFF_PR);
-    const int e0 = t * PER;
-    int cnt = 0;
-    for (int e = e0; e < e0 + PER; ++e)
-        if (e < np && (e == 0 || uint32_t(key[e] >> 16) != uint32_t(key[e - 1] >> 16))) ++cnt;
-    tsum[t] = cnt;
-    __syncthreads();
-    if (t < 32) {  // exclusive scan of the per-thread counts by one warp (LANE_N per lane)
-        int v[LANE_N], run = 0;
-        for (int q = 0; q < LANE_N; ++q) {
-            v[q] = run;
-            run += tsum[t * LANE_N + q];
+    } else {
+        for (int a = t - 512; a < I.P; a += 512) {
+            const double al = I.alpha[a];
+            if (!isfinite(al)) set_status(status, DEV_NONFINITE_INPUT);
+            double s0, c0;
+            sincos(0.5 * al, &s0, &c0);
+            const double s1 = (s0 + c0) * M_SQRT1_2, c1 = (c0 - s0) * M_SQRT1_2;  // alpha/2 +- pi/4, as in k_prepare
+            const double s2 = (s0 - c0) * M_SQRT1_2, c2 = (c0 + s0) * M_SQRT1_2;
+            I.cs[a] = make_double2(c0, s0);
+            I.cs[I.P + a] = make_double2(c1, s1);
+            I.cs[2 * I.P + a] = make_double2(c2, s2);
         }
-        int incl = run;
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (t >= o) incl += y;
-        }
-        const int base = incl - run;
-        for (int q = 0; q < LANE_N; ++q) tsum[t * LANE_N + q] = base + v[q];
-        if (t == 31) reinterpret_cast<int*>(tb)[0] = incl;  // number of pair classes
     }
     __syncthreads();
-    int cid = tsum[t];
-    for (int e = e0; e < e0 + PER && e < np; ++e) {
-        const uint32_t x = uint32_t(key[e] >> 16);
-        if (e == 0 || x != uint32_t(key[e - 1] >> 16)) {
-            cx[cid] = x;
-            co[cid] = e;
-            ++cid;
+    {  // thread t: the class of mask t -- its pairs, its place, its number
+        int total = 0;
+#pragma unroll
+        for (int v = 0; v < WHT_RANK_WARPS; ++v) {
+            const int c = cnt[v][t];
+            cnt[v][t] = (unsigned short)total;  // pairs of earlier warps
+            total += c;
         }
-        const int p = int(key[e] & 0xFFFFu), l = p & 0xFF, m = p >> 8;
-        pr[e] = uint16_t(p);
-        const uint32_t zl = sz[l], zm = sz[m];
-        reinterpret_cast<uint16_t*>(tb + WHT_OFF_EZ)[e] = uint16_t((zl ^ zm) & uint32_t(N - 1));
+        int at = total, cls = total > 0;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, at, o), k = __shfl_up_sync(0xffffffffu, cls, o);
+            if (lane >= o) {
+                at += y;
+                cls += k;
+            }
+        }
+        if (lane == 31) {
+            part[w] = at;
+            cpart[w] = cls;
+        }
+        __syncthreads();
+        int p0 = part[lane], c0 = cpart[lane];
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, p0, o), k = __shfl_up_sync(0xffffffffu, c0, o);
+            if (lane >= o) {
+                p0 += y;
+                c0 += k;
+            }
+        }
+        const int pw = w ? __shfl_sync(0xffffffffu, p0, w - 1) : 0, cw = w ? __shfl_sync(0xffffffffu, c0, w - 1) : 0;
+        start[t] = pw + at - total;
+        if (total > 0) {
+            reinterpret_cast<uint32_t*>(tb + WHT_OFF_CX)[cw + cls - 1] = uint32_t(t);
+            reinterpret_cast<int*>(tb + WHT_OFF_CO)[cw + cls - 1] = pw + at - total;
+        }
+        if (t == WHT_CT - 1) {
+            reinterpret_cast<int*>(tb)[0] = cw + cls;
+            reinterpret_cast<int*>(tb + WHT_OFF_CO)[cw + cls] = np;
+        }
+        if (t == 0) {
+            double sum = 0.0;
+            for (int k = 0; k < 8; ++k) sum += red[k];
+            s_bn2 = sum;
+            *I.bn2 = sum;
+            if (!(sum > 0.0) || !isfinite(sum)) set_status(status, DEV_BAD_NORM);
+            *reinterpret_cast<int*>(tb + WHT_OFF_BIM) = s_im;
+        }
+    }
+    __syncthreads();
+    if (w < 8 && I.b) {
+        const double sc2 = F64 ? scalbn(1.0, -w64_bexp(s_bn2)) : 0.0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int j = t + 256 * k;
+            if (j >= N) break;
+            if (F64) {
+                const Fx re = fx_from(b[k].x * sc2), im = fx_from(b[k].y * sc2);
+                reinterpret_cast<int4*>(I.bf)[j] = make_int4(re.h, re.l, im.h, im.l);
+            }
+            else reinterpret_cast<float2*>(I.bf)[j] = make_float2((float)b[k].x, (float)b[k].y);
+        }
+    }
+    for (int e = WHT_CT - 1 - t; e < np; e += WHT_CT) {
+        int l, m;
+        wht_pair(e, l, m);
+        const uint32_t x = sx[l] ^ sx[m], zl = sz[l];
+        const int at = start[x] + cnt[e / run][x] + rank[e];
+        reinterpret_cast<uint16_t*>(tb + WHT_OFF_PR)[at] = uint16_t(l | (m << 8));
+        reinterpret_cast<uint16_t*>(tb + WHT_OFF_EZ)[at] = uint16_t(zl ^ sz[m]);
+        const double2 a = sc[l], c = sc[m];
+        const double wr = a.x * c.x + a.y * c.y;  // Re w_lm
         const float sg = ((__popc(zl & x) & 1) ? -1.f : 1.f) * (l < m ? 2.f : 1.f);  // exact scaling
         if (F64) {
-            reinterpret_cast<double*>(tb + WHT_OFF_EK)[e] = (double)sg * I.w[l * L + m].x;
+            reinterpret_cast<double*>(tb + WHT_OFF_EK)[at] = (double)sg * wr;
         } else {
-            const float4 wv = I.wf[l * L + m];
-            reinterpret_cast<float2*>(tb + WHT_OFF_EK)[e] = make_float2(sg * wv.x, sg * wv.y);
+            const float hi = (float)wr;
+            reinterpret_cast<float2*>(tb + WHT_OFF_EK)[at] = make_float2(sg * hi, sg * (float)(wr - (double)hi));
         }
     }
-    if (t == WHT_CT - 1) co[tsum[WHT_CT - 1] + cnt] = np;  // the end of the last class
-    __shared__ int sfirst[64];  // term k is the first with its mask
-    if (t < L) {
-        bool f = true;
-        for (int q = 0; q < t && f; ++q) f = sx[q] != sx[t];
-        sfirst[t] = f ? 1 : 0;
+    if (w == 15 || w == 14) {  // term k is the first with its mask
+        const int k = t - 448;
+        bool f = k < L;
+        for (int q = 0; q < k && f; ++q) f = sx[q] != sx[k];
+        const unsigned m = __ballot_sync(0xffffffffu, f);
+        if (lane == 0) s_first[w - 14] = m;
     }
     __syncthreads();
-    if (t < L) {  // term classes by x_l: rank and class number of term l from counts
+    if (t >= 512 && t - 512 < L) {  // term classes by x_l: rank and class number of the term from counts
         uint32_t* dx = reinterpret_cast<uint32_t*>(tb + WHT_OFF_DX);
         int* dof = reinterpret_cast<int*>(tb + WHT_OFF_DO);
-        uint16_t* dt = reinterpret_cast<uint16_t*>(tb + WHT_OFF_DT);
-        const uint32_t xl = sx[t];
-        int below = 0, rank = 0, cls = 0, nd = 0;
+        const int l = t - 512;
+        const uint32_t xl = sx[l];
+        int below = 0, place = 0, cls = 0, nd = 0;
         bool first = true;
         for (int k = 0; k < L; ++k) {
             const uint32_t xk = sx[k];
-            const bool kfirst = sfirst[k] != 0;
+            const bool kfirst = (s_first[k >> 5] >> (k & 31)) & 1u;
             if (xk < xl) {
                 ++below;
                 if (kfirst) ++cls;
             }
-            if (xk < xl || (xk == xl && k < t)) ++rank;
-            if (xk == xl && k < t) first = false;
+            if (xk < xl || (xk == xl && k < l)) ++place;
+            if (xk == xl && k < l) first = false;
             if (kfirst) ++nd;
         }
-        dt[rank] = uint16_t(t);
+        reinterpret_cast<uint16_t*>(tb + WHT_OFF_DT)[place] = uint16_t(l);
         if (first) {
             dx[cls] = xl;
             dof[cls] = below;
         }
-        if (t == 0) {
+        if (l == 0) {
             dof[nd] = L;
             reinterpret_cast<int*>(tb)[1] = nd;
         }
     }
-    __syncthreads();  // the table is complete: record what it was built from
-    if (t < L) {
-        kx[t] = I.xm[t];
-        kz[t] = I.zm[t];
-        kc[t] = I.coef[t];
-    }
-    if (t == 0) *kL = tag;
-    __syncthreads();  // every word of the table is written
-    const unsigned long long sum = wht_checksum(tb, red);
-    if (t == 0) *ksum = sum;
 }
 
 // Unnormalised Walsh-Hadamard transform of a warp's vector, v[r] at index
@@ -2823,24 +2836,18 @@ inline size_t wht_smem_bytes(int Pmax) {
 // DVQLS_FP64 with L <= 64 and n <= 10: the same classes, for the same terms.
 // The FP64 tiles spend one DFMA per term and amplitude on a pipe that issues 2
 // per clock and SM (n = 10, L = 64: 2.2 M DFMAs, 1.1 M cycles per state).  Here
-// the transforms run in 64-bit fixed point on the integer pipes: the state has
-// norm one, so sum_i |psi[i] psi[i ^ x]| <= 1 and every partial sum of a
-// transform stays within 1.0 = 2^62 -- the adds are exact.  An amplitude and a
-// product are rounded once each, to 2^-63 absolute (an FP64 rounding of an
-// amplitude near 2^-5, the mean at n = 10, is 2^-58).  What is left on the FP64
-// pipe is the state build and one FMA per term for the weighted sums.
+// the state (build_state_fx) and the transforms run in 64-bit fixed point on the
+// integer pipes: sum_i |psi[i] psi[i ^ x]| <= 1, so every partial sum of a
+// transform stays within 1.0 = 2^60 and the adds are exact; a product is rounded
+// once, at 2^-60.  The FP64 pipe keeps one FMA per term for the weighted sums.
 // One CTA of 8 warps per item, two CTAs per SM (the transform of 2^10 values
 // holds 64 registers a lane), so one CTA's state build overlaps the other's
 // transforms.
-// n = 10, L = 64, 101 shifts of one system: 623 us by the tiles, 72 us by the
-// classes; 48 systems of n = 6..10: 8,646 us against 600 us.
+// n = 10, L = 64, 101 shifts of one system: 623 us by the tiles, 46 us by the
+// classes (72 with an FP64 state); 48 systems of n = 6..10: 8,646 us against 331
+// (600).  A state of n = 10 takes 20 k cycles of a CTA, its 29 transforms and 2,080
+// lookups 31 k; both are bound by the integer multiply-adds and adds.
 constexpr int W64_ROW = (1 << WHT_MAXN) + (1 << WHT_MAXN) / 32;
-
-// a b for a, b in fixed point, rounded to nearest.
-__device__ __forceinline__ long long w64_mul(long long a, long long b) {
-    const unsigned long long lo = (unsigned long long)a * (unsigned long long)b;
-    return (__mul64hi(a, b) << 2) + (long long)(lo >> 62) + (long long)((lo >> 61) & 1ull);
-}
 
 // Transform of v (index (r << 5) | lane) into the warp's row, at i + (i >> 5)
 // for 2^10 values (A = 32: through the row, lane bits become register bits), else at i.
@@ -2888,7 +2895,7 @@ __device__ __forceinline__ void w64_transform(long long (&v)[A], long long* row,
 // the term classes of one state q, dealt to the warps; the warp's sums of its
 // lanes in D (flavour 0) and E (the others), delta~ to dre / dim.
 template <int A, int LOGA>
-__device__ void w64_item(const Inst& I, int s, const long long* q, long long* row, double* dre, double* dim,
+__device__ void w64_item(const Inst& I, int s, const Fx* q, long long* row, double* dre, double* dim,
                          const uint32_t* szl, double& D, double& E, int lane) {
     constexpr bool PAD = A == 32;
     const int n = I.n, N = 1 << n, L = I.L, w = threadIdx.x >> 5, lm = N < 32 ? N - 1 : 31;
@@ -2903,7 +2910,6 @@ __device__ void w64_item(const Inst& I, int s, const long long* q, long long* ro
     const int* dof = reinterpret_cast<const int*>(tb + WHT_OFF_DO);
     const uint16_t* dt = reinterpret_cast<const uint16_t*>(tb + WHT_OFF_DT);
     double2* Gp = (s == 0 && I.Gpart) ? reinterpret_cast<double2*>(I.Gpart) : nullptr;
-    const double unit = scalbn(1.0, -W64_FRAC);
     const int parts = 1 + *reinterpret_cast<const int*>(tb + WHT_OFF_BIM);
     const int pairs = ncls * I.F, jobs = pairs + (I.local ? 0 : nd * parts);
     auto at = [&](uint32_t z) { return row[PAD ? z + (z >> 5) : z]; };
@@ -2912,14 +2918,15 @@ __device__ void w64_item(const Inst& I, int s, const long long* q, long long* ro
         long long v[A];
         if (j >= pairs) {
             const int c = (j - pairs) / parts, part = (j - pairs) - c * parts, x = int(dx[c]);
-            const longlong2* qb = reinterpret_cast<const longlong2*>(I.bf);
+            const int4* qb = reinterpret_cast<const int4*>(I.bf);
 #pragma unroll
             for (int r = 0; r < A; ++r) {  // conj(b[i ^ x]) psi[i], its real or imaginary part
                 const int i = (r << 5) | (lane & lm), k = (i ^ x) & (N - 1);
-                v[r] = w64_mul(part ? -qb[k].y : qb[k].x, q[i]);
+                const int4 bb = qb[k];
+                v[r] = fx_mul(part ? fx_neg(Fx{bb.z, bb.w}) : Fx{bb.x, bb.y}, q[i]);
             }
             w64_transform<A, LOGA>(v, row, N, lane);
-            const double sc = scalbn(1.0, w64_bexp(*I.bn2) - W64_FRAC);
+            const double sc = scalbn(1.0, w64_bexp(*I.bn2) - FX_BITS);
             for (int e = dof[c] + lane; e < dof[c + 1]; e += 32) {
                 const int l = dt[e];
                 (part ? dim : dre)[l] = (double)at(szl[l] & uint32_t(N - 1)) * sc;
@@ -2932,7 +2939,7 @@ __device__ void w64_item(const Inst& I, int s, const long long* q, long long* ro
 #pragma unroll
         for (int r = 0; r < A; ++r) {
             const int i = (r << 5) | (lane & lm);
-            v[r] = w64_mul(q[i], q[(i ^ x) & (N - 1)]);  // masks >= 2^n are reported, never followed
+            v[r] = fx_mul(q[i], q[(i ^ x) & (N - 1)]);  // masks >= 2^n are reported, never followed
         }
         w64_transform<A, LOGA>(v, row, N, lane);
         const int e0 = co[c], e1 = co[c + 1];
@@ -2947,7 +2954,7 @@ __device__ void w64_item(const Inst& I, int s, const long long* q, long long* ro
         if (Gp)  // the beta output of the unshifted state
             for (int e = e0 + lane; e < e1; e += 32) {
                 const int p = pr[e], l = p & 0xFF, m = p >> 8;
-                double beta = (double)at(ez[e]) * unit;
+                double beta = (double)at(ez[e]) * 0x1p-60;
                 if (__popc(szl[l] & uint32_t(x)) & 1) beta = -beta;
                 Gp[(long long)l * L + m] = make_double2(beta, 0.0);
                 Gp[(long long)m * L + l] = make_double2(beta, 0.0);
@@ -2956,8 +2963,8 @@ __device__ void w64_item(const Inst& I, int s, const long long* q, long long* ro
     }
 }
 
-inline size_t w64_smem_bytes(int Pmax) {
-    return 8 * (f64_state_doubles(WHT_MAXN, Pmax) + (size_t(1) << WHT_MAXN) + 8 * size_t(W64_ROW));
+inline size_t w64_smem_bytes(int Pmax) {  // transform rows, then the state build's room
+    return 64 * size_t(W64_ROW) + fx_smem(WHT_MAXN, Pmax);
 }
 
 __global__ void __launch_bounds__(WHT_NT, 2) k_terms_wht64(const Inst* __restrict__ insts, int count, long long total,
@@ -2970,9 +2977,7 @@ __global__ void __launch_bounds__(WHT_NT, 2) k_terms_wht64(const Inst* __restric
     __shared__ double2 redT[2];
     __shared__ long long s_item;
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
-    long long* q = reinterpret_cast<long long*>(smem);        // 2^WHT_MAXN
-    long long* row = q + (1 << WHT_MAXN) + w * W64_ROW;         // this warp's transform row
-    double* st = reinterpret_cast<double*>(q + (1 << WHT_MAXN) + 8 * W64_ROW);
+    long long* row = reinterpret_cast<long long*>(smem) + w * W64_ROW;  // this warp's transform row
     for (;;) {
         if (t == 0) s_item = (long long)atomicAdd(queue, 1ull);
         __syncthreads();
@@ -2980,15 +2985,12 @@ __global__ void __launch_bounds__(WHT_NT, 2) k_terms_wht64(const Inst* __restric
         __syncthreads();
         if (gi >= total) break;
         const Inst& I = insts[find_instance(insts, count, gi)];
-        const int s = int(gi - I.item_base), L = I.L, N = 1 << I.n;
+        const int s = int(gi - I.item_base), L = I.L;
         if (t < TT) {
             szl[t] = t < L ? I.zm[t] : 0u;
             dre[t] = dim[t] = 0.0;
         }
-        build_state_f64(st, I.n, I.d, I.P, I.cs, s + I.s0);
-        const double one = scalbn(1.0, W64_FRAC);
-        for (int i = t; i < N; i += WHT_NT) q[i] = __double2ll_rn(st[f64_pad(i)] * one);
-        __syncthreads();
+        const Fx* q = build_state_fx(smem + 64 * W64_ROW, I.n, I.d, I.P, I.cs, s + I.s0);  // ends with a barrier
         double D = 0.0, E = 0.0;
         switch (I.n) {
             case 10: w64_item<32, 5>(I, s, q, row, dre, dim, szl, D, E, lane); break;
@@ -3021,7 +3023,7 @@ __global__ void __launch_bounds__(WHT_NT, 2) k_terms_wht64(const Inst* __restric
             if (lane == 0) redT[w] = T;
         }
         __syncthreads();
-        const double unit = scalbn(1.0, -W64_FRAC);
+        const double unit = 0x1p-60;
         if (t == 0) {
             double Ds = 0.0, Es = 0.0;
             for (int k = 0; k < WHT_NT / 32; ++k) {
@@ -3043,35 +3045,34 @@ template <typename R>
 __global__ void __launch_bounds__(NT) k_combine(const Inst* __restrict__ insts, int* status) {
     pdl_wait();
     using R2 = typename V2<R>::t;
+    __shared__ double sN[2 * MAX_ANGLES + 1], sD[2 * MAX_ANGLES + 1];  // N_s (local cost: E_s) and D_s
     const Inst I = insts[blockIdx.x];
     const int t = threadIdx.x, T = I.T, ks = I.ks, L = I.L;
     const double bn2 = *I.bn2;
     for (int s = t; s < I.S; s += NT) {
-        double2 D = make_double2(0.0, 0.0), Tv = make_double2(0.0, 0.0);
+        double D = 0.0;
+        double2 Tv = make_double2(0.0, 0.0);
         const double2* dp = I.Dpart + (long long)s * I.F * T * T * ks;
-        for (int e = 0; e < T * T * ks; ++e) {
-            D.x += dp[e].x;
-            D.y += dp[e].y;
-        }
+#pragma unroll 4
+        for (int e = 0; e < T * T * ks; ++e) D += dp[e].x;
+        sD[s] = D;
         if (I.local) {  // E_s = sum over the gamma flavors (real parts)
             double E = 0.0;
+#pragma unroll 4
             for (int e = T * T * ks; e < I.F * T * T * ks; ++e) E += dp[e].x;
-            I.NsDs[3 * s] = E;
-            I.NsDs[3 * s + 1] = D.x;
-            I.NsDs[3 * s + 2] = D.y;
+            sN[s] = E;
             continue;
         }
         const double2* tp = I.Tpart + (long long)s * T * ks;
+#pragma unroll 4
         for (int e = 0; e < T * ks; ++e) {
             Tv.x += tp[e].x;
             Tv.y += tp[e].y;
         }
-        I.NsDs[3 * s] = (Tv.x * Tv.x + Tv.y * Tv.y) / bn2;
-        I.NsDs[3 * s + 1] = D.x;
-        I.NsDs[3 * s + 2] = D.y;
+        sN[s] = (Tv.x * Tv.x + Tv.y * Tv.y) / bn2;
     }
     __syncthreads();
-    const double N0 = I.NsDs[0], D0 = I.NsDs[1];
+    const double N0 = sN[0], D0 = sD[0];
     // Global cost: C = 1 - N/D.  Local cost: C_L = 1/2 - E / (2 n D) (N holds E).
     const double scale = I.local ? 0.5 / I.n : 1.0;
     if (t == 0) {
@@ -3080,8 +3081,8 @@ __global__ void __launch_bounds__(NT) k_combine(const Inst* __restrict__ insts, 
     }
     if (I.grad && I.S > 1)
         for (int k = t; k < I.P; k += NT) {
-            const double dN = 0.5 * (I.NsDs[3 * (2 * k + 1)] - I.NsDs[3 * (2 * k + 2)]);
-            const double dD = 0.5 * (I.NsDs[3 * (2 * k + 1) + 1] - I.NsDs[3 * (2 * k + 2) + 1]);
+            const double dN = 0.5 * (sN[2 * k + 1] - sN[2 * k + 2]);
+            const double dD = 0.5 * (sD[2 * k + 1] - sD[2 * k + 2]);
             I.grad[k] = -scale * (dN * D0 - N0 * dD) / (D0 * D0);
         }
     if (I.beta) {
@@ -3220,18 +3221,15 @@ static int launch_pass(dvqls_ctx* ctx, cudaStream_t st, const Inst* dtable, cons
     // One profiling mark per kernel, so the launch counts are exact.  The
     // prepare kernel also resets the work queue.
     if (marks) prof_begin(ctx, 0);
-    k_prepare<<<dim3(ps.count, ps.prep_parts + (ps.tc && ps.bop_fused ? ps.bop_parts : 0)), NT, 0, st>>>(
+    if (ps.wht)
+        (ps.fp32 ? k_wht_prepare<false> : k_wht_prepare<true>)<<<ps.count, WHT_CT, 0, st>>>(dtable, ctx->d_status, ctx->d_queue);
+    else
+        k_prepare<<<dim3(ps.count, ps.prep_parts + (ps.tc && ps.bop_fused ? ps.bop_parts : 0)), NT, 0, st>>>(
         dtable, ctx->d_status, ctx->d_queue, ps.prep_parts);
     if (marks) prof_end(ctx);
     if (ps.tc && !ps.bop_fused) {
         if (marks) prof_begin(ctx, 0);
         DVQLS_CUDA_TRY(ctx, launch_pdl(k_prep_bop, dim3(ps.count, ps.bop_parts), dim3(256), 0, st, dtable));
-        if (marks) prof_end(ctx);
-    }
-    if (ps.wht) {
-        if (marks) prof_begin(ctx, 0);
-        DVQLS_CUDA_TRY(ctx, launch_pdl(ps.fp32 ? k_wht_classes<false> : k_wht_classes<true>, dim3(ps.count), dim3(WHT_CT), 0,
-                                       st, dtable));
         if (marks) prof_end(ctx);
     }
     if (ps.tc && ps.st_grid > 0) {  // shifted states of the on-chip instances, packed for the term kernel
@@ -3502,10 +3500,10 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
         Off& o = off[i];
         const size_t L = h.L;
         o.ctil = ar.reserve(L * 16);
-        // pair weights w_lm for the CUDA-core and Walsh-Hadamard kernels (the
-        // tensor-core epilogue forms its weights from c~ alone)
-        o.w = tc ? 0 : ar.reserve(L * L * 16);
-        o.wf = fp32 && !tc ? ar.reserve(L * L * 16) : 0;  // float-float weights of the FP32 term kernels
+        // pair weights w_lm for the CUDA-core kernels (the tensor-core epilogue and
+        // the class table form theirs from c~)
+        o.w = tc || wht ? 0 : ar.reserve(L * L * 16);
+        o.wf = fp32 && !tc && !wht ? ar.reserve(L * L * 16) : 0;  // float-float weights of the FP32 term kernels
         o.cf = fp32 ? ar.reserve(L * 16) : 0;
         o.bop = tc && !local ? ar.reserve(size_t(tc_bop_stages(h.N)) * TC_BOP_STAGE) : 0;
         o.wht = wht ? ar.reserve(WHT_TABLE_BYTES) : 0;
@@ -3577,8 +3575,8 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
         I.s0 = range ? range->s0 : 0;
         I.local = local ? 1 : 0;
         I.ctil = (double2*)(ws + o.ctil);
-        I.w = tc ? nullptr : (double2*)(ws + o.w);
-        I.wf = fp32 && !tc ? (float4*)(ws + o.wf) : nullptr;
+        I.w = tc || wht ? nullptr : (double2*)(ws + o.w);
+        I.wf = fp32 && !tc && !wht ? (float4*)(ws + o.wf) : nullptr;
         I.cf = fp32 ? (float4*)(ws + o.cf) : nullptr;
         I.bop = tc && !local ? (void*)(ws + o.bop) : nullptr;
         I.wht = wht ? (void*)(ws + o.wht) : nullptr;
