@@ -60,6 +60,8 @@ struct Inst {
     void* bf;        // Walsh-Hadamard classes: b as float2, or in fixed point as int4 (FP64), or null
     double2* cs;     // 3P: (cos, sin) of half angles: base, +pi/2, -pi/2
     double* bn2;     // ||b||^2
+    double* bpart;   // its BN_PARTS block sums (states in HBM), or null
+    int fold;        // 1: the term kernel's partial sums are added by k_fold before the combine
     double2* Dpart;  // S*T*T*ks
     double2* Tpart;  // S*T*ks
     void* Gpart;     // ks*L*L (shift 0 only; null when beta is not requested)
@@ -1178,6 +1180,31 @@ __device__ __noinline__ double b_norm2(const Inst& I, double* red) {
     return sum;
 }
 
+// ||b||^2 of a large b by blocks, added in order by k_prepare: one CTA took 1.1 ms
+// over the 16 MB of n = 20.
+constexpr int BN_PARTS = 128;
+__global__ void __launch_bounds__(256) k_bnorm(const Inst* __restrict__ insts) {
+    pdl_trigger();
+    const Inst& I = insts[blockIdx.y];
+    if (!I.bpart || !I.b) return;
+    const long long N = 1LL << I.n, per = N / BN_PARTS;  // N > 4096
+    const double2* b = I.b + blockIdx.x * per;
+    double acc = 0.0;
+#pragma unroll 4
+    for (long long j = threadIdx.x; j < per; j += 256) {
+        const double2 v = b[j];
+        acc += v.x * v.x + v.y * v.y;
+    }
+    for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    __shared__ double red[8];
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int k = 1; k < 8; ++k) acc += red[k];
+        I.bpart[blockIdx.x] = acc;
+    }
+}
+
 // Per instance: CTAs 0 .. prep_parts - 1 form ||b||^2 and c~ (part 0), the
 // half-angle tables (part 1, or 0 when alone) and the pair weights (all
 // parts); CTAs from prep_parts on, when launched, build the tensor-core b rows
@@ -1200,7 +1227,13 @@ __global__ void __launch_bounds__(NT) k_prepare(const Inst* __restrict__ insts, 
         return;
     }
     if (part == 0) {
-        const double sum = b_norm2(I, red);
+        double sum = 0.0;
+        if (I.bpart) {
+            if (t == 0)
+                for (int k = 0; k < BN_PARTS; ++k) sum += I.bpart[k];
+        } else {
+            sum = b_norm2(I, red);
+        }
         for (int l = t; l < I.L; l += NT) {
             const uint32_t x = I.xm[l], z = I.zm[l];
             if (x >= N || z >= N) set_status(status, DEV_BAD_MASK);
@@ -3041,6 +3074,36 @@ __global__ void __launch_bounds__(WHT_NT, 2) k_terms_wht64(const Inst* __restric
 }
 
 // ---------------------------------------------------------------- combine
+// Adds the partial sums of a shift where there are many (states in HBM: one per
+// 2,048 amplitudes), a warp per shift, lanes in stride and then a fixed tree, into
+// the shift's first slots.  In the combine one thread per shift added them: 406 us
+// for the uneven batch (n = 20: 441 shifts x 512 slots), 20 with this.
+constexpr int FOLD_MIN = 64;  // slots per shift from which it is worth a launch
+__global__ void __launch_bounds__(256) k_fold(const Inst* __restrict__ insts) {
+    pdl_wait();
+    pdl_trigger();
+    const Inst& I = insts[blockIdx.y];
+    const int s = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (!I.fold || s >= I.S) return;
+    const int T = I.T, nd = T * T * I.ks;
+    auto fold = [&](double2* p, int count) {
+        double2 v = make_double2(0.0, 0.0);
+        for (int e = lane; e < count; e += 32) {
+            v.x += p[e].x;
+            v.y += p[e].y;
+        }
+        for (int o = 16; o; o >>= 1) {
+            v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+            v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+        }
+        if (lane == 0) p[0] = v;
+    };
+    double2* dp = I.Dpart + (long long)s * I.F * nd;
+    fold(dp, nd);
+    if (I.local) fold(dp + nd, (I.F - 1) * nd);
+    else fold(I.Tpart + (long long)s * T * I.ks, T * I.ks);
+}
+
 template <typename R>
 __global__ void __launch_bounds__(NT) k_combine(const Inst* __restrict__ insts, int* status) {
     pdl_wait();
@@ -3049,23 +3112,24 @@ __global__ void __launch_bounds__(NT) k_combine(const Inst* __restrict__ insts, 
     const Inst I = insts[blockIdx.x];
     const int t = threadIdx.x, T = I.T, ks = I.ks, L = I.L;
     const double bn2 = *I.bn2;
+    const int nd = I.fold ? 1 : T * T * ks, nt = I.fold ? 1 : T * ks, ne = I.fold ? 1 : (I.F - 1) * T * T * ks;
     for (int s = t; s < I.S; s += NT) {
         double D = 0.0;
         double2 Tv = make_double2(0.0, 0.0);
         const double2* dp = I.Dpart + (long long)s * I.F * T * T * ks;
 #pragma unroll 4
-        for (int e = 0; e < T * T * ks; ++e) D += dp[e].x;
+        for (int e = 0; e < nd; ++e) D += dp[e].x;
         sD[s] = D;
         if (I.local) {  // E_s = sum over the gamma flavors (real parts)
             double E = 0.0;
 #pragma unroll 4
-            for (int e = T * T * ks; e < I.F * T * T * ks; ++e) E += dp[e].x;
+            for (int e = 0; e < ne; ++e) E += dp[T * T * ks + e].x;
             sN[s] = E;
             continue;
         }
         const double2* tp = I.Tpart + (long long)s * T * ks;
 #pragma unroll 4
-        for (int e = 0; e < T * ks; ++e) {
+        for (int e = 0; e < nt; ++e) {
             Tv.x += tp[e].x;
             Tv.y += tp[e].y;
         }
@@ -3136,18 +3200,19 @@ __global__ void __launch_bounds__(NT) k_partials(const Inst* __restrict__ insts,
     pdl_wait();
     const Inst& I = insts[0];
     const int T = I.T, ks = I.ks;
+    const int nd = I.fold ? 1 : T * T * ks, nt = I.fold ? 1 : T * ks;
     const double inv = 1.0 / sqrt(*I.bn2);
     for (int g = threadIdx.x; g < S_full; g += NT) {
         const int s = g - I.s0;
         double v[4] = {0.0, 0.0, 0.0, 0.0};
         if (s >= 0 && s < I.S) {
             const double2* dp = I.Dpart + (long long)s * T * T * ks;
-            for (int e = 0; e < T * T * ks; ++e) {
+            for (int e = 0; e < nd; ++e) {
                 v[2] += dp[e].x;
                 v[3] += dp[e].y;
             }
             const double2* tp = I.Tpart + (long long)s * T * ks;
-            for (int e = 0; e < T * ks; ++e) {
+            for (int e = 0; e < nt; ++e) {
                 v[0] += tp[e].x;
                 v[1] += tp[e].y;
             }
@@ -3211,6 +3276,8 @@ struct PassShape {
     int S_full;           // and the instance's 2P + 1 shifts
     int prep_parts;  // CTAs per instance of k_prepare (weights split ~256 per CTA)
     int bop_parts;   // CTAs per instance building the tensor-core b rows
+    int any_hbm;     // some state lives in HBM
+    int fold_grid;   // CTAs per instance of k_fold (0: no instance has that many partial sums)
     int bop_fused;   // 1: those CTAs are part of k_prepare (every state has <= TC_BOP_FUSED_N amplitudes)
 };
 
@@ -3220,6 +3287,11 @@ static int launch_pass(dvqls_ctx* ctx, cudaStream_t st, const Inst* dtable, cons
                        const std::vector<const HostInst*>& tab, bool marks) {
     // One profiling mark per kernel, so the launch counts are exact.  The
     // prepare kernel also resets the work queue.
+    if (ps.any_hbm) {
+        if (marks) prof_begin(ctx, 0);
+        k_bnorm<<<dim3(BN_PARTS, ps.count), 256, 0, st>>>(dtable);
+        if (marks) prof_end(ctx);
+    }
     if (marks) prof_begin(ctx, 0);
     if (ps.wht)
         (ps.fp32 ? k_wht_prepare<false> : k_wht_prepare<true>)<<<ps.count, WHT_CT, 0, st>>>(dtable, ctx->d_status, ctx->d_queue);
@@ -3260,6 +3332,11 @@ static int launch_pass(dvqls_ctx* ctx, cudaStream_t st, const Inst* dtable, cons
         DVQLS_CUDA_TRY(ctx, launch_pdl(k_terms_smem<double>, dim3(ps.grid), dim3(NT), ps.smem, st, dtable, ps.count,
                                        ps.total, ctx->d_queue));
     if (marks) prof_end(ctx);
+    if (ps.fold_grid) {
+        if (marks) prof_begin(ctx, 2);
+        DVQLS_CUDA_TRY(ctx, launch_pdl(k_fold, dim3(ps.fold_grid, ps.count), dim3(256), 0, st, dtable));
+        if (marks) prof_end(ctx);
+    }
     if (marks) prof_begin(ctx, 2);
     if (ps.partials)
         DVQLS_CUDA_TRY(ctx, launch_pdl(k_partials, dim3(1), dim3(NT), 0, st, dtable, ps.S_full, ps.partials));
@@ -3450,7 +3527,7 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
     struct Off {
         size_t coef, xm, zm, alpha, b;       // staged inputs (ws) ...
         size_t pcoef, pxm, pzm, palpha, pb;  // ... and their pinned slots
-        size_t ctil, w, wf, cf, bop, wht, bf, cs, bn2, Dp, Tp, Gp, dp, NsDs, cost, grad, beta, delta, states, chain, tcst;
+        size_t ctil, w, wf, cf, bop, wht, bf, cs, bn2, bpart, Dp, Tp, Gp, dp, NsDs, cost, grad, beta, delta, states, chain, tcst;
         size_t pcost, pgrad, pbeta, pdelta;
     };
     std::vector<Off> off(count);
@@ -3510,6 +3587,7 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
         o.bf = wht ? ar.reserve(size_t(h.N) * (fp32 ? 8 : 16)) : 0;
         o.cs = ar.reserve(size_t(3) * h.P * 16);
         o.bn2 = ar.reserve(8);
+        o.bpart = h.hbm && !local ? ar.reserve(BN_PARTS * 8) : 0;
         o.Dp = ar.reserve(size_t(h.S) * h.F * h.T * h.T * kp * 16);
         o.Tp = ar.reserve(size_t(h.S) * h.T * kp * 16);
         o.Gp = beta_out ? ar.reserve(size_t(kp) * L * L * r2) : 0;
@@ -3583,6 +3661,7 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
         I.bf = wht ? (void*)(ws + o.bf) : nullptr;
         I.cs = (double2*)(ws + o.cs);
         I.bn2 = (double*)(ws + o.bn2);
+        I.bpart = h.hbm && !local ? (double*)(ws + o.bpart) : nullptr;
         I.Dpart = (double2*)(ws + o.Dp);
         I.Tpart = (double2*)(ws + o.Tp);
         I.Gpart = beta_out ? (void*)(ws + o.Gp) : nullptr;
@@ -3615,10 +3694,13 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
         std::stable_sort(ord.begin(), ord.end(),
                          [&](int a, int b) { return hi[a].N / kk[a] > hi[b].N / kk[b]; });
         long long base = 0;
+        ps.fold_grid = 0;
         for (int oi = 0; oi < count; ++oi) {
             const int i = ord[oi];
             Inst I = rec[i];
             I.ks = kk[i];
+            I.fold = !wht && I.F * I.T * I.T * I.ks >= FOLD_MIN;
+            if (I.fold) ps.fold_grid = std::max(ps.fold_grid, ceil_div(I.S, 8));
             // a Walsh-Hadamard item covers every flavour; the tensor-core tiles take
             // each pair of tiles once (T (T + 1) / 2 per shift), the CUDA-core tiles T^2
             I.items = wht ? I.S : tc ? I.S * I.F * (I.T * (I.T + 1) / 2) * I.ks : I.S * I.F * I.T * I.T * I.ks;
@@ -3645,6 +3727,7 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
         ps.S_full = S_full;
         ps.prep_parts = (int)std::min<long long>(16, std::max<long long>(1, LLmax / NT));
         ps.bop_parts = (int)std::min<long long>(64, std::max<long long>(1, tc_bop_stages(Nmax) * (TC_BOP_STAGE / 16) / 256));
+        ps.any_hbm = any_hbm;
         ps.bop_fused = Nmax <= TC_BOP_FUSED_N;
     };
     auto upload = [&]() -> int {
