@@ -19,6 +19,7 @@ int set_error(dvqls_ctx* ctx, int code, const char* fmt, ...) {
 
 bool is_device_ptr(const dvqls_ctx* ctx, const void* p) {
     if (!p) return false;
+    if (p >= ctx->own_lo && p < ctx->own_hi) return true;
     auto& seen = const_cast<dvqls_ctx*>(ctx)->host_ptrs;
     if (seen.count(p)) return false;
     cudaPointerAttributes a;
@@ -296,6 +297,7 @@ extern "C" void dvqls_destroy(dvqls_ctx* ctx) {
     dvqls::release_graph_cache(ctx);
     if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
     if (ctx->ws) cudaFree(ctx->ws);
+    if (ctx->opt_pin) cudaFreeHost(ctx->opt_pin);
     if (ctx->pin) cudaFreeHost(ctx->pin);
     if (ctx->d_status) cudaFree(ctx->d_status);
     if (ctx->h_status) cudaFreeHost(ctx->h_status);

@@ -66,6 +66,10 @@ struct dvqls_ctx {
     // Pinned word the status is read into (an asynchronous copy, then one
     // stream synchronisation).
     int* h_status = nullptr;
+    // Pinned words the optimizer reads its costs and fidelities into, kept
+    // between calls (at most two doubles per instance of the largest batch).
+    double* opt_pin = nullptr;
+    size_t opt_pin_cap = 0;
 
     // Pinned staging is reused by every call: pin_event marks the last
     // host-to-device copy out of it; it is waited on before the next write.
@@ -96,6 +100,9 @@ struct dvqls_ctx {
     // allocations, so the answer cannot turn into "device"; at worst memory
     // that became managed there is staged through the pinned buffer.
     std::unordered_set<const void*> host_ptrs;
+    // Device memory that a running call of this context owns ([lo, hi), or
+    // empty): its addresses need no query either (the optimizer's cost passes).
+    const char *own_lo = nullptr, *own_hi = nullptr;
 
     // Cached batched-call state (see terms.cu): the last captured graph of a
     // cost pass, the private stream graphs are captured on, and the

@@ -505,20 +505,25 @@ __global__ void __launch_bounds__(CGR_T) k_cg_diag(int n, const LcuGroups* __res
     else cgr_solve<EPT, false>(n, G, re, im, b, x, sp, tol, max_iter, out);
 }
 
-// One Adam update of the active angles: element i is angle gmap[i], whose
-// instance has the bias corrections c1[i] = 1 - beta1^t and c2[i] = 1 - beta2^t.
+// One Adam update of the active angles: element i is angle gmap[i].  p1[k] and
+// p2[k] hold beta1^t and beta2^t of angle k's instance, formed as products in
+// the order of its updates (a copy per angle: no update has to wait for another),
+// so nothing is uploaded between iterations.
 __global__ void k_adam(int count, const int* __restrict__ gmap, const double* __restrict__ g, double* alpha,
-                       double* m, double* v, double lr, double b1, double b2, double eps, const double* __restrict__ c1,
-                       const double* __restrict__ c2) {
+                       double* m, double* v, double lr, double b1, double b2, double eps, double* p1, double* p2) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= count) return;
     const int k = gmap[i];
+    const double q1 = __dmul_rn(p1[k], b1), q2 = __dmul_rn(p2[k], b2);  // not fused into 1 - q: the host forms them so
+    p1[k] = q1;
+    p2[k] = q2;
+    const double c1 = 1.0 - q1, c2 = 1.0 - q2;
     const double gi = g[i];
     const double mi = b1 * m[k] + (1.0 - b1) * gi;
     const double vi = b2 * v[k] + (1.0 - b2) * gi * gi;
     m[k] = mi;
     v[k] = vi;
-    alpha[k] -= lr * (mi / c1[i]) / (sqrt(vi / c2[i]) + eps);
+    alpha[k] -= lr * (mi / c1) / (sqrt(vi / c2) + eps);
 }
 
 // cudaMalloc'd block owned by one optimizer call.
@@ -920,10 +925,10 @@ static int optimize(dvqls_ctx* ctx, int count, const dvqls_instance* inst, const
     Arena ar;
     const size_t o_al = ar.reserve(size_t(Pt) * 8), o_m = ar.reserve(size_t(Pt) * 8), o_v = ar.reserve(size_t(Pt) * 8);
     const size_t o_g = ar.reserve(size_t(Pt) * 8), o_gm = ar.reserve(size_t(Pt) * 4);
-    const size_t o_c1 = ar.reserve(size_t(Pt) * 8), o_c2 = ar.reserve(size_t(Pt) * 8);
+    const size_t o_p1 = ar.reserve(size_t(Pt) * 8), o_p2 = ar.reserve(size_t(Pt) * 8);
     const size_t o_x = ar.reserve(size_t(Nt) * 16), o_b = ar.reserve(size_t(Nt) * 16);
     const size_t o_c = ar.reserve(size_t(Lt) * 16), o_xm = ar.reserve(size_t(Lt) * 4), o_zm = ar.reserve(size_t(Lt) * 4);
-    const size_t o_cost = ar.reserve(size_t(count) * 8), o_F = ar.reserve(size_t(count) * 8);
+    const size_t o_cost = ar.reserve(size_t(count) * 16);  // costs, then fidelities: one copy to the host
     const size_t o_cs = ar.reserve(size_t(Pt) * 16), o_ft = ar.reserve(sizeof(FidInst) * count);
     DevBlock blk;
     if (cudaMalloc(&blk.p, ar.total()) != cudaSuccess) {
@@ -931,15 +936,31 @@ static int optimize(dvqls_ctx* ctx, int count, const dvqls_instance* inst, const
         return set_error(ctx, DVQLS_ERR_ALLOC, "optimizer state of %zu bytes", ar.total());
     }
     char* base = blk.p;
+    if (ctx->opt_pin_cap < size_t(count) * 16) {
+        if (ctx->opt_pin) cudaFreeHost(ctx->opt_pin);
+        ctx->opt_pin = nullptr;
+        ctx->opt_pin_cap = 0;
+        if (cudaMallocHost(&ctx->opt_pin, size_t(count) * 16) != cudaSuccess) {
+            cudaGetLastError();
+            return set_error(ctx, DVQLS_ERR_ALLOC, "pinned results of %d instances", count);
+        }
+        ctx->opt_pin_cap = size_t(count) * 16;
+    }
+    struct OwnScope {  // run_batch's arguments below lie in the block
+        dvqls_ctx* c;
+        ~OwnScope() { c->own_lo = c->own_hi = nullptr; }
+    } own{ctx};
+    ctx->own_lo = base;
+    ctx->own_hi = base + ar.total();
     double* alpha = (double*)(base + o_al);
     double* m = (double*)(base + o_m);
     double* v = (double*)(base + o_v);
     double* g = (double*)(base + o_g);
     int* gmap = (int*)(base + o_gm);
     double* costs = (double*)(base + o_cost);
-    double* F = (double*)(base + o_F);
-    double* c1d = (double*)(base + o_c1);
-    double* c2d = (double*)(base + o_c2);
+    double* F = costs + count;
+    double* p1d = (double*)(base + o_p1);
+    double* p2d = (double*)(base + o_p2);
     // Adam state: zero moments and no updates, or the caller's checkpoint.  The
     // bias corrections 1 - beta^t are kept as products formed on the host in
     // the same order as a run that never stopped, so a resumed run continues
@@ -960,6 +981,17 @@ static int optimize(dvqls_ctx* ctx, int count, const dvqls_instance* inst, const
     } else {
         DVQLS_CUDA_TRY(ctx, cudaMemsetAsync(m, 0, size_t(Pt) * 8, ctx->stream));
         DVQLS_CUDA_TRY(ctx, cudaMemsetAsync(v, 0, size_t(Pt) * 8, ctx->stream));
+    }
+    {
+        std::vector<double> hp(size_t(Pt) * 2);
+        for (int i = 0; i < count; ++i)
+            for (long long k = aoff[i]; k < aoff[i + 1]; ++k) {
+                hp[size_t(k)] = p1[i];
+                hp[size_t(Pt + k)] = p2[i];
+            }
+        DVQLS_CUDA_TRY(ctx, cudaMemcpyAsync(p1d, hp.data(), size_t(Pt) * 8, cudaMemcpyHostToDevice, ctx->stream));
+        DVQLS_CUDA_TRY(ctx, cudaMemcpyAsync(p2d, hp.data() + Pt, size_t(Pt) * 8, cudaMemcpyHostToDevice, ctx->stream));
+        DVQLS_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
     }
     std::vector<dvqls_instance> dinst(count);
     std::vector<FidInst> fid(count);
@@ -1001,13 +1033,12 @@ static int optimize(dvqls_ctx* ctx, int count, const dvqls_instance* inst, const
     DVQLS_CUDA_TRY(ctx, allow_dynamic_smem((const void*)k_fidelity));
     std::vector<int> active(count);
     for (int i = 0; i < count; ++i) active[i] = i;
-    std::vector<double> hF(count), hC(count);
+    const double *hC = ctx->opt_pin, *hF = ctx->opt_pin + count;
     std::vector<int> hmap;
     std::vector<dvqls_instance> ainst;
     std::vector<FidInst> afid;
     bool dirty = true;
     long long Pa = 0;
-    std::vector<double> hc1, hc2;
     int rc = DVQLS_OK;
     for (int it = 0; it <= opt->max_iter && !active.empty(); ++it) {
         if (dirty) {
@@ -1029,8 +1060,7 @@ static int optimize(dvqls_ctx* ctx, int count, const dvqls_instance* inst, const
         k_fidelity<<<na, FT, fsmem, ctx->stream>>>((const FidInst*)(base + o_ft), ctx->d_status);
         rc = run_batch(ctx, na, ainst.data(), opt->precision, true, costs, g, nullptr, nullptr, false);
         if (rc) return rc;
-        DVQLS_CUDA_TRY(ctx, cudaMemcpyAsync(hF.data(), F, size_t(count) * 8, cudaMemcpyDeviceToHost, ctx->stream));
-        DVQLS_CUDA_TRY(ctx, cudaMemcpyAsync(hC.data(), costs, size_t(na) * 8, cudaMemcpyDeviceToHost, ctx->stream));
+        DVQLS_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->opt_pin, costs, size_t(count) * 16, cudaMemcpyDeviceToHost, ctx->stream));
         rc = sync_and_check(ctx);
         if (rc) return rc;
         std::vector<int> still;
@@ -1069,20 +1099,9 @@ static int optimize(dvqls_ctx* ctx, int count, const dvqls_instance* inst, const
             dirty = true;
         }
         if (active.empty() || Pa == 0) break;
-        hc1.clear();
-        hc2.clear();
-        for (int i : active) {  // the update of instance i is its (steps[i] + 1)-th
-            p1[i] *= opt->beta1;
-            p2[i] *= opt->beta2;
-            ++steps[i];
-            hc1.insert(hc1.end(), size_t(P[i]), 1.0 - p1[i]);
-            hc2.insert(hc2.end(), size_t(P[i]), 1.0 - p2[i]);
-        }
-        DVQLS_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
-        DVQLS_CUDA_TRY(ctx, cudaMemcpy(c1d, hc1.data(), hc1.size() * 8, cudaMemcpyHostToDevice));
-        DVQLS_CUDA_TRY(ctx, cudaMemcpy(c2d, hc2.data(), hc2.size() * 8, cudaMemcpyHostToDevice));
-        k_adam<<<ceil_div(Pa, 256), 256, 0, ctx->stream>>>(int(Pa), gmap, g, alpha, m, v, opt->lr, opt->beta1,
-                                                          opt->beta2, opt->eps, c1d, c2d);
+        for (int i : active) ++steps[i];
+        k_adam<<<ceil_div(Pa, 64), 64, 0, ctx->stream>>>(int(Pa), gmap, g, alpha, m, v, opt->lr, opt->beta1, opt->beta2,
+                                                         opt->eps, p1d, p2d);
         DVQLS_CUDA_TRY(ctx, cudaGetLastError());
     }
     DVQLS_CUDA_TRY(ctx, cudaMemcpyAsync(alpha_out, alpha, size_t(Pt) * 8, cudaMemcpyDefault, ctx->stream));
