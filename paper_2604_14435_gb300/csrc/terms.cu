@@ -982,21 +982,31 @@ constexpr int HBM_KQ = 11;
 // Work split.  The shifted states are built before the term kernel
 // (k_tc_states; packed pairs hi | (2 lo) << 16 of 2^12 psi, L2-resident), so
 // the term kernel only streams.  One CTA per SM (it allocates tensor memory)
-// with three warp roles:
-//   - 16 builder warps take items from the queue, load an item's state into
-//     shared memory in four copies (copy t holds psi[k ^ t], so a term's 16
-//     amplitudes of a block are four aligned 16-byte loads: the low two bits
-//     of x_l pick the copy, the next two permute the loads), and write the
-//     operands of each stage (K-major, no swizzle: core matrices of 8 rows x
-//     16 bytes; LBO 128 B between the two halves of a k-step, SBO 256 B between
-//     8-row groups, 18 row groups per k-step: 2 lo rows in groups 0..7, hi
-//     rows in 8..15, the b rows in 16, zeros in 17) into a ring of TC_NSTG
-//     stages, one term's 16 amplitudes at two places of the stage per thread;
+// with four warp roles, three of them once per half (two halves of the CTA work
+// on their own items):
+//   - a loader warp takes the half's items from the queue and prepares the next
+//     one (masks, packed state, parameters) while the builders are on this one;
+//   - 8 builder warps lay the state out in shared memory (split arrays or
+//     copies permuted by the low bits of x_l, so a term's 16 amplitudes of a
+//     block are a few aligned 16-byte loads) and write the operands of each
+//     stage (K-major, no swizzle: core matrices of 8 rows x 16 bytes; LBO 128 B
+//     between the two halves of a k-step, SBO 256 B between 8-row groups, 18 row
+//     groups per k-step: 2 lo rows in groups 0..7, hi rows in 8..15, the b rows
+//     in 16, zeros in 17) into the half's stages of a ring of TC_NSTG, one term's
+//     16 amplitudes at two places of the stage per thread;
 //   - one MMA warp issues each stage into the accumulator of its block and
 //     commits the stage's buffer back to the builders;
 //   - 4 epilogue warps (one per quarter of the tensor-memory lanes) fold each
 //     finished accumulator block, read out an item's Gram and delta and weight
 //     them, while the builders and the MMA warp go on with the next items.
+// What bounds it: no one role.  With the MMAs left out a batch of 32 took 165 us of
+// 181, without building 164, without weighting 178: hand-overs in a chain, and the
+// fetch of instructions for roles that share an SM's four schedulers.  Hence an MMA warp, an
+// epilogue and a loader per half (in place of one MMA warp and eight epilogue warps that
+// polled for both, and an item set-up in the builders), suspended waits, and one code for
+// both kinds of stage: n = 10, L = 64, 32 instances 182 -> 163 us per pass, the local
+// cost 2,504 -> 2,168, L = 256 (8 instances, depth 6) 782 -> 692, two n = 20 instances and
+// 62 small ones 53.0 -> 47.9 ms.
 // The tensor core adds each MMA's sum into the accumulator with a rounding
 // that is not to nearest (measured: a one-sided drift of ~2^-24 |acc| per
 // MMA), so an accumulator block covers TC_FLUSH stages and the epilogue folds
@@ -1011,15 +1021,17 @@ constexpr int HBM_KQ = 11;
 // gives up raises the abort flag, every role stops at its next check, the MMA
 // warp waits for its issued MMAs before the tensor memory is freed, and the
 // host gets DVQLS_ERR_TIMEOUT.
-// Served for tiles with L <= 64 (T = 1) of the global cost.
 constexpr int TCK = 128;            // amplitudes per stage of a diagonal tile: 8 MMA k-steps of 16
 constexpr int TC_BW = 16;           // builder warps
 constexpr int TC_BT = 32 * TC_BW;   // builder threads: one 16-amplitude half-row of one term per stage each
-constexpr int TC_EW = 8;            // epilogue warps, two per quarter of the tensor-memory lanes
+constexpr int TC_EW = 4;            // epilogue warps of a half, one per quarter of the tensor-memory lanes
 constexpr int TC_ET = 32 * TC_EW;
-constexpr int TCT = TC_BT + 32 + TC_ET;  // builders, the MMA warp, the epilogue warps
+constexpr int TCT = TC_BT + 2 * (32 + TC_ET + 32);  // builders, then per half an MMA warp, the epilogue warps, a loader
+constexpr int TC_LOAD_NMAX = 10;         // states up to 2^10 amplitudes are loaded ahead, where there is room
+// Shared memory per half for states of up to 2^n amplitudes loaded ahead (n = 0: none).
+__host__ __device__ inline int tc_load_bytes(int n) { return n > 0 ? 4 << n : 0; }
 constexpr int TC_NSTG = 4;          // operand stages in flight
-constexpr int TC_NIT = 4;           // item records in flight from the builders to the epilogue
+constexpr int TC_NIT = 4;           // item records in flight from a loader to its epilogue
 constexpr int TC_FLUSH = 4;         // stages per accumulator block (8 MMAs of each Gram entry per stage)
 constexpr int TC_NB = 144;          // row groups per k-step x 8: 2 lo and hi of 64 terms, b rows, zero rows
 constexpr uint32_t TC_ACC1 = 256;   // tensor-memory columns of builder half h: 256 h ..
@@ -1100,9 +1112,9 @@ inline size_t tc_psi_region(int nmax_smem, int copy_nmax, int split_nmax) {
 }
 // A state region for each builder half; the shared-memory readout of the
 // epilogue only for passes that return beta or delta (no other item touches it).
-inline size_t tc_smem_bytes(int nmax_smem, int copy_nmax, int split_nmax, bool readout) {
+inline size_t tc_smem_bytes(int nmax_smem, int copy_nmax, int split_nmax, bool readout, int load_nmax = 0) {
     return 1024 + (size_t)TC_NSTG * TC_STAGE_BYTES + 2 * tc_psi_region(nmax_smem, copy_nmax, split_nmax) +
-           (readout ? TC_EPI_BYTES : 0);
+           2 * tc_load_bytes(load_nmax) + (readout ? TC_EPI_BYTES : 0);
 }
 // Stages of the b rows of an instance with 2^n amplitudes.
 __host__ __device__ inline long long tc_bop_stages(long long N) { return (N + TCK - 1) / TCK; }
@@ -1344,20 +1356,9 @@ __device__ __forceinline__ uint64_t tc_desc(uint32_t addr) {
 __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t phase) {
     uint32_t done;
     asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
         : "=r"(done)
-        : "r"(bar), "r"(phase)
-        : "memory");
-    return done != 0;
-}
-// Non-blocking test of an mbarrier phase: for loops that poll several
-// barriers, where a blocking try_wait on one could hold up work on another.
-__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t phase) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(done)
-        : "r"(bar), "r"(phase)
+        : "r"(bar), "r"(phase), "r"(10000u)
         : "memory");
     return done != 0;
 }
@@ -1421,28 +1422,21 @@ __device__ __forceinline__ int tc_off16(int row, int kk) {
     return (((kk >> 4) * (TC_NB / 8) + (row >> 3)) * 2 + ((kk >> 3) & 1)) * 128 + (row & 7) * 16;
 }
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
+    uint32_t r[8];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-    for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
+    for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(r[j]);
 }
-
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16]) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};" ::"r"(
-            taddr),
-        "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])), "r"(__float_as_uint(v[3])),
-        "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])), "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7])),
-        "r"(__float_as_uint(v[8])), "r"(__float_as_uint(v[9])), "r"(__float_as_uint(v[10])),
-        "r"(__float_as_uint(v[11])), "r"(__float_as_uint(v[12])), "r"(__float_as_uint(v[13])),
-        "r"(__float_as_uint(v[14])), "r"(__float_as_uint(v[15]))
-        : "memory");
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const float (&v)[8]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr),
+                 "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])),
+                 "r"(__float_as_uint(v[3])), "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])),
+                 "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7]))
+                 : "memory");
 }
 
 __device__ __forceinline__ float2 tmem_ld2(uint32_t taddr) {
@@ -1459,8 +1453,7 @@ __device__ __forceinline__ void tmem_st2(uint32_t taddr, float2 v) {
 }
 
 // One finished accumulator block (slot columns hb + slot ..) folded by an
-// epilogue warp whose tensor-memory lanes are 32 q .. 32 q + 31 (Gram columns
-// 32 ch .. 32 ch + 31; the delta columns when ch = 0).  Off-diagonal pair
+// epilogue warp whose tensor-memory lanes are 32 q .. 32 q + 31.  Off-diagonal pair
 // (`off`): lanes 0..63 are the first tile's hi rows and lanes 64..127 its lo
 // rows, each against hi + lo of the second tile (two MMAs into the same 64
 // columns; lo lo, ~2^-22 of the product, rides along).  Diagonal tile: lanes
@@ -1477,50 +1470,50 @@ __device__ __forceinline__ void tmem_st2(uint32_t taddr, float2 v) {
 // float-float for the main quadrant, FP32 for the correction quadrant (2 lo hi^T,
 // or a pair's lo rows), SB skipped when every Im c~_m is zero (`imz`) -- and the
 // delta columns are returned in dr.
-__device__ __forceinline__ void tc_fold(uint32_t tmem, uint32_t hb, uint32_t slot, int q, int ch, int lane, bool first,
+__device__ __forceinline__ void tc_fold(uint32_t tmem, uint32_t hb, uint32_t slot, int q, int lane, bool first,
                                         bool last, bool off, bool toX, float* X, float2* XD, const float4* cB,
                                         float& SA, float& EA, float& SB, float& EB, float2& dr, bool imz) {
     const uint32_t base = tmem + ((32u * uint32_t(q)) << 16), acc = hb + slot * TC_SLOT;
     const int xr = (q & 1) * 32 + lane;  // row within the lane half
     float* Xq = X + (q >> 1) * TC_X;
 #pragma unroll 1
-    for (int g = 2 * ch; g < 2 * ch + 2; ++g) {  // this warp's 32 of the quadrant's 64 columns
-        float v[16];
-        tmem_ld16(base + acc + 16 * g, v);
+    for (int g = 0; g < 8; ++g) {  // the quadrant's 64 columns
+        float v[8];
+        tmem_ld8(base + acc + 8 * g, v);
         if (!first) {
-            float u[16];
-            tmem_ld16(base + hb + TC_SUM + 16 * g, u);
+            float u[8];
+            tmem_ld8(base + hb + TC_SUM + 8 * g, u);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) v[j] += u[j];
+            for (int j = 0; j < 8; ++j) v[j] += u[j];
         }
         if (last && toX) {
 #pragma unroll
-            for (int j = 0; j < 16; ++j) Xq[xr * 65 + 16 * g + j] = v[j];
+            for (int j = 0; j < 8; ++j) Xq[xr * 65 + 8 * g + j] = v[j];
         } else if (last && (off ? q >= 2 : q < 2)) {
             // the correction quadrant (2 lo hi^T of a diagonal tile, or the lo rows of a pair's
             // first tile) is ~2^-10 of the main one: FP32 products and sums leave its rounding
             // near 2^-34 of the weighted sum
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const float4 cm = cB[16 * g + j];  // one address per warp: a broadcast
+            for (int j = 0; j < 8; ++j) {
+                const float4 cm = cB[8 * g + j];  // one address per warp: a broadcast
                 SA = fmaf(cm.x, v[j], SA);
                 if (!imz) SB = fmaf(cm.z, v[j], SB);
             }
         } else if (last && imz) {  // every Im c~_m of the columns is zero: the second form is zero
 #pragma unroll
-            for (int j = 0; j < 16; ++j) ff_mac(SA, EA, cB[16 * g + j].x, cB[16 * g + j].y, v[j]);
+            for (int j = 0; j < 8; ++j) ff_mac(SA, EA, cB[8 * g + j].x, cB[8 * g + j].y, v[j]);
         } else if (last) {
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const float4 cm = cB[16 * g + j];  // one address per warp: a broadcast
+            for (int j = 0; j < 8; ++j) {
+                const float4 cm = cB[8 * g + j];  // one address per warp: a broadcast
                 ff_mac(SA, EA, cm.x, cm.y, v[j]);
                 ff_mac(SB, EB, cm.z, cm.w, v[j]);
             }
         } else {
-            tmem_st16(base + hb + TC_SUM + 16 * g, v);
+            tmem_st8(base + hb + TC_SUM + 8 * g, v);
         }
     }
-    if (ch == 0 && !off) {  // the delta columns
+    if (!off) {  // the delta columns
         const float2 d0 = tmem_ld2(base + acc + 64);
         float2 dv;
         if (q < 2) {
@@ -1543,7 +1536,7 @@ __device__ __forceinline__ void tc_fold(uint32_t tmem, uint32_t hb, uint32_t slo
 
 // A builder thread's share of a stage: the 16 amplitudes jb .. jb + 15 of one
 // term at k = kk0 .. kk0 + 15, hi into row rhi of dhi and the low part into
-// row rlo of dlo (doubled as stored, or halved back when HALVE).  psi_hl holds
+// row rlo of dlo (doubled as stored, or halved back when `halve`).  psi_hl holds
 // the Na amplitudes of the state's block that contains the sources (Na = N for
 // states in shared memory).  With jb a multiple of 16, the sources j ^ x_l of the
 // block are rb | (i ^ xlo) with rb = (jb ^ x_l) & ~15: a permutation of 16
@@ -1564,13 +1557,12 @@ __device__ __forceinline__ uint32_t halve2(uint32_t v) {
 // oh, ol: byte offsets tc_off16(rhi, kk0), tc_off16(rlo, kk0) of the two rows
 // (kk0 a multiple of 16, so the second 8 amplitudes sit 128 bytes further).
 // The split arrays' stride is recomputed here from Na rather than passed in:
-// one argument fewer live across the stage loop keeps the kernel's spills
-// at a few bytes under its 72-register cap.
-template <bool HBM, bool HALVE>
+// one argument fewer live across the stage loop of a kernel at its 72-register cap.
+template <bool HBM>
 __device__ __forceinline__ void tc_build_half(const uint32_t* psi_hl, const float* psi_g, int N, int Na, int jb, int kend,
                                               bool act, uint32_t xl, uint32_t zl, const uint32_t (&sgn)[8],
                                               unsigned char* dhi, int oh, unsigned char* dlo, int ol, bool copies,
-                                              bool split) {
+                                              bool split, bool halve) {
     const uint32_t xhi = xl & ~15u, xlo = xl & 15u & uint32_t(N - 1);
     const int nval = act ? min(16, max(0, kend - jb)) : 0;
     const uint32_t rb = (uint32_t(jb) ^ xhi) & uint32_t(N - 1) & ~15u;
@@ -1636,7 +1628,7 @@ __device__ __forceinline__ void tc_build_half(const uint32_t* psi_hl, const floa
         lo.y = lw[4 * g + 1] ^ sgn[4 * g + 1] ^ flip;
         lo.z = lw[4 * g + 2] ^ sgn[4 * g + 2] ^ flip;
         lo.w = lw[4 * g + 3] ^ sgn[4 * g + 3] ^ flip;
-        if (HALVE) {
+        if (halve) {
             lo.x = halve2(lo.x);
             lo.y = halve2(lo.y);
             lo.z = halve2(lo.z);
@@ -1648,24 +1640,39 @@ __device__ __forceinline__ void tc_build_half(const uint32_t* psi_hl, const floa
 }
 
 // Warp roles: two builder halves of 8 warps (warps 0..7 and 8..15), each
-// running its own items -- its own queue fetches, state layout, masks, two of
+// running its own items -- its own loader, state layout, masks, two of
 // the ring's stages (slots 2h, 2h + 1), item records and two accumulator slots
 // (TMEM columns 256 h .., its blocks alternating between them) -- so one
-// half's item set-up (fetch, state load, masks) overlaps the other half's
-// stages; warp 16 issues the MMAs of both halves, taking whichever half has a
-// stage ready; warps 17..24 run the epilogue of both, taking whichever
-// accumulator block has finished (both poll with non-blocking test_wait, so a
-// barrier of one half never holds up the other).  Hand-overs, per half h: a
-// stage by its `full` mbarrier (the half's 256 builder threads arrive after a
-// proxy fence; the stage record -- address of the hi array, first / last stage
-// of an accumulator block, pair flag -- is written first) and back by `empty`
-// (the MMA warp's commit); an accumulator block by accf[h][slot] (commit after
-// its last stage) and back by acce[h][slot] (every epilogue thread, after its
-// tensor-memory loads); an item record (instance, shift, amplitude part, tile
-// item, stages, flavour) by itf[h][r] and back by ite[h][r].  Every wait
-// gives up after budget_ns nanoseconds; a thread that has seen the abort flag
-// waits no more.
+// half's item set-up overlaps the other half's stages; per half one warp that
+// issues its MMAs (warps 16, 17), four epilogue warps (18..21 and 22..25) and the
+// loader (26, 27).  Every role waits on one barrier at a time, in the hardware's
+// suspended wait: one MMA warp and one epilogue group that polled both halves'
+// barriers took a quarter of the SM's issue slots.
+// Hand-overs, per half h: an item by ldf[h] (masks in sxl and szl, the rest in
+// s_item, a state of up to 2^TC_LOAD_NMAX amplitudes in the load area when the
+// layout leaves room for it) and back by lde[h], when every builder warp has it in
+// registers; a stage by its `full` mbarrier (every builder thread arrives after a proxy
+// fence; the stage record -- operand address, first / last stage of an accumulator
+// block, pair flag -- is written first) and back by `empty` (the MMA warp's
+// commit); an accumulator block by
+// accf[h][slot] (commit after its last stage) and back by acce[h][slot] (every
+// epilogue warp, after its tensor-memory loads); an item's record (instance,
+// shift, amplitude part, tile item, stages, flavour) by itf[h][r] and back by
+// ite[h][r].  Every wait gives up after budget_ns nanoseconds; a thread that has
+// seen the abort flag waits no more.
 constexpr int TC_HT = TC_BT / 2;  // threads of a builder half
+// What the builders need of an item (with its masks and, if it is staged, its state).
+struct TcItem {
+    int N, nch, kbeg, kend;
+    int off;     // pair stages; -1: no more items
+    int kind;    // bits: 1 split arrays, 2 packed copies, 4 a block of a state in HBM, 8 gather from HBM, 16 state
+                 // by registers, 32 staged
+    int cnt[2];  // terms of the item's two tiles
+    int Na;      // amplitudes in shared memory
+    const float* psi_g;
+    const void* state;  // the packed state
+    const uint4* bop;   // the b rows of the item's first stage, or null
+};
 __global__ void __launch_bounds__(TCT, 1) k_terms_tc(const Inst* __restrict__ insts, int count, long long total,
                                                      unsigned long long* queue, int* status, int copy_nmax,
                                                      int split_range, int psi_half, long long budget_ns) {
@@ -1673,15 +1680,14 @@ __global__ void __launch_bounds__(TCT, 1) k_terms_tc(const Inst* __restrict__ in
     pdl_trigger();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ __align__(8) unsigned long long fullb[TC_NSTG], emptyb[TC_NSTG], accf[2][2], acce[2][2],
-        itf[2][TC_NIT], ite[2][TC_NIT], drainb;
+        itf[2][TC_NIT], ite[2][TC_NIT], drainb[2], ldf[2], lde[2];
     __shared__ uint32_t srec[TC_NSTG][2];
     __shared__ int4 irec[2][TC_NIT];
-    __shared__ int4 s_cur[2];  // epilogue: the item record each half is on
     __shared__ uint32_t s_tmem;
-    __shared__ long long s_item[2];
-    __shared__ int s_abort, s_pick;
+    __shared__ TcItem s_item[2];  // per half: the next item, from its loader
+    __shared__ int s_abort, s_xlock;  // s_xlock: a half's epilogue is using X, XD
     __shared__ uint32_t sxl[2][128], szl[2][128];  // per half: masks of the item's tile (and of a pair's second)
-    __shared__ float sred[3][2][TC_EW];
+    __shared__ float sred[2][3][2][TC_EW];
     __shared__ __align__(16) float4 scf[2][128];  // per half: c~ of the item's two tiles (zero past L)
     __shared__ long long s_ibase[TC_MAXC];  // item bases of the first TC_MAXC instances
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
@@ -1692,7 +1698,7 @@ __global__ void __launch_bounds__(TCT, 1) k_terms_tc(const Inst* __restrict__ in
     }
     // The readout (X, XD) is allocated only when the pass returns beta or delta; only
     // shift-0 items of such a pass touch it.
-    float* X = reinterpret_cast<float*>(base + TC_NSTG * TC_STAGE_BYTES + 2 * psi_half);
+    float* X = reinterpret_cast<float*>(base + TC_NSTG * TC_STAGE_BYTES + 2 * psi_half + 2 * tc_load_bytes(split_range >> 16));
     float2* XD = reinterpret_cast<float2*>(X + 2 * TC_X);
     if (t == 0) {
         for (int k = 0; k < TC_NSTG; ++k) {
@@ -1702,16 +1708,19 @@ __global__ void __launch_bounds__(TCT, 1) k_terms_tc(const Inst* __restrict__ in
         for (int k = 0; k < 2; ++k) {
             for (int sl = 0; sl < 2; ++sl) {
                 asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&accf[k][sl])), "r"(1));
-                asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&acce[k][sl])), "r"(TC_ET));
+                asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&acce[k][sl])), "r"(TC_EW));
             }
             for (int r = 0; r < TC_NIT; ++r) {
                 asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&itf[k][r])), "r"(1));
-                asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&ite[k][r])), "r"(1));
+                asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&ite[k][r])), "r"(TC_EW));
             }
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&drainb[k])), "r"(1));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&ldf[k])), "r"(1));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&lde[k])), "r"(TC_HT / 32));
         }
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&drainb)), "r"(1));
         asm volatile("fence.mbarrier_init.release.cluster;");
         s_abort = 0;
+        s_xlock = 0;
     }
     // Rows 4..7 of row group 16 and row group 17 of every k-step of every stage
     // stay zero (a diagonal stage's MMA reads them as B rows 68..79; the pair
@@ -1750,124 +1759,81 @@ __global__ void __launch_bounds__(TCT, 1) k_terms_tc(const Inst* __restrict__ in
         const int ohd = tc_off16(TC_HIROW + l, sub * 16), old = tc_off16(l, sub * 16);
         const int ohp = tc_off16(l, 32 * psp), olp = tc_off16(64 + l, 32 * psp);
         uint32_t eph = 0u, pend = 0u;   // bit q: parity of empty[2h + q] to wait for; stage in flight
-        uint32_t iph = 0u, iused = 0u;  // item ring (thread 0 of the half): parity of ite[h][r]; slot used
-        int ir = 0;
-        uint32_t gc = 0u;  // stages the half has handed over
+        uint32_t lph = 0u;  // parity of ldf[h]
+        uint32_t gc = 0u;   // stages the half has handed over
         bool ab = false;
-        long long cur = total, nxt = total;  // thread 0 of the half: this item and the next from the queue
-        if (tt == 0) {
-            cur = (long long)atomicAdd(queue, 1ull);
-            nxt = cur < total ? (long long)atomicAdd(queue, 1ull) : total;
-        }
+        const uint4* lds = reinterpret_cast<const uint4*>(base + TC_NSTG * TC_STAGE_BYTES + 2 * psi_half + h * tc_load_bytes(split_range >> 16));
         for (;;) {
-            if (tt == 0) s_item[h] = (aborted(&s_abort) || ab) ? total : cur;
+            if (lane == 0 && !ab) ab = aborted(&s_abort) || !mbar_wait(su32(&ldf[h]), lph, budget_ns);
+            lph ^= 1u;
+            // every warp has the item, and is done with the one before it
             ab = bar_or(bar, TC_HT, ab);
-            const long long gi = s_item[h];
-            ab = bar_or(bar, TC_HT, ab);
-            if (ab || gi >= total) break;
-            if (tt == 0) {  // the next queue position, fetched while this item runs
-                cur = nxt;
-                nxt = cur < total && !aborted(&s_abort) ? (long long)atomicAdd(queue, 1ull) : total;
-            }
-            const int ii = find_instance_cached(insts, s_ibase, count, gi);
-            const Inst& I = insts[ii];
-            const int local = int(gi - I.item_base);
-            const int n = I.n, N = 1 << n, L = I.L, ks = I.ks, T = I.T, NU = T * (T + 1) / 2;
-            const int ksi = local % ks, u = (local / ks) % NU, f = (local / ks / NU) % I.F, s = (local / ks / NU) / I.F;
-            int tl, tm;
-            tc_tile_pair(u, T, tl, tm);
-            // a pair of different tiles, or a local-cost flavour f > 0 (the second side's
-            // strings X_j A_m = sigma(x_m ^ e_j, z_m), j = f - 1): stages of 64 amplitudes,
-            // [hi; lo] rows on both sides
-            const bool off = tl != tm || f > 0;
-            const uint32_t xflip = f > 0 ? (1u << (f - 1)) : 0u;
-            const int kper = N / ks, kbeg = ksi * kper, kend = kbeg + kper;
+            if (ab) break;
+            const TcItem& it = s_item[h];
+            if (it.off < 0) break;
+            const int N = it.N, nch = it.nch, kbeg = it.kbeg, kend = it.kend, Na = it.Na;
+            const bool off = it.off != 0, blk = it.kind & 4, split = it.kind & 1, copies = it.kind & 2, gl = it.kind & 8;
             const int step = off ? TCK / 2 : TCK;
-            const int nch = (kend - kbeg + step - 1) / step;
-            if (tt == 0) {  // the item's record for the epilogue
-                if ((iused >> ir) & 1u) {
-                    if (!ab && (aborted(&s_abort) || !mbar_wait(su32(&ite[h][ir]), (iph >> ir) & 1u, budget_ns)))
-                        ab = true;
-                    iph ^= 1u << ir;
+            const int side = off ? pside : 0, jb0 = off ? 32 * psp : 16 * sub;
+            const int oh = off ? ohp : ohd, ol = off ? olp : old;
+            const bool act = l < it.cnt[side];
+            const uint32_t xl = xs[side * 64 + l], zl = zs[side * 64 + l];
+            const float* psi_g = it.psi_g;
+            const uint4* bop = it.bop;
+            const int sst = 2 * Na + 16;  // bytes of one split array
+            unsigned char* pb = reinterpret_cast<unsigned char*>(psi_hl);
+            // Group tt of 8 amplitudes (Na / 8 <= 256 groups of a staged state or an HBM block): its packed
+            // words p_i = hi_i | (2 lo)_i << 16.
+            uint32_t pw[8];
+            const bool regs = it.kind & 16, mine = 8 * tt < Na;
+            if (regs) {
+                if (mine) {
+                    uint4 p0, p1;
+                    if (it.kind & 32) {
+                        p0 = lds[2 * tt];
+                        p1 = lds[2 * tt + 1];
+                    } else {
+                        p0 = __ldcg(reinterpret_cast<const uint4*>(it.state) + 2 * tt);
+                        p1 = __ldcg(reinterpret_cast<const uint4*>(it.state) + 2 * tt + 1);
+                    }
+                    pw[0] = p0.x; pw[1] = p0.y; pw[2] = p0.z; pw[3] = p0.w;
+                    pw[4] = p1.x; pw[5] = p1.y; pw[6] = p1.z; pw[7] = p1.w;
                 }
-                iused |= 1u << ir;
-                irec[h][ir] = make_int4(ii, s, ksi | (u << 16), nch | (f << 16));  // ksi < 2^16
-                mbar_arrive(su32(&itf[h][ir]));
-            }
-            ir = (ir + 1) % TC_NIT;
-            if (tt < 128) {
-                const int gt = (tt < 64 ? tl : tm) * TT + (tt & 63);
-                xs[tt] = gt < L ? I.xm[gt] ^ (tt < 64 ? 0u : xflip) : 0u;
-                zs[tt] = gt < L ? I.zm[gt] : 0u;
-            }
-            const float* psi_g = I.states ? reinterpret_cast<const float*>(I.states) + (size_t)s * N : nullptr;
-            // A state in HBM whose item reads only its own block of HBM_K amplitudes
-            // (every X-mask of the item's tiles below HBM_K) is staged once in shared
-            // memory and gathered from there like an on-chip state.
-            bool blk = false;
-            if (I.states) {
-                const int gt = (tt < 64 ? tl : tm) * TT + (tt & 63);
-                const bool far = tt < 128 && gt < L && xs[tt] >= uint32_t(HBM_K);
-                blk = kper == HBM_K && !bar_or(bar, TC_HT, far);
-            }
-            const int Na = blk ? int(HBM_K) : N;  // amplitudes in shared memory
-            // split_range: the largest n of the split arrays in bits 0..7, the smallest (at least 4) in 8..15
-            const int sn = blk ? HBM_KQ : n;
-            const bool split = (!I.states || blk) && tc_split(sn, split_range & 255) && sn >= (split_range >> 8);
-            const bool copies = !split && (!I.states || blk) && tc_copies(blk ? HBM_KQ : n, copy_nmax);
-            const int sst = tc_split_stride(blk ? HBM_KQ : n);  // bytes of one split array
-            if (blk) {  // the item's block of the FP32 state in HBM, split into packed pairs here
-                // the FP32 block lands in the last copy's room (with copies) or in place
-                float* stage = reinterpret_cast<float*>(psi_hl + (copies ? 3 * (Na + 8) : 0));
-                for (int k = 4 * tt; k < Na; k += 4 * TC_HT)
-                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(su32(stage + k)),
-                                 "l"(__cvta_generic_to_global(psi_g + kbeg + k))
-                                 : "memory");
-                asm volatile("cp.async.commit_group;\n\tcp.async.wait_all;" ::: "memory");
-                bar_n(bar, TC_HT);
-                float vb[HBM_K / TC_HT];
+            } else if (blk) {  // the item's block of the FP32 state in HBM, split into packed pairs here
+                if (mine) {
+                    const float4* src = reinterpret_cast<const float4*>(psi_g + kbeg) + 2 * tt;
+                    const float4 f0 = src[0], f1 = src[1];
+                    const float fv[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
 #pragma unroll
-                for (int e = 0; e < HBM_K / TC_HT; ++e) vb[e] = stage[tt * (HBM_K / TC_HT) + e];
-                bar_n(bar, TC_HT);
-                const int ncp = copies ? 4 : 1;
-#pragma unroll
-                for (int e = 0; e < HBM_K / TC_HT; ++e) {
-                    const int k = tt * (HBM_K / TC_HT) + e;
-                    const uint32_t v = split_h2l(vb[e] * TC_SCALE);
-                    for (int t3 = 0; t3 < ncp; ++t3) psi_hl[t3 * (Na + 8) + (k ^ t3)] = v;
+                    for (int e = 0; e < 8; ++e) pw[e] = split_h2l(fv[e] * TC_SCALE);
                 }
-            } else if (!I.states) {  // the packed state of shift s (built by k_tc_states)
-                const uint32_t* src = reinterpret_cast<const uint32_t*>(I.tcst) + (size_t)s * N;
-                // split arrays: the packed words land in the room of the last two lo copies
-                uint32_t* dst = split ? reinterpret_cast<uint32_t*>(reinterpret_cast<unsigned char*>(psi_hl) + 14 * sst)
-                                      : psi_hl;
+            } else if (!gl) {  // a larger (or a tiny) packed state, into place
+                const uint32_t* src = reinterpret_cast<const uint32_t*>(it.state);
                 if (N >= 4) {
                     for (int k = 4 * tt; k < N; k += 4 * TC_HT)
-                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(su32(dst + k)),
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(su32(psi_hl + k)),
                                      "l"(__cvta_generic_to_global(src + k))
                                      : "memory");
                     asm volatile("cp.async.commit_group;\n\tcp.async.wait_all;" ::: "memory");
                 } else if (tt < N) {
-                    dst[tt] = src[tt];
+                    psi_hl[tt] = src[tt];
                 }
             }
-            ab = bar_or(bar, TC_HT, ab);
-            if (split) {
-                // Group gi of 8 amplitudes (one per thread: N / 8 <= 128 groups): its packed words
-                // p_i = hi_i | (2 lo)_i << 16 go to the hi and lo copies t = 0..7, whose words j hold
-                // elements (2j) ^ t, (2j + 1) ^ t of the group: word j ^ (t >> 1) of the pairs in order
-                // (t even) or swapped (t odd).
-                unsigned char* pb = reinterpret_cast<unsigned char*>(psi_hl);
-                const int gi = tt;
-                uint4 p0 = make_uint4(0u, 0u, 0u, 0u), p1 = p0;
-                if (gi < N / 8) {
-                    const uint4* stg = reinterpret_cast<const uint4*>(pb + 14 * sst);
-                    p0 = stg[2 * gi];
-                    p1 = stg[2 * gi + 1];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(su32(&lde[h]));  // this warp has read the item, its masks and its state
+            const bool halve = off && !regs && !blk;  // the low parts of a pair are halved back in the gather, or here
+            if ((regs || blk) && mine) {
+                if (off) {
+                    const __half2 hv = __floats2half2_rn(1.f, 0.5f);
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const __half2 v = __hmul2(*reinterpret_cast<__half2*>(&pw[k]), hv);
+                        pw[k] = *reinterpret_cast<const uint32_t*>(&v);
+                    }
                 }
-                bar_n(bar, TC_HT);  // every staged word is read before the copies overwrite them
-                if (gi < N / 8) {
-                    const uint32_t pw[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
+                if (split) {
+                    // hi and lo copies t = 0..7, whose words j hold elements (2j) ^ t, (2j + 1) ^ t of the
+                    // group: word j ^ (t >> 1) of the pairs in order (t even) or swapped (t odd)
                     uint32_t HP[4], HS[4], LP[4], LS[4];
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
@@ -1881,14 +1847,23 @@ __global__ void __launch_bounds__(TCT, 1) k_terms_tc(const Inst* __restrict__ in
                         const int u = t8 >> 1;
                         const uint32_t* H = (t8 & 1) ? HS : HP;
                         const uint32_t* Lw = (t8 & 1) ? LS : LP;
-                        *reinterpret_cast<uint4*>(pb + t8 * sst + 16 * gi) = make_uint4(H[0 ^ u], H[1 ^ u], H[2 ^ u], H[3 ^ u]);
-                        *reinterpret_cast<uint4*>(pb + (8 + t8) * sst + 16 * gi) =
+                        *reinterpret_cast<uint4*>(pb + t8 * sst + 16 * tt) = make_uint4(H[0 ^ u], H[1 ^ u], H[2 ^ u], H[3 ^ u]);
+                        *reinterpret_cast<uint4*>(pb + (8 + t8) * sst + 16 * tt) =
                             make_uint4(Lw[0 ^ u], Lw[1 ^ u], Lw[2 ^ u], Lw[3 ^ u]);
                     }
+                } else {  // packed copies t (or one): psi[k ^ t] at word t (Na + 8) + k
+                    const int ncp = copies ? 4 : 1;
+#pragma unroll
+                    for (int t3 = 0; t3 < 4; ++t3) {
+                        if (t3 >= ncp) break;
+                        uint4* d = reinterpret_cast<uint4*>(psi_hl + t3 * (Na + 8) + 8 * tt);
+                        d[0] = make_uint4(pw[0 ^ t3], pw[1 ^ t3], pw[2 ^ t3], pw[3 ^ t3]);
+                        d[1] = make_uint4(pw[4 ^ t3], pw[5 ^ t3], pw[6 ^ t3], pw[7 ^ t3]);
+                    }
                 }
-                bar_n(bar, TC_HT);
             }
-            if (copies && !blk) {  // copy t: psi[k ^ t] at word t (N + 8) + k
+            bar_n(bar, TC_HT);
+            if (copies && !regs && !blk) {  // copy t: psi[k ^ t] at word t (N + 8) + k
                 for (int k = tt; k < N; k += TC_HT) {
                     const uint32_t v = psi_hl[k];
 #pragma unroll
@@ -1896,9 +1871,6 @@ __global__ void __launch_bounds__(TCT, 1) k_terms_tc(const Inst* __restrict__ in
                 }
                 bar_n(bar, TC_HT);
             }
-            const int side = off ? pside : 0;
-            const bool act = (side ? tm : tl) * TT + l < L;
-            const uint32_t xl = xs[side * 64 + l], zl = zs[side * 64 + l];
             uint32_t sgn[8];  // word g: sign bits of elements 2g (bit 15) and 2g + 1 (bit 31) of a 16-block
             {
                 const uint32_t xlo = xl & 15u & uint32_t(N - 1);
@@ -1907,7 +1879,6 @@ __global__ void __launch_bounds__(TCT, 1) k_terms_tc(const Inst* __restrict__ in
                     sgn[g] = ((__popc(zl & 15u & (uint32_t(2 * g) ^ xlo)) & 1) ? 0x8000u : 0u) |
                              ((__popc(zl & 15u & (uint32_t(2 * g + 1) ^ xlo)) & 1) ? 0x80000000u : 0u);
             }
-            const bool gl = I.states && !blk;  // gather from the state in HBM
             for (int c = 0; c < nch; ++c, ++gc) {
                 const int q = int(gc & 1u), st = 2 * h + q;
                 if ((pend >> q) & 1u) {  // the MMAs that read this buffer last time must be done
@@ -1919,42 +1890,30 @@ __global__ void __launch_bounds__(TCT, 1) k_terms_tc(const Inst* __restrict__ in
                 unsigned char* zhi = base + st * TC_STAGE_BYTES;
                 unsigned char* zlo = zhi + TC_OPND_BYTES;
                 const int j0 = kbeg + c * step;
-                const bool brow = !off && I.bop && tt < TC_BOP_STAGE / 16;
+                const bool brow = bop && tt < TC_BOP_STAGE / 16;
                 if (brow) {  // the stage's b rows (j0 is a multiple of TCK), copied while the terms are built
-                    const uint4* srcb = reinterpret_cast<const uint4*>(I.bop) + (long long)(j0 / TCK) * (TC_BOP_STAGE / 16) + tt;
+                    const uint4* srcb = bop + c * (TC_BOP_STAGE / 16) + tt;
                     const int ks8 = tt >> 3, kh = (tt >> 2) & 1, br = tt & 3;
                     const uint32_t dst = su32(zhi + ks8 * TC_KSTEP_BYTES + TC_BROW + kh * 128 + br * 16);
                     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n\tcp.async.commit_group;" ::"r"(dst),
                                  "l"(__cvta_generic_to_global(srcb))
                                  : "memory");
                 }
-                if (!off) {
-                    // diagonal: amplitudes kk = 64 hf + 16 sub .. of the stage, hi to row
-                    // TC_HIROW + l and 2 lo to row l of the same k-steps
+                // Two blocks of 16 amplitudes of the thread's term, one code for both kinds of stage
+                // (a second copy of it for pairs cost 5 % of a batch that mixes them, in instruction fetches):
+                // diagonal: amplitudes kk = 64 hf + 16 sub .. of the stage, hi to row TC_HIROW + l and 2 lo to
+                // row l of the same k-steps; pair: the side's array (hi array: first tile, 2 lo array:
+                // second), hi to row l and lo (halved back) to row 64 + l
+                unsigned char* dst = side ? zlo : zhi;
 #pragma unroll 1
-                    for (int hf = 0; hf < 2; ++hf) {
-                        const int jb = j0 + hf * (TCK / 2) + sub * 16, dk = hf * TC_OFF_HALF;
-                        if (gl)
-                            tc_build_half<true, false>(nullptr, psi_g, N, Na, jb, kend, act, xl, zl, sgn, zhi,
-                                                       ohd + dk, zhi, old + dk, false, false);
-                        else
-                            tc_build_half<false, false>(psi_hl, nullptr, N, Na, jb, kend, act, xl, zl, sgn, zhi,
-                                                        ohd + dk, zhi, old + dk, copies, split);
-                    }
-                } else {
-                    // pair: the side's array (hi array: first tile, 2 lo array: second),
-                    // hi to row l and lo (halved back) to row 64 + l
-                    unsigned char* dst = pside ? zlo : zhi;
-#pragma unroll 1
-                    for (int qb = 0; qb < 2; ++qb) {
-                        const int jb = j0 + (2 * psp + qb) * 16, dk = qb * TC_KSTEP_BYTES;
-                        if (gl)
-                            tc_build_half<true, true>(nullptr, psi_g, N, Na, jb, kend, act, xl, zl, sgn, dst, ohp + dk,
-                                                      dst, olp + dk, false, false);
-                        else
-                            tc_build_half<false, true>(psi_hl, nullptr, N, Na, jb, kend, act, xl, zl, sgn, dst, ohp + dk,
-                                                       dst, olp + dk, copies, split);
-                    }
+                for (int hf = 0; hf < 2; ++hf) {
+                    const int jb = j0 + jb0 + (off ? 16 * hf : hf * (TCK / 2)), dk = off ? hf * TC_KSTEP_BYTES : hf * TC_OFF_HALF;
+                    if (gl)
+                        tc_build_half<true>(nullptr, psi_g, N, Na, jb, kend, act, xl, zl, sgn, dst, oh + dk, dst, ol + dk,
+                                            false, false, off);
+                    else
+                        tc_build_half<false>(psi_hl, nullptr, N, Na, jb, kend, act, xl, zl, sgn, dst, oh + dk, dst, ol + dk,
+                                             copies, split, halve);
                 }
                 if (brow) asm volatile("cp.async.wait_all;" ::: "memory");
                 if (tt == 0) {
@@ -1967,58 +1926,46 @@ __global__ void __launch_bounds__(TCT, 1) k_terms_tc(const Inst* __restrict__ in
                 pend |= 1u << q;
             }
         }
-        // No more items: an exit stage for the MMA warp and an exit record for
-        // the epilogue (their waits are bounded whatever happens here).
+        // No more items: an exit stage for the MMA warp (its waits are bounded whatever happens here).
         {
             const int q = int(gc & 1u), st = 2 * h + q;
             if (((pend >> q) & 1u) && !ab && !aborted(&s_abort)) mbar_wait(su32(&emptyb[st]), (eph >> q) & 1u, budget_ns);
             if (tt == 0) srec[st][0] = TC_EXIT;
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             mbar_arrive(su32(&fullb[st]));
-            if (tt == 0) {
-                if (((iused >> ir) & 1u) && !ab && !aborted(&s_abort))
-                    mbar_wait(su32(&ite[h][ir]), (iph >> ir) & 1u, budget_ns);
-                irec[h][ir] = make_int4(-1, 0, 0, 0);
-                mbar_arrive(su32(&itf[h][ir]));
-            }
         }
         if (ab) s_abort = 1;
-    } else if (w == TC_BW) {  // ------------------------------------------------------------- MMA warp
+    } else if (w < TC_BW + 2) {  // ---------------------------------------------------- MMA warp of half h
         if (lane == 0) {
-            // per half h: next ring slot (bit h), parity of full[2h + q] (bit 2h + q), accumulator slot
-            // of the block in progress (bit h) and of the next block (bit h); per accumulator slot sl of
-            // half h (bit 2h + sl): parity of acce[h][sl], slot used before; done (bit h)
-            uint32_t nq = 0u, fph = 0u, csl = 0u, nsl = 0u, aph = 0u, aused = 0u, done = 0u;
-            unsigned long long idle0 = gtimer_ns();
-            while (done != 3u) {
-                bool progressed = false;
-                for (int h = 0; h < 2; ++h) {
-                    if ((done >> h) & 1u) continue;
-                    const int q = (nq >> h) & 1, st = 2 * h + q;
-                    if (!mbar_test(su32(&fullb[st]), (fph >> st) & 1u)) continue;
-                    asm volatile("tcgen05.fence::after_thread_sync;");
-                    const uint32_t hb = srec[st][0], fl = srec[st][1];
-                    if (hb != TC_EXIT && (fl & 1u)) {
-                        // first stage of a block: its slot must have been read out by the epilogue
-                        // (the block before last of this half); the other half meanwhile
-                        const uint32_t sl = (nsl >> h) & 1u, sb = 2u * h + sl;
-                        if ((aused >> sb) & 1u) {
-                            if (!mbar_test(su32(&acce[h][sl]), (aph >> sb) & 1u)) continue;
-                            aph ^= 1u << sb;
-                            asm volatile("tcgen05.fence::after_thread_sync;");
+            const int h = w - TC_BW;
+            // per ring slot q: parity of full[2h + q]; the accumulator slot of the block in progress and of the
+            // next one; per slot: parity of acce[h][sl], used before
+            uint32_t nq = 0u, fph = 0u, sl = 0u, nsl = 0u, aph = 0u, aused = 0u;
+            for (;;) {
+                const int q = int(nq), st = 2 * h + q;
+                if (aborted(&s_abort) || !mbar_wait(su32(&fullb[st]), (fph >> q) & 1u, budget_ns)) {
+                    s_abort = 1;
+                    break;
+                }
+                fph ^= 1u << q;
+                nq ^= 1u;
+                asm volatile("tcgen05.fence::after_thread_sync;");
+                const uint32_t hb = srec[st][0], fl = srec[st][1];
+                if (hb == TC_EXIT) break;
+                if (fl & 1u) {  // first stage of a block: the block before last has left its slot
+                    sl = nsl;
+                    nsl ^= 1u;
+                    if ((aused >> sl) & 1u) {
+                        if (aborted(&s_abort) || !mbar_wait(su32(&acce[h][sl]), (aph >> sl) & 1u, budget_ns)) {
+                            s_abort = 1;
+                            break;
                         }
-                        aused |= 1u << sb;
-                        csl = (csl & ~(1u << h)) | (sl << h);
-                        nsl ^= 1u << h;
+                        aph ^= 1u << sl;
+                        asm volatile("tcgen05.fence::after_thread_sync;");
                     }
-                    fph ^= 1u << st;
-                    nq ^= 1u << h;
-                    progressed = true;
-                    if (hb == TC_EXIT) {
-                        done |= 1u << h;
-                        continue;
-                    }
-                    const uint32_t sl = (csl >> h) & 1u;
+                    aused |= 1u << sl;
+                }
+                {
                     const uint32_t lb = hb + TC_OPND_BYTES, tm = s_tmem + uint32_t(h) * TC_ACC1 + sl * TC_SLOT;
                     if (fl & 4u) {  // pair: [hi; lo] of the first tile against hi, then lo, of the second
                         const uint64_t dA = tc_desc(hb), dB = tc_desc(lb);
@@ -2065,80 +2012,179 @@ __global__ void __launch_bounds__(TCT, 1) k_terms_tc(const Inst* __restrict__ in
                         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                             su32(&accf[h][sl])));
                 }
-                if (progressed) {
-                    idle0 = gtimer_ns();
-                } else if (aborted(&s_abort) || (long long)(gtimer_ns() - idle0) > budget_ns) {
-                    s_abort = 1;
-                    break;
-                }
             }
             // Every MMA issued has completed before the tensor memory is freed.
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                su32(&drainb)));
-            if (!mbar_wait(su32(&drainb), 0u, TC_DRAIN_NS)) s_abort = 1;
+                su32(&drainb[h])));
+            if (!mbar_wait(su32(&drainb[h]), 0u, TC_DRAIN_NS)) s_abort = 1;
         }
         __syncwarp();
-    } else {  // ----------------------------------------------------------------------------- epilogue
-        const int et = t - (TC_BT + 32), ew = et >> 5, q = w & 3, ch = ew >> 2;  // q: this warp's TMEM lane quarter
-        // Thread 0 keeps, per half, the item-ring position, the ring's parities and
-        // whether it holds the current record, and the accumulator slot of the
-        // half's next block with the parities of accf; every thread keeps the
-        // block count.
-        uint32_t fph = 0u, aph = 0u, esl = 0u, have = 0u, done = 0u;
-        int r[2] = {0, 0}, blkc[2] = {0, 0}, last_pick = 1;
-        bool ab = false;
-        for (;;) {
-            if (et == 0) {  // the half whose accumulator block is ready next
-                int pick = -1, pslot = 0;
-                const unsigned long long t0 = gtimer_ns();
-                for (;;) {
-                    for (int k = 1; k <= 2 && pick < 0; ++k) {
-                        const int hh = (last_pick + k) & 1;
-                        if ((done >> hh) & 1u) continue;
-                        if (!((have >> hh) & 1u)) {
-                            const uint32_t pb = hh * TC_NIT + r[hh];
-                            if (!mbar_test(su32(&itf[hh][r[hh]]), (fph >> pb) & 1u)) continue;
-                            fph ^= 1u << pb;
-                            const int4 rc = irec[hh][r[hh]];
-                            s_cur[hh] = rc;
-                            if (rc.x < 0) {
-                                done |= 1u << hh;
-                                continue;
-                            }
-                            have |= 1u << hh;
-                        }
-                        const uint32_t sl = (esl >> hh) & 1u, sb = 2u * hh + sl;
-                        if (mbar_test(su32(&accf[hh][sl]), (aph >> sb) & 1u)) {
-                            aph ^= 1u << sb;
-                            esl ^= 1u << hh;
-                            pick = hh;
-                            pslot = int(sl);
-                        }
-                    }
-                    if (pick >= 0 || done == 3u) break;
-                    if (aborted(&s_abort) || (long long)(gtimer_ns() - t0) > budget_ns) {
-                        pick = -2;
-                        break;
-                    }
-                }
-                if (pick >= 0) last_pick = pick;
-                s_pick = pick | (pslot << 4);
+    } else if (w >= TC_BW + 2 + 2 * TC_EW) {  // ------------------------------------------- loader of half h
+        // Takes the half's items from the queue and prepares each while the builders are on the one
+        // before it: decodes it, leaves its masks, its packed state (up to 2^TC_LOAD_NMAX amplitudes; a
+        // block of a state in HBM is brought into L2) and its parameters in shared memory, and passes its
+        // record to the epilogue.
+        const int h = w - (TC_BW + 2 + 2 * TC_EW);
+        uint32_t* xs = sxl[h];
+        uint32_t* zs = szl[h];
+        unsigned char* lds = base + TC_NSTG * TC_STAGE_BYTES + 2 * psi_half + h * tc_load_bytes(split_range >> 16);
+        uint32_t eph = 0u, iph = 0u, iused = 0u;  // parities of lde[h] and ite[h][r]; record slot used
+        int ir = 0;
+        bool used = false, ab = false;
+        auto wait = [&](uint32_t bar, uint32_t phase) {
+            int ok = 1;
+            if (lane == 0) ok = !aborted(&s_abort) && mbar_wait(bar, phase, budget_ns);
+            return __shfl_sync(0xffffffffu, ok, 0) != 0;
+        };
+        auto record = [&](int4 rec) {  // to the epilogue
+            if ((iused >> ir) & 1u) {
+                if (!wait(su32(&ite[h][ir]), (iph >> ir) & 1u)) return false;
+                iph ^= 1u << ir;
             }
-            bar_n(3, TC_ET);
-            const int pick = s_pick < 0 ? s_pick : (s_pick & 15), slot = s_pick < 0 ? 0 : (s_pick >> 4);
-            if (pick == -2) ab = true;
-            if (pick < 0) break;
-            const int4 rc = s_cur[pick];
+            iused |= 1u << ir;
+            if (lane == 0) {
+                irec[h][ir] = rec;
+                mbar_arrive(su32(&itf[h][ir]));
+            }
+            ir = (ir + 1) % TC_NIT;
+            return true;
+        };
+        for (;;) {
+            // One item ahead, not two: the last items of the queue spread evenly.
+            if (used) {
+                if (!wait(su32(&lde[h]), eph)) {  // the builders have read the item before
+                    ab = true;
+                    break;
+                }
+                eph ^= 1u;
+            }
+            used = true;
+            long long gi = 0;
+            if (lane == 0) gi = (long long)atomicAdd(queue, 1ull);
+            gi = __shfl_sync(0xffffffffu, gi, 0);
+            TcItem it;
+            it.off = -1;
+            uint32_t mx[4], mz[4];
+            int4 rec = make_int4(-1, 0, 0, 0);
+            const void* src = nullptr;
+            if (gi < total) {
+                const int ii = find_instance_cached(insts, s_ibase, count, gi);
+                const Inst& I = insts[ii];
+                int local = int(gi - I.item_base);
+                const int n = I.n, N = 1 << n, L = I.L, ks = I.ks, T = I.T, NU = T * (T + 1) / 2;
+                const int ksi = local % ks;
+                local /= ks;
+                const int u = local % NU;
+                local /= NU;
+                const int f = local % I.F, s = local / I.F;
+                int tl, tm;
+                tc_tile_pair(u, T, tl, tm);
+                // a pair of different tiles, or a local-cost flavour f > 0 (the second side's
+                // strings X_j A_m = sigma(x_m ^ e_j, z_m), j = f - 1): stages of 64 amplitudes,
+                // [hi; lo] rows on both sides
+                it.off = tl != tm || f > 0;
+                const uint32_t xflip = f > 0 ? (1u << (f - 1)) : 0u;
+                const int kper = N / ks, step = it.off ? TCK / 2 : TCK;
+                it.N = N;
+                it.kbeg = ksi * kper;
+                it.kend = it.kbeg + kper;
+                it.nch = (kper + step - 1) / step;
+                it.cnt[0] = min(TT, L - tl * TT);
+                it.cnt[1] = min(TT, L - tm * TT);
+                bool far = false;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int e = lane + 32 * k, gt = (e < 64 ? tl : tm) * TT + (e & 63);
+                    mx[k] = gt < L ? I.xm[gt] ^ (e < 64 ? 0u : xflip) : 0u;
+                    mz[k] = gt < L ? I.zm[gt] : 0u;
+                    far |= mx[k] >= uint32_t(HBM_K);
+                }
+                it.psi_g = I.states ? reinterpret_cast<const float*>(I.states) + (size_t)s * N : nullptr;
+                // A state in HBM whose item reads only its own block of HBM_K amplitudes (every X-mask
+                // of the item's tiles below HBM_K) is staged in shared memory by the builders and
+                // gathered from there like an on-chip state.
+                const bool blk = I.states && kper == HBM_K && !__any_sync(0xffffffffu, far);
+                it.Na = blk ? int(HBM_K) : N;
+                // split_range: the largest n of the split arrays in bits 0..7, the smallest (at least 4) in
+                // 8..15, the largest n loaded ahead in 16.. (0: no room for it)
+                const int sn = blk ? HBM_KQ : n;
+                const bool sm = !I.states || blk;
+                const bool split = sm && tc_split(sn, split_range & 255) && sn >= ((split_range >> 8) & 255);
+                const bool copies = !split && sm && tc_copies(sn, copy_nmax);
+                const bool regs = !I.states && n >= 3 && (1 << n) <= 8 * TC_HT, staged = regs && n <= (split_range >> 16);
+                it.kind = (split ? 1 : 0) | (copies ? 2 : 0) | (blk ? 4 : 0) | (I.states && !blk ? 8 : 0) | (regs ? 16 : 0) | (staged ? 32 : 0);
+                it.state = I.states ? nullptr : reinterpret_cast<const uint32_t*>(I.tcst) + (size_t)s * N;
+                it.bop = !it.off && I.bop ? reinterpret_cast<const uint4*>(I.bop) + (long long)(it.kbeg / TCK) * (TC_BOP_STAGE / 16) : nullptr;
+                if (staged) src = it.state;
+                if (blk)
+                    for (int k = lane; k < int(HBM_K) * 4 / 128; k += 32)
+                        asm volatile("prefetch.global.L2 [%0];" ::"l"(__cvta_generic_to_global(it.psi_g + it.kbeg + 32 * k)));
+                rec = make_int4(ii, s, ksi | (u << 16), it.nch | (f << 16));  // ksi < 2^16
+            }
+            if (it.off >= 0) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    xs[lane + 32 * k] = mx[k];
+                    zs[lane + 32 * k] = mz[k];
+                }
+                if (src)
+                    for (int k = 16 * lane; k < 4 * it.N; k += 16 * 32)
+                        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(su32(lds + k)),
+                                     "l"(__cvta_generic_to_global(reinterpret_cast<const unsigned char*>(src) + k))
+                                     : "memory");
+                asm volatile("cp.async.commit_group;\n\tcp.async.wait_all;" ::: "memory");
+            }
+            if (lane == 0) s_item[h] = it;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(su32(&ldf[h]));
+            if (!record(rec)) {
+                ab = true;
+                break;
+            }
+            if (it.off < 0) break;
+        }
+        if (ab) s_abort = 1;
+    } else {  // ----------------------------------------------------------------------------- epilogue
+        const int ee = t - (TC_BT + 64), h = ee / TC_ET, et = ee % TC_ET, ew = et >> 5, q = w & 3;  // q: TMEM lane quarter
+        const int ebar = 3 + h;
+        // item-ring position and its parities, the accumulator slot of the half's next block with the
+        // parities of accf, the block within the item
+        uint32_t fph = 0u, aph = 0u, slot = 0u;
+        int r = 0, b = 0;
+        bool ab = false;
+        // Every warp waits by itself (its first lane); a wait that gives up ends the whole half together.
+        auto wait = [&](uint32_t bar, uint32_t phase) {
+            int ok = 1;
+            if (lane == 0) ok = !aborted(&s_abort) && mbar_wait(bar, phase, budget_ns);
+            return __shfl_sync(0xffffffffu, ok, 0) != 0;
+        };
+        int4 rc = make_int4(-1, 0, 0, 0);
+        for (;;) {
+            if (b == 0) {
+                const bool ok = wait(su32(&itf[h][r]), (fph >> r) & 1u);
+                if (ok) rc = irec[h][r];
+                if (bar_or(ebar, TC_ET, !ok)) {
+                    ab = true;
+                    break;
+                }
+                fph ^= 1u << r;
+                if (rc.x < 0) break;
+            }
+            if (bar_or(ebar, TC_ET, !wait(su32(&accf[h][slot]), (aph >> slot) & 1u))) {
+                ab = true;
+                break;
+            }
+            aph ^= 1u << slot;
             const Inst& I = insts[rc.x];
             const int s = rc.y, ksi = rc.z & 0xFFFF, u = rc.z >> 16, nch = rc.w & 0xFFFF, f = rc.w >> 16;
             const int L = I.L, ks = I.ks, T = I.T;
             int tl, tm;
             tc_tile_pair(u, T, tl, tm);
             const bool off = tl != tm || f > 0;
-            const int nblk = (nch + TC_FLUSH - 1) / TC_FLUSH, b = blkc[pick];
+            const int nblk = (nch + TC_FLUSH - 1) / TC_FLUSH;
             const bool lastb = b + 1 == nblk;
-            float4* cfh = scf[pick];
-            if (b == 0 && et < 128) {  // c~ of the item's two tiles, fetched while its blocks run
+            float4* cfh = scf[h];
+            if (b == 0) {  // c~ of the item's two tiles, fetched while its blocks run
                 const int gl = ((et >> 6) ? tm : tl) * TT + (et & 63);
                 if (gl < L)
                     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n\tcp.async.commit_group;" ::"r"(
@@ -2155,25 +2201,42 @@ __global__ void __launch_bounds__(TCT, 1) k_terms_tc(const Inst* __restrict__ in
             bool imz = false;  // the column weights c~_m of the item are all real (a real A gives real c~)
             if (lastb && !toX) {
                 asm volatile("cp.async.wait_all;" ::: "memory");
-                bar_n(3, TC_ET);  // c~ of the item's tiles is in cfh
+                bar_n(ebar, TC_ET);  // c~ of the item's tiles is in cfh
                 const float4 c0 = cfh[(off ? 64 : 0) + lane], c1 = cfh[(off ? 64 : 0) + 32 + lane];
                 imz = __all_sync(0xffffffffu, c0.z == 0.f && c0.w == 0.f && c1.z == 0.f && c1.w == 0.f);
             }
             float SA = 0.f, EA = 0.f, SB = 0.f, EB = 0.f;
             float2 dr = make_float2(0.f, 0.f);
+            if (lastb && toX) {  // one half at a time in X, XD (a few items of a pass)
+                int got = 1;
+                if (et == 0) {
+                    const unsigned long long t0 = gtimer_ns();
+                    while (atomicCAS(&s_xlock, 0, 1) != 0)
+                        if (aborted(&s_abort) || (long long)(gtimer_ns() - t0) > budget_ns) {
+                            got = 0;
+                            break;
+                        }
+                }
+                if (bar_or(ebar, TC_ET, !got)) {
+                    ab = true;
+                    break;
+                }
+            }
             asm volatile("tcgen05.fence::after_thread_sync;");
-            tc_fold(s_tmem, uint32_t(pick) * TC_ACC1, uint32_t(slot), q, ch, lane, b == 0, lastb, off, toX, X, XD,
+            tc_fold(s_tmem, uint32_t(h) * TC_ACC1, slot, q, lane, b == 0, lastb, off, toX, X, XD,
                     cfh + (off ? 64 : 0), SA, EA, SB, EB, dr, imz);
             asm volatile("tcgen05.fence::before_thread_sync;");
-            mbar_arrive(su32(&acce[pick][slot]));
-            blkc[pick] = lastb ? 0 : b + 1;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(su32(&acce[h][slot]));
+            slot ^= 1u;
             if (!lastb) {
-                bar_n(3, TC_ET);  // s_pick and s_cur are read before thread 0 writes them again
+                ++b;
                 continue;
             }
+            b = 0;
             if (toX) {
                 asm volatile("cp.async.wait_all;" ::: "memory");
-                bar_n(3, TC_ET);  // the readout is in X (and XD), c~ in cfh
+                bar_n(ebar, TC_ET);  // the readout is in X (and XD), c~ in cfh
             }
             const int nl = min(TT, L - tl * TT);  // terms in the first tile
             const float* Xu = X;
@@ -2192,7 +2255,7 @@ __global__ void __launch_bounds__(TCT, 1) k_terms_tc(const Inst* __restrict__ in
                 E += fac * cl.x * EA;
                 ff_mac(S, E, fac * cl.z, fac * cl.w, SB);
                 E += fac * cl.z * EB;
-                if (!off && ch == 0 && a < nl && !I.local) {  // this quadrant's part of delta~_a
+                if (!off && a < nl && !I.local) {  // this quadrant's part of delta~_a
                     const float dsc = 1.f / (TC_SCALE * tc_bscale(*I.bn2));  // exact: a power of two
                     const float2 dacc = make_float2(dr.x * dsc, -dr.y * dsc);  // conj(b) phi
                     ff_mac(TrS, TrE, cl.x, cl.y, dacc.x);
@@ -2209,14 +2272,14 @@ __global__ void __launch_bounds__(TCT, 1) k_terms_tc(const Inst* __restrict__ in
                 // of the first tile and b of the second (for flavour f > 0, gamma^j_ab);
                 // different tiles stand for both orders of the pair (the Gram, gamma^j
                 // and Re w are symmetric), so those count twice (exact doubling).  Thread
-                // et takes row a = et / 4 and columns 8 (et % 4) + j, 32 + 8 (et % 4) + j
-                // (j < 8: one bank per lane); terms past L have c~ = 0 and zero rows.
+                // et takes row a = et / 2 and columns 16 g + 8 (et % 2) + j (g < 4, j < 8);
+                // terms past L have c~ = 0.
                 const float4* cB = cfh + (off ? 64 : 0);
-                const int a = et >> 2, cq = et & 3;
+                const int a = et >> 1, cq = et & 1;
                 float SA = 0.f, EA = 0.f, SB = 0.f, EB = 0.f;
-#pragma unroll
-                for (int k = 0; k < 16; ++k) {
-                    const int bc = ((k >> 3) << 5) | (cq << 3) | (k & 7);
+#pragma unroll 4
+                for (int k = 0; k < 32; ++k) {
+                    const int bc = ((k >> 3) << 4) | (cq << 3) | (k & 7);
                     const float g = Xu[a * 65 + bc] + Xl[a * 65 + bc];
                     const float4 cm = cB[bc];
                     ff_mac(SA, EA, cm.x, cm.y, g);
@@ -2258,21 +2321,23 @@ __global__ void __launch_bounds__(TCT, 1) k_terms_tc(const Inst* __restrict__ in
             ff_warp_sum(TrS, TrE);
             ff_warp_sum(TiS, TiE);
             if (lane == 0) {
-                sred[0][0][ew] = S;
-                sred[0][1][ew] = E;
-                sred[1][0][ew] = TrS;
-                sred[1][1][ew] = TrE;
-                sred[2][0][ew] = TiS;
-                sred[2][1][ew] = TiE;
+                sred[h][0][0][ew] = S;
+                sred[h][0][1][ew] = E;
+                sred[h][1][0][ew] = TrS;
+                sred[h][1][1][ew] = TrE;
+                sred[h][2][0][ew] = TiS;
+                sred[h][2][1][ew] = TiE;
+                mbar_arrive(su32(&ite[h][r]));  // this warp has read the item's record
             }
-            bar_n(3, TC_ET);
+            bar_n(ebar, TC_ET);  // and is done with X, XD and cfh
+            r = (r + 1) % TC_NIT;
             if (et == 0) {  // FP64 only for the final pairs, added in a fixed order
                 double qv[3];
                 for (int k = 0; k < 3; ++k) {
                     float S2 = 0.f, E2 = 0.f;
                     for (int v = 0; v < TC_EW; ++v) {
-                        ff_add(S2, E2, sred[k][0][v]);
-                        E2 += sred[k][1][v];
+                        ff_add(S2, E2, sred[h][k][0][v]);
+                        E2 += sred[h][k][1][v];
                     }
                     qv[k] = (double)S2 + (double)E2;
                 }
@@ -2283,12 +2348,12 @@ __global__ void __launch_bounds__(TCT, 1) k_terms_tc(const Inst* __restrict__ in
                 I.Dpart[slot2 * ks + ksi] = make_double2(qv[0] * (double)TC_UNSCALE, 0.0);
                 if (tl != tm) I.Dpart[(slot2 + 1) * ks + ksi] = make_double2(0.0, 0.0);
                 else if (f == 0 && !I.local) I.Tpart[((long long)s * T + tl) * ks + ksi] = make_double2(qv[1], qv[2]);
-                // the half's item record is free again
-                mbar_arrive(su32(&ite[pick][r[pick]]));
-                r[pick] = (r[pick] + 1) % TC_NIT;
-                have &= ~(1u << pick);
+                if (toX) {
+                    __threadfence_block();
+                    atomicExch(&s_xlock, 0);
+                }
             }
-            bar_n(3, TC_ET);  // X, sred and s_cur are free again
+            bar_n(ebar, TC_ET);  // sred is free again
         }
         asm volatile("cp.async.wait_all;" ::: "memory");  // no copy into shared memory outlives the CTA
         if (ab) s_abort = 1;
@@ -3077,7 +3142,7 @@ __global__ void __launch_bounds__(WHT_NT, 2) k_terms_wht64(const Inst* __restric
 // Adds the partial sums of a shift where there are many (states in HBM: one per
 // 2,048 amplitudes), a warp per shift, lanes in stride and then a fixed tree, into
 // the shift's first slots.  In the combine one thread per shift added them: 406 us
-// for the uneven batch (n = 20: 441 shifts x 512 slots), 20 with this.
+// for the uneven batch (n = 20: 441 shifts x 512 slots), 14 with this and 9 left in the combine.
 constexpr int FOLD_MIN = 64;  // slots per shift from which it is worth a launch
 __global__ void __launch_bounds__(256) k_fold(const Inst* __restrict__ insts) {
     pdl_wait();
@@ -3268,6 +3333,7 @@ struct PassShape {
     int copy_nmax;   // tensor-core kernel: states of 2^4 .. 2^copy_nmax amplitudes kept in four copies (0: none)
     int split_nmax;  // tensor-core kernel: states of 2^split_nmin .. 2^split_nmax amplitudes kept as split
     int split_nmin;  // hi / lo arrays (split_nmax 0: none)
+    int load_nmax;   // tensor-core kernel: states of up to 2^load_nmax amplitudes loaded ahead (0: none)
     int psi_region;  // tensor-core kernel: shared bytes of a builder half's state copies
     int st_grid;     // tensor-core pass: CTAs per instance of k_tc_states (0: no state in shared memory)
     int st_smem;     // and its dynamic shared bytes
@@ -3323,7 +3389,8 @@ static int launch_pass(dvqls_ctx* ctx, cudaStream_t st, const Inst* dtable, cons
                                        ps.total, ctx->d_queue));
     else if (ps.tc)
         DVQLS_CUDA_TRY(ctx, launch_pdl(k_terms_tc, dim3(ps.grid), dim3(TCT), ps.smem, st, dtable, ps.count, ps.total,
-                                       ctx->d_queue, ctx->d_status, ps.copy_nmax, ps.split_nmax | (ps.split_nmin << 8), ps.psi_region,
+                                       ctx->d_queue, ctx->d_status, ps.copy_nmax, ps.split_nmax | (ps.split_nmin << 8) | (ps.load_nmax << 16),
+                                       ps.psi_region,
                                        ps.budget_ns));
     else if (ps.fp32)
         DVQLS_CUDA_TRY(ctx, launch_pdl(k_terms_smem<float>, dim3(ps.grid), dim3(NT), ps.smem, st, dtable, ps.count,
@@ -3461,7 +3528,7 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
     bool wht = precision == DVQLS_FP32_WHT || precision == DVQLS_FP64;
     for (const auto& h : hi) wht = wht && h.T == 1 && h.n <= WHT_MAXN;
     bool tc = !wht && (precision == DVQLS_FP32_TC || (precision == DVQLS_FP32_WHT && !local));
-    int copy_nmax = 0, split_nmax = 0;
+    int copy_nmax = 0, split_nmax = 0, load_nmax = 0;
     const bool readout = beta_out || delta_out;
     // the tensor-core kernel's shared state region: the largest on-chip state, and
     // a staged block of HBM_K amplitudes when some state lives in HBM
@@ -3478,6 +3545,10 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
             if (tc_smem_bytes(tc_nsm, c, 0, readout) + fa.sharedSizeBytes <= (size_t)optin) copy_nmax = c;
         for (int c = std::min(TC_SPLIT_NMAX, tc_nsm); tc && c >= 4 && !split_nmax; --c)
             if (tc_smem_bytes(tc_nsm, copy_nmax, c, readout) + fa.sharedSizeBytes <= (size_t)optin) split_nmax = c;
+        // room to load the on-chip states ahead, if the layouts leave it
+        const int ld = any_smem ? std::min(nmax, TC_LOAD_NMAX) : 0;
+        if (tc && ld >= 3 && tc_smem_bytes(tc_nsm, copy_nmax, split_nmax, readout, ld) + fa.sharedSizeBytes <= (size_t)optin)
+            load_nmax = ld;
     }
     // The tensor-core pass builds the on-chip states in a kernel of its own.
     int st_grid = 0;
@@ -3490,7 +3561,7 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
             }
     if (st_grid > 0) DVQLS_CUDA_TRY(ctx, allow_dynamic_smem((const void*)k_tc_states));
     const size_t smem = wht  ? (fp32 ? wht_smem_bytes(Pmax) : w64_smem_bytes(Pmax))
-                        : tc ? tc_smem_bytes(tc_nsm, copy_nmax, split_nmax, readout)
+                        : tc ? tc_smem_bytes(tc_nsm, copy_nmax, split_nmax, readout, load_nmax)
                         : fp32 ? smem_bytes<float>(nmax, Pmax) : smem_bytes<double>(nmax, Pmax);
     const size_t r2 = fp32 ? 8 : 16;
     auto kfun = wht ? (fp32 ? (const void*)k_terms_wht : (const void*)k_terms_wht64)
@@ -3718,6 +3789,7 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
         ps.smem = smem;
         ps.copy_nmax = copy_nmax;
         ps.split_nmax = split_use;
+        ps.load_nmax = load_nmax;
         ps.split_nmin = split_min;
         ps.psi_region = tc ? (int)tc_psi_region(tc_nsm, copy_nmax, split_nmax) : 0;
         ps.st_grid = st_grid;
