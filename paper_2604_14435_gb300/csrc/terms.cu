@@ -1004,9 +1004,11 @@ constexpr int HBM_KQ = 11;
 // fetch of instructions for roles that share an SM's four schedulers.  Hence an MMA warp, an
 // epilogue and a loader per half (in place of one MMA warp and eight epilogue warps that
 // polled for both, and an item set-up in the builders), suspended waits, and one code for
-// both kinds of stage: n = 10, L = 64, 32 instances 182 -> 163 us per pass, the local
-// cost 2,504 -> 2,168, L = 256 (8 instances, depth 6) 782 -> 692, two n = 20 instances and
-// 62 small ones 53.0 -> 47.9 ms.
+// both kinds of stage: n = 10, L = 64, 32 instances 182 -> 158 us per pass, the local
+// cost 2,504 -> 2,116, L = 256 (8 instances, depth 6) 782 -> 677, two n = 20 instances and
+// 62 small ones 53.0 -> 47.2 ms.  Now without building 131 us of 163, without MMAs 148,
+// without weighting 160.  Stages of half the size (twice as many in the ring) took 201:
+// what a stage costs is its hand-over as much as its work.
 // The tensor core adds each MMA's sum into the accumulator with a rounding
 // that is not to nearest (measured: a one-sided drift of ~2^-24 |acc| per
 // MMA), so an accumulator block covers TC_FLUSH stages and the epilogue folds
@@ -1369,8 +1371,7 @@ __device__ __forceinline__ unsigned long long gtimer_ns() {
 }
 // Waits for phase `phase` of an mbarrier for at most budget_ns nanoseconds of
 // the global timer (and at most 2^32 tries, should the timer not advance).
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t phase, long long budget_ns) {
-    if (mbar_try(bar, phase)) return true;
+__device__ __forceinline__ bool mbar_wait_on(uint32_t bar, uint32_t phase, long long budget_ns) {
     const unsigned long long t0 = gtimer_ns();
     for (long long it = 0; it < (1LL << 32); ++it) {
         if (mbar_try(bar, phase)) return true;
@@ -1378,8 +1379,17 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t phase, long lon
     }
     return false;
 }
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t phase, long long budget_ns) {
+    return mbar_try(bar, phase) || mbar_wait_on(bar, phase, budget_ns);
+}
 // The abort flag as other roles may have just written it.
 __device__ __forceinline__ bool aborted(const int* f) { return *reinterpret_cast<const volatile int*>(f) != 0; }
+// A wait that has already been met reads one barrier and nothing else (a look at the
+// abort flag before each wait, on the chain of every stage, cost 2.5 %); one that has
+// not is given up at once when the CTA has aborted.
+__device__ __forceinline__ bool role_wait(const int* abort, uint32_t bar, uint32_t phase, long long budget_ns) {
+    return mbar_try(bar, phase) || (!aborted(abort) && mbar_wait_on(bar, phase, budget_ns));
+}
 
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
     asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}\n" ::"r"(bar) : "memory");
@@ -1764,7 +1774,7 @@ __global__ void __launch_bounds__(TCT, 1) k_terms_tc(const Inst* __restrict__ in
         bool ab = false;
         const uint4* lds = reinterpret_cast<const uint4*>(base + TC_NSTG * TC_STAGE_BYTES + 2 * psi_half + h * tc_load_bytes(split_range >> 16));
         for (;;) {
-            if (lane == 0 && !ab) ab = aborted(&s_abort) || !mbar_wait(su32(&ldf[h]), lph, budget_ns);
+            if (lane == 0 && !ab) ab = !role_wait(&s_abort, su32(&ldf[h]), lph, budget_ns);
             lph ^= 1u;
             // every warp has the item, and is done with the one before it
             ab = bar_or(bar, TC_HT, ab);
@@ -1882,7 +1892,7 @@ __global__ void __launch_bounds__(TCT, 1) k_terms_tc(const Inst* __restrict__ in
             for (int c = 0; c < nch; ++c, ++gc) {
                 const int q = int(gc & 1u), st = 2 * h + q;
                 if ((pend >> q) & 1u) {  // the MMAs that read this buffer last time must be done
-                    if (!ab && (aborted(&s_abort) || !mbar_wait(su32(&emptyb[st]), (eph >> q) & 1u, budget_ns)))
+                    if (!ab && (!role_wait(&s_abort, su32(&emptyb[st]), (eph >> q) & 1u, budget_ns)))
                         ab = true;
                     eph ^= 1u << q;
                     pend &= ~(1u << q);
@@ -1943,7 +1953,7 @@ __global__ void __launch_bounds__(TCT, 1) k_terms_tc(const Inst* __restrict__ in
             uint32_t nq = 0u, fph = 0u, sl = 0u, nsl = 0u, aph = 0u, aused = 0u;
             for (;;) {
                 const int q = int(nq), st = 2 * h + q;
-                if (aborted(&s_abort) || !mbar_wait(su32(&fullb[st]), (fph >> q) & 1u, budget_ns)) {
+                if (!role_wait(&s_abort, su32(&fullb[st]), (fph >> q) & 1u, budget_ns)) {
                     s_abort = 1;
                     break;
                 }
@@ -1956,7 +1966,7 @@ __global__ void __launch_bounds__(TCT, 1) k_terms_tc(const Inst* __restrict__ in
                     sl = nsl;
                     nsl ^= 1u;
                     if ((aused >> sl) & 1u) {
-                        if (aborted(&s_abort) || !mbar_wait(su32(&acce[h][sl]), (aph >> sl) & 1u, budget_ns)) {
+                        if (!role_wait(&s_abort, su32(&acce[h][sl]), (aph >> sl) & 1u, budget_ns)) {
                             s_abort = 1;
                             break;
                         }
@@ -2033,7 +2043,7 @@ __global__ void __launch_bounds__(TCT, 1) k_terms_tc(const Inst* __restrict__ in
         bool used = false, ab = false;
         auto wait = [&](uint32_t bar, uint32_t phase) {
             int ok = 1;
-            if (lane == 0) ok = !aborted(&s_abort) && mbar_wait(bar, phase, budget_ns);
+            if (lane == 0) ok = role_wait(&s_abort, bar, phase, budget_ns);
             return __shfl_sync(0xffffffffu, ok, 0) != 0;
         };
         auto record = [&](int4 rec) {  // to the epilogue
@@ -2155,7 +2165,7 @@ __global__ void __launch_bounds__(TCT, 1) k_terms_tc(const Inst* __restrict__ in
         // Every warp waits by itself (its first lane); a wait that gives up ends the whole half together.
         auto wait = [&](uint32_t bar, uint32_t phase) {
             int ok = 1;
-            if (lane == 0) ok = !aborted(&s_abort) && mbar_wait(bar, phase, budget_ns);
+            if (lane == 0) ok = role_wait(&s_abort, bar, phase, budget_ns);
             return __shfl_sync(0xffffffffu, ok, 0) != 0;
         };
         int4 rc = make_int4(-1, 0, 0, 0);
