@@ -38,41 +38,41 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // FP32 products on 64 x 64 tiles, 4 x 4 outputs per thread, the operands of 16
-// steps of k staged in shared memory with the next 16 in registers meanwhile.
-// One row of threads per k needs two 16-byte shared loads for 16 FMAs, which
-// the FMA pipe bounds.  64 x 64 (not larger) so that the batch of 2,000 with 256
-// hidden units still gives 128 CTAs.  Loads are single floats: the weights
-// start at any multiple of four bytes in the flat parameter vector.  A training
-// step of that batch: 96 us of kernels, against 840 with 16 x 16 tiles, no split
-// over the batch (16 CTAs for the 256 x 256 gradient) and bias gradients of one
-// thread per column.
+// steps of k staged in shared memory by asynchronous copies, three tiles ahead.
+// One row of threads per k needs two 16-byte shared loads for 16 FMAs, which the
+// FMA pipe bounds; but a CTA has its SM to itself here, so a tile's 512 cycles of
+// FMAs do not cover a load from L2 one tile ahead (in registers: 123 us for the step
+// below; with copies three ahead 110).  64 x 64 (not larger) so that the batch of 2,000
+// with 256 hidden units still gives 128 CTAs.  A training step of that batch took 605 us
+// with 16 x 16 tiles, no split over the batch (16 CTAs for the 256 x 256 gradient) and
+// bias gradients of one thread per column.  Two groups of 256 threads per CTA, each with
+// every other tile of k, gave 114.
 constexpr int GT = 64, GK = 16, GTH = 256;
 
-// Operand element (row, k) of a tile: row-major with k contiguous (KMAJOR) or
-// with the row contiguous.
+constexpr int GSTG = 4;  // tiles of k in shared memory: three on the way while one is multiplied
+
+struct GemmSmem {
+    float A[GSTG][GK][GT + 4], B[GSTG][GK][GT + 4];
+};
+
+// Operand tile (rows row0 .., k0 .. k0 + GK - 1) into S[k][row], zero outside, by
+// asynchronous copies: row-major with k contiguous (KMAJOR) or with the row
+// contiguous.  Single floats: a matrix of the flat parameter vector starts at any
+// multiple of four bytes.
 template <bool KMAJOR>
-__device__ __forceinline__ void gemm_fetch(const float* __restrict__ P, long long ld, int row0, int rows, int k0, int kend,
-                                           float (&v)[4]) {
+__device__ __forceinline__ void gemm_fetch(float (*S)[GT + 4], const float* __restrict__ P, long long ld, int row0, int rows,
+                                           int k0, int kend) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         const int e = threadIdx.x + q * GTH;
         const int r = KMAJOR ? e / GK : e % GT, k = KMAJOR ? e % GK : e / GT;
-        v[q] = (row0 + r < rows && k0 + k < kend) ? (KMAJOR ? P[(row0 + r) * ld + k0 + k] : P[(k0 + k) * ld + row0 + r])
-                                                  : 0.f;
+        const bool in = row0 + r < rows && k0 + k < kend;
+        const float* src = in ? (KMAJOR ? P + (row0 + r) * ld + k0 + k : P + (k0 + k) * ld + row0 + r) : P;
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(&S[k][r])),
+                     "l"(__cvta_generic_to_global(src)), "r"(in ? 4 : 0)
+                     : "memory");
     }
 }
-template <bool KMAJOR>
-__device__ __forceinline__ void gemm_stash(float (*S)[GT + 4], const float (&v)[4]) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int e = threadIdx.x + q * GTH;
-        S[KMAJOR ? e % GK : e / GT][KMAJOR ? e / GK : e % GT] = v[q];
-    }
-}
-
-struct GemmSmem {
-    float A[2][GK][GT + 4], B[2][GK][GT + 4];
-};
 
 // acc[i][j] = sum over k in [k0, kend) of A(m0 + 4 ty + i, k) B(k, n0 + 4 tx + j);
 // rsum (threads below 64, when wanted): the sum over k of A(m0 + t, k).
@@ -85,18 +85,21 @@ __device__ __forceinline__ void gemm_tile(GemmSmem& sm, const float* __restrict_
     for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-    float va[4], vb[4];
-    gemm_fetch<AK>(A, lda, m0, M, k0, kend, va);
-    gemm_fetch<BK>(B, ldb, n0, N, k0, kend, vb);
-    int buf = 0;
-    for (int k = k0; k < kend; k += GK, buf ^= 1) {
-        gemm_stash<AK>(sm.A[buf], va);
-        gemm_stash<BK>(sm.B[buf], vb);
-        __syncthreads();  // the other buffer was read before the last barrier
-        if (k + GK < kend) {
-            gemm_fetch<AK>(A, lda, m0, M, k + GK, kend, va);
-            gemm_fetch<BK>(B, ldb, n0, N, k + GK, kend, vb);
+    const int tiles = (kend - k0 + GK - 1) / GK;
+    auto issue = [&](int u) {  // one group of copies per tile, empty past the last
+        if (u < tiles) {
+            gemm_fetch<AK>(sm.A[u % GSTG], A, lda, m0, M, k0 + u * GK, kend);
+            gemm_fetch<BK>(sm.B[u % GSTG], B, ldb, n0, N, k0 + u * GK, kend);
         }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+#pragma unroll
+    for (int u = 0; u < GSTG - 1; ++u) issue(u);
+    for (int u = 0; u < tiles; ++u) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(GSTG - 2) : "memory");
+        __syncthreads();  // tile u is there for all threads, and all have read tile u - 1
+        issue(u + GSTG - 1);
+        const int buf = u % GSTG;
 #pragma unroll
         for (int q = 0; q < GK; ++q) {
             const float4 a = *reinterpret_cast<const float4*>(&sm.A[buf][q][4 * ty]);
