@@ -74,6 +74,12 @@ typedef enum {
 /* Arithmetic of the state build and the term reductions.  The FP32 paths
  * keep the coefficient-weighted L^2 sum, the cost ratio and the gradient
  * combine in FP64.
+ *   DVQLS_FP64:    FP64 states and term reductions.  When every instance has
+ *                  L <= 64 and n <= 10 the terms come by Walsh-Hadamard
+ *                  classes (as DVQLS_FP32_WHT below) with state, products and
+ *                  transforms in 64-bit fixed point (units of 2^-60): the
+ *                  same accuracy as the FP64 tiles (1e-12 of the parity
+ *                  tests; 1.2e-15 measured at n = 10), in less time.
  *   DVQLS_FP32:    FP32 states, FP32 term reductions on the CUDA cores.
  *   DVQLS_FP32_TC: FP32 states; the term Gram on the tensor cores
  *                  (tcgen05 kind::f16: every amplitude, scaled by 2^12,
@@ -257,7 +263,8 @@ typedef struct {
  * 2^9 amplitudes, or packed copies) where they fit -- on the real inputs (the
  * fastest of three passes per candidate) and keeps the fastest for the
  * context (an autotuner; that call is synchronous), unless dvqls_set_tuning
- * fixed the choices.  The kernel sequence of a
+ * fixed the choices.  Passes by Walsh-Hadamard classes have neither split
+ * nor layout and time nothing.  The kernel sequence of a
  * pass is captured once as a CUDA graph and replayed while the instance
  * table (shapes and pointers) is unchanged; with profiling enabled, or when
  * the caller is capturing the stream, kernels are launched directly.
@@ -484,8 +491,8 @@ int dvqls_ws_load(dvqls_ctx* ctx, const char* path, dvqls_ws** out);
  * code running inside a memory pool or allocator that owns the whole device,
  * a real-time loop whose allocation pattern is fixed, or a plugin host that
  * forbids cudaMalloc.  It computes what dvqls_cost_grad computes in
- * DVQLS_FP64 or DVQLS_FP32 (the same kernels; no beta / delta output)
- * without a context: it calls no cudaMalloc, cudaFree, cudaMallocHost or
+ * DVQLS_FP64 or DVQLS_FP32 (always the CUDA-core tiles; no beta / delta
+ * output) without a context: it calls no cudaMalloc, cudaFree, cudaMallocHost or
  * other allocating routine.
  *
  * Its scratch is one fixed device array of DVQLS_NOALLOC_SCRATCH_BYTES
