@@ -58,14 +58,18 @@ __global__ void __launch_bounds__(FT) k_fidelity(const FidInst* __restrict__ ins
     __shared__ double rnx[FT / 32];
     const FidInst I = insts[blockIdx.x];
     const int N = 1 << I.n;
+    bool bad = false;
     for (int a = threadIdx.x; a < I.P; a += FT) {
         const double al = I.alpha[a];
-        if (!isfinite(al)) atomicCAS(status, 0, DEV_NONFINITE_INPUT);
+        if (!isfinite(al)) {
+            atomicCAS(status, 0, DEV_NONFINITE_INPUT);
+            bad = true;
+        }
         double s, c;
         sincos(0.5 * al, &s, &c);
         I.cs[a] = make_double2(c, s);
     }
-    __syncthreads();
+    bad = __syncthreads_or(bad);  // fixed point holds no NaN
     const Fx* psi = build_state_fx(smem, I.n, I.d, I.P, I.cs, 0);
     double2 ov = make_double2(0.0, 0.0), nx = make_double2(0.0, 0.0);
     for (int j = threadIdx.x; j < N; j += FT) {
@@ -95,7 +99,7 @@ __global__ void __launch_bounds__(FT) k_fidelity(const FidInst* __restrict__ ins
     }
     if (threadIdx.x == 0) {
         if (!(nx.x > 0.0) || !isfinite(nx.x)) atomicCAS(status, 0, DEV_BAD_NORM);
-        *I.F = (ov.x * ov.x + ov.y * ov.y) / nx.x;
+        *I.F = bad ? __longlong_as_double(0x7ff8000000000000LL) : (ov.x * ov.x + ov.y * ov.y) / nx.x;
     }
 }
 

@@ -2407,7 +2407,8 @@ constexpr size_t WHT_OFF_DT = WHT_OFF_DO + 4 * 65;                  // uint16 te
 constexpr size_t WHT_OFF_EZ = (WHT_OFF_DT + 2 * 64 + 15) & ~size_t(15);  // uint16 z_l ^ z_m by class
 constexpr size_t WHT_OFF_EK = (WHT_OFF_EZ + 2 * WHT_MAXP + 15) & ~size_t(15);  // signed weights by class: float2, or
                                                                                // double (FP64)
-constexpr size_t WHT_OFF_BIM = WHT_OFF_EK + 8 * WHT_MAXP;  // int: b has a nonzero imaginary part
+constexpr size_t WHT_OFF_BIM = WHT_OFF_EK + 8 * WHT_MAXP;  // int: bit 0 b has a nonzero imaginary part, bit 1 an angle
+                                                           // is not finite
 constexpr size_t WHT_TABLE_BYTES = WHT_OFF_BIM + 16;          // header: int pair classes, term classes
 // Fixed point of the FP64 classes (units of 2^-FX_BITS): b is scaled by a power
 // of two so that ||b|| <= 1.
@@ -2448,7 +2449,7 @@ __global__ void __launch_bounds__(WHT_CT) k_wht_prepare(const Inst* __restrict__
     __shared__ unsigned short cnt[WHT_RANK_WARPS][BINS], rank[WHT_MAXP];
     __shared__ int start[BINS], part[32], cpart[32];
     __shared__ double red[8], s_bn2;
-    __shared__ int s_im;
+    __shared__ int s_im, s_bad;
     __shared__ unsigned s_first[2];
     const Inst I = insts[blockIdx.x];
     const int L = I.L, t = threadIdx.x, w = t >> 5, lane = t & 31, np = L * (L + 1) / 2;
@@ -2456,7 +2457,7 @@ __global__ void __launch_bounds__(WHT_CT) k_wht_prepare(const Inst* __restrict__
     unsigned char* tb = reinterpret_cast<unsigned char*>(I.wht);
     if (queue && blockIdx.x == 0 && t == 0) *queue = 0ull;  // the term kernel's work queue
     for (int k = t; k < WHT_RANK_WARPS * BINS / 2; k += WHT_CT) reinterpret_cast<uint32_t*>(cnt)[k] = 0u;
-    if (t == 0) s_im = 0;
+    if (t == 0) s_im = s_bad = 0;
     if (t < L) {
         const uint32_t x = I.xm[t], z = I.zm[t];
         const double2 c = I.coef[t];
@@ -2505,7 +2506,10 @@ __global__ void __launch_bounds__(WHT_CT) k_wht_prepare(const Inst* __restrict__
     } else {
         for (int a = t - 512; a < I.P; a += 512) {
             const double al = I.alpha[a];
-            if (!isfinite(al)) set_status(status, DEV_NONFINITE_INPUT);
+            if (!isfinite(al)) {
+                set_status(status, DEV_NONFINITE_INPUT);
+                s_bad = 1;
+            }
             double s0, c0;
             sincos(0.5 * al, &s0, &c0);
             const double s1 = (s0 + c0) * M_SQRT1_2, c1 = (c0 - s0) * M_SQRT1_2;  // alpha/2 +- pi/4, as in k_prepare
@@ -2561,7 +2565,7 @@ __global__ void __launch_bounds__(WHT_CT) k_wht_prepare(const Inst* __restrict__
             s_bn2 = sum;
             *I.bn2 = sum;
             if (!(sum > 0.0) || !isfinite(sum)) set_status(status, DEV_BAD_NORM);
-            *reinterpret_cast<int*>(tb + WHT_OFF_BIM) = s_im;
+            *reinterpret_cast<int*>(tb + WHT_OFF_BIM) = s_im | s_bad << 1;
         }
     }
     __syncthreads();
@@ -2776,7 +2780,7 @@ __device__ void wht_item(const Inst& I, int s, const float* psi, const float2* s
     const uint16_t* dt = reinterpret_cast<const uint16_t*>(tb + WHT_OFF_DT);
     // One list of transforms for the warps: the pair classes, then the term
     // classes (Re, and Im when b has an imaginary part: dim stays zero else).
-    const int parts = 1 + *reinterpret_cast<const int*>(tb + WHT_OFF_BIM);
+    const int parts = 1 + (*reinterpret_cast<const int*>(tb + WHT_OFF_BIM) & 1);
     const int jobs = ncls + nd * parts;
 #pragma unroll 1
     for (int j = w; j < jobs; j += WHT_NT / 32) {
@@ -2957,6 +2961,12 @@ inline size_t wht_smem_bytes(int Pmax) {
 // lookups 31 k; both are bound by the integer multiply-adds and adds.
 constexpr int W64_ROW = (1 << WHT_MAXN) + (1 << WHT_MAXN) / 32;
 
+// Value of one fixed-point unit, from an instance's class table: NaN when one of its
+// angles is not finite (reported in the status word; fixed point itself holds no NaN).
+__device__ __forceinline__ double w64_unit(const unsigned char* tb) {
+    return *reinterpret_cast<const int*>(tb + WHT_OFF_BIM) & 2 ? __longlong_as_double(0x7ff8000000000000LL) : 0x1p-60;
+}
+
 // Transform of v (index (r << 5) | lane) into the warp's row, at i + (i >> 5)
 // for 2^10 values (A = 32: through the row, lane bits become register bits), else at i.
 template <int A, int LOGA>
@@ -3018,7 +3028,7 @@ __device__ void w64_item(const Inst& I, int s, const Fx* q, long long* row, doub
     const int* dof = reinterpret_cast<const int*>(tb + WHT_OFF_DO);
     const uint16_t* dt = reinterpret_cast<const uint16_t*>(tb + WHT_OFF_DT);
     double2* Gp = (s == 0 && I.Gpart) ? reinterpret_cast<double2*>(I.Gpart) : nullptr;
-    const int parts = 1 + *reinterpret_cast<const int*>(tb + WHT_OFF_BIM);
+    const int parts = 1 + (*reinterpret_cast<const int*>(tb + WHT_OFF_BIM) & 1);
     const int pairs = ncls * I.F, jobs = pairs + (I.local ? 0 : nd * parts);
     auto at = [&](uint32_t z) { return row[PAD ? z + (z >> 5) : z]; };
 #pragma unroll 1
@@ -3034,7 +3044,7 @@ __device__ void w64_item(const Inst& I, int s, const Fx* q, long long* row, doub
                 v[r] = fx_mul(part ? fx_neg(Fx{bb.z, bb.w}) : Fx{bb.x, bb.y}, q[i]);
             }
             w64_transform<A, LOGA>(v, row, N, lane);
-            const double sc = scalbn(1.0, w64_bexp(*I.bn2) - FX_BITS);
+            const double sc = scalbn(w64_unit(tb), w64_bexp(*I.bn2));
             for (int e = dof[c] + lane; e < dof[c + 1]; e += 32) {
                 const int l = dt[e];
                 (part ? dim : dre)[l] = (double)at(szl[l] & uint32_t(N - 1)) * sc;
@@ -3062,7 +3072,7 @@ __device__ void w64_item(const Inst& I, int s, const Fx* q, long long* row, doub
         if (Gp)  // the beta output of the unshifted state
             for (int e = e0 + lane; e < e1; e += 32) {
                 const int p = pr[e], l = p & 0xFF, m = p >> 8;
-                double beta = (double)at(ez[e]) * 0x1p-60;
+                double beta = (double)at(ez[e]) * w64_unit(tb);
                 if (__popc(szl[l] & uint32_t(x)) & 1) beta = -beta;
                 Gp[(long long)l * L + m] = make_double2(beta, 0.0);
                 Gp[(long long)m * L + l] = make_double2(beta, 0.0);
@@ -3131,8 +3141,8 @@ __global__ void __launch_bounds__(WHT_NT, 2) k_terms_wht64(const Inst* __restric
             if (lane == 0) redT[w] = T;
         }
         __syncthreads();
-        const double unit = 0x1p-60;
         if (t == 0) {
+            const double unit = w64_unit(reinterpret_cast<const unsigned char*>(I.wht));
             double Ds = 0.0, Es = 0.0;
             for (int k = 0; k < WHT_NT / 32; ++k) {
                 Ds += red[k];

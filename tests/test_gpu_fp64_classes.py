@@ -97,3 +97,29 @@ def test_table_follows_the_precision(dv, ctx):
         cost, grad = np.zeros(1), np.zeros(alpha.size)
         dv.dvqls_cost_grad(ctx, an, alpha, lcu, bb, prec, cost, grad)
         assert abs(cost[0] - ref["cost"]) <= tol * max(1.0, abs(ref["cost"])), prec
+
+
+def test_non_finite_angles_give_nan(dv, ctx):
+    """Fixed point holds no NaN: an instance with one is reported and its outputs are NaN; the others are right."""
+    n, d, L = 6, 2, 20
+    P = n * (d + 1)
+    coef, xs, zs, b = problem(n, L, 3, "band")
+    alpha = wl.random_angles(2 * P, 5)
+    alpha[3] = np.nan
+    ref = oterms.cost_grad(n, d, alpha[P:], b / np.linalg.norm(b), coef, xs, zs)
+    dev = [torch.tensor(v, device="cuda") for v in (cvec(coef), xs.view(np.int32), zs.view(np.int32), cvec(b), alpha)]
+    an, lcu = dv.make_ansatz(n, d), dv.make_lcu(L, dev[0], dev[1], dev[2])
+    for local in (False, True):
+        costs, grads = torch.zeros(2, device="cuda", dtype=torch.float64), torch.zeros(2 * P, device="cuda", dtype=torch.float64)
+        arr = dv.make_instances([(an, lcu, dev[4][:P], dev[3]), (an, lcu, dev[4][P:], dev[3])])
+        call = dv.dvqls_local_cost_grad_batched if local else dv.dvqls_cost_grad_batched
+        with pytest.raises(dv.DvqlsError) as e:
+            call(ctx, arr, dv.DVQLS_FP64, costs, grads)
+            dv.dvqls_sync(ctx)
+        assert e.value.code == dv.DVQLS_ERR_INVALID_ARG
+        c, g = costs.cpu().numpy(), grads.cpu().numpy()
+        assert np.isnan(c[0]) and np.isnan(g[:P]).all()
+        if not local:
+            assert abs(c[1] - ref["cost"]) <= 1e-12 and np.abs(g[P:] - ref["grad"]).max() <= 1e-12
+        else:
+            assert np.isfinite(c[1]) and np.isfinite(g[P:]).all()
