@@ -1004,9 +1004,9 @@ constexpr int HBM_KQ = 11;
 // fetch of instructions for roles that share an SM's four schedulers.  Hence an MMA warp, an
 // epilogue and a loader per half (in place of one MMA warp and eight epilogue warps that
 // polled for both, and an item set-up in the builders), suspended waits, and one code for
-// both kinds of stage: n = 10, L = 64, 32 instances 182 -> 158 us per pass, the local
-// cost 2,504 -> 2,116, L = 256 (8 instances, depth 6) 782 -> 677, two n = 20 instances and
-// 62 small ones 53.0 -> 47.2 ms.  Now without building 131 us of 163, without MMAs 148,
+// both kinds of stage: n = 10, L = 64, 32 instances 182 -> 159 us per pass, the local
+// cost 2,504 -> 2,122, L = 256 (8 instances, depth 6) 782 -> 681, two n = 20 instances and
+// 62 small ones 53.0 -> 47.3 ms.  Now without building 131 us of 163, without MMAs 148,
 // without weighting 160.  Stages of half the size (twice as many in the ring) took 201:
 // what a stage costs is its hand-over as much as its work.
 // The tensor core adds each MMA's sum into the accumulator with a rounding
@@ -2041,9 +2041,18 @@ __global__ void __launch_bounds__(TCT, 1) k_terms_tc(const Inst* __restrict__ in
         uint32_t eph = 0u, iph = 0u, iused = 0u;  // parities of lde[h] and ite[h][r]; record slot used
         int ir = 0;
         bool used = false, ab = false;
+        // The builders take an item when they have built the one before it, with a bounded wait per
+        // stage: the loader waits that many times over, and no longer than until the CTA aborts.
+        int stages = 0, before = 0;  // of the item published last, and of the one before it
         auto wait = [&](uint32_t bar, uint32_t phase) {
             int ok = 1;
-            if (lane == 0) ok = role_wait(&s_abort, bar, phase, budget_ns);
+            if (lane == 0) {
+                const long long limit = budget_ns * (stages + before + 4);
+                const unsigned long long t0 = gtimer_ns();
+                long long tries = 1LL << 32;  // as mbar_wait's
+                do ok = mbar_try(bar, phase);
+                while (!ok && --tries && !aborted(&s_abort) && (long long)(gtimer_ns() - t0) <= limit);
+            }
             return __shfl_sync(0xffffffffu, ok, 0) != 0;
         };
         auto record = [&](int4 rec) {  // to the epilogue
@@ -2144,6 +2153,8 @@ __global__ void __launch_bounds__(TCT, 1) k_terms_tc(const Inst* __restrict__ in
                                      : "memory");
                 asm volatile("cp.async.commit_group;\n\tcp.async.wait_all;" ::: "memory");
             }
+            before = stages;
+            stages = it.off >= 0 ? it.nch : 0;
             if (lane == 0) s_item[h] = it;
             __syncwarp();
             if (lane == 0) mbar_arrive(su32(&ldf[h]));
