@@ -46,7 +46,8 @@ cudaError_t allow_dynamic_smem(const void* fn) {
     return e;
 }
 
-int ensure_workspace(dvqls_ctx* ctx, size_t bytes) {
+int ensure_workspace(dvqls_ctx* ctx, size_t bytes, size_t table_bytes) {
+    if (ctx->last_table.size() != table_bytes) ctx->last_table.clear();
     if (bytes <= ctx->ws_cap) return DVQLS_OK;
     DVQLS_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
     ctx->last_table.clear();

@@ -75,7 +75,9 @@ struct dvqls_ctx {
     // host-to-device copy out of it; it is waited on before the next write.
     cudaEvent_t pin_event = nullptr;
     bool pin_event_live = false;
-    // Last instance table uploaded by the batched call (skipped when equal).
+    // The instance table at the start of the workspace, as the batched call
+    // uploaded it (an equal one is not uploaded again); empty when another call
+    // has planned the workspace since.
     std::vector<char> last_table;
 
     // Kernel timing (dvqls_profile_*): event pairs not yet read, a pool of
@@ -154,7 +156,12 @@ class Arena {
     size_t total_ = 0;
 };
 
-int ensure_workspace(dvqls_ctx* ctx, size_t bytes);
+// Makes `bytes` of workspace available to the caller, who may write all of it:
+// the instance table that the batched cost pass left at its start (last_table)
+// counts as overwritten from then on.  Only run_batch, which puts its own table
+// of table_bytes there and everything else behind it, keeps a table of that size,
+// unless the workspace moves.
+int ensure_workspace(dvqls_ctx* ctx, size_t bytes, size_t table_bytes = 0);
 // Wait until no copy out of the pinned staging is pending, so it can be
 // written again; pin_release records the end of the copies just enqueued.
 int pin_acquire(dvqls_ctx* ctx);

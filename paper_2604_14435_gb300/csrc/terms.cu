@@ -3699,7 +3699,7 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
         o.chain = h.hbm && h.S + h.s0 > 1 ? ar.reserve((2 * size_t(h.d) + 1) * size_t(h.N) * (r2 / 2)) : 0;
         o.tcst = tc && !h.hbm ? ar.reserve(size_t(h.S) * size_t(h.N) * 4) : 0;     // packed FP16 pairs
     }
-    int rc = ensure_workspace(ctx, ar.total());
+    int rc = ensure_workspace(ctx, ar.total(), sizeof(Inst) * count);
     if (!rc) rc = ensure_pinned(ctx, pin.total());
     if (rc) return rc;
     char* ws = ctx->ws;
