@@ -267,7 +267,11 @@ typedef struct {
  * nor layout and time nothing.  The kernel sequence of a
  * pass is captured once as a CUDA graph and replayed while the instance
  * table (shapes and pointers) is unchanged; with profiling enabled, or when
- * the caller is capturing the stream, kernels are launched directly.
+ * the caller is capturing the stream, kernels are launched directly.  A pass
+ * that the caller captured brings its instance table with every launch of the
+ * graph; it works in the context's workspace, so the graph serves until a
+ * larger call makes that grow, and not at the same time as other work of the
+ * context.
  * Errors: as dvqls_cost_grad, for any instance; INVALID_ARG for count < 1
  * (an empty batch) or inst NULL. */
 int dvqls_cost_grad_batched(dvqls_ctx* ctx, int count, const dvqls_instance* inst,

@@ -3446,18 +3446,33 @@ static int launch_pass(dvqls_ctx* ctx, cudaStream_t st, const Inst* dtable, cons
     return DVQLS_OK;
 }
 
+// The instance table in kernel arguments, for a caller that is capturing the
+// stream: a captured copy would read the pinned staging when the graph is
+// launched, after other calls have written it, and the table in the workspace may
+// belong to another call by then.
+struct TableChunk {
+    uint4 w[224];  // of 4 KB of arguments
+};
+__global__ void __launch_bounds__(224) k_put_table(TableChunk c, int count, uint4* dst) {
+    if (int(threadIdx.x) < count) dst[threadIdx.x] = c.w[threadIdx.x];
+}
+
+static bool is_capturing(dvqls_ctx* ctx) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(ctx->stream, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return cap != cudaStreamCaptureStatusNone;
+}
+
 // Replays a captured graph of the pass when the launch (table bytes and
 // shape) is the one captured last; otherwise captures it on the context's
 // private capture stream first.  Profiling and callers that are capturing
 // the stream themselves get direct launches.
 static int run_pass(dvqls_ctx* ctx, const Inst* dtable, const PassShape& ps, const std::vector<const HostInst*>& tab,
-                    const std::vector<char>& table_bytes) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(ctx->stream, &cap) != cudaSuccess) {
-        cudaGetLastError();
-        cap = cudaStreamCaptureStatusActive;
-    }
-    if (ctx->profiling || cap != cudaStreamCaptureStatusNone)
+                    const std::vector<char>& table_bytes, bool capturing) {
+    if (ctx->profiling || capturing)
         return launch_pass(ctx, ctx->stream, dtable, ps, tab, ctx->profiling);
     std::vector<char> key(table_bytes);
     const char* pk = reinterpret_cast<const char*>(&ps);
@@ -3779,7 +3794,8 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
         I.delta = delta_out ? (double2*)(ws + o.delta) : nullptr;
     }
     const Inst* dtable = (const Inst*)(ws + o_table);
-    const size_t tbytes = sizeof(Inst) * count;
+    const size_t tbytes = sizeof(Inst) * count;  // its room in the workspace is rounded up to 256 bytes
+    const bool capturing = is_capturing(ctx);
 
     rc = flush_in(ctx);
     if (rc) return rc;
@@ -3835,6 +3851,17 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
     };
     auto upload = [&]() -> int {
         const char* tb = reinterpret_cast<const char*>(table.data());
+        if (capturing) {  // the graph brings it with every launch; the next call outside it uploads its own
+            ctx->last_table.clear();
+            for (size_t at = 0; at < tbytes; at += sizeof(TableChunk)) {
+                TableChunk c{};
+                const size_t bytes = std::min(sizeof c, tbytes - at);
+                memcpy(&c, tb + at, bytes);
+                k_put_table<<<1, 224, 0, ctx->stream>>>(c, ceil_div(bytes, 16), (uint4*)((char*)dtable + at));
+            }
+            DVQLS_CUDA_TRY(ctx, cudaGetLastError());
+            return DVQLS_OK;
+        }
         if (ctx->last_table.size() == tbytes && memcmp(ctx->last_table.data(), tb, tbytes) == 0) return DVQLS_OK;
         if (all_device) {
             int r = pin_acquire(ctx);
@@ -3916,7 +3943,7 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
     if (rc) return rc;
     {
         DVQLS_NVTX("dvqls pass kernels");
-        rc = run_pass(ctx, dtable, ps, tab, ctx->last_table);
+        rc = run_pass(ctx, dtable, ps, tab, ctx->last_table, capturing);
     }
     if (rc) return rc;
 
