@@ -1199,10 +1199,10 @@ __device__ __noinline__ double b_norm2(const Inst& I, double* red) {
 constexpr int BN_PARTS = 128;
 __global__ void __launch_bounds__(256) k_bnorm(const Inst* __restrict__ insts) {
     pdl_trigger();
-    const Inst& I = insts[blockIdx.y];
+    const Inst& I = insts[blockIdx.x];
     if (!I.bpart || !I.b) return;
     const long long N = 1LL << I.n, per = N / BN_PARTS;  // N > 4096
-    const double2* b = I.b + blockIdx.x * per;
+    const double2* b = I.b + blockIdx.y * per;
     double acc = 0.0;
 #pragma unroll 4
     for (long long j = threadIdx.x; j < per; j += 256) {
@@ -1215,7 +1215,7 @@ __global__ void __launch_bounds__(256) k_bnorm(const Inst* __restrict__ insts) {
     __syncthreads();
     if (threadIdx.x == 0) {
         for (int k = 1; k < 8; ++k) acc += red[k];
-        I.bpart[blockIdx.x] = acc;
+        I.bpart[blockIdx.y] = acc;
     }
 }
 
@@ -3178,8 +3178,8 @@ constexpr int FOLD_MIN = 64;  // slots per shift from which it is worth a launch
 __global__ void __launch_bounds__(256) k_fold(const Inst* __restrict__ insts) {
     pdl_wait();
     pdl_trigger();
-    const Inst& I = insts[blockIdx.y];
-    const int s = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const Inst& I = insts[blockIdx.x];
+    const int s = blockIdx.y * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (!I.fold || s >= I.S) return;
     const int T = I.T, nd = T * T * I.ks;
     auto fold = [&](double2* p, int count) {
@@ -3386,7 +3386,7 @@ static int launch_pass(dvqls_ctx* ctx, cudaStream_t st, const Inst* dtable, cons
     // prepare kernel also resets the work queue.
     if (ps.any_hbm) {
         if (marks) prof_begin(ctx, 0);
-        k_bnorm<<<dim3(BN_PARTS, ps.count), 256, 0, st>>>(dtable);
+        k_bnorm<<<dim3(ps.count, BN_PARTS), 256, 0, st>>>(dtable);  // a grid's y extent ends at 65,535
         if (marks) prof_end(ctx);
     }
     if (marks) prof_begin(ctx, 0);
@@ -3432,7 +3432,7 @@ static int launch_pass(dvqls_ctx* ctx, cudaStream_t st, const Inst* dtable, cons
     if (marks) prof_end(ctx);
     if (ps.fold_grid) {
         if (marks) prof_begin(ctx, 2);
-        DVQLS_CUDA_TRY(ctx, launch_pdl(k_fold, dim3(ps.fold_grid, ps.count), dim3(256), 0, st, dtable));
+        DVQLS_CUDA_TRY(ctx, launch_pdl(k_fold, dim3(ps.count, ps.fold_grid), dim3(256), 0, st, dtable));
         if (marks) prof_end(ctx);
     }
     if (marks) prof_begin(ctx, 2);
