@@ -2972,10 +2972,17 @@ inline size_t wht_smem_bytes(int Pmax) {
 // lookups 31 k; both are bound by the integer multiply-adds and adds.
 constexpr int W64_ROW = (1 << WHT_MAXN) + (1 << WHT_MAXN) / 32;
 
-// Value of one fixed-point unit, from an instance's class table: NaN when one of its
-// angles is not finite (reported in the status word; fixed point itself holds no NaN).
-__device__ __forceinline__ double w64_unit(const unsigned char* tb) {
-    return *reinterpret_cast<const int*>(tb + WHT_OFF_BIM) & 2 ? __longlong_as_double(0x7ff8000000000000LL) : 0x1p-60;
+// Factor of an instance's results, from its class table: NaN when one of its angles
+// is not finite (reported in the status word; fixed point itself holds no NaN).
+__device__ __forceinline__ double w64_valid(const unsigned char* tb) {
+    return *reinterpret_cast<const int*>(tb + WHT_OFF_BIM) & 2 ? __longlong_as_double(0x7ff8000000000000LL) : 1.0;
+}
+// The value of v units of 2^-60, at most 1: a weight is multiplied by that, not by v,
+// which would take weights above 1e289 past the largest double.  The scale is a
+// subtraction from the exponent (v = 0 has none).
+__device__ __forceinline__ double w64_value(long long v) {
+    const double d = (double)v;
+    return __hiloint2double(__double2hiint(d) - (v != 0 ? FX_BITS << 20 : 0), __double2loint(d));
 }
 
 // Transform of v (index (r << 5) | lane) into the warp's row, at i + (i >> 5)
@@ -3041,7 +3048,7 @@ __device__ void w64_item(const Inst& I, int s, const Fx* q, long long* row, doub
     double2* Gp = (s == 0 && I.Gpart) ? reinterpret_cast<double2*>(I.Gpart) : nullptr;
     const int parts = 1 + (*reinterpret_cast<const int*>(tb + WHT_OFF_BIM) & 1);
     const int pairs = ncls * I.F, jobs = pairs + (I.local ? 0 : nd * parts);
-    auto at = [&](uint32_t z) { return row[PAD ? z + (z >> 5) : z]; };
+    auto at = [&](uint32_t z) { return w64_value(row[PAD ? z + (z >> 5) : z]); };
 #pragma unroll 1
     for (int j = w; j < jobs; j += WHT_NT / 32) {
         long long v[A];
@@ -3055,10 +3062,10 @@ __device__ void w64_item(const Inst& I, int s, const Fx* q, long long* row, doub
                 v[r] = fx_mul(part ? fx_neg(Fx{bb.z, bb.w}) : Fx{bb.x, bb.y}, q[i]);
             }
             w64_transform<A, LOGA>(v, row, N, lane);
-            const double sc = scalbn(w64_unit(tb), w64_bexp(*I.bn2));
+            const double sc = scalbn(w64_valid(tb), w64_bexp(*I.bn2));
             for (int e = dof[c] + lane; e < dof[c + 1]; e += 32) {
                 const int l = dt[e];
-                (part ? dim : dre)[l] = (double)at(szl[l] & uint32_t(N - 1)) * sc;
+                (part ? dim : dre)[l] = at(szl[l] & uint32_t(N - 1)) * sc;
             }
             __syncwarp();
             continue;
@@ -3073,17 +3080,17 @@ __device__ void w64_item(const Inst& I, int s, const Fx* q, long long* row, doub
         w64_transform<A, LOGA>(v, row, N, lane);
         const int e0 = co[c], e1 = co[c + 1];
         if (f == 0) {
-            for (int e = e0 + lane; e < e1; e += 32) D = fma(ek[e], (double)at(ez[e]), D);
+            for (int e = e0 + lane; e < e1; e += 32) D = fma(ek[e], at(ez[e]), D);
         } else {
             for (int e = e0 + lane; e < e1; e += 32) {
                 const double k = ek[e];
-                E = fma((szl[pr[e] & 0xFF] >> (f - 1)) & 1u ? -k : k, (double)at(ez[e]), E);
+                E = fma((szl[pr[e] & 0xFF] >> (f - 1)) & 1u ? -k : k, at(ez[e]), E);
             }
         }
         if (Gp)  // the beta output of the unshifted state
             for (int e = e0 + lane; e < e1; e += 32) {
                 const int p = pr[e], l = p & 0xFF, m = p >> 8;
-                double beta = (double)at(ez[e]) * w64_unit(tb);
+                double beta = at(ez[e]) * w64_valid(tb);
                 if (__popc(szl[l] & uint32_t(x)) & 1) beta = -beta;
                 Gp[(long long)l * L + m] = make_double2(beta, 0.0);
                 Gp[(long long)m * L + l] = make_double2(beta, 0.0);
@@ -3153,14 +3160,14 @@ __global__ void __launch_bounds__(WHT_NT, 2) k_terms_wht64(const Inst* __restric
         }
         __syncthreads();
         if (t == 0) {
-            const double unit = w64_unit(reinterpret_cast<const unsigned char*>(I.wht));
+            const double valid = w64_valid(reinterpret_cast<const unsigned char*>(I.wht));
             double Ds = 0.0, Es = 0.0;
             for (int k = 0; k < WHT_NT / 32; ++k) {
                 Ds += red[k];
                 if (I.local) Es += redE[k];
             }
-            I.Dpart[(long long)s * I.F] = make_double2(Ds * unit, 0.0);
-            if (I.local) I.Dpart[(long long)s * I.F + 1] = make_double2(Es * unit, 0.0);
+            I.Dpart[(long long)s * I.F] = make_double2(Ds * valid, 0.0);
+            if (I.local) I.Dpart[(long long)s * I.F + 1] = make_double2(Es * valid, 0.0);
             else I.Tpart[s] = make_double2(redT[0].x + redT[1].x, redT[0].y + redT[1].y);
         } else if (I.local && t >= 2 && t < I.F) {  // slot 0 of a shift holds D, slot 1 E, the rest zero
             I.Dpart[(long long)s * I.F + t] = make_double2(0.0, 0.0);
