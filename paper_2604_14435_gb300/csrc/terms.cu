@@ -2419,14 +2419,14 @@ constexpr size_t WHT_OFF_EZ = (WHT_OFF_DT + 2 * 64 + 15) & ~size_t(15);  // uint
 constexpr size_t WHT_OFF_EK = (WHT_OFF_EZ + 2 * WHT_MAXP + 15) & ~size_t(15);  // signed weights by class: float2, or
                                                                                // double (FP64)
 constexpr size_t WHT_OFF_BIM = WHT_OFF_EK + 8 * WHT_MAXP;  // int: bit 0 b has a nonzero imaginary part, bit 1 an angle
-                                                           // is not finite
+                                                           // is not finite, bit 2 ||b||^2 is zero or not finite
 constexpr size_t WHT_TABLE_BYTES = WHT_OFF_BIM + 16;          // header: int pair classes, term classes
 // Fixed point of the FP64 classes (units of 2^-FX_BITS): b is scaled by a power
 // of two so that ||b|| <= 1.
 __device__ __forceinline__ int w64_bexp(double bn2) {
     int ex;
     frexp(sqrt(bn2), &ex);  // ||b|| <= 2^ex
-    return min(max(ex, -1000), 1000);  // an invalid ||b||^2 is reported by k_prepare
+    return min(max(ex, -1000), 1000);  // an invalid ||b||^2 is reported and marked in the table
 }
 
 // What a class pass needs of one instance (one CTA each), in one launch: the
@@ -2575,8 +2575,9 @@ __global__ void __launch_bounds__(WHT_CT) k_wht_prepare(const Inst* __restrict__
             for (int k = 0; k < 8; ++k) sum += red[k];
             s_bn2 = sum;
             *I.bn2 = sum;
-            if (!(sum > 0.0) || !isfinite(sum)) set_status(status, DEV_BAD_NORM);
-            *reinterpret_cast<int*>(tb + WHT_OFF_BIM) = s_im | s_bad << 1;
+            const bool bad_norm = !(sum > 0.0) || !isfinite(sum);
+            if (bad_norm) set_status(status, DEV_BAD_NORM);
+            *reinterpret_cast<int*>(tb + WHT_OFF_BIM) = s_im | s_bad << 1 | bad_norm << 2;
         }
     }
     __syncthreads();
@@ -2972,10 +2973,11 @@ inline size_t wht_smem_bytes(int Pmax) {
 // lookups 31 k; both are bound by the integer multiply-adds and adds.
 constexpr int W64_ROW = (1 << WHT_MAXN) + (1 << WHT_MAXN) / 32;
 
-// Factor of an instance's results, from its class table: NaN when one of its angles
-// is not finite (reported in the status word; fixed point itself holds no NaN).
-__device__ __forceinline__ double w64_valid(const unsigned char* tb) {
-    return *reinterpret_cast<const int*>(tb + WHT_OFF_BIM) & 2 ? __longlong_as_double(0x7ff8000000000000LL) : 1.0;
+// Factor of an instance's results, from its class table: NaN when one of the bits
+// `bad` is set (2: an angle is not finite; 4: ||b||^2 is zero or not finite; both are
+// reported in the status word, but fixed point itself holds no NaN).
+__device__ __forceinline__ double w64_valid(const unsigned char* tb, int bad) {
+    return *reinterpret_cast<const int*>(tb + WHT_OFF_BIM) & bad ? __longlong_as_double(0x7ff8000000000000LL) : 1.0;
 }
 // The value of v units of 2^-60, at most 1: a weight is multiplied by that, not by v,
 // which would take weights above 1e289 past the largest double.  The scale is a
@@ -3062,7 +3064,7 @@ __device__ void w64_item(const Inst& I, int s, const Fx* q, long long* row, doub
                 v[r] = fx_mul(part ? fx_neg(Fx{bb.z, bb.w}) : Fx{bb.x, bb.y}, q[i]);
             }
             w64_transform<A, LOGA>(v, row, N, lane);
-            const double sc = scalbn(w64_valid(tb), w64_bexp(*I.bn2));
+            const double sc = scalbn(w64_valid(tb, 2 | 4), w64_bexp(*I.bn2));
             for (int e = dof[c] + lane; e < dof[c + 1]; e += 32) {
                 const int l = dt[e];
                 (part ? dim : dre)[l] = at(szl[l] & uint32_t(N - 1)) * sc;
@@ -3090,7 +3092,7 @@ __device__ void w64_item(const Inst& I, int s, const Fx* q, long long* row, doub
         if (Gp)  // the beta output of the unshifted state
             for (int e = e0 + lane; e < e1; e += 32) {
                 const int p = pr[e], l = p & 0xFF, m = p >> 8;
-                double beta = at(ez[e]) * w64_valid(tb);
+                double beta = at(ez[e]) * w64_valid(tb, 2);
                 if (__popc(szl[l] & uint32_t(x)) & 1) beta = -beta;
                 Gp[(long long)l * L + m] = make_double2(beta, 0.0);
                 Gp[(long long)m * L + l] = make_double2(beta, 0.0);
@@ -3160,7 +3162,7 @@ __global__ void __launch_bounds__(WHT_NT, 2) k_terms_wht64(const Inst* __restric
         }
         __syncthreads();
         if (t == 0) {
-            const double valid = w64_valid(reinterpret_cast<const unsigned char*>(I.wht));
+            const double valid = w64_valid(reinterpret_cast<const unsigned char*>(I.wht), 2);
             double Ds = 0.0, Es = 0.0;
             for (int k = 0; k < WHT_NT / 32; ++k) {
                 Ds += red[k];

@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 import torch
 
+from oracle import terms as oterms
 from paper_2604_14435_gb300 import workloads as wl
 
 from test_gpu_terms import cvec, random_problem
@@ -31,3 +32,33 @@ def test_large_and_small_coefficients(dv, ctx, n, L, scale):
     assert abs(got[1][1] - got[0][1]) <= 1e-13 * max(1.0, abs(got[0][1]))
     assert np.all(np.abs(got[1][2][:, 2] / scale / scale - got[0][2][:, 2]) <= 1e-13 * np.abs(got[0][2][:, 2]))
     assert np.all(np.abs(got[1][2][:, :2] / scale - got[0][2][:, :2]) <= 1e-13 * np.abs(got[0][2][:, :2]).max())
+
+
+@pytest.mark.parametrize("bad", [np.inf, np.nan, 1e200, 0.0])  # an entry; 1e200: ||b||^2 overflows; 0: all of b
+@pytest.mark.parametrize("n", [3, 6, 10])
+def test_bad_norm_gives_nan(dv, ctx, n, bad):
+    """A right-hand side without a finite, positive norm is reported and its instance's outputs are NaN; the other
+    instance of the batch is right."""
+    d, L = 1, 12
+    P = n * (d + 1)
+    rng = np.random.default_rng(n)
+    coef, xs, zs, b = random_problem(rng, n, L)
+    ref = oterms.cost_grad(n, d, wl.random_angles(P, 3), b, coef, xs, zs)
+    wrong = b.copy()
+    if bad == 0.0:
+        wrong[:] = 0.0
+    else:
+        wrong[1] = bad
+    dev = [torch.tensor(v, device="cuda") for v in (cvec(coef), xs.view(np.int32), zs.view(np.int32),
+                                                    wl.random_angles(P, 3), cvec(wrong), cvec(b))]
+    an, lcu = dv.make_ansatz(n, d), dv.make_lcu(L, dev[0], dev[1], dev[2])
+    costs, grads = (torch.zeros(m, device="cuda", dtype=torch.float64) for m in (2, 2 * P))
+    arr = dv.make_instances([(an, lcu, dev[3], dev[4]), (an, lcu, dev[3], dev[5])])
+    with pytest.raises(dv.DvqlsError) as e:
+        dv.dvqls_cost_grad_batched(ctx, arr, dv.DVQLS_FP64, costs, grads)
+        dv.dvqls_sync(ctx)
+    assert e.value.code == dv.DVQLS_ERR_INVALID_ARG
+    c, g = costs.cpu().numpy(), grads.cpu().numpy()
+    assert np.isnan(c[0]) and np.isnan(g[:P]).all()
+    assert abs(c[1] - ref["cost"]) <= 1e-12 * max(1.0, abs(ref["cost"]))
+    assert np.all(np.abs(g[P:] - ref["grad"]) <= 1e-12 * np.maximum(1.0, np.abs(ref["grad"])))
