@@ -54,8 +54,7 @@ __device__ double2 block_sum2_all(double2 v, double2* red) {
 // One CTA per instance; the state in fixed point (build_state_fx), the overlap in FP64.
 __global__ void __launch_bounds__(FT) k_fidelity(const FidInst* __restrict__ insts, int* status) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ double2 red[FT / 32];
-    __shared__ double rnx[FT / 32];
+    __shared__ double2 red[FT / 32];  // no more: what is left is for the angles (fx_smem)
     const FidInst I = insts[blockIdx.x];
     const int N = 1 << I.n;
     bool bad = false;
@@ -84,14 +83,14 @@ __global__ void __launch_bounds__(FT) k_fidelity(const FidInst* __restrict__ ins
         ov.y += __shfl_xor_sync(0xffffffffu, ov.y, o);
         nx.x += __shfl_xor_sync(0xffffffffu, nx.x, o);
     }
-    if ((threadIdx.x & 31) == 0) {
-        red[threadIdx.x >> 5] = ov;
-        rnx[threadIdx.x >> 5] = nx.x;
-    }
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ov;
+    __syncthreads();
+    ov = red[threadIdx.x & 7];
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = nx;
     __syncthreads();
     if (threadIdx.x >= 8) return;
-    ov = red[threadIdx.x];
-    nx.x = rnx[threadIdx.x];
+    nx = red[threadIdx.x];
     for (int o = 4; o; o >>= 1) {
         ov.x += __shfl_xor_sync(0xffu, ov.x, o);
         ov.y += __shfl_xor_sync(0xffu, ov.y, o);
