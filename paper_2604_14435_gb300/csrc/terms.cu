@@ -2419,7 +2419,8 @@ constexpr size_t WHT_OFF_EZ = (WHT_OFF_DT + 2 * 64 + 15) & ~size_t(15);  // uint
 constexpr size_t WHT_OFF_EK = (WHT_OFF_EZ + 2 * WHT_MAXP + 15) & ~size_t(15);  // signed weights by class: float2, or
                                                                                // double (FP64)
 constexpr size_t WHT_OFF_BIM = WHT_OFF_EK + 8 * WHT_MAXP;  // int: bit 0 b has a nonzero imaginary part, bit 1 an angle
-                                                           // is not finite, bit 2 ||b||^2 is zero or not finite
+                                                           // is not finite, bit 2 ||b||^2 is zero or not finite;
+                                                           // then (FP64) int: the weights' exponent
 constexpr size_t WHT_TABLE_BYTES = WHT_OFF_BIM + 16;          // header: int pair classes, term classes
 // Fixed point of the FP64 classes (units of 2^-FX_BITS): b is scaled by a power
 // of two so that ||b|| <= 1.
@@ -2460,7 +2461,7 @@ __global__ void __launch_bounds__(WHT_CT) k_wht_prepare(const Inst* __restrict__
     __shared__ unsigned short cnt[WHT_RANK_WARPS][BINS], rank[WHT_MAXP];
     __shared__ int start[BINS], part[32], cpart[32];
     __shared__ double red[8], s_bn2;
-    __shared__ int s_im, s_bad;
+    __shared__ int s_im, s_bad, s_exp;
     __shared__ unsigned s_first[2];
     const Inst I = insts[blockIdx.x];
     const int L = I.L, t = threadIdx.x, w = t >> 5, lane = t & 31, np = L * (L + 1) / 2;
@@ -2468,7 +2469,10 @@ __global__ void __launch_bounds__(WHT_CT) k_wht_prepare(const Inst* __restrict__
     unsigned char* tb = reinterpret_cast<unsigned char*>(I.wht);
     if (queue && blockIdx.x == 0 && t == 0) *queue = 0ull;  // the term kernel's work queue
     for (int k = t; k < WHT_RANK_WARPS * BINS / 2; k += WHT_CT) reinterpret_cast<uint32_t*>(cnt)[k] = 0u;
-    if (t == 0) s_im = s_bad = 0;
+    if (t == 0) {
+        s_im = s_bad = 0;
+        s_exp = -1000;
+    }
     if (t < L) {
         const uint32_t x = I.xm[t], z = I.zm[t];
         const double2 c = I.coef[t];
@@ -2482,6 +2486,10 @@ __global__ void __launch_bounds__(WHT_CT) k_wht_prepare(const Inst* __restrict__
         if (I.cf) I.cf[t] = split_ff(r);
     }
     __syncthreads();
+    if (F64 && t < L) {
+        const double a = fmax(fabs(sc[t].x), fabs(sc[t].y));
+        atomicMax(&s_exp, ((__double2hiint(a) >> 20) & 0x7ff) - 1023);
+    }
     double2 b[4];  // warps 0 .. 7: the instance's b (the local cost's is implied)
     if (w < 8) {
         double acc = !I.b && t == 0 ? 1.0 : 0.0;
@@ -2531,6 +2539,11 @@ __global__ void __launch_bounds__(WHT_CT) k_wht_prepare(const Inst* __restrict__
         }
     }
     __syncthreads();
+    if (F64 && t < L) {  // weights of c~ 2^-s_exp, which is below 2: their sums in units of 2^-60 stay in range
+        const double f = scalbn(1.0, -s_exp);  // exact
+        sc[t].x *= f;
+        sc[t].y *= f;
+    }
     {  // thread t: the class of mask t -- its pairs, its place, its number
         int total = 0;
 #pragma unroll
@@ -2577,7 +2590,7 @@ __global__ void __launch_bounds__(WHT_CT) k_wht_prepare(const Inst* __restrict__
             *I.bn2 = sum;
             const bool bad_norm = !(sum > 0.0) || !isfinite(sum);
             if (bad_norm) set_status(status, DEV_BAD_NORM);
-            *reinterpret_cast<int*>(tb + WHT_OFF_BIM) = s_im | s_bad << 1 | bad_norm << 2;
+            *reinterpret_cast<int2*>(tb + WHT_OFF_BIM) = make_int2(s_im | s_bad << 1 | bad_norm << 2, 2 * s_exp);
         }
     }
     __syncthreads();
@@ -2979,13 +2992,9 @@ constexpr int W64_ROW = (1 << WHT_MAXN) + (1 << WHT_MAXN) / 32;
 __device__ __forceinline__ double w64_valid(const unsigned char* tb, int bad) {
     return *reinterpret_cast<const int*>(tb + WHT_OFF_BIM) & bad ? __longlong_as_double(0x7ff8000000000000LL) : 1.0;
 }
-// The value of v units of 2^-60, at most 1: a weight is multiplied by that, not by v,
-// which would take weights above 1e289 past the largest double.  The scale is a
-// subtraction from the exponent (v = 0 has none).
-__device__ __forceinline__ double w64_value(long long v) {
-    const double d = (double)v;
-    return __hiloint2double(__double2hiint(d) - (v != 0 ? FX_BITS << 20 : 0), __double2loint(d));
-}
+// Exponent of an instance's weights: the table holds them for c~ scaled down by half of it, so
+// that no weight times a transform value in units of 2^-60 leaves the range of a double.
+__device__ __forceinline__ int w64_wexp(const unsigned char* tb) { return reinterpret_cast<const int*>(tb + WHT_OFF_BIM)[1]; }
 
 // Transform of v (index (r << 5) | lane) into the warp's row, at i + (i >> 5)
 // for 2^10 values (A = 32: through the row, lane bits become register bits), else at i.
@@ -3050,7 +3059,7 @@ __device__ void w64_item(const Inst& I, int s, const Fx* q, long long* row, doub
     double2* Gp = (s == 0 && I.Gpart) ? reinterpret_cast<double2*>(I.Gpart) : nullptr;
     const int parts = 1 + (*reinterpret_cast<const int*>(tb + WHT_OFF_BIM) & 1);
     const int pairs = ncls * I.F, jobs = pairs + (I.local ? 0 : nd * parts);
-    auto at = [&](uint32_t z) { return w64_value(row[PAD ? z + (z >> 5) : z]); };
+    auto at = [&](uint32_t z) { return (double)row[PAD ? z + (z >> 5) : z]; };
 #pragma unroll 1
     for (int j = w; j < jobs; j += WHT_NT / 32) {
         long long v[A];
@@ -3064,7 +3073,7 @@ __device__ void w64_item(const Inst& I, int s, const Fx* q, long long* row, doub
                 v[r] = fx_mul(part ? fx_neg(Fx{bb.z, bb.w}) : Fx{bb.x, bb.y}, q[i]);
             }
             w64_transform<A, LOGA>(v, row, N, lane);
-            const double sc = scalbn(w64_valid(tb, 2 | 4), w64_bexp(*I.bn2));
+            const double sc = scalbn(w64_valid(tb, 2 | 4), w64_bexp(*I.bn2) - FX_BITS);
             for (int e = dof[c] + lane; e < dof[c + 1]; e += 32) {
                 const int l = dt[e];
                 (part ? dim : dre)[l] = at(szl[l] & uint32_t(N - 1)) * sc;
@@ -3092,7 +3101,7 @@ __device__ void w64_item(const Inst& I, int s, const Fx* q, long long* row, doub
         if (Gp)  // the beta output of the unshifted state
             for (int e = e0 + lane; e < e1; e += 32) {
                 const int p = pr[e], l = p & 0xFF, m = p >> 8;
-                double beta = at(ez[e]) * w64_valid(tb, 2);
+                double beta = at(ez[e]) * scalbn(w64_valid(tb, 2), -FX_BITS);
                 if (__popc(szl[l] & uint32_t(x)) & 1) beta = -beta;
                 Gp[(long long)l * L + m] = make_double2(beta, 0.0);
                 Gp[(long long)m * L + l] = make_double2(beta, 0.0);
@@ -3162,14 +3171,16 @@ __global__ void __launch_bounds__(WHT_NT, 2) k_terms_wht64(const Inst* __restric
         }
         __syncthreads();
         if (t == 0) {
-            const double valid = w64_valid(reinterpret_cast<const unsigned char*>(I.wht), 2);
+            const unsigned char* tb = reinterpret_cast<const unsigned char*>(I.wht);
+            const double valid = w64_valid(tb, 2);
+            const int we = w64_wexp(tb) - FX_BITS;
             double Ds = 0.0, Es = 0.0;
             for (int k = 0; k < WHT_NT / 32; ++k) {
                 Ds += red[k];
                 if (I.local) Es += redE[k];
             }
-            I.Dpart[(long long)s * I.F] = make_double2(Ds * valid, 0.0);
-            if (I.local) I.Dpart[(long long)s * I.F + 1] = make_double2(Es * valid, 0.0);
+            I.Dpart[(long long)s * I.F] = make_double2(scalbn(Ds * valid, we), 0.0);
+            if (I.local) I.Dpart[(long long)s * I.F + 1] = make_double2(scalbn(Es * valid, we), 0.0);
             else I.Tpart[s] = make_double2(redT[0].x + redT[1].x, redT[0].y + redT[1].y);
         } else if (I.local && t >= 2 && t < I.F) {  // slot 0 of a shift holds D, slot 1 E, the rest zero
             I.Dpart[(long long)s * I.F + t] = make_double2(0.0, 0.0);
