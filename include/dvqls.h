@@ -76,10 +76,17 @@ typedef enum {
  * combine in FP64.
  *   DVQLS_FP64:    FP64 states and term reductions.  When every instance has
  *                  L <= 64 and n <= 10 the terms come by Walsh-Hadamard
- *                  classes (as DVQLS_FP32_WHT below) with state, products and
- *                  transforms in 64-bit fixed point (units of 2^-60): the
- *                  same accuracy as the FP64 tiles (1e-12 of the parity
- *                  tests; 1.2e-15 measured at n = 10), in less time.
+ *                  classes (as DVQLS_FP32_WHT below) with transforms in
+ *                  64-bit fixed point, in less time and no less accurate
+ *                  than the FP64 tiles (against extended precision, systems
+ *                  of n = 3..10: gradients 1.4e-15 to 3e-15 off in the mean,
+ *                  the tiles' 2.5e-15 to 4e-15).  A state spread over its
+ *                  amplitudes is in fixed point too; where the products of
+ *                  one class are small (angles near zero, a right-hand side
+ *                  of few entries) the evaluation takes an FP64 state and
+ *                  units that follow the size of the products, so that small
+ *                  overlaps keep the relative accuracy of FP64 sums; such an
+ *                  evaluation takes about twice the time.
  *   DVQLS_FP32:    FP32 states, FP32 term reductions on the CUDA cores.
  *   DVQLS_FP32_TC: FP32 states; the term Gram on the tensor cores
  *                  (tcgen05 kind::f16: every amplitude, scaled by 2^12,

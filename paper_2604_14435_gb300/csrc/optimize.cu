@@ -51,10 +51,10 @@ __device__ double2 block_sum2_all(double2 v, double2* red) {
     return s;
 }
 
-// One CTA per instance; the state in fixed point (build_state_fx), the overlap in FP64.
+// One CTA per instance; the state and the overlap in FP64 (build_state_f64).
 __global__ void __launch_bounds__(FT) k_fidelity(const FidInst* __restrict__ insts, int* status) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ double2 red[FT / 32];  // no more: what is left is for the angles (fx_smem)
+    __shared__ double2 red[FT / 32];  // no more: the rest is for the angles and amplitudes, 16 bytes each
     const FidInst I = insts[blockIdx.x];
     const int N = 1 << I.n;
     bool bad = false;
@@ -68,12 +68,13 @@ __global__ void __launch_bounds__(FT) k_fidelity(const FidInst* __restrict__ ins
         sincos(0.5 * al, &s, &c);
         I.cs[a] = make_double2(c, s);
     }
-    bad = __syncthreads_or(bad);  // fixed point holds no NaN
-    const Fx* psi = build_state_fx(smem, I.n, I.d, I.P, I.cs, 0);
+    bad = __syncthreads_or(bad);  // the scaled rotations lose a NaN
+    double *psi, *other;
+    build_state_f64<DVQLS_MAX_SMEM_QUBITS>(smem, I.n, I.d, I.P, I.cs, 0, psi, other);
     double2 ov = make_double2(0.0, 0.0), nx = make_double2(0.0, 0.0);
     for (int j = threadIdx.x; j < N; j += FT) {
         const double2 x = I.xhat[j];
-        const double p = fx_to(psi[j]);  // the state is real
+        const double p = psi[j];  // the state is real
         ov.x += x.x * p;  // conj(x) p
         ov.y -= x.y * p;
         nx.x += x.x * x.x + x.y * x.y;
@@ -579,7 +580,7 @@ extern "C" int dvqls_fidelity(dvqls_ctx* ctx, const dvqls_ansatz* an, const doub
     I.F = (double*)(ctx->ws + o_F);
     memcpy(ctx->pin + p_t, &I, sizeof I);
     DVQLS_CUDA_TRY(ctx, cudaMemcpyAsync(ctx->ws + o_t, ctx->pin + p_t, sizeof I, cudaMemcpyHostToDevice, ctx->stream));
-    const size_t smem = fx_smem(n, P);
+    const size_t smem = 16 * size_t(P + N);  // f64_smem(n, P) or a little more: the depths served stay what they were
     DVQLS_CUDA_TRY(ctx, allow_dynamic_smem((const void*)k_fidelity));
     k_fidelity<<<1, FT, smem, ctx->stream>>>((const FidInst*)(ctx->ws + o_t), ctx->d_status);
     DVQLS_CUDA_TRY(ctx, cudaGetLastError());
@@ -1032,7 +1033,7 @@ static int optimize(dvqls_ctx* ctx, int count, const dvqls_instance* inst, const
         results[i].fidelity = NAN;
     }
     size_t fsmem = 0;
-    for (int i = 0; i < count; ++i) fsmem = std::max(fsmem, fx_smem(inst[i].ansatz.n, P[i]));
+    for (int i = 0; i < count; ++i) fsmem = std::max(fsmem, 16 * size_t(P[i] + N[i]));  // as dvqls_fidelity
     DVQLS_CUDA_TRY(ctx, allow_dynamic_smem((const void*)k_fidelity));
     std::vector<int> active(count);
     for (int i = 0; i < count; ++i) active[i] = i;

@@ -352,18 +352,18 @@ __device__ inline void build_state_regs(void* psi, float* scratch, float2* scs, 
     group_sync(bar, 256);
 }
 
-// ---- The state in 64-bit fixed point, for 256 threads, n <= 12 (FP64 precision).
+// ---- The state in 64-bit fixed point, for 256 threads, n <= 10 (FP64 precision).
 //
 // FP64 instructions issue at 1/64 of the FP32 rate, six integer multiply-adds
 // and a shift in less time than one of them.  The state has norm
 // one, so every amplitude and every cos and sin is h 2^30 + l in units of 2^-60
 // (|h| <= 2^30, l in [-2^29, 2^29)), and c a + t b is six multiply-adds and a
-// shift, rounded to nearest at 2^-60; the two products of low parts, below a
-// quarter of that unit and of mean zero, are dropped.  An FP64 rotation rounds an
-// amplitude near 2^-5 (the mean at n = 10) at 2^-58, so this is no less exact
-// (gradients of 48 systems of n = 6..10 against a 64-bit reference: 8.5e-16
-// relative, FP64 states 1.1e-15).
-// n = 10, depth 4: 20 k cycles for a state and CTA, 60 k in FP64 with the state in
+// shift.  It is rounded at 2^-60 and leaves out the two products of low parts, a
+// quarter of that unit each at most: an error of one unit at most.  An FP64 rotation
+// rounds an amplitude near 2^-5 (the mean at n = 10) at 2^-58, so this is no less exact
+// for amplitudes of that size; small ones lose relative accuracy, and whoever sums up
+// products of them takes the FP64 state instead (build_state_f64).
+// n = 10, depth 4: 18 k cycles of an SM for a state, 60 k in FP64 with the state in
 // shared memory.
 constexpr int FX_BITS = 60;
 struct Fx {
@@ -376,7 +376,6 @@ __device__ __forceinline__ Fx fx_split(long long y) {  // y: the value + 2^29
     return r;
 }
 __device__ __forceinline__ Fx fx_from(double v) { return fx_split(__double2ll_rn(v * 0x1p60) + (1LL << 29)); }
-__device__ __forceinline__ double fx_to(Fx a) { return double((long long)a.h * (1LL << 30) + a.l) * 0x1p-60; }
 __device__ __forceinline__ Fx fx_neg(Fx a) { return Fx{-a.h, -a.l}; }  // l = -2^29 gives 2^29, which the products take
 // a b in units of 2^-60, rounded to nearest.
 __device__ __forceinline__ long long fx_mul(Fx a, Fx b) {
@@ -487,7 +486,7 @@ __device__ void fx_warp(Fx* out, const int4* ang, const Fx* lowt, const Fx* high
     }
 }
 
-// psi(alpha_s): returns where its 2^n amplitudes lie in smem (fx_smem(n, P)
+// psi(alpha_s), n <= 10: returns where its 2^n amplitudes lie in smem (fx_smem(n, P)
 // bytes).  cs as for build_state_real.  Whole CTA of 256 threads; ends with a
 // barrier.
 __device__ inline Fx* build_state_fx(unsigned char* smem, int n, int d, int P, const double2* cs, int s) {
@@ -515,20 +514,20 @@ __device__ inline Fx* build_state_fx(unsigned char* smem, int n, int d, int P, c
     for (int e = t ^ 255; e < nlow + nh; e += 256) {
         const bool lo = e < nlow;
         const int i = lo ? e : e - nlow, q0 = lo ? 0 : nl, q1 = lo ? nl : n;
-        double v = 1.0;
+        // in fixed point: a table entry is shared by 32 amplitudes, whose sums would show FP64
+        // roundings of it (2^-53 of itself) where roundings of each amplitude average out
+        Fx v{1 << 30, 0};
         for (int q = q0; q < q1; ++q) {
             const double2 c = angle(q);
-            v *= ((i >> (q - q0)) & 1) ? c.y : c.x;
+            v = fx_split(fx_mul(v, fx_from(((i >> (q - q0)) & 1) ? c.y : c.x)) + (1LL << 29));
         }
-        (lo ? lowt : hight)[i] = fx_from(v);
+        (lo ? lowt : hight)[i] = v;
     }
     __syncthreads();
     switch (n) {
         case 8: fx_multiwarp<1, 0>(out, scr, angw, lowt, hight, n, d, t); break;
         case 9: fx_multiwarp<2, 1>(out, scr, angw, lowt, hight, n, d, t); break;
         case 10: fx_multiwarp<4, 2>(out, scr, angw, lowt, hight, n, d, t); break;
-        case 11: fx_multiwarp<8, 3>(out, scr, angw, lowt, hight, n, d, t); break;
-        case 12: fx_multiwarp<16, 4>(out, scr, angw, lowt, hight, n, d, t); break;
         default:
             if (t < 32) {
                 if (n == 7) fx_warp<4, 2>(out, angw, lowt, hight, n, d, t);
@@ -539,6 +538,221 @@ __device__ inline Fx* build_state_fx(unsigned char* smem, int n, int d, int P, c
     }
     __syncthreads();
     return out;
+}
+
+// ---- The state in FP64 registers, for 256 threads, n <= 12.
+//
+// FP64 instructions issue at 1/64 of the FP32 rate and bound this, so a rotation runs
+// in scaled form (ry_scaled): one FMA per amplitude, and the factors, multiplied
+// together by a warp, once per group of layers.  Every amplitude keeps its relative
+// accuracy, whatever its size.  n = 10, depth 4: 31 k cycles of an SM per state (40 k
+// FMAs are 20 k), the fixed-point state above 18 k.
+
+// Ratio of an Ry in scaled form: |ratio| <= 1 leaves bit 62 clear, it is set for the
+// sine form.  (A NaN is reported by whoever formed the angles' table.)
+__device__ __forceinline__ long long ry64_pack(double2 v) {  // v: (cos, sin)
+    const bool sf = fabs(v.y) > fabs(v.x);
+    return __double_as_longlong(sf ? v.x / v.y : v.y / v.x) | (long long)sf << 62;
+}
+__device__ __forceinline__ double flip_sign(double v, int flip) {  // flip: 0 or the sign bit
+    return __hiloint2double(__double2hiint(v) ^ flip, __double2loint(v));
+}
+
+// Layers whose factors are applied together: at most 64 rotations, each of which lets
+// the amplitudes grow by sqrt(2) at most.
+__host__ __device__ inline int ry64_group(int n) { return 64 / n; }
+__host__ __device__ inline int ry64_groups(int n, int P) { return (P / n - 1 + ry64_group(n) - 1) / ry64_group(n); }
+
+// The product of the factors of rotations first .. first + count - 1 (count <= 64), by
+// a warp; angle(a) is (cos, sin).  Formed as 64-bit significands (2^-63 relative per
+// product, as FP64 products would not be) and rounded once.
+template <class Angle>
+__device__ __forceinline__ double ry64_factor(int first, int count, int lane, const Angle& angle) {
+    unsigned long long m = 1ull << 63;  // m 2^(e - 63)
+    int e = 0, neg = 0;
+    auto times = [&](unsigned long long m2, int e2, int neg2) {
+        m = __umul64hi(m, m2);
+        e += e2 + 1;
+        if (!(m >> 63)) {
+            m <<= 1;
+            --e;
+        }
+        neg ^= neg2;
+    };
+    for (int k = lane; k < count; k += 32) {
+        const double2 v = angle(first + k);
+        const unsigned long long f = (unsigned long long)__double_as_longlong(fabs(v.y) > fabs(v.x) ? v.y : v.x);
+        times((f | 1ull << 52) << 11, int((f >> 52) & 0x7ff) - 1023, int(f >> 63));
+    }
+    for (int o = 16; o; o >>= 1) {
+        const unsigned long long m2 = __shfl_xor_sync(0xffffffffu, m, o);
+        const int e2 = __shfl_xor_sync(0xffffffffu, e, o), neg2 = __shfl_xor_sync(0xffffffffu, neg, o);
+        times(m2, e2, neg2);
+    }
+    const double f = scalbn((double)m, e - 63);
+    return neg ? -f : f;
+}
+
+// Ry of the qubits on lane bits b0 .. b0 + nb - 1 and on the register bits.
+template <int A>
+__device__ __forceinline__ void ry64_lanes(double (&v)[A], int lane, int b0, int nb, const long long* ang) {
+    for (int j = 0; j < nb; ++j) {
+        const long long q = ang[j];
+        const double r = __longlong_as_double(q & ~(1LL << 62));
+        const bool sf = (q >> 62) & 1;
+        const int flip = (lane >> (b0 + j)) & 1 ? 0 : int(0x80000000u);
+#pragma unroll
+        for (int k = 0; k < A; ++k) {
+            const double p = flip_sign(__shfl_xor_sync(0xffffffffu, v[k], 1 << (b0 + j)), flip);
+            v[k] = fma(r, sf ? v[k] : p, sf ? p : v[k]);
+        }
+    }
+}
+template <int A, int LOGA>
+__device__ __forceinline__ void ry64_regs(double (&v)[A], const long long* ang) {
+#pragma unroll
+    for (int kb = 0; kb < LOGA; ++kb) {
+        const long long q = ang[kb];
+        const double r = __longlong_as_double(q & ~(1LL << 62));
+        const bool sf = (q >> 62) & 1;
+#pragma unroll
+        for (int k = 0; k < A; ++k)
+            if (!((k >> kb) & 1)) {
+                const double a0 = v[k], a1 = v[k | (1 << kb)];
+                v[k] = fma(r, sf ? a0 : -a1, sf ? -a1 : a0);
+                v[k | (1 << kb)] = fma(r, sf ? a1 : a0, sf ? a0 : a1);
+            }
+    }
+}
+
+// Shared memory of build_state_f64, in bytes: the ratios and the groups' factors, two
+// buffers of 2^n amplitudes.
+__host__ __device__ inline size_t f64_angle_bytes(int n, int P) {
+    return (8 * size_t(P + ry64_groups(n, P)) + 15) & ~size_t(15);
+}
+__host__ __device__ inline size_t f64_smem(int n, int P) { return f64_angle_bytes(n, P) + (size_t(16) << n); }
+
+// n >= 8: A = 2^n / 256 amplitudes per thread.  Mapping 0: i = (r << 8) | (w << 5) |
+// lane (qubits 0..4 on lanes, 5..7 on warps), mapping 1: i = (r << 8) | (lane << 3) | w
+// (3..7 on lanes, 0..2 on warps); one transpose per layer brings the three
+// qubits of the warp bits onto lanes, alternating the mappings, as
+// state_regs_multiwarp.
+template <int A, int LOGA>
+__device__ void f64_multiwarp(double* out, double* scr, const long long* ang, const double* fac, const double2* c0, int n,
+                              int d, int t) {
+    const int lane = t & 31, w = t >> 5, N = 1 << n, G = ry64_group(n);
+    auto index = [&](int M, int r) { return M == 0 ? (r << 8) | (w << 5) | lane : (r << 8) | (lane << 3) | w; };
+    double v[A];
+#pragma unroll
+    for (int r = 0; r < A; ++r) {
+        const int i = index(0, r);
+        v[r] = 1.0;
+        for (int q = 0; q < n; ++q) v[r] *= ((i >> q) & 1) ? c0[q].y : c0[q].x;
+    }
+    int M = 0, g = 0;
+    for (int layer = 1; layer <= d; ++layer) {
+        const long long* la = ang + layer * n;
+#pragma unroll
+        for (int r = 0; r < A; ++r) v[r] = flip_sign(v[r], czring_parity(index(M, r), n) << 31);
+        ry64_lanes<A>(v, lane, 0, 5, la + (M == 0 ? 0 : 3));
+        ry64_regs<A, LOGA>(v, la + 8);
+        double* buf = scr + (layer & 1) * N;
+#pragma unroll
+        for (int r = 0; r < A; ++r) buf[fx_at(index(M, r))] = v[r];
+        __syncthreads();
+        M ^= 1;
+#pragma unroll
+        for (int r = 0; r < A; ++r) v[r] = buf[fx_at(index(M, r))];
+        // mapping 0: lanes 0..2 hold qubits 0..2; mapping 1: lanes 2..4 hold qubits 5..7
+        ry64_lanes<A>(v, lane, M == 0 ? 0 : 2, 3, la + (M == 0 ? 0 : 5));
+        if (layer == d || layer == (g + 1) * G) {
+            const double f = fac[g++];
+#pragma unroll
+            for (int r = 0; r < A; ++r) v[r] *= f;
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < A; ++r) out[index(M, r)] = v[r];
+}
+
+// n <= 7: one warp holds the state, A = max(1, 2^n / 32) amplitudes per lane.
+template <int A, int LOGA>
+__device__ void f64_warp(double* out, const long long* ang, const double* fac, const double2* c0, int n, int d, int lane) {
+    const int N = 1 << n, li = N < 32 ? lane & (N - 1) : lane, nl = n < 5 ? n : 5, G = ry64_group(n);
+    double v[A];
+#pragma unroll
+    for (int r = 0; r < A; ++r) {
+        const int i = (r << 5) | li;
+        v[r] = 1.0;
+        for (int q = 0; q < n; ++q) v[r] *= ((i >> q) & 1) ? c0[q].y : c0[q].x;
+    }
+    int g = 0;
+    for (int layer = 1; layer <= d; ++layer) {
+        const long long* la = ang + layer * n;
+#pragma unroll
+        for (int r = 0; r < A; ++r) v[r] = flip_sign(v[r], czring_parity((r << 5) | li, n) << 31);
+        ry64_lanes<A>(v, lane, 0, nl, la);
+        ry64_regs<A, LOGA>(v, la + 5);
+        if (layer == d || layer == (g + 1) * G) {
+            const double f = fac[g++];
+#pragma unroll
+            for (int r = 0; r < A; ++r) v[r] *= f;
+        }
+    }
+    if (lane < N || N >= 32) {
+#pragma unroll
+        for (int r = 0; r < A; ++r) out[(r << 5) | lane] = v[r];
+    }
+}
+
+// psi(alpha_s) in `out`, 2^n doubles of smem (f64_smem(n, P) bytes); as many in `other`
+// are free afterwards.  cs as for build_state_real; n <= NMAX.  Whole CTA of 256
+// threads; ends with a barrier.
+template <int NMAX>
+__device__ inline void build_state_f64(unsigned char* smem, int n, int d, int P, const double2* cs, int s, double*& out,
+                                       double*& other) {
+    const int N = 1 << n, t = threadIdx.x, lane = t & 31, w = t >> 5;
+    long long* ang = reinterpret_cast<long long*>(smem);
+    double* fac = reinterpret_cast<double*>(ang + P);
+    double* scr = reinterpret_cast<double*>(smem + f64_angle_bytes(n, P));  // two buffers; the first layer's (cos, sin)
+    double2* c0 = reinterpret_cast<double2*>(scr);                          // start in the one first written at layer 2
+    // the result: not the buffer of the last transpose, whose reads may still go on
+    out = scr + (n < 8 ? 1 : (d + 1) & 1) * N;
+    other = out == scr ? scr + N : scr;
+    int k = -1, which = 0;
+    if (s > 0) {
+        k = (s - 1) >> 1;
+        which = ((s - 1) & 1) ? 2 : 1;
+    }
+    auto angle = [&](int a) { return cs[(a == k ? which : 0) * P + a]; };
+    const int G = ry64_group(n), groups = ry64_groups(n, P);
+    for (int g = w; g < groups; g += 8) {
+        const int first = n * (1 + g * G);
+        const double f = ry64_factor(first, min(n * G, P - first), lane, angle);
+        if (lane == 0) fac[g] = f;
+    }
+    for (int a = n + (t ^ 128); a < P; a += 256) ang[a] = ry64_pack(angle(a));
+    if (t < n) c0[t] = angle(t);  // on |0>: a product state
+    __syncthreads();
+    switch (n) {
+        case 8: f64_multiwarp<1, 0>(out, scr, ang, fac, c0, n, d, t); break;
+        case 9: f64_multiwarp<2, 1>(out, scr, ang, fac, c0, n, d, t); break;
+        case 10: f64_multiwarp<4, 2>(out, scr, ang, fac, c0, n, d, t); break;
+        case 11:
+            if constexpr (NMAX >= 11) f64_multiwarp<8, 3>(out, scr, ang, fac, c0, n, d, t);
+            break;
+        case 12:
+            if constexpr (NMAX >= 12) f64_multiwarp<16, 4>(out, scr, ang, fac, c0, n, d, t);
+            break;
+        default:
+            if (t < 32) {
+                if (n == 7) f64_warp<4, 2>(out, ang, fac, c0, n, d, t);
+                else if (n == 6) f64_warp<2, 1>(out, ang, fac, c0, n, d, t);
+                else f64_warp<1, 0>(out, ang, fac, c0, n, d, t);
+            }
+            break;
+    }
+    __syncthreads();
 }
 
 }  // namespace dvqls

@@ -26,6 +26,7 @@
 #include <algorithm>
 #include <mutex>
 #include <string>
+#include <type_traits>
 
 #include "internal.cuh"
 #include "state.cuh"
@@ -2423,11 +2424,11 @@ constexpr size_t WHT_OFF_BIM = WHT_OFF_EK + 8 * WHT_MAXP;  // int: bit 0 b has a
                                                            // then (FP64) int: the weights' exponent
 constexpr size_t WHT_TABLE_BYTES = WHT_OFF_BIM + 16;          // header: int pair classes, term classes
 // Fixed point of the FP64 classes (units of 2^-FX_BITS): b is scaled by a power
-// of two so that ||b|| <= 1.
+// of two, 2^-ex, so that ||b|| <= 3/2.
 __device__ __forceinline__ int w64_bexp(double bn2) {
     int ex;
-    frexp(sqrt(bn2), &ex);  // ||b|| <= 2^ex
-    return min(max(ex, -1000), 1000);  // an invalid ||b||^2 is reported and marked in the table
+    const double m = frexp(sqrt(bn2), &ex);  // ||b|| = m 2^ex, 1/2 <= m < 1
+    return min(max(m <= 0.75 ? ex - 1 : ex, -1000), 1000);  // an invalid ||b||^2 is reported and marked in the table
 }
 
 // What a class pass needs of one instance (one CTA each), in one launch: the
@@ -2539,7 +2540,7 @@ __global__ void __launch_bounds__(WHT_CT) k_wht_prepare(const Inst* __restrict__
         }
     }
     __syncthreads();
-    if (F64 && t < L) {  // weights of c~ 2^-s_exp, which is below 2: their sums in units of 2^-60 stay in range
+    if (F64 && t < L) {  // weights of c~ 2^-s_exp, which is below 2: their sums in units of 2^-62 stay in range
         const double f = scalbn(1.0, -s_exp);  // exact
         sc[t].x *= f;
         sc[t].y *= f;
@@ -2974,16 +2975,24 @@ inline size_t wht_smem_bytes(int Pmax) {
 // The FP64 tiles spend one DFMA per term and amplitude on a pipe that issues 2
 // per clock and SM (n = 10, L = 64: 2.2 M DFMAs, 1.1 M cycles per state).  Here
 // the state (build_state_fx) and the transforms run in 64-bit fixed point on the
-// integer pipes: sum_i |psi[i] psi[i ^ x]| <= 1, so every partial sum of a
-// transform stays within 1.0 = 2^60 and the adds are exact; a product is rounded
-// once, at 2^-60.  The FP64 pipe keeps one FMA per term for the weighted sums.
+// integer pipes: sum_i |psi[i] psi[i ^ x]| <= 1 = 2^62, and |b[i ^ x] psi[i]| sums up to 3/2 at
+// most (w64_bexp), so every partial sum of a transform stays within 64 bits and the adds
+// are exact; a product is rounded once, at 2^-62.  The FP64 pipe keeps one FMA per term for the weighted sums.
 // One CTA of 8 warps per item, two CTAs per SM (the transform of 2^10 values
 // holds 64 registers a lane), so one CTA's state build overlaps the other's
 // transforms.
-// n = 10, L = 64, 101 shifts of one system: 623 us by the tiles, 46 us by the
-// classes (72 with an FP64 state); 48 systems of n = 6..10: 8,646 us against 331
-// (600).  A state of n = 10 takes 20 k cycles of a CTA, its 29 transforms and 2,080
-// lookups 31 k; both are bound by the integer multiply-adds and adds.
+//
+// Fixed point has an absolute error, FP64 sums one relative to the size of their terms.
+// A class's products are summed up in magnitude on the way; where that is below
+// W64_FULL (angles near zero, a right-hand side of few entries), the item starts over
+// with its state in FP64 (build_state_f64) and every class in a unit of its own, 2^-62 of a
+// bound on that sum (from the exponents of its products, within a factor of 8): an
+// overlap is then as accurate as an FP64 sum of its terms, however small they are.
+// n = 10, L = 64, 101 shifts of one system: 623 us by the tiles, 36 us by the
+// classes; 48 systems of n = 6..10 at random angles: 8,646 us against 336 (317 without the
+// magnitudes, 444 with the FP64 state and units for every item).  A state of n = 10 takes
+// 20 k cycles of a CTA, its 29 transforms and 2,080 lookups 31 k; both are bound by the
+// integer multiply-adds and adds.
 constexpr int W64_ROW = (1 << WHT_MAXN) + (1 << WHT_MAXN) / 32;
 
 // Factor of an instance's results, from its class table: NaN when one of the bits
@@ -2993,8 +3002,75 @@ __device__ __forceinline__ double w64_valid(const unsigned char* tb, int bad) {
     return *reinterpret_cast<const int*>(tb + WHT_OFF_BIM) & bad ? __longlong_as_double(0x7ff8000000000000LL) : 1.0;
 }
 // Exponent of an instance's weights: the table holds them for c~ scaled down by half of it, so
-// that no weight times a transform value in units of 2^-60 leaves the range of a double.
+// that no weight times a transform value in units of 2^-62 leaves the range of a double.
 __device__ __forceinline__ int w64_wexp(const unsigned char* tb) { return reinterpret_cast<const int*>(tb + WHT_OFF_BIM)[1]; }
+// a b in units of 2^-62, rounded to nearest (without the product of the low parts, below a
+// unit); EVEN: ties to even.  A factor of few bits, as the entries of b = |+> are, makes a tie of
+// one product in eight or sixteen, and rounded up they would add up in a transform's first value
+// (n = 10, depth 1: T 3e-17 off, 7e-18 to even).
+template <bool EVEN>
+__device__ __forceinline__ long long w64_mul(int2 a, int2 b) {
+    long long x = (1LL << 27) - EVEN + (long long)a.x * b.y + (long long)a.y * b.x;
+    if (EVEN) x += ((x + 1 - (1LL << 27)) >> 28) & 1;
+    return (x >> 28) + (long long)a.x * b.x * 4;
+}
+// Magnitude of its products, in units of 2^-30, from which a class is taken in fixed point:
+// 1/32.  Its errors come to 2^-58 at n = 10 (1,024 roundings at 2^-62, amplitudes that are
+// 2^-59 off), an FP64 rounding of that sum, and less for fewer products.
+constexpr unsigned W64_FULL = 1u << 25;
+
+// A product's operand in parts: an FP64 value (h 2^30 + l) 2^(e - 60), its significand in
+// two signed parts, |h| < 2^31, |l| < 2^30, exact (a zero or a subnormal has the least
+// exponent and no leading one).
+__device__ __forceinline__ int fl_exp(double v) { return max((__double2hiint(v) >> 20) & 0x7ff, 1) - 1023; }
+__device__ __forceinline__ int2 fl_parts(double v) {
+    const int hi = __double2hiint(v), lo = __double2loint(v);
+    const int m = (hi & 0xfffff) | ((hi >> 20) & 0x7ff ? 1 << 20 : 0);
+    const int h = (m << 10) | int(uint32_t(lo) >> 22), l = (lo & 0x3fffff) << 8;
+    return hi < 0 ? make_int2(-h, -l) : make_int2(h, l);
+}
+// a b 2^(62 - E), rounded to nearest, ties to even, for products below 2^(E - 1) (down = E - 3 -
+// the sum of their exponents, not negative).  The product of the low parts, below 2^-60 of
+// a full product, is dropped.
+__device__ __forceinline__ long long fl_mul(int2 a, int2 b, int down) {
+    const long long p = (long long)a.x * b.x + (((long long)a.x * b.y + (long long)a.y * b.x) >> 30);
+    const int sh = min(down, 63);
+    const long long q = p >> sh >> 1;  // the next bit decides, or those below it, or the last one kept
+    return q + ((p >> sh & 1) && ((q & 1) || p >> sh << sh != p));
+}
+// Whether a class's products, of magnitude `mag` over this lane (2^-30; a floor counts a
+// negative product's by one more at most), sum up to less than W64_FULL; tells the others.
+__device__ __forceinline__ bool w64_sparse(unsigned mag, int n, int lane, int* sparse) {
+    mag = __reduce_add_sync(0xffffffffu, n < 5 && lane >> n ? 0u : mag);
+    if (mag >= W64_FULL) return false;
+    if (lane == 0) *reinterpret_cast<volatile int*>(sparse) = 1;
+    return true;
+}
+// v[r] = the products of a(r) and q(r), FP64 values in parts (fl_parts, fl_exp), of a lane
+// in the unit 2^ex that is returned: 2^-62 of a bound 2^E on the sum of the magnitudes of the
+// warp's products (each below 2^(s + 2), s the sum of its exponents, so that every
+// s <= E - 3; `live`: no other lane holds the same products).  Rolled loops, through the
+// warp's row: few instructions and registers for the path that is taken seldom.
+template <int A, class Exps, class Mul>
+__device__ __forceinline__ int w64_products(long long (&v)[A], const Exps& exps, const Mul& mul, long long* row, int lane,
+                                            bool live) {
+    int top = -4096;
+#pragma unroll 2
+    for (int r = 0; r < A; ++r) top = max(top, exps(r));
+    top = __reduce_max_sync(0xffffffffu, top);
+    unsigned sum = A;  // units of 2^(top - 20); what the shifts drop is below one unit each
+#pragma unroll 2
+    for (int r = 0; r < A; ++r) sum += (1u << 20) >> min(top - exps(r), 31);
+    sum = __reduce_add_sync(0xffffffffu, live ? sum : 0u);
+    const int E = top + 2 - 20 + (32 - __clz(sum));
+#pragma unroll 2
+    for (int r = 0; r < A; ++r) row[(r << 5) | lane] = mul(r, E - 3 - exps(r));
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < A; ++r) v[r] = row[(r << 5) | lane];
+    __syncwarp();
+    return E - 62;
+}
 
 // Transform of v (index (r << 5) | lane) into the warp's row, at i + (i >> 5)
 // for 2^10 values (A = 32: through the row, lane bits become register bits), else at i.
@@ -3039,11 +3115,13 @@ __device__ __forceinline__ void w64_transform(long long (&v)[A], long long* row,
 }
 
 // The pair classes (flavours 0..n of the local cost) and, for the global cost,
-// the term classes of one state q, dealt to the warps; the warp's sums of its
-// lanes in D (flavour 0) and E (the others), delta~ to dre / dim.
-template <int A, int LOGA>
-__device__ void w64_item(const Inst& I, int s, const Fx* q, long long* row, double* dre, double* dim,
-                         const uint32_t* szl, double& D, double& E, int lane) {
+// the term classes of one state, dealt to the warps; the warp's sums of its
+// lanes in D (flavour 0) and E (the others), delta~ to dre / dim.  FIXED: the state q is in
+// fixed point, and *sparse is set, and everything left, when a class is not full;
+// else q is in parts, with the exponents qe.
+template <int A, int LOGA, bool FIXED>
+__device__ void w64_item(const Inst& I, int s, const int2* q, const int* qe, long long* row, double* dre, double* dim,
+                         const uint32_t* szl, double& D, double& E, int lane, int* sparse) {
     constexpr bool PAD = A == 32;
     const int n = I.n, N = 1 << n, L = I.L, w = threadIdx.x >> 5, lm = N < 32 ? N - 1 : 31;
     const unsigned char* tb = reinterpret_cast<const unsigned char*>(I.wht);
@@ -3062,46 +3140,76 @@ __device__ void w64_item(const Inst& I, int s, const Fx* q, long long* row, doub
     auto at = [&](uint32_t z) { return (double)row[PAD ? z + (z >> 5) : z]; };
 #pragma unroll 1
     for (int j = w; j < jobs; j += WHT_NT / 32) {
+        if (FIXED && *reinterpret_cast<volatile int*>(sparse)) return;
         long long v[A];
+        int ex = -62;  // the transform's unit is 2^ex
         if (j >= pairs) {
             const int c = (j - pairs) / parts, part = (j - pairs) - c * parts, x = int(dx[c]);
-            const int4* qb = reinterpret_cast<const int4*>(I.bf);
+            // conj(b[i ^ x]) psi[i], its real or imaginary part (negated)
+            if (FIXED) {
+                const int2* qb = reinterpret_cast<const int2*>(I.bf) + part;
+                unsigned mag = 0u;
 #pragma unroll
-            for (int r = 0; r < A; ++r) {  // conj(b[i ^ x]) psi[i], its real or imaginary part
-                const int i = (r << 5) | (lane & lm), k = (i ^ x) & (N - 1);
-                const int4 bb = qb[k];
-                v[r] = fx_mul(part ? fx_neg(Fx{bb.z, bb.w}) : Fx{bb.x, bb.y}, q[i]);
+                for (int r = 0; r < A; ++r) {
+                    const int i = (r << 5) | (lane & lm), k = (i ^ x) & (N - 1);
+                    v[r] = w64_mul<true>(qb[2 * k], q[i]);
+                    mag = __sad(int(v[r] >> 32), 0, mag);
+                }
+                if (w64_sparse(mag, n, lane, sparse)) return;
+                ex += w64_bexp(*I.bn2);
+            } else {
+                const double* b = reinterpret_cast<const double*>(I.b) + part;
+                auto i = [&](int r) { return (r << 5) | (lane & lm); };
+                auto bv = [&](int r) { return b[2 * ((i(r) ^ x) & (N - 1))]; };
+                ex = w64_products<A>(v, [&](int r) { return qe[i(r)] + fl_exp(bv(r)); },
+                                     [&](int r, int down) { return fl_mul(fl_parts(bv(r)), q[i(r)], down); }, row, lane,
+                                     lane < N || N >= 32);
             }
             w64_transform<A, LOGA>(v, row, N, lane);
-            const double sc = scalbn(w64_valid(tb, 2 | 4), w64_bexp(*I.bn2) - FX_BITS);
             for (int e = dof[c] + lane; e < dof[c + 1]; e += 32) {
                 const int l = dt[e];
-                (part ? dim : dre)[l] = at(szl[l] & uint32_t(N - 1)) * sc;
+                const double d = scalbn(at(szl[l] & uint32_t(N - 1)), ex) * w64_valid(tb, 2 | 4);
+                (part ? dim : dre)[l] = part ? -d : d;
             }
             __syncwarp();
             continue;
         }
         const int f = j / ncls, c = j - f * ncls;
         const int x = int(cx[c] ^ (f ? 1u << (f - 1) : 0u));  // X_j between the two terms (local cost)
+        if (FIXED) {
+            unsigned mag = 0u;
 #pragma unroll
-        for (int r = 0; r < A; ++r) {
-            const int i = (r << 5) | (lane & lm);
-            v[r] = fx_mul(q[i], q[(i ^ x) & (N - 1)]);  // masks >= 2^n are reported, never followed
+            for (int r = 0; r < A; ++r) {
+                const int i = (r << 5) | (lane & lm);
+                v[r] = w64_mul<false>(q[i], q[(i ^ x) & (N - 1)]);  // masks >= 2^n are reported, never followed
+                mag = __sad(int(v[r] >> 32), 0, mag);
+            }
+            if (w64_sparse(mag, n, lane, sparse)) return;
+        } else {
+            auto i = [&](int r) { return (r << 5) | (lane & lm); };
+            auto k = [&](int r) { return (i(r) ^ x) & (N - 1); };
+            ex = w64_products<A>(v, [&](int r) { return qe[i(r)] + qe[k(r)]; },
+                                 [&](int r, int down) { return fl_mul(q[i(r)], q[k(r)], down); }, row, lane,
+                                 lane < N || N >= 32);
         }
         w64_transform<A, LOGA>(v, row, N, lane);
         const int e0 = co[c], e1 = co[c + 1];
+        double sum = 0.0;  // of the class, in its unit
         if (f == 0) {
-            for (int e = e0 + lane; e < e1; e += 32) D = fma(ek[e], at(ez[e]), D);
+            for (int e = e0 + lane; e < e1; e += 32) sum = fma(ek[e], at(ez[e]), sum);
         } else {
             for (int e = e0 + lane; e < e1; e += 32) {
                 const double k = ek[e];
-                E = fma((szl[pr[e] & 0xFF] >> (f - 1)) & 1u ? -k : k, at(ez[e]), E);
+                sum = fma((szl[pr[e] & 0xFF] >> (f - 1)) & 1u ? -k : k, at(ez[e]), sum);
             }
         }
+        if (!FIXED) sum = scalbn(sum, ex + 62);
+        if (f == 0) D += sum;
+        else E += sum;
         if (Gp)  // the beta output of the unshifted state
             for (int e = e0 + lane; e < e1; e += 32) {
                 const int p = pr[e], l = p & 0xFF, m = p >> 8;
-                double beta = at(ez[e]) * scalbn(w64_valid(tb, 2), -FX_BITS);
+                double beta = scalbn(at(ez[e]), ex) * w64_valid(tb, 2);
                 if (__popc(szl[l] & uint32_t(x)) & 1) beta = -beta;
                 Gp[(long long)l * L + m] = make_double2(beta, 0.0);
                 Gp[(long long)m * L + l] = make_double2(beta, 0.0);
@@ -3123,6 +3231,7 @@ __global__ void __launch_bounds__(WHT_NT, 2) k_terms_wht64(const Inst* __restric
     __shared__ double dre[TT], dim[TT], red[WHT_NT / 32], redE[WHT_NT / 32];
     __shared__ double2 redT[2];
     __shared__ long long s_item;
+    __shared__ int s_sparse;
     const int t = threadIdx.x, w = t >> 5, lane = t & 31;
     long long* row = reinterpret_cast<long long*>(smem) + w * W64_ROW;  // this warp's transform row
     for (;;) {
@@ -3137,15 +3246,36 @@ __global__ void __launch_bounds__(WHT_NT, 2) k_terms_wht64(const Inst* __restric
             szl[t] = t < L ? I.zm[t] : 0u;
             dre[t] = dim[t] = 0.0;
         }
-        const Fx* q = build_state_fx(smem + 64 * W64_ROW, I.n, I.d, I.P, I.cs, s + I.s0);  // ends with a barrier
+        if (t == 0) s_sparse = 0;
         double D = 0.0, E = 0.0;
-        switch (I.n) {
-            case 10: w64_item<32, 5>(I, s, q, row, dre, dim, szl, D, E, lane); break;
-            case 9: w64_item<16, 4>(I, s, q, row, dre, dim, szl, D, E, lane); break;
-            case 8: w64_item<8, 3>(I, s, q, row, dre, dim, szl, D, E, lane); break;
-            case 7: w64_item<4, 2>(I, s, q, row, dre, dim, szl, D, E, lane); break;
-            case 6: w64_item<2, 1>(I, s, q, row, dre, dim, szl, D, E, lane); break;
-            default: w64_item<1, 0>(I, s, q, row, dre, dim, szl, D, E, lane); break;  // n <= 5
+        auto classes = [&](auto fixed, const int2* q, const int* qe) {
+            constexpr bool FIXED = decltype(fixed)::value;
+            switch (I.n) {
+                case 10: w64_item<32, 5, FIXED>(I, s, q, qe, row, dre, dim, szl, D, E, lane, &s_sparse); break;
+                case 9: w64_item<16, 4, FIXED>(I, s, q, qe, row, dre, dim, szl, D, E, lane, &s_sparse); break;
+                case 8: w64_item<8, 3, FIXED>(I, s, q, qe, row, dre, dim, szl, D, E, lane, &s_sparse); break;
+                case 7: w64_item<4, 2, FIXED>(I, s, q, qe, row, dre, dim, szl, D, E, lane, &s_sparse); break;
+                case 6: w64_item<2, 1, FIXED>(I, s, q, qe, row, dre, dim, szl, D, E, lane, &s_sparse); break;
+                default: w64_item<1, 0, FIXED>(I, s, q, qe, row, dre, dim, szl, D, E, lane, &s_sparse); break;  // n <= 5
+            }
+        };
+        unsigned char* room = smem + 64 * W64_ROW;
+        const Fx* fx = build_state_fx(room, I.n, I.d, I.P, I.cs, s + I.s0);  // ends with a barrier
+        classes(std::true_type{}, reinterpret_cast<const int2*>(fx), nullptr);
+        __syncthreads();
+        if (s_sparse) {
+            double *psi, *other;
+            build_state_f64<WHT_MAXN>(room, I.n, I.d, I.P, I.cs, s + I.s0, psi, other);  // ends with a barrier
+            int2* q = reinterpret_cast<int2*>(psi);
+            int* qe = reinterpret_cast<int*>(other);
+            for (int i = t; i < 1 << I.n; i += WHT_NT) {
+                const double v = psi[i];
+                q[i] = fl_parts(v);
+                qe[i] = fl_exp(v);
+            }
+            D = E = 0.0;
+            __syncthreads();
+            classes(std::false_type{}, q, qe);
         }
         for (int o = 16; o; o >>= 1) D += __shfl_xor_sync(0xffffffffu, D, o);
         if (I.local)
@@ -3173,7 +3303,7 @@ __global__ void __launch_bounds__(WHT_NT, 2) k_terms_wht64(const Inst* __restric
         if (t == 0) {
             const unsigned char* tb = reinterpret_cast<const unsigned char*>(I.wht);
             const double valid = w64_valid(tb, 2);
-            const int we = w64_wexp(tb) - FX_BITS;
+            const int we = w64_wexp(tb) - 62;
             double Ds = 0.0, Es = 0.0;
             for (int k = 0; k < WHT_NT / 32; ++k) {
                 Ds += red[k];
