@@ -3055,15 +3055,15 @@ template <int A, class Exps, class Mul>
 __device__ __forceinline__ int w64_products(long long (&v)[A], const Exps& exps, const Mul& mul, long long* row, int lane,
                                             bool live) {
     int top = -4096;
-#pragma unroll 2
+#pragma unroll 8
     for (int r = 0; r < A; ++r) top = max(top, exps(r));
     top = __reduce_max_sync(0xffffffffu, top);
     unsigned sum = A;  // units of 2^(top - 20); what the shifts drop is below one unit each
-#pragma unroll 2
+#pragma unroll 8
     for (int r = 0; r < A; ++r) sum += (1u << 20) >> min(top - exps(r), 31);
     sum = __reduce_add_sync(0xffffffffu, live ? sum : 0u);
     const int E = top + 2 - 20 + (32 - __clz(sum));
-#pragma unroll 2
+#pragma unroll 8
     for (int r = 0; r < A; ++r) row[(r << 5) | lane] = mul(r, E - 3 - exps(r));
     __syncwarp();
 #pragma unroll
@@ -3114,18 +3114,33 @@ __device__ __forceinline__ void w64_transform(long long (&v)[A], long long* row,
     __syncwarp();
 }
 
-// The pair classes (flavours 0..n of the local cost) and, for the global cost,
-// the term classes of one state, dealt to the warps; the warp's sums of its
-// lanes in D (flavour 0) and E (the others), delta~ to dre / dim.  FIXED: the state q is in
+// Transforms of a state: the pair classes (flavours 0..n of the local cost) and, for
+// the global cost, the term classes (Re, and Im when b has an imaginary part).
+__device__ __forceinline__ int w64_jobs(const Inst& I) {
+    const unsigned char* tb = reinterpret_cast<const unsigned char*>(I.wht);
+    const int ncls = reinterpret_cast<const int*>(tb)[0], nd = reinterpret_cast<const int*>(tb)[1];
+    return ncls * I.F + (I.local ? 0 : nd * (1 + (*reinterpret_cast<const int*>(tb + WHT_OFF_BIM) & 1)));
+}
+// Where the states of a pass leave room on the GPU, a state's transforms are dealt to several
+// CTAs, which all build it: up to I.ks parts, of W64_PART transforms (one round of a CTA's warps)
+// at least; a CTA without a part ends at once.  Masks that share few classes give few
+// parts, random masks (a class per pair nearly) many: one state of n = 10, L = 64 65 us, its
+// local cost 80 (one CTA per state 343 and 2,883; the tiles, which split the amplitudes, 140
+// both); 101 states with 29 transforms each take the 36 us that one CTA per state takes.
+// Parts of 16 transforms left two of 304 CTAs' items on one SM there (47 us).
+constexpr int W64_PART = 8;
+
+// The transforms first, first + step, ... of one state, each by a warp; the warp's sums of
+// its lanes in D (flavour 0) and E (the others), delta~ to dre / dim.  FIXED: the state q is in
 // fixed point, and *sparse is set, and everything left, when a class is not full;
 // else q is in parts, with the exponents qe.
 template <int A, int LOGA, bool FIXED>
 __device__ void w64_item(const Inst& I, int s, const int2* q, const int* qe, long long* row, double* dre, double* dim,
-                         const uint32_t* szl, double& D, double& E, int lane, int* sparse) {
+                         const uint32_t* szl, double& D, double& E, int lane, int* sparse, int first, int step) {
     constexpr bool PAD = A == 32;
-    const int n = I.n, N = 1 << n, L = I.L, w = threadIdx.x >> 5, lm = N < 32 ? N - 1 : 31;
+    const int n = I.n, N = 1 << n, L = I.L, lm = N < 32 ? N - 1 : 31;
     const unsigned char* tb = reinterpret_cast<const unsigned char*>(I.wht);
-    const int ncls = reinterpret_cast<const int*>(tb)[0], nd = reinterpret_cast<const int*>(tb)[1];
+    const int ncls = reinterpret_cast<const int*>(tb)[0];
     const uint32_t* cx = reinterpret_cast<const uint32_t*>(tb + WHT_OFF_CX);
     const int* co = reinterpret_cast<const int*>(tb + WHT_OFF_CO);
     const uint16_t* pr = reinterpret_cast<const uint16_t*>(tb + WHT_OFF_PR);
@@ -3135,11 +3150,12 @@ __device__ void w64_item(const Inst& I, int s, const int2* q, const int* qe, lon
     const int* dof = reinterpret_cast<const int*>(tb + WHT_OFF_DO);
     const uint16_t* dt = reinterpret_cast<const uint16_t*>(tb + WHT_OFF_DT);
     double2* Gp = (s == 0 && I.Gpart) ? reinterpret_cast<double2*>(I.Gpart) : nullptr;
+    double* dp = (s == 0 && I.dpart) ? reinterpret_cast<double*>(I.dpart) : nullptr;
     const int parts = 1 + (*reinterpret_cast<const int*>(tb + WHT_OFF_BIM) & 1);
-    const int pairs = ncls * I.F, jobs = pairs + (I.local ? 0 : nd * parts);
+    const int pairs = ncls * I.F, jobs = w64_jobs(I);
     auto at = [&](uint32_t z) { return (double)row[PAD ? z + (z >> 5) : z]; };
 #pragma unroll 1
-    for (int j = w; j < jobs; j += WHT_NT / 32) {
+    for (int j = first; j < jobs; j += step) {
         if (FIXED && *reinterpret_cast<volatile int*>(sparse)) return;
         long long v[A];
         int ex = -62;  // the transform's unit is 2^ex
@@ -3170,6 +3186,10 @@ __device__ void w64_item(const Inst& I, int s, const int2* q, const int* qe, lon
                 const int l = dt[e];
                 const double d = scalbn(at(szl[l] & uint32_t(N - 1)), ex) * w64_valid(tb, 2 | 4);
                 (part ? dim : dre)[l] = part ? -d : d;
+                if (dp) {  // the delta output of the unshifted state
+                    dp[2 * l + part] = part ? -d : d;
+                    if (parts == 1) dp[2 * l + 1] = 0.0;
+                }
             }
             __syncwarp();
             continue;
@@ -3241,29 +3261,42 @@ __global__ void __launch_bounds__(WHT_NT, 2) k_terms_wht64(const Inst* __restric
         __syncthreads();
         if (gi >= total) break;
         const Inst& I = insts[find_instance(insts, count, gi)];
-        const int s = int(gi - I.item_base), L = I.L;
+        // items of an instance: part 0 of every state first, so that states spread over the SMs
+        const int local = int(gi - I.item_base), s = local % I.S, part = local / I.S, L = I.L, ks = I.ks;
+        const int live = min(ks, max(1, w64_jobs(I) / W64_PART));
+        double2* Dp = I.Dpart + (long long)s * I.F * ks + part;
+        if (part >= live) {
+            for (int f = t; f < I.F; f += WHT_NT) Dp[f * ks] = make_double2(0.0, 0.0);
+            if (!I.local && t == 0) I.Tpart[(long long)s * ks + part] = make_double2(0.0, 0.0);
+            continue;
+        }
         if (t < TT) {
             szl[t] = t < L ? I.zm[t] : 0u;
             dre[t] = dim[t] = 0.0;
         }
         if (t == 0) s_sparse = 0;
         double D = 0.0, E = 0.0;
+        const int first = part * (WHT_NT / 32) + w, step = live * (WHT_NT / 32);
         auto classes = [&](auto fixed, const int2* q, const int* qe) {
             constexpr bool FIXED = decltype(fixed)::value;
             switch (I.n) {
-                case 10: w64_item<32, 5, FIXED>(I, s, q, qe, row, dre, dim, szl, D, E, lane, &s_sparse); break;
-                case 9: w64_item<16, 4, FIXED>(I, s, q, qe, row, dre, dim, szl, D, E, lane, &s_sparse); break;
-                case 8: w64_item<8, 3, FIXED>(I, s, q, qe, row, dre, dim, szl, D, E, lane, &s_sparse); break;
-                case 7: w64_item<4, 2, FIXED>(I, s, q, qe, row, dre, dim, szl, D, E, lane, &s_sparse); break;
-                case 6: w64_item<2, 1, FIXED>(I, s, q, qe, row, dre, dim, szl, D, E, lane, &s_sparse); break;
-                default: w64_item<1, 0, FIXED>(I, s, q, qe, row, dre, dim, szl, D, E, lane, &s_sparse); break;  // n <= 5
+                case 10: w64_item<32, 5, FIXED>(I, s, q, qe, row, dre, dim, szl, D, E, lane, &s_sparse, first, step); break;
+                case 9: w64_item<16, 4, FIXED>(I, s, q, qe, row, dre, dim, szl, D, E, lane, &s_sparse, first, step); break;
+                case 8: w64_item<8, 3, FIXED>(I, s, q, qe, row, dre, dim, szl, D, E, lane, &s_sparse, first, step); break;
+                case 7: w64_item<4, 2, FIXED>(I, s, q, qe, row, dre, dim, szl, D, E, lane, &s_sparse, first, step); break;
+                case 6: w64_item<2, 1, FIXED>(I, s, q, qe, row, dre, dim, szl, D, E, lane, &s_sparse, first, step); break;
+                default: w64_item<1, 0, FIXED>(I, s, q, qe, row, dre, dim, szl, D, E, lane, &s_sparse, first, step); break;  // n <= 5
             }
         };
         unsigned char* room = smem + 64 * W64_ROW;
-        const Fx* fx = build_state_fx(room, I.n, I.d, I.P, I.cs, s + I.s0);  // ends with a barrier
-        classes(std::true_type{}, reinterpret_cast<const int2*>(fx), nullptr);
-        __syncthreads();
-        if (s_sparse) {
+        bool sparse = I.d == 0;  // a product state nearly always is
+        if (!sparse) {
+            const Fx* fx = build_state_fx(room, I.n, I.d, I.P, I.cs, s + I.s0);  // ends with a barrier
+            classes(std::true_type{}, reinterpret_cast<const int2*>(fx), nullptr);
+            __syncthreads();
+            sparse = s_sparse;
+        }
+        if (sparse) {
             double *psi, *other;
             build_state_f64<WHT_MAXN>(room, I.n, I.d, I.P, I.cs, s + I.s0, psi, other);  // ends with a barrier
             int2* q = reinterpret_cast<int2*>(psi);
@@ -3291,7 +3324,6 @@ __global__ void __launch_bounds__(WHT_NT, 2) k_terms_wht64(const Inst* __restric
                 const double2 c = I.ctil[t];
                 const double dr = dre[t], di = dim[t];
                 T = make_double2(c.x * dr - c.y * di, c.x * di + c.y * dr);
-                if (s == 0 && I.dpart) reinterpret_cast<double2*>(I.dpart)[t] = make_double2(dr, di);
             }
             for (int o = 16; o; o >>= 1) {
                 T.x += __shfl_xor_sync(0xffffffffu, T.x, o);
@@ -3309,11 +3341,11 @@ __global__ void __launch_bounds__(WHT_NT, 2) k_terms_wht64(const Inst* __restric
                 Ds += red[k];
                 if (I.local) Es += redE[k];
             }
-            I.Dpart[(long long)s * I.F] = make_double2(scalbn(Ds * valid, we), 0.0);
-            if (I.local) I.Dpart[(long long)s * I.F + 1] = make_double2(scalbn(Es * valid, we), 0.0);
-            else I.Tpart[s] = make_double2(redT[0].x + redT[1].x, redT[0].y + redT[1].y);
-        } else if (I.local && t >= 2 && t < I.F) {  // slot 0 of a shift holds D, slot 1 E, the rest zero
-            I.Dpart[(long long)s * I.F + t] = make_double2(0.0, 0.0);
+            Dp[0] = make_double2(scalbn(Ds * valid, we), 0.0);
+            if (I.local) Dp[ks] = make_double2(scalbn(Es * valid, we), 0.0);
+            else I.Tpart[(long long)s * ks + part] = make_double2(redT[0].x + redT[1].x, redT[0].y + redT[1].y);
+        } else if (I.local && t >= 2 && t < I.F) {  // flavour 0 of a shift holds D, flavour 1 E, the rest zero
+            Dp[t * ks] = make_double2(0.0, 0.0);
         }
         __syncthreads();
     }
@@ -3359,6 +3391,7 @@ __global__ void __launch_bounds__(NT) k_combine(const Inst* __restrict__ insts, 
     const int t = threadIdx.x, T = I.T, ks = I.ks, L = I.L;
     const double bn2 = *I.bn2;
     const int nd = I.fold ? 1 : T * T * ks, nt = I.fold ? 1 : T * ks, ne = I.fold ? 1 : (I.F - 1) * T * T * ks;
+    const int no = I.wht ? 1 : ks;  // parts of the beta and delta outputs (a class is one CTA's)
     for (int s = t; s < I.S; s += NT) {
         double D = 0.0;
         double2 Tv = make_double2(0.0, 0.0);
@@ -3400,7 +3433,7 @@ __global__ void __launch_bounds__(NT) k_combine(const Inst* __restrict__ insts, 
         const long long LL = (long long)L * L;
         for (long long e = t; e < LL; e += NT) {
             double gr = 0.0, gi = 0.0;
-            for (int k = 0; k < ks; ++k) {
+            for (int k = 0; k < no; ++k) {
                 gr += (double)G[k * LL + e].x;
                 gi += (double)G[k * LL + e].y;
             }
@@ -3419,7 +3452,7 @@ __global__ void __launch_bounds__(NT) k_combine(const Inst* __restrict__ insts, 
         const double inv = 1.0 / sqrt(bn2);
         for (int l = t; l < L; l += NT) {
             double vr = 0.0, vi = 0.0;
-            for (int k = 0; k < ks; ++k) {
+            for (int k = 0; k < no; ++k) {
                 vr += (double)dpp[(long long)k * L + l].x;
                 vi += (double)dpp[(long long)k * L + l].y;
             }
@@ -3782,8 +3815,14 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
     auto tuned = ctx->tune.find(sig);
     const bool fixed = ctx->fixed_split > 0;  // dvqls_set_tuning
     const bool tuning = any_smem && !wht && tuned == ctx->tune.end() && !fixed;
+    long long states = 0;
+    for (const auto& h : hi) states += h.S;
+    auto w64_parts = [&](const HostInst& h) {  // by the most transforms that the masks can ask for
+        const long long pairs = std::min<long long>(h.N, h.L * (h.L + 1) / 2), terms = std::min<long long>(h.N, h.L);
+        return (int)std::max<long long>(1, std::min(slots / states, (h.F * pairs + (local ? 0 : 2 * terms)) / W64_PART));
+    };
     auto ks_for = [&](const HostInst& h, int ks) {  // tensor-core items start on whole 128-amplitude stages
-        if (wht) return 1;                            // a class item covers a whole state
+        if (wht) return fp32 ? 1 : w64_parts(h);      // a class item covers a whole state, or part of its transforms
         return h.hbm ? (int)std::max<long long>(1, h.N / HBM_K)
                      : (int)std::min<long long>(ks, std::max<long long>(1, h.N / (tc ? TCK : JC)));
     };
@@ -3857,8 +3896,8 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
         o.bpart = h.hbm && !local ? ar.reserve(BN_PARTS * 8) : 0;
         o.Dp = ar.reserve(size_t(h.S) * h.F * h.T * h.T * kp * 16);
         o.Tp = ar.reserve(size_t(h.S) * h.T * kp * 16);
-        o.Gp = beta_out ? ar.reserve(size_t(kp) * L * L * r2) : 0;
-        o.dp = delta_out ? ar.reserve(size_t(kp) * L * r2) : 0;
+        o.Gp = beta_out ? ar.reserve(size_t(wht ? 1 : kp) * L * L * r2) : 0;
+        o.dp = delta_out ? ar.reserve(size_t(wht ? 1 : kp) * L * r2) : 0;
         o.NsDs = ar.reserve(size_t(h.S) * 24);
         o.states = h.hbm ? ar.reserve(size_t(h.S) * size_t(h.N) * (r2 / 2)) : 0;  // real amplitudes
         o.chain = h.hbm && h.S + h.s0 > 1 ? ar.reserve((2 * size_t(h.d) + 1) * size_t(h.N) * (r2 / 2)) : 0;
@@ -3967,11 +4006,11 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
             const int i = ord[oi];
             Inst I = rec[i];
             I.ks = kk[i];
-            I.fold = !wht && I.F * I.T * I.T * I.ks >= FOLD_MIN;
+            I.fold = I.F * I.T * I.T * I.ks >= FOLD_MIN;
             if (I.fold) ps.fold_grid = std::max(ps.fold_grid, ceil_div(I.S, 8));
-            // a Walsh-Hadamard item covers every flavour; the tensor-core tiles take
+            // a Walsh-Hadamard item covers every flavour (FP64: or a part of the transforms); the tensor-core tiles take
             // each pair of tiles once (T (T + 1) / 2 per shift), the CUDA-core tiles T^2
-            I.items = wht ? I.S : tc ? I.S * I.F * (I.T * (I.T + 1) / 2) * I.ks : I.S * I.F * I.T * I.T * I.ks;
+            I.items = wht ? I.S * I.ks : tc ? I.S * I.F * (I.T * (I.T + 1) / 2) * I.ks : I.S * I.F * I.T * I.T * I.ks;
             I.item_base = base;
             base += I.items;
             table[oi] = I;
