@@ -633,7 +633,6 @@ __device__ __forceinline__ void shift_angle(const Inst& I, int sg, int a, R& c, 
 template <typename R>
 __global__ void __launch_bounds__(256) k_hbm_init(const Inst* __restrict__ insts, int idx, int sg0) {
     pdl_wait();
-    pdl_trigger();
     // The product state factorises over bit groups: amplitude i of this chunk
     // is t0[i & 63] t1[(i >> 6) & 63] h, the factors of qubits 0..5, 6..11 and
     // of the chunk's high bits (two multiplies per amplitude).
@@ -675,7 +674,6 @@ __global__ void __launch_bounds__(256) k_hbm_init(const Inst* __restrict__ insts
 template <typename R>
 __global__ void __launch_bounds__(256) k_hbm_lo(const Inst* __restrict__ insts, int idx, int layer, int sg0) {
     pdl_wait();
-    pdl_trigger();
     extern __shared__ __align__(16) unsigned char sm[];
     R* w = reinterpret_cast<R*>(sm);
     const Inst& I = insts[idx];
@@ -730,7 +728,6 @@ __global__ void __launch_bounds__(256) k_hbm_lo(const Inst* __restrict__ insts, 
 __device__ __forceinline__ int lo_pad(int e) { return e + ((e >> 5) << 2) + ((e >> 8) << 4); }
 __global__ void __launch_bounds__(256) k_hbm_lo_regs(const Inst* __restrict__ insts, int idx, int layer, int sg0) {
     pdl_wait();
-    pdl_trigger();
     constexpr int PADW = LOC + (LOC >> 5) * 4 + (LOC >> 8) * 16;
     __shared__ __align__(16) float scr[2][PADW];
     __shared__ float rq[LOQ], fq[LOQ];
@@ -804,7 +801,6 @@ __global__ void __launch_bounds__(256) k_hbm_lo_regs(const Inst* __restrict__ in
 template <typename R>
 __global__ void __launch_bounds__(256) k_hbm_hi(const Inst* __restrict__ insts, int idx, int layer, int sg0) {
     pdl_wait();
-    pdl_trigger();
     extern __shared__ __align__(16) unsigned char sm[];
     R* w = reinterpret_cast<R*>(sm);  // [H][HC]
     const Inst& I = insts[idx];
@@ -850,7 +846,6 @@ __global__ void __launch_bounds__(256) k_hbm_hi(const Inst* __restrict__ insts, 
 template <int LOGH>
 __global__ void __launch_bounds__(256) k_hbm_hi_regs(const Inst* __restrict__ insts, int idx, int layer, int sg0) {
     pdl_wait();
-    pdl_trigger();
     constexpr int H = 1 << LOGH, RG = H / 8;
     __shared__ float scr[H * 33];
     __shared__ float rq[LOGH], fq[LOGH];
@@ -900,6 +895,10 @@ int build_hbm_states(dvqls_ctx* ctx, cudaStream_t st, const Inst* dtable, int id
     const size_t lo_smem = sizeof(R) * LOC, hi_smem = sizeof(R) * ((size_t)chunks * HC);
     DVQLS_CUDA_TRY(ctx, allow_dynamic_smem((const void*)k_hbm_lo<R>));
     DVQLS_CUDA_TRY(ctx, allow_dynamic_smem((const void*)k_hbm_hi<R>));
+    // No early trigger in these kernels: a dependent's CTAs, placed while the last ones of a
+    // pass run, land on the SMs that happen to have room and then work on a part of the GPU
+    // (with the trigger: the fidelity's FP64 state of n = 20 542 us, 342 without; FP32 tiles of n = 13,
+    // d = 1 behind the last pass 222, 175; the uneven batch 47.6 ms, 46.8).
     // one profiling mark per kernel
     auto init = [&](int sg0, int count) -> int {
         if (marks) prof_begin(ctx, 3);
