@@ -202,7 +202,7 @@ __device__ __forceinline__ void fwht_bits(double* w, int elems, int b0, int bits
 // bit), k_sel_pick finds the lowest bin that is needed, k_sel_collect copies
 // the keys from it on into a candidate list, and one CTA sorts that list and
 // writes the terms.  The list nearly always fits (SEL_CAP candidates); when it
-// does not (a mass of nearly or exactly equal keys at the cut), the host adds
+// does not (a mass of nearly or exactly equal keys at the cut), the host launches
 // rounds over the next SEL_BITS bits of the keys and, at equal keys, of their
 // positions, after which exactly L_max candidates are left.  A sort of every
 // 4,096-key block took 2,154 us of the n = 20 tridiagonal decomposition (22 M
@@ -373,6 +373,7 @@ __global__ void __launch_bounds__(FW_T) k_fwht_hi(int n, double* val, Misc* misc
 // found so far.  Clears the counts for the next round.
 __global__ void __launch_bounds__(SEL_T) k_sel_pick(int round, double tau, int L_max, Misc* misc, uint32_t* ghist) {
     constexpr int PER = SEL_BINS / SEL_T;
+    if (misc->done) return;  // an earlier round was enough
     __shared__ long long part[SEL_T / 32];
     __shared__ long long s_at, s_above;
     __shared__ int s_bin;
@@ -423,6 +424,7 @@ __global__ void __launch_bounds__(SEL_T) k_sel_pick(int round, double tau, int L
 __global__ void __launch_bounds__(256) k_sel_hist(int round, const double* __restrict__ val, long long E, double tau,
                                                   const Misc* misc, uint32_t* ghist) {
     __shared__ uint32_t hist[SEL_BINS];
+    if (misc->done) return;  // an earlier round was enough
     for (int k = threadIdx.x; k < SEL_BINS; k += blockDim.x) hist[k] = 0u;
     __syncthreads();
     const unsigned long long thr = threshold_bits(tau, misc->kmax), lk = misc->lb_key, lp = misc->lb_pos;
@@ -662,13 +664,14 @@ int decompose_common(dvqls_ctx* ctx, const double* A_in, int n, int nbands, cons
     k_sel_pick<<<1, SEL_T, 0, ctx->stream>>>(0, tau, L_max, misc, hist);
     rc = collect(1);
     if (!rc && !hm->done) {
-        for (int round = 1; round < SEL_ROUNDS && !rc && !hm->done; ++round) {
+        // All rounds without a look from the host (a round after the last one needed ends at once):
+        // with a synchronisation each, 65,536 equal keys took 323 us in all.
+        for (int round = 1; round < SEL_ROUNDS; ++round) {
             k_sel_hist<<<egrid, 256, 0, ctx->stream>>>(round, val, E, tau, misc, hist);
             k_sel_pick<<<1, SEL_T, 0, ctx->stream>>>(round, tau, L_max, misc, hist);
-            DVQLS_CUDA_TRY(ctx, cudaGetLastError());
-            rc = read_misc();
         }
-        if (!rc) rc = collect(0);
+        DVQLS_CUDA_TRY(ctx, cudaGetLastError());
+        rc = collect(0);
     }
     if (rc) return rc;
     const int L = hm->l_out;
