@@ -12,6 +12,7 @@
 // order, so gradients are deterministic.  Parameters are one flat FP32 vector:
 // W1 [H x I], b1 [H], W2 [H x H], b2 [H], W3 [O x H], b3 [O] (row-major).
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 
 #include "internal.cuh"
@@ -126,7 +127,7 @@ __device__ __forceinline__ float gelu_grad(float x) {
 enum Epilogue {
     EPI_GELU,  // C = GELU(Z), Z = product + bias
     EPI_BIAS,  // C = product + bias
-    EPI_LOSS,  // C = mask (product + bias - target), and the CTA's parts of the loss
+    EPI_LOSS,  // C = scale mask (product + bias - target), and the CTA's parts of the loss
     EPI_BACK,  // C = product GELU'(Z)
 };
 
@@ -137,7 +138,7 @@ template <int EPI, bool BK, int R = 4>
 __global__ void __launch_bounds__(GTH) k_gemm(int M, int N, int K, const float* __restrict__ A, const float* __restrict__ B,
                                               int ldb, const float* __restrict__ bias, float* Z, float* C,
                                               const float* __restrict__ target, const float* __restrict__ mask,
-                                              float* part) {
+                                              float* part, float scale) {
     pdl_wait();
     __shared__ GemmSmem sm;
     const int m0 = blockIdx.y * (16 * R), n0 = blockIdx.x * GT, tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -166,7 +167,7 @@ __global__ void __launch_bounds__(GTH) k_gemm(int M, int N, int K, const float* 
                 const float mk = mask[at], e = v - target[at];
                 s1 += mk * e * e;
                 s2 += mk;
-                v = mk * e;
+                v = mk * e * scale;
             }
             C[at] = v;
         }
@@ -192,7 +193,7 @@ __global__ void __launch_bounds__(GTH) k_gemm(int M, int N, int K, const float* 
 }
 
 // The gradients of the three weight matrices and biases, before the factor
-// 2 / sum M: job q is gW[m, n] = sum_b D[b, m] Hq[b, n] (rows of D: the layer's
+// 2 / (scale sum M): job q is gW[m, n] = sum_b D[b, m] Hq[b, n] (rows of D: the layer's
 // derivative; rows of Hq: its input) and gb[m] = sum_b D[b, m].  Grid: (tiles of
 // all three jobs, splits of the batch); split s writes its sums to part[s np ..].
 struct GradJob {
@@ -234,7 +235,7 @@ struct AdamArgs {
 // leaves the loss sums in lossbuf.
 __global__ void __launch_bounds__(256) k_grad_update(long long np, int splits, const float* __restrict__ part,
                                                      int nloss, const float* __restrict__ lpart, float* lossbuf,
-                                                     float* grad, float* p, float* m, float* v, AdamArgs a) {
+                                                     float* grad, float* p, float* m, float* v, AdamArgs a, float unscale) {
     pdl_wait();
     __shared__ float red[2];
     if (threadIdx.x < 32) {  // the same sums in the same order in every CTA
@@ -264,7 +265,7 @@ __global__ void __launch_bounds__(256) k_grad_update(long long np, int splits, c
     }
     __syncthreads();
     if (i >= np) return;
-    g *= red[1] > 0.f ? 2.f / red[1] : 0.f;
+    g *= red[1] > 0.f ? 2.f * unscale / red[1] : 0.f;
     if (grad) {
         grad[i] = g;
         return;
@@ -375,6 +376,10 @@ Params params_of(const dvqls_ws* w) {
 
 dim3 gemm_grid(int M, int N) { return dim3(ceil_div(N, GT), ceil_div(M, GT)); }
 
+// The power of two that takes the place of 1 / sum M in back-propagation, where sum M is not known
+// yet: a derivative summed over the batch stays in the range of its mean.
+float loss_scale(const dvqls_ws* w, int B) { return ldexpf(1.f, -int(std::ceil(std::log2(double(B) * w->O)))); }
+
 // Hidden layers, then y (loss = false) or the loss parts and dy = M (y - t).
 int forward(dvqls_ws* w, const Views& a, int B, bool loss) {
     dvqls_ctx* ctx = w->ctx;
@@ -387,15 +392,15 @@ int forward(dvqls_ws* w, const Views& a, int B, bool loss) {
     auto layer = [&](auto tall, auto flat, int N, int K, const float* in, const float* W, const float* b, float* z, float* out) {
         if (low(N))
             return launch(ctx, flat, dim3(ceil_div(N, GT), ceil_div(B, 16)), B, N, K, in, W, K, b, z, out, nullptr, nullptr,
-                          nullptr);
-        return launch(ctx, tall, gemm_grid(B, N), B, N, K, in, W, K, b, z, out, nullptr, nullptr, nullptr);
+                          nullptr, 1.f);
+        return launch(ctx, tall, gemm_grid(B, N), B, N, K, in, W, K, b, z, out, nullptr, nullptr, nullptr, 1.f);
     };
     int rc = layer(k_gemm<EPI_GELU, true>, k_gemm<EPI_GELU, true, 1>, H, I, a.X, p.W1, p.b1, a.z1, a.h1);
     if (!rc) rc = layer(k_gemm<EPI_GELU, true>, k_gemm<EPI_GELU, true, 1>, H, H, a.h1, p.W2, p.b2, a.z2, a.h2);
     if (rc) return rc;
     if (loss)
         return launch(ctx, k_gemm<EPI_LOSS, true>, gemm_grid(B, O), B, O, H, a.h2, p.W3, H, p.b3, nullptr, a.dy, a.T, a.M,
-                      a.lpart);
+                      a.lpart, loss_scale(w, B));
     return layer(k_gemm<EPI_BIAS, true>, k_gemm<EPI_BIAS, true, 1>, O, H, a.h2, p.W3, p.b3, nullptr, a.y);
 }
 
@@ -407,10 +412,10 @@ int backward(dvqls_ws* w, const Views& a, int B, const AdamArgs* adam) {
     const Params p = params_of(w);
     // d2[b, h] = sum_o dy[b, o] W3[o, h] GELU'(z2), d1[b, k] = sum_h d2[b, h] W2[h, k] GELU'(z1)
     int rc = launch(ctx, k_gemm<EPI_BACK, false>, gemm_grid(B, H), B, H, O, a.dy, p.W3, H, nullptr, a.z2, a.d2, nullptr,
-                    nullptr, nullptr);
+                    nullptr, nullptr, 1.f);
     if (!rc)
         rc = launch(ctx, k_gemm<EPI_BACK, false>, gemm_grid(B, H), B, H, H, a.d2, p.W2, H, nullptr, a.z1, a.d1, nullptr,
-                    nullptr, nullptr);
+                    nullptr, nullptr, 1.f);
     if (rc) return rc;
     GradJobs jobs;
     int tiles = 0;
@@ -428,7 +433,7 @@ int backward(dvqls_ws* w, const Views& a, int B, const AdamArgs* adam) {
     if (rc) return rc;
     const dim3 lg = gemm_grid(B, O);
     return launch(ctx, k_grad_update, dim3(ceil_div(w->np, 256)), w->np, ceil_div(B, per), a.gpart, int(lg.x * lg.y), a.lpart,
-                  w->lossbuf, adam ? nullptr : w->grad, w->params, w->m, w->v, adam ? *adam : AdamArgs{});
+                  w->lossbuf, adam ? nullptr : w->grad, w->params, w->m, w->v, adam ? *adam : AdamArgs{}, 1.f / loss_scale(w, B));
 }
 
 int copy_in(dvqls_ws* w, float* dst, const float* src, long long n) {
