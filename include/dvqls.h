@@ -511,7 +511,7 @@ int dvqls_ws_load(dvqls_ctx* ctx, const char* path, dvqls_ws** out);
  * process exits.  A request whose scratch exceeds it is rejected with
  * INVALID_ARG.  The scratch it needs is, in bytes (each term rounded up to
  * 256): sizeof record + 256 + 16 L + 16 L^2 + 48 P + 8 + 16 S T^2 k
- * + 16 S T k + 24 S, with S = 2P+1, T = ceil(L/64) and k <= 8 the split of
+ * + 16 S T k, with S = 2P+1, T = ceil(L/64) and k <= 8 the split of
  * the amplitude range, plus 16 L^2 + 16 L in DVQLS_FP32 (the weights as
  * float pairs).  With the largest split (k = 8), n = 10, depth 4 (P = 50)
  * fits up to L = 160 in FP32 and L = 200 in FP64 on any GPU.

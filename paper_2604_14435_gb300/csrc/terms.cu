@@ -67,7 +67,6 @@ struct Inst {
     double2* Tpart;  // S*T*ks
     void* Gpart;     // ks*L*L (shift 0 only; null when beta is not requested)
     void* dpart;     // ks*L   (shift 0 only; null when delta is not requested)
-    double* NsDs;    // 3S: N_s, Re D_s, Im D_s
     void* states;    // n > 12: the S shifted states in HBM (S x N), else null
     void* chain;     // n > 12: the unshifted state after every pass (2d + 1 states), or null when S = 1
     void* tcst;      // tensor-core pass, n <= 12: the S shifted states as packed FP16 pairs (S x N words), else null
@@ -110,38 +109,16 @@ __device__ __forceinline__ double2 ctil_of(const Inst& I, int l) {
     }
 }
 
-// Per-instance tables of a pass (Sec. 2.3 Stage I inputs).  Grid (instances,
-// parts): part 0 checks the inputs, forms ||b||^2 and c~; every part takes its
-// share of the shift angle tables and of the L^2 weights w_lm = conj(c~_l) c~_m.
 // Programmatic dependent launch: the kernels of a pass after the first are
 // launched so that their CTAs may start while the previous kernel finishes;
 // each waits for the previous grid's completion (and its memory) before its
 // first dependent access, and lets the next kernel start once all its CTAs
-// are running.  Launched without the attribute, both are no-ops.
+// are running (the passes over states in HBM do not, see build_hbm_states).
+// Launched without the attribute, both are no-ops.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-
 // ------------------------------------------------------------ term tiles
-template <typename R>
-__device__ __forceinline__ void load4(const typename V2<R>::t* p, typename V2<R>::t (&v)[4]);
-template <>
-__device__ __forceinline__ void load4<float>(const float2* p, float2 (&v)[4]) {
-    const float4 a = reinterpret_cast<const float4*>(p)[0];
-    const float4 b = reinterpret_cast<const float4*>(p)[1];
-    v[0] = make_float2(a.x, a.y);
-    v[1] = make_float2(a.z, a.w);
-    v[2] = make_float2(b.x, b.y);
-    v[3] = make_float2(b.z, b.w);
-}
-template <>
-__device__ __forceinline__ void load4<double>(const double2* p, double2 (&v)[4]) {
-    v[0] = p[0];
-    v[1] = p[1];
-    v[2] = p[2];
-    v[3] = p[3];
-}
-
 __device__ __forceinline__ double2 block_sum2(double2 v, double2* red) {
     for (int o = 16; o; o >>= 1) {
         v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
@@ -153,30 +130,6 @@ __device__ __forceinline__ double2 block_sum2(double2 v, double2* red) {
     double2 s = make_double2(0.0, 0.0);
     if (threadIdx.x == 0)
         for (int k = 0; k < NT / 32; ++k) {
-            s.x += red[k].x;
-            s.y += red[k].y;
-        }
-    return s;  // valid in thread 0
-}
-
-// One work item (see the file comment).  Item u of a shift: u < T is the
-// diagonal tile (u, u); u >= T is half h of the off-diagonal tile pair
-// (tl < tm) number (u - T) / 2.  Only blocks with l <= m are computed:
-// beta_ml = conj(beta_lm) exactly, so the pair contributes 2 Re(w_lm G~_lm) to
-// D_s and nothing to its imaginary part.  Threads: two K-groups of KSLOT task
-// slots; each active slot owns one 4 x 4 block of complex products and
-// accumulates it over its K-group's half of every chunk, in registers.
-__device__ __forceinline__ double2 block_sum2_n(double2 v, double2* red, int nthreads) {
-    for (int o = 16; o; o >>= 1) {
-        v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
-        v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
-    }
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    double2 s = make_double2(0.0, 0.0);
-    if (threadIdx.x == 0)
-        for (int k = 0; k < nthreads / 32; ++k) {
             s.x += red[k].x;
             s.y += red[k].y;
         }
@@ -252,6 +205,13 @@ __device__ __forceinline__ void store4r<double>(double* p, const double (&v)[4])
 // every phi_l[j] = (-1)^popc(z_l & (j ^ x_l)) psi[j ^ x_l] is real and the
 // Gram G~ is real symmetric: one FMA per product, and delta_l = sum_j
 // conj(b_j) phi_l[j] takes Re b and Im b separately.
+// One work item (see the file comment).  Item u of a shift: u < T is the
+// diagonal tile (u, u); u >= T is half h of the off-diagonal tile pair
+// (tl < tm) number (u - T) / 2.  Only blocks with l <= m are computed:
+// beta_ml = conj(beta_lm) exactly, so the pair contributes 2 Re(w_lm G~_lm) to
+// D_s and nothing to its imaginary part.  Threads: two K-groups of KSLOT task
+// slots; each active slot owns one 4 x 4 block of complex products and
+// accumulates it over its K-group's half of every chunk, in registers.
 template <typename R>
 __device__ void process_item(const Inst& I, int local, unsigned char* smem, uint32_t* smask, double2* red) {
     using R2 = typename V2<R>::t;
@@ -1219,6 +1179,8 @@ __global__ void __launch_bounds__(256) k_bnorm(const Inst* __restrict__ insts) {
     }
 }
 
+// Per-instance tables of a pass (Sec. 2.3 Stage I inputs): the input checks, ||b||^2, c~, the
+// shift angle tables and the L^2 weights w_lm = conj(c~_l) c~_m.
 // Per instance: CTAs 0 .. prep_parts - 1 form ||b||^2 and c~ (part 0), the
 // half-angle tables (part 1, or 0 when alone) and the pair weights (all
 // parts); CTAs from prep_parts on, when launched, build the tensor-core b rows
@@ -1790,7 +1752,6 @@ __global__ void __launch_bounds__(TCT, 1) k_terms_tc(const Inst* __restrict__ in
             const uint32_t xl = xs[side * 64 + l], zl = zs[side * 64 + l];
             const float* psi_g = it.psi_g;
             const uint4* bop = it.bop;
-            const int sst = 2 * Na + 16;  // bytes of one split array
             unsigned char* pb = reinterpret_cast<unsigned char*>(psi_hl);
             // Group tt of 8 amplitudes (Na / 8 <= 256 groups of a staged state or an HBM block): its packed
             // words p_i = hi_i | (2 lo)_i << 16.
@@ -1842,6 +1803,7 @@ __global__ void __launch_bounds__(TCT, 1) k_terms_tc(const Inst* __restrict__ in
                     }
                 }
                 if (split) {
+                    const int sst = 2 * Na + 16;  // bytes of one split array
                     // hi and lo copies t = 0..7, whose words j hold elements (2j) ^ t, (2j + 1) ^ t of the
                     // group: word j ^ (t >> 1) of the pairs in order (t even) or swapped (t odd)
                     uint32_t HP[4], HS[4], LP[4], LS[4];
@@ -1872,15 +1834,6 @@ __global__ void __launch_bounds__(TCT, 1) k_terms_tc(const Inst* __restrict__ in
                     }
                 }
             }
-            bar_n(bar, TC_HT);
-            if (copies && !regs && !blk) {  // copy t: psi[k ^ t] at word t (N + 8) + k
-                for (int k = tt; k < N; k += TC_HT) {
-                    const uint32_t v = psi_hl[k];
-#pragma unroll
-                    for (int t3 = 1; t3 < 4; ++t3) psi_hl[t3 * (N + 8) + (k ^ t3)] = v;
-                }
-                bar_n(bar, TC_HT);
-            }
             uint32_t sgn[8];  // word g: sign bits of elements 2g (bit 15) and 2g + 1 (bit 31) of a 16-block
             {
                 const uint32_t xlo = xl & 15u & uint32_t(N - 1);
@@ -1889,6 +1842,7 @@ __global__ void __launch_bounds__(TCT, 1) k_terms_tc(const Inst* __restrict__ in
                     sgn[g] = ((__popc(zl & 15u & (uint32_t(2 * g) ^ xlo)) & 1) ? 0x8000u : 0u) |
                              ((__popc(zl & 15u & (uint32_t(2 * g + 1) ^ xlo)) & 1) ? 0x80000000u : 0u);
             }
+            bar_n(bar, TC_HT);
             for (int c = 0; c < nch; ++c, ++gc) {
                 const int q = int(gc & 1u), st = 2 * h + q;
                 if ((pend >> q) & 1u) {  // the MMAs that read this buffer last time must be done
@@ -3832,7 +3786,7 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
     struct Off {
         size_t coef, xm, zm, alpha, b;       // staged inputs (ws) ...
         size_t pcoef, pxm, pzm, palpha, pb;  // ... and their pinned slots
-        size_t ctil, w, wf, cf, bop, wht, bf, cs, bn2, bpart, Dp, Tp, Gp, dp, NsDs, cost, grad, beta, delta, states, chain, tcst;
+        size_t ctil, w, wf, cf, bop, wht, bf, cs, bn2, bpart, Dp, Tp, Gp, dp, cost, grad, beta, delta, states, chain, tcst;
         size_t pcost, pgrad, pbeta, pdelta;
     };
     std::vector<Off> off(count);
@@ -3897,7 +3851,6 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
         o.Tp = ar.reserve(size_t(h.S) * h.T * kp * 16);
         o.Gp = beta_out ? ar.reserve(size_t(wht ? 1 : kp) * L * L * r2) : 0;
         o.dp = delta_out ? ar.reserve(size_t(wht ? 1 : kp) * L * r2) : 0;
-        o.NsDs = ar.reserve(size_t(h.S) * 24);
         o.states = h.hbm ? ar.reserve(size_t(h.S) * size_t(h.N) * (r2 / 2)) : 0;  // real amplitudes
         o.chain = h.hbm && h.S + h.s0 > 1 ? ar.reserve((2 * size_t(h.d) + 1) * size_t(h.N) * (r2 / 2)) : 0;
         o.tcst = tc && !h.hbm ? ar.reserve(size_t(h.S) * size_t(h.N) * 4) : 0;     // packed FP16 pairs
@@ -3971,7 +3924,6 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
         I.Tpart = (double2*)(ws + o.Tp);
         I.Gpart = beta_out ? (void*)(ws + o.Gp) : nullptr;
         I.dpart = delta_out ? (void*)(ws + o.dp) : nullptr;
-        I.NsDs = (double*)(ws + o.NsDs);
         I.states = h.hbm ? (void*)(ws + o.states) : nullptr;
         I.chain = h.hbm && h.S + h.s0 > 1 ? (void*)(ws + o.chain) : nullptr;
         I.tcst = tc && !h.hbm ? (void*)(ws + o.tcst) : nullptr;
@@ -4382,8 +4334,8 @@ extern "C" int dvqls_combine_partials(dvqls_ctx* ctx, int n, int depth, const do
 }
 
 // ------------------------------------------------- allocation-free variant
-// dvqls_cost_grad_noalloc runs the same three kernels as dvqls_cost_grad for
-// one instance, but takes its scratch (instance record, weights, per-item
+// dvqls_cost_grad_noalloc runs the prepare, tile and combine kernels for one instance
+// (in FP64 also where dvqls_cost_grad takes the Walsh-Hadamard classes), but takes its scratch (instance record, weights, per-item
 // partial sums, queue counter, status word) from the file-scope device array
 // below instead of a context workspace, so it needs no cudaMalloc, no pinned
 // staging and no context.  Every GPU that loads the library holds the array
@@ -4482,7 +4434,6 @@ extern "C" int dvqls_cost_grad_noalloc(void* stream_arg, const dvqls_ansatz* ans
     const size_t o_bn2 = ar.reserve(8);
     const size_t o_Dp = ar.reserve(size_t(S) * T * T * ks * 16);
     const size_t o_Tp = ar.reserve(size_t(S) * T * ks * 16);
-    const size_t o_NsDs = ar.reserve(size_t(S) * 24);
     if (ar.total() > NOALLOC_BYTES) return DVQLS_ERR_INVALID_ARG;  // beyond the fixed scratch
     char* base = nullptr;
     int rc = noalloc_scratch_address(&base);
@@ -4513,7 +4464,6 @@ extern "C" int dvqls_cost_grad_noalloc(void* stream_arg, const dvqls_ansatz* ans
     I.bn2 = (double*)(base + o_bn2);
     I.Dpart = (double2*)(base + o_Dp);
     I.Tpart = (double2*)(base + o_Tp);
-    I.NsDs = (double*)(base + o_NsDs);
     I.cost = cost;
     I.grad = grad;
     Inst* table = (Inst*)(base + o_table);
