@@ -56,9 +56,14 @@ int ensure_workspace(dvqls_ctx* ctx, size_t bytes, size_t table_bytes) {
     ctx->ws = nullptr;
     ctx->ws_cap = 0;
     size_t cap = bytes + bytes / 4 + (1 << 20);
-    if (cudaMalloc(&ctx->ws, cap) != cudaSuccess) {
+    if (cudaMalloc(&ctx->ws, cap) != cudaSuccess) {  // no room to spare: what the call needs
         cudaGetLastError();
-        return set_error(ctx, DVQLS_ERR_ALLOC, "device workspace of %zu bytes", cap);
+        cap = bytes;
+        if (cudaMalloc(&ctx->ws, cap) != cudaSuccess) {
+            cudaGetLastError();
+            ctx->ws = nullptr;
+            return set_error(ctx, DVQLS_ERR_ALLOC, "device workspace of %zu bytes", cap);
+        }
     }
     ctx->ws_cap = cap;
     return DVQLS_OK;
