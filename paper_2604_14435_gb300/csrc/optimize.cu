@@ -237,7 +237,10 @@ __global__ void __launch_bounds__(CGT) k_cg(int n, int L, const double2* coef, c
 // costs one multiply-add per amplitude and distinct mask instead of one per
 // term (7 against 64 for the top terms of a tridiagonal matrix), and only its
 // real half when every diagonal and the right-hand side are real.  FP64 bounds
-// these solves: its instructions issue at 1/64 of the FP32 rate.
+// these solves: its instructions issue at 1/64 of the FP32 rate.  At n = 12 the 16
+// amplitudes of a thread spill (424 bytes), which the diagonals still outweigh: 64 right-hand
+// sides with 33 terms on 9 masks 4,159 us term by term, 620 here; with 61 terms on 61 masks,
+// complex, 6,451 and 2,794.
 constexpr int GRP_MAXL = 2048;  // terms the grouping kernel takes
 constexpr int GRP_MAXX = 64;    // distinct masks the solver takes; more: term by term
 constexpr int CGR_T = 256;

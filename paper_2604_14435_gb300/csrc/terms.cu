@@ -2928,9 +2928,10 @@ inline size_t wht_smem_bytes(int Pmax) {
 // The FP64 tiles spend one DFMA per term and amplitude on a pipe that issues 2
 // per clock and SM (n = 10, L = 64: 2.2 M DFMAs, 1.1 M cycles per state).  Here
 // the state (build_state_fx) and the transforms run in 64-bit fixed point on the
-// integer pipes: sum_i |psi[i] psi[i ^ x]| <= 1 = 2^62, and |b[i ^ x] psi[i]| sums up to 3/2 at
-// most (w64_bexp), so every partial sum of a transform stays within 64 bits and the adds
-// are exact; a product is rounded once, at 2^-62.  The FP64 pipe keeps one FMA per term for the weighted sums.
+// integer pipes: sum_i |psi[i] psi[i ^ x]| <= 1 = 2^62, and |b[i ^ x] psi[i]| sums up to
+// 3/2 at most (w64_bexp), so every partial sum of a transform stays within 64 bits and
+// the adds are exact; a product is rounded once, at 2^-62.  The FP64 pipe keeps one FMA
+// per term for the weighted sums.
 // One CTA of 8 warps per item, two CTAs per SM (the transform of 2^10 values
 // holds 64 registers a lane), so one CTA's state build overlaps the other's
 // transforms.
@@ -2942,10 +2943,11 @@ inline size_t wht_smem_bytes(int Pmax) {
 // bound on that sum (from the exponents of its products, within a factor of 8): an
 // overlap is then as accurate as an FP64 sum of its terms, however small they are.
 // n = 10, L = 64, 101 shifts of one system: 623 us by the tiles, 36 us by the
-// classes; 48 systems of n = 6..10 at random angles: 8,646 us against 336 (317 without the
-// magnitudes, 444 with the FP64 state and units for every item).  A state of n = 10 takes
-// 20 k cycles of a CTA, its 29 transforms and 2,080 lookups 31 k; both are bound by the
-// integer multiply-adds and adds.
+// classes; 48 systems of n = 6..10 at random angles: 8,646 us against 345 (317 with products
+// at 2^-60 and without the magnitudes, 444 with the FP64 state and units for every
+// item; at angles below 1e-3, where every item starts over, 32 systems of n = 10 15.6 ms
+// against 1.4).  A state of n = 10 takes 20 k cycles of a CTA, its 29 transforms and
+// 2,080 lookups 31 k; both are bound by the integer multiply-adds and adds.
 constexpr int W64_ROW = (1 << WHT_MAXN) + (1 << WHT_MAXN) / 32;
 
 // Factor of an instance's results, from its class table: NaN when one of the bits
