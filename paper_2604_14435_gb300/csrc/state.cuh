@@ -625,6 +625,20 @@ __device__ __forceinline__ void ry64_regs(double (&v)[A], const long long* ang) 
     }
 }
 
+// The first layer on |0>, a product state: the factors of the qubits below nt, by the bits of i,
+// then those of the register bits.
+template <int A, int LOGA>
+__device__ __forceinline__ void ry64_product(double (&v)[A], int i, int nt, const double2* c0) {
+    v[0] = 1.0;
+    for (int q = 0; q < nt; ++q) v[0] *= ((i >> q) & 1) ? c0[q].y : c0[q].x;
+#pragma unroll
+    for (int kb = 0; kb < LOGA; ++kb)
+#pragma unroll
+        for (int r = 0; r < (1 << kb); ++r) {
+            v[r | (1 << kb)] = v[r] * c0[nt + kb].y;
+            v[r] *= c0[nt + kb].x;
+        }
+}
 // Shared memory of build_state_f64, in bytes: the ratios and the groups' factors, two
 // buffers of 2^n amplitudes.
 __host__ __device__ inline size_t f64_angle_bytes(int n, int P) {
@@ -643,12 +657,7 @@ __device__ void f64_multiwarp(double* out, double* scr, const long long* ang, co
     const int lane = t & 31, w = t >> 5, N = 1 << n, G = ry64_group(n);
     auto index = [&](int M, int r) { return M == 0 ? (r << 8) | (w << 5) | lane : (r << 8) | (lane << 3) | w; };
     double v[A];
-#pragma unroll
-    for (int r = 0; r < A; ++r) {
-        const int i = index(0, r);
-        v[r] = 1.0;
-        for (int q = 0; q < n; ++q) v[r] *= ((i >> q) & 1) ? c0[q].y : c0[q].x;
-    }
+    ry64_product<A, LOGA>(v, (w << 5) | lane, 8, c0);
     int M = 0, g = 0;
     for (int layer = 1; layer <= d; ++layer) {
         const long long* la = ang + layer * n;
@@ -680,12 +689,7 @@ template <int A, int LOGA>
 __device__ void f64_warp(double* out, const long long* ang, const double* fac, const double2* c0, int n, int d, int lane) {
     const int N = 1 << n, li = N < 32 ? lane & (N - 1) : lane, nl = n < 5 ? n : 5, G = ry64_group(n);
     double v[A];
-#pragma unroll
-    for (int r = 0; r < A; ++r) {
-        const int i = (r << 5) | li;
-        v[r] = 1.0;
-        for (int q = 0; q < n; ++q) v[r] *= ((i >> q) & 1) ? c0[q].y : c0[q].x;
-    }
+    ry64_product<A, LOGA>(v, li, nl, c0);
     int g = 0;
     for (int layer = 1; layer <= d; ++layer) {
         const long long* la = ang + layer * n;
