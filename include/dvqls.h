@@ -79,8 +79,8 @@ typedef enum {
  *                  classes (as DVQLS_FP32_WHT below) with transforms in
  *                  64-bit fixed point, in less time and no less accurate
  *                  than the FP64 tiles (against extended precision, systems
- *                  of n = 3..10: gradients 1.4e-15 to 3e-15 off in the mean,
- *                  the tiles' 2.5e-15 to 4e-15).  A state spread over its
+ *                  of n = 3..10: gradients 1.3e-15 to 1.2e-14 off in the mean,
+ *                  the tiles' 2.2e-15 to 2.1e-14).  A state spread over its
  *                  amplitudes is in fixed point too; where the products of
  *                  one class are small (angles near zero, a right-hand side
  *                  of few entries) the evaluation takes an FP64 state and
