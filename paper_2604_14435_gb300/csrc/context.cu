@@ -46,8 +46,18 @@ cudaError_t allow_dynamic_smem(const void* fn) {
     return e;
 }
 
+bool is_capturing(dvqls_ctx* ctx) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(ctx->stream, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return cap != cudaStreamCaptureStatusNone;
+}
+
 int ensure_workspace(dvqls_ctx* ctx, size_t bytes, size_t table_bytes) {
-    if (ctx->last_table.size() != table_bytes) ctx->last_table.clear();
+    ctx->ws_in_graph = ctx->ws_in_graph || is_capturing(ctx);
+    if (ctx->ws_in_graph || ctx->last_table.size() != table_bytes) ctx->last_table.clear();
     if (bytes <= ctx->ws_cap) return DVQLS_OK;
     DVQLS_CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
     ctx->last_table.clear();

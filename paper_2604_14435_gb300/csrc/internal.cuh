@@ -79,6 +79,9 @@ struct dvqls_ctx {
     // uploaded it (an equal one is not uploaded again); empty when another call
     // has planned the workspace since.
     std::vector<char> last_table;
+    // A graph of the caller's writes the workspace: the caller captured a call of this
+    // context, and may launch the graph between any two others (no table is kept then).
+    bool ws_in_graph = false;
 
     // Kernel timing (dvqls_profile_*): event pairs not yet read, a pool of
     // reusable events, and per-phase totals.
@@ -160,8 +163,10 @@ class Arena {
 // the instance table that the batched cost pass left at its start (last_table)
 // counts as overwritten from then on.  Only run_batch, which puts its own table
 // of table_bytes there and everything else behind it, keeps a table of that size,
-// unless the workspace moves.
+// unless the workspace moves or the caller has captured a call of the context.
 int ensure_workspace(dvqls_ctx* ctx, size_t bytes, size_t table_bytes = 0);
+// Whether the caller is capturing the context's stream (or its state cannot be read).
+bool is_capturing(dvqls_ctx* ctx);
 // Wait until no copy out of the pinned staging is pending, so it can be
 // written again; pin_release records the end of the copies just enqueued.
 int pin_acquire(dvqls_ctx* ctx);

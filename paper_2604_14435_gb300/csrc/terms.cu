@@ -3595,15 +3595,6 @@ __global__ void __launch_bounds__(224) k_put_table(TableChunk c, int count, uint
     if (int(threadIdx.x) < count) dst[threadIdx.x] = c.w[threadIdx.x];
 }
 
-static bool is_capturing(dvqls_ctx* ctx) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(ctx->stream, &cap) != cudaSuccess) {
-        cudaGetLastError();
-        return true;
-    }
-    return cap != cudaStreamCaptureStatusNone;
-}
-
 // Replays a captured graph of the pass when the launch (table bytes and
 // shape) is the one captured last; otherwise captures it on the context's
 // private capture stream first.  Profiling and callers that are capturing
@@ -3993,8 +3984,7 @@ int run_batch(dvqls_ctx* ctx, int count, const dvqls_instance* inst, int precisi
     };
     auto upload = [&]() -> int {
         const char* tb = reinterpret_cast<const char*>(table.data());
-        if (capturing) {  // the graph brings it with every launch; the next call outside it uploads its own
-            ctx->last_table.clear();
+        if (capturing) {  // the graph brings it with every launch
             for (size_t at = 0; at < tbytes; at += sizeof(TableChunk)) {
                 TableChunk c{};
                 const size_t bytes = std::min(sizeof c, tbytes - at);

@@ -68,3 +68,58 @@ def test_captured_pass(dv, prec, count):
         right(1)
     finally:
         dv.dvqls_destroy(ctx)
+
+
+@pytest.mark.parametrize("prec", [0, 2, 3])
+def test_direct_calls_around_a_launch_of_the_graph(dv, prec):
+    """A launch of the graph leaves its own table in the workspace, and the context is not
+    told: a direct call equal to the one before it brings its table again.  The same
+    sums on the same inputs: equal bits."""
+    n, d, L, count = 6, 1, 12, 2
+    P = n * (d + 1)
+    rng = np.random.default_rng(7)
+    an = dv.make_ansatz(n, d)
+    batches = []
+    for k in range(2):  # the captured batch, and another one of the same shape
+        keep, items = [], []
+        for i in range(count):
+            coef, xs, zs, b = random_problem(rng, n, L)
+            t = [torch.tensor(v, device="cuda") for v in (cvec(coef), xs.view(np.int32), zs.view(np.int32), cvec(b),
+                                                          wl.random_angles(P, 70 + 2 * k + i))]
+            keep.append(t)
+            items.append((an, dv.make_lcu(L, t[0], t[1], t[2]), t[4], t[3]))
+        out = [torch.zeros(m, device="cuda", dtype=torch.float64) for m in (count, count * P)]
+        batches.append((dv.make_instances(items), out, keep))
+    torch.cuda.synchronize()
+    stream = torch.cuda.Stream()
+    ctx = dv.dvqls_create(0, stream.cuda_stream)
+
+    def taken(k):  # the results of batch k, which are cleared
+        torch.cuda.synchronize()
+        dv.dvqls_sync(ctx)
+        r = [o.cpu().numpy().copy() for o in batches[k][1]]
+        for o in batches[k][1]:
+            o.zero_()
+        torch.cuda.synchronize()
+        return r
+
+    def direct(k):
+        dv.dvqls_cost_grad_batched(ctx, batches[k][0], prec, *batches[k][1])
+        return taken(k)
+
+    try:
+        dv.dvqls_set_tuning(ctx, 1, 0)
+        first = [direct(k) for k in range(2)]
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream, capture_error_mode="thread_local"):
+            dv.dvqls_cost_grad_batched(ctx, batches[0][0], prec, *batches[0][1])
+        for k in (1, 0, 1):
+            for a, b in zip(first[k], direct(k)):
+                assert np.array_equal(a, b)
+            graph.replay()
+            for a, b in zip(first[0], taken(0)):
+                assert np.array_equal(a, b)
+            for a, b in zip(first[k], direct(k)):
+                assert np.array_equal(a, b)
+    finally:
+        dv.dvqls_destroy(ctx)
