@@ -3111,7 +3111,8 @@ __device__ void w64_item(const Inst& I, int s, const int2* q, const int* qe, lon
     auto at = [&](uint32_t z) { return (double)row[PAD ? z + (z >> 5) : z]; };
 #pragma unroll 1
     for (int j = first; j < jobs; j += step) {
-        if (FIXED && *reinterpret_cast<volatile int*>(sparse)) return;
+        // the same answer for all lanes, which may read at different times
+        if (FIXED && __any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(sparse))) return;
         long long v[A];
         int ex = -62;  // the transform's unit is 2^ex
         if (j >= pairs) {
